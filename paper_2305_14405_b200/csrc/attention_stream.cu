@@ -9,8 +9,8 @@
 // this kernel computes Q K^T TWICE: a first sweep over the keys only for the row maximum, a second
 // sweep for the exponentials.  The tensor pipe is idle most of the time in this ALU-bound kernel, so
 // the second Q K^T is free, and the footprint drops to 128 tensor-memory columns and ~50 KB of
-// shared memory per softmax group (plus Q and the table): three CTAs fit on an SM and one
-// CTA's loads, MMAs and hand-offs overlap the others' arithmetic.  Any L that is a multiple of 128.
+// shared memory (plus Q and the table): three CTAs fit on an SM and one CTA's loads, MMAs and hand-offs
+// overlap the others' arithmetic.
 //
 // CTAs are persistent: one resident wave (three per SM) walks over the (batch, head, 128-query block) tiles.
 // Barriers, tensor memory and the replicated table are set up once per CTA; every mbarrier's phase is a running
@@ -18,27 +18,27 @@
 // and first K chunks, after its last P V the next first V chunk, and the next tile's first product starts as
 // soon as the softmax warps have read the accumulator out of tensor memory.
 //
-// The 16-bit P tile of the one-group form never touches shared memory: the softmax warps write it to 32 further
-// tensor-memory columns (tcgen05.st) and P V takes its A operand from there; the shared-memory pipe, which the
-// table lookups load most, loses the tile's stores and the tensor core's reads of it.
+// The 16-bit P tile never touches shared memory: the softmax warps write it to further tensor-memory columns
+// (tcgen05.st) and P V takes its A operand from there; the shared-memory pipe, which the table lookups load most,
+// loses the tile's stores and the tensor core's reads of it.
 //
-// A group is one control warp and four softmax warps, an independent pipeline that owns 128
-// tensor-memory columns [S_g | O_g], two K stages, a V stage and a P tile.  A CTA has NG = 1 or 2
-// groups (template parameter; only NG = 1 is built, see nm_launch_attention_stream); with two, the groups split
-// the keys: in sweep 1 group g takes the
-// 128-key chunks g, g+NG, ... (scores over all 128 columns, K staged in its two K stages and,
-// alternately, in its P tile); in sweep 2 the 64-key chunks g, g+NG, ... (scores in S_g, accumulator
-// O_g); row maxima and sums are exchanged through shared memory and the accumulators summed in the
-// epilogue.
+// RAGGED form (an L that is not a multiple of 128, otherwise the CUDA-core kernel's): the tensor maps fill rows
+// beyond the sequence with zeros, the scores of keys beyond L are masked in the last chunk only, and warps whose
+// 32 queries all lie beyond L keep the barriers' pace without arithmetic.  The CUDA-core kernel holds its
+// probabilities in fp32, so this form does not round them to 16 bits: e = hi + lo, two 16-bit terms (the error of
+// the pair is at most 2^-18 e in bf16, against the 2^-9 of the result's own rounding), and P V runs once per term.
+// The second term's 32 columns make it two CTAs per SM instead of three.  B 7, L 333, 12 heads: 2368 us on the CUDA
+// cores, 21.3 us here; B 1, L 37: 13.4 and 7.0 us.
 //
-//   warps 0..NG-1     control warp of group g: TMA loads (the group's K chunks through two stages, its V
-//                     chunks through one) and the tcgen05.mma for S_g = Q K_c^T and O_g += P_c V_c (V as
-//                     an MN-major operand).  It sleeps in a named barrier (bar.sync) that the group's
-//                     softmax warps signal with bar.arrive, so hand-offs cost no polling.
-//   warps NG..5NG-1   softmax, one per tensor-memory lane quarter and group: tcgen05.ld, row maximum
-//                     (sweep 1); PWL exp, row sum, bf16 P tile in the swizzled K-major layout (sweep 2);
-//                     PWL reciprocal, scaling, store (optionally as int8 codes for the int8 encoder).
+//   warp 0            control: TMA loads (K chunks through two stages, V chunks through one) and the tcgen05.mma
+//                     for S = Q K_c^T and O += P_c V_c (V as an MN-major operand).  It sleeps in a named barrier
+//                     (bar.sync) that the softmax warps signal with bar.arrive, so hand-offs cost no polling.
+//   warps 1..4        softmax, one per tensor-memory lane quarter: tcgen05.ld, row maximum (sweep 1); PWL exp, row
+//                     sum, P tile (sweep 2); PWL reciprocal, scaling, store (optionally as int8 codes for the int8
+//                     encoder).
 #include <string.h>
+
+#include <type_traits>
 
 #include "nm_common.cuh"
 
@@ -72,6 +72,10 @@ template <> struct AT<__nv_bfloat16> {
         __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
         return *reinterpret_cast<uint32_t*>(&h);
     }
+    static __device__ __forceinline__ float2 unpack(uint32_t w)
+    {
+        return make_float2(__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u));
+    }
 };
 template <> struct AT<__half> {
     static constexpr uint32_t fmt = 0;
@@ -81,6 +85,7 @@ template <> struct AT<__half> {
         __half2 h = __floats2half2_rn(a, b);
         return *reinterpret_cast<uint32_t*>(&h);
     }
+    static __device__ __forceinline__ float2 unpack(uint32_t w) { return __half22float2(*reinterpret_cast<__half2*>(&w)); }
 };
 
 // 16 packed words of this thread's row into 16 consecutive tensor-memory columns (the mirror of the 16-column read)
@@ -131,88 +136,75 @@ __device__ __forceinline__ Tile tile_decode(const TileGeom& gm, int t)
 struct LoadCtx {
     const CUtensorMap *tmQ, *tmK, *tmV;
     uint8_t *q_s, *k_st, *p_s, *v_st;
-    uint64_t *bar_q, *bar_k1_full, *bar_v_full;   // bar_k1_full: [group][2]
+    uint64_t *bar_q, *bar_k1_full, *bar_v_full;   // bar_k1_full: [2]
     int n128;
 };
-// Q and each group's first two 128-key chunks of sweep 1 (stage 0 = the group's two K stages, stage 1 = its P
-// tile).  One thread; the buffers must be free.
-template <int NG>
+// Q and the first two 128-key chunks of sweep 1 (stage 0 = the two K stages, stage 1 = the buffer p_s).  One
+// thread; the buffers must be free.
 __device__ __forceinline__ void load_tile_head(const LoadCtx& c, const Tile& t)
 {
     nm_mbar_expect_tx(c.bar_q, BQ * ROWB);
     nm_tma_load_3d(c.q_s, c.tmQ, t.g * HD, t.qb * BQ, t.b, c.bar_q);
 #pragma unroll
-    for (int gi = 0; gi < NG; ++gi) {
-#pragma unroll
-        for (int st = 0; st < 2; ++st) {
-            const int c128 = gi + NG * st;
-            if (c128 >= c.n128) break;
-            uint8_t* dst = st == 0 ? c.k_st + (size_t)gi * 2 * STAGE : c.p_s + (size_t)gi * PBUF;
-            uint64_t* bar = c.bar_k1_full + gi * 2 + st;
-            nm_mbar_expect_tx(bar, 2 * STAGE);
-            nm_tma_load_3d(dst, c.tmK, t.g * HD, c128 * 2 * CK, t.b, bar);
-            nm_tma_load_3d(dst + STAGE, c.tmK, t.g * HD, c128 * 2 * CK + CK, t.b, bar);
-        }
+    for (int st = 0; st < 2; ++st) {
+        if (st >= c.n128) break;
+        uint8_t* dst = st == 0 ? c.k_st : c.p_s;
+        uint64_t* bar = c.bar_k1_full + st;
+        nm_mbar_expect_tx(bar, 2 * STAGE);
+        nm_tma_load_3d(dst, c.tmK, t.g * HD, st * 2 * CK, t.b, bar);
+        nm_tma_load_3d(dst + STAGE, c.tmK, t.g * HD, st * 2 * CK + CK, t.b, bar);
     }
 }
-// The group's first V chunk of a tile (one thread; the V stage must be free).
-__device__ __forceinline__ void load_first_v(const LoadCtx& c, const Tile& t, int gi)
+// The first V chunk of a tile (one thread; the V stage must be free).
+__device__ __forceinline__ void load_first_v(const LoadCtx& c, const Tile& t)
 {
-    nm_mbar_expect_tx(c.bar_v_full + gi, STAGE);
-    nm_tma_load_3d(c.v_st + (size_t)gi * STAGE, c.tmV, t.g * HD, gi * CK, t.b, c.bar_v_full + gi);
+    nm_mbar_expect_tx(c.bar_v_full, STAGE);
+    nm_tma_load_3d(c.v_st, c.tmV, t.g * HD, 0, t.b, c.bar_v_full);
 }
 
-// NG = softmax groups per CTA: 2 (320 threads, 256 tensor-memory columns, two CTAs per SM) or
-// 1 (160 threads, 128 columns, three CTAs per SM: more tiles in flight per SM, fewer warps per tile).
-template <typename T, bool CLAMP_HI, int NG>
-__global__ void __launch_bounds__(160 * NG, NG == 1 ? 3 : 2)
+template <typename T, bool CLAMP_HI, bool RAGGED>
+__global__ void __launch_bounds__(160, RAGGED ? 2 : 3)
 attention_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                         const __grid_constant__ CUtensorMap tmV, const SArgs a)
 {
     constexpr uint32_t IDESC_QK = nm_idesc(1, AT<T>::fmt, 0, 0, BQ, CK);   // S chunk: 128 x 64
     constexpr uint32_t IDESC_PV = nm_idesc(1, AT<T>::fmt, 0, 1, BQ, HD);   // O: 128 x 64, V MN-major
     constexpr uint32_t IDESC_QK1 = nm_idesc(1, AT<T>::fmt, 0, 0, BQ, 2 * CK);   // sweep 1: 128 x 128
-    constexpr uint32_t TMEM_COLS = 128 * NG;   // S0 | O0 (| S1 | O1); sweep 1 writes 128 keys over [S_g | O_g]
-    constexpr int NSOFT = 128 * NG;            // softmax threads
-    constexpr uint32_t GRP_COLS = 128;    // tensor-memory columns of a group
-    constexpr uint32_t O_OFF = 64;        // O_g within the group's columns
-    // One group per CTA: the 16-bit P tile goes through tensor memory (a second allocation of 32 columns: 64 keys,
-    // two per column) and is the A operand of P V from there; three CTAs hold 3 x (128 + 32) of the SM's 512
-    // columns.  That takes the P tile's stores, its reads by the tensor core and the proxy fence off the shared-
-    // memory pipe, which the table lookups load most.  With two groups the columns do not suffice (2 CTAs x 320).
-    constexpr bool PT = NG == 1;
-    constexpr uint32_t P_COLS = 32;
+    constexpr uint32_t TMEM_COLS = 128;   // S | O; sweep 1 writes 128 keys over [S | O]
+    constexpr uint32_t O_OFF = 64;
+    // The 16-bit P tile goes through a second allocation of 32 columns (64 keys, two per column) and is the A operand
+    // of P V from there; three CTAs hold 3 x (128 + 32) of the SM's 512 columns.  RAGGED: 32 more for the low terms.
+    constexpr uint32_t P_COLS = RAGGED ? 64 : 32;
+    constexpr int P_TERMS = RAGGED ? 2 : 1;
 
     extern __shared__ uint8_t smem_raw[];
-    __shared__ uint64_t bar_q, bar_drain[NG];
-    __shared__ uint64_t bar_k_full[NG][2], bar_k1_full[NG][2], bar_v_full[NG], bar_s_full[NG], bar_p_empty[NG];
+    __shared__ uint64_t bar_q, bar_drain;
+    __shared__ uint64_t bar_k_full[2], bar_k1_full[2], bar_v_full, bar_s_full, bar_p_empty;
     __shared__ uint32_t tmem_slot, tmem_slot_p;
     __shared__ int abort_flag;
-    __shared__ float s_red[NG][BQ];
 
     const int L = a.L;
-    const int n = L / CK;      // chunks (even: L is a multiple of 128)
-    const int half = n / NG;   // chunks per group in sweep 2: group g takes g, g+NG, ...
-    const int n128 = L / (2 * CK);   // 128-key chunks of sweep 1: group g takes g, g+NG, ...
+    const int n = RAGGED ? (L + CK - 1) / CK : L / CK;                    // 64-key chunks of sweep 2
+    const int n128 = RAGGED ? (L + 2 * CK - 1) / (2 * CK) : L / (2 * CK);   // 128-key chunks of sweep 1
     uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     uint8_t* q_s = base;                       // 16 KB
-    uint8_t* k_st = q_s + BQ * ROWB;           // [group][2] x 8 KB
-    uint8_t* v_st = k_st + NG * 2 * STAGE;     // [group] x 8 KB
-    uint8_t* p_s = v_st + NG * STAGE;          // [group] x 16 KB
-    float2* rep = reinterpret_cast<float2*>(p_s + NG * PBUF);   // (n_exp + 1) x 16 copies
+    uint8_t* k_st = q_s + BQ * ROWB;           // 2 x 8 KB
+    uint8_t* v_st = k_st + 2 * STAGE;          // 8 KB
+    uint8_t* p_s = v_st + STAGE;               // 16 KB: sweep 1's second K stage
+    float2* rep = reinterpret_cast<float2*>(p_s + PBUF);   // (n_exp + 1) x 16 copies
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     // A CTA walks over the (batch, head, 128-query block) tiles blockIdx.x, blockIdx.x + gridDim.x, ...: barriers,
     // tensor memory and the replicated table are set up once, and the control warp fetches the next tile's Q,
     // first K chunks and first V chunk while the softmax warps finish the current one.
-    const int blocks_per_seq = L / BQ;
+    const int blocks_per_seq = n128;   // BQ = 2 CK
     const int n_tiles = a.B * a.heads * blocks_per_seq;
     const TileGeom geom = {blocks_per_seq, a.heads};
     auto tile_of = [geom](int t) { return tile_decode(geom, t); };
     LoadCtx lc;
     lc.tmQ = &tmQ; lc.tmK = &tmK; lc.tmV = &tmV;
     lc.q_s = q_s; lc.k_st = k_st; lc.p_s = p_s; lc.v_st = v_st;
-    lc.bar_q = &bar_q; lc.bar_k1_full = &bar_k1_full[0][0]; lc.bar_v_full = &bar_v_full[0];
+    lc.bar_q = &bar_q; lc.bar_k1_full = &bar_k1_full[0]; lc.bar_v_full = &bar_v_full;
     lc.n128 = n128;
 
     if (threadIdx.x == 0) {
@@ -221,158 +213,144 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
         nm_prefetch_tmap(&tmK);
         nm_prefetch_tmap(&tmV);
         nm_mbar_init(&bar_q, 1);
-        for (int i = 0; i < NG; ++i) {
-            nm_mbar_init(&bar_drain[i], 1);
-            nm_mbar_init(&bar_k_full[i][0], 1);
-            nm_mbar_init(&bar_k_full[i][1], 1);
-            nm_mbar_init(&bar_k1_full[i][0], 1);
-            nm_mbar_init(&bar_k1_full[i][1], 1);
-            nm_mbar_init(&bar_v_full[i], 1);
-            nm_mbar_init(&bar_s_full[i], 1);
-            nm_mbar_init(&bar_p_empty[i], 1);
-        }
+        nm_mbar_init(&bar_drain, 1);
+        nm_mbar_init(&bar_k_full[0], 1);
+        nm_mbar_init(&bar_k_full[1], 1);
+        nm_mbar_init(&bar_k1_full[0], 1);
+        nm_mbar_init(&bar_k1_full[1], 1);
+        nm_mbar_init(&bar_v_full, 1);
+        nm_mbar_init(&bar_s_full, 1);
+        nm_mbar_init(&bar_p_empty, 1);
         nm_fence_barrier_init();
         // The first copies go out before the rest of the set-up (tensor-memory allocation, table
-        // replication, block barrier), so that their latency overlaps it: Q, each group's first two
-        // 128-key chunks of sweep 1 (stage 0 = the group's two K stages, stage 1 = its P tile, which
-        // sweep 1 does not use otherwise) and its first V chunk.
+        // replication, block barrier), so that their latency overlaps it: Q, the first two 128-key chunks
+        // of sweep 1 and the first V chunk.
         nm_grid_dependency_wait();   // Q, K, V come from the previous kernel
         if ((int)blockIdx.x < n_tiles) {
             const Tile t0 = tile_of((int)blockIdx.x);
-            load_tile_head<NG>(lc, t0);
-            for (int gi = 0; gi < NG; ++gi) load_first_v(lc, t0, gi);
+            load_tile_head(lc, t0);
+            load_first_v(lc, t0);
         }
     }
-    if (warp == NG - 1) {
+    if (warp == 0) {
         nm_tmem_alloc(&tmem_slot, TMEM_COLS);
-        if constexpr (PT) nm_tmem_alloc(&tmem_slot_p, P_COLS);
+        nm_tmem_alloc(&tmem_slot_p, P_COLS);
         nm_tmem_relinquish();
-    }
-    if (warp >= NG) {
+    } else {
         // 16-way replicated exp table: entry s, copy c at rep[s*16 + c].  A 64-bit warp load is served
         // half a warp at a time, so 16 copies already make arbitrary lookups conflict-free.  One extra
         // entry (a copy of the last) lets input 0 of a table whose range ends at 0 go unclamped.
         const int ne = a.n_exp;
-        for (int i = threadIdx.x - 32 * NG; i < (ne + 1) * 16; i += NSOFT) rep[i] = a.t_exp->kb[min(i >> 4, ne - 1)];
+        for (int i = threadIdx.x - 32; i < (ne + 1) * 16; i += 128) rep[i] = a.t_exp->kb[min(i >> 4, ne - 1)];
     }
     nm_tc_fence_before();
     __syncthreads();
     nm_tc_fence_after();
     const uint32_t tmem_base = tmem_slot;
-    const uint32_t tmem_p = PT ? tmem_slot_p : 0u;
+    const uint32_t tmem_p = tmem_slot_p;
     volatile int* abortp = &abort_flag;
     nm_grid_launch_dependents();   // the next kernel may start its set-up
     nm_grid_dependency_wait();     // Q, K, V come from the previous kernel
 
-    if (warp < NG) {
-        // ------------------------------------------------ control warp of group `warp`
+    if (warp == 0) {
+        // ------------------------------------------------ control warp
         // Runs with all 32 lanes (barrier tests, counters and descriptors stay warp-uniform); one
         // elected lane issues the TMA and tcgen05 instructions.  It sleeps in a named barrier until
-        // its group's four softmax warps have arrived there, so signalling costs no polling:
+        // the four softmax warps have arrived there, so signalling costs no polling:
         //   S-consumed(i): chunk i's scores are in registers -> K stage i & 1 is free (load the chunk
         //                  after next into it) and S is free (issue Q K^T for the next chunk);
-        //   P-ready(j):    the bf16 P tile of the j-th chunk of sweep 2 is in shared memory -> O += P V.
-        const int gi = NG == 1 ? 0 : warp;
-        const uint32_t bar_sc = 2 + 2 * gi, bar_pr = 3 + 2 * gi, bar_oc = 6 + gi;
-        const int cnt1 = (n128 - gi + NG - 1) / NG;   // the group's 128-key chunks in sweep 1
-        uint8_t* my_k = k_st + (size_t)gi * 2 * STAGE;
-        uint8_t* my_v = v_st + (size_t)gi * STAGE;
-        uint8_t* my_p = p_s + (size_t)gi * PBUF;
-        const uint32_t my_tmem = tmem_base + (uint32_t)gi * GRP_COLS;
+        //   P-ready(j):    the P tile of the j-th chunk of sweep 2 is in tensor memory -> O += P V.
+        const uint32_t bar_sc = 2, bar_pr = 3, bar_oc = 6;
         auto wait = [&](uint64_t* bar, uint32_t parity) {
             return __all_sync(0xffffffffu, nm_mbar_wait_relaxed<20>(bar, parity, abortp, a.status)) != 0;
         };
         bool ok = true;
         const uint64_t qdesc = nm_smem_desc_sw128(nm_smem_u32(q_s));
         // completions consumed so far on each barrier (they run on from tile to tile)
-        uint32_t q_cnt = 0, k1_cnt0 = 0, k1_cnt1 = 0, k_cnt0 = 0, k_cnt1 = 0, v_cnt = 0, pv_cnt = 0;
+        uint32_t q_cnt = 0, k1_cnt0 = 0, k1_cnt1 = 0, k_cnt0 = 0, k_n128 = 0, v_cnt = 0, pv_cnt = 0;
         for (int tile = (int)blockIdx.x, ti = 0; tile < n_tiles; tile += (int)gridDim.x, ++ti) {
             const Tile t = tile_of(tile);
             const int g = t.g, b = t.b;
             const bool more = tile + (int)gridDim.x < n_tiles;
             if (ok && !wait(&bar_q, q_cnt & 1u)) ok = false;
             ++q_cnt;
-            // the previous tile's epilogue has read O out of tensor memory (sweep 1 writes over [S_g | O_g])
+            // the previous tile's epilogue has read O out of tensor memory (sweep 1 writes over [S | O])
             if (ti > 0) asm volatile("bar.sync %0, %1;" ::"r"(bar_oc), "n"(160) : "memory");
-            // ---- sweep 1: [S_g | O_g] = Q K^T for 128 keys at a time; K stage i & 1 (0: the two K stages
+            // ---- sweep 1: [S | O] = Q K^T for 128 keys at a time; K stage i & 1 (0: the two K stages
             // taken together, 1: the P tile)
             auto issue_qk1 = [&](int i) {
                 const uint32_t par = ((i & 1) ? k1_cnt1 : k1_cnt0) & 1u;
                 if (i & 1) ++k1_cnt1; else ++k1_cnt0;
                 if (!ok) return;
-                if (!wait(&bar_k1_full[gi][i & 1], par)) { ok = false; return; }
+                if (!wait(&bar_k1_full[i & 1], par)) { ok = false; return; }
                 nm_tc_fence_after();
-                const uint64_t kdesc = nm_smem_desc_sw128(nm_smem_u32((i & 1) ? my_p : my_k));
+                const uint64_t kdesc = nm_smem_desc_sw128(nm_smem_u32((i & 1) ? p_s : k_st));
                 if (nm_elect_one()) {
 #pragma unroll
-                    for (int k = 0; k < 4; ++k) nm_mma_f16(my_tmem, qdesc + 2 * k, kdesc + 2 * k, IDESC_QK1, k != 0);
-                    nm_tc_commit(&bar_s_full[gi]);
+                    for (int k = 0; k < 4; ++k) nm_mma_f16(tmem_base, qdesc + 2 * k, kdesc + 2 * k, IDESC_QK1, k != 0);
+                    nm_tc_commit(&bar_s_full);
                 }
                 __syncwarp();
             };
-            if (cnt1 > 0) issue_qk1(0);
-            for (int i = 0; i < cnt1; ++i) {
+            if (n128 > 0) issue_qk1(0);
+            for (int i = 0; i < n128; ++i) {
                 asm volatile("bar.sync %0, %1;" ::"r"(bar_sc), "n"(160) : "memory");   // S-consumed: chunk i is in registers
-                if (i + 1 < cnt1) issue_qk1(i + 1);
-                if (ok && i + 2 < cnt1 && nm_elect_one()) {   // its MMAs are complete: the stage takes the chunk after next
-                    uint8_t* dst = (i & 1) ? my_p : my_k;
-                    const int key0 = (gi + NG * (i + 2)) * 2 * CK;
-                    nm_mbar_expect_tx(&bar_k1_full[gi][i & 1], 2 * STAGE);
-                    nm_tma_load_3d(dst, &tmK, g * HD, key0, b, &bar_k1_full[gi][i & 1]);
-                    nm_tma_load_3d(dst + STAGE, &tmK, g * HD, key0 + CK, b, &bar_k1_full[gi][i & 1]);
+                if (i + 1 < n128) issue_qk1(i + 1);
+                if (ok && i + 2 < n128 && nm_elect_one()) {   // its MMAs are complete: the stage takes the chunk after next
+                    uint8_t* dst = (i & 1) ? p_s : k_st;
+                    const int key0 = (i + 2) * 2 * CK;
+                    nm_mbar_expect_tx(&bar_k1_full[i & 1], 2 * STAGE);
+                    nm_tma_load_3d(dst, &tmK, g * HD, key0, b, &bar_k1_full[i & 1]);
+                    nm_tma_load_3d(dst + STAGE, &tmK, g * HD, key0 + CK, b, &bar_k1_full[i & 1]);
                 }
                 __syncwarp();
             }
-            // ---- sweep 2: the group's j-th chunk is the 64 keys of chunk g + NG*j; K stage j & 1
+            // ---- sweep 2: chunk j is 64 keys; K stage j & 1
             auto load_k = [&](int j) {
                 if (ok && nm_elect_one()) {
-                    nm_mbar_expect_tx(&bar_k_full[gi][j & 1], STAGE);
-                    nm_tma_load_3d(my_k + (size_t)(j & 1) * STAGE, &tmK, g * HD, (gi + NG * j) * CK, b, &bar_k_full[gi][j & 1]);
+                    nm_mbar_expect_tx(&bar_k_full[j & 1], STAGE);
+                    nm_tma_load_3d(k_st + (size_t)(j & 1) * STAGE, &tmK, g * HD, j * CK, b, &bar_k_full[j & 1]);
                 }
                 __syncwarp();
             };
-            auto issue_qk = [&](int j) {   // S_g = Q K^T
-                const uint32_t par = ((j & 1) ? k_cnt1 : k_cnt0) & 1u;
-                if (j & 1) ++k_cnt1; else ++k_cnt0;
+            auto issue_qk = [&](int j) {   // S = Q K^T
+                const uint32_t par = ((j & 1) ? k_n128 : k_cnt0) & 1u;
+                if (j & 1) ++k_n128; else ++k_cnt0;
                 if (!ok) return;
-                if (!wait(&bar_k_full[gi][j & 1], par)) { ok = false; return; }
+                if (!wait(&bar_k_full[j & 1], par)) { ok = false; return; }
                 nm_tc_fence_after();
-                const uint64_t kdesc = nm_smem_desc_sw128(nm_smem_u32(my_k + (size_t)(j & 1) * STAGE));
+                const uint64_t kdesc = nm_smem_desc_sw128(nm_smem_u32(k_st + (size_t)(j & 1) * STAGE));
                 if (nm_elect_one()) {
 #pragma unroll
-                    for (int k = 0; k < 4; ++k) nm_mma_f16(my_tmem, qdesc + 2 * k, kdesc + 2 * k, IDESC_QK, k != 0);
-                    nm_tc_commit(&bar_s_full[gi]);
+                    for (int k = 0; k < 4; ++k) nm_mma_f16(tmem_base, qdesc + 2 * k, kdesc + 2 * k, IDESC_QK, k != 0);
+                    nm_tc_commit(&bar_s_full);
                 }
                 __syncwarp();
             };
             load_k(0);   // every MMA of sweep 1 has completed: the K stages are free
-            if (half > 1) load_k(1);
+            if (n > 1) load_k(1);
             issue_qk(0);
-            for (int j = 0; j < half; ++j) {
+            for (int j = 0; j < n; ++j) {
                 asm volatile("bar.sync %0, %1;" ::"r"(bar_sc), "n"(160) : "memory");   // S-consumed(j)
-                if (j + 1 < half) issue_qk(j + 1);
-                if (j + 2 < half) load_k(j + 2);
-                if constexpr (NG == 1) {
-                    // Last chunk: every Q K^T of the tile has completed, so Q, the K stages and the P tile (which
-                    // only sweep 1 uses when P goes through tensor memory) take the next tile's first loads now.
-                    if (j + 1 == half && more && ok && nm_elect_one()) load_tile_head<NG>(lc, tile_of(tile + (int)gridDim.x));
-                    __syncwarp();
-                }
+                if (j + 1 < n) issue_qk(j + 1);
+                if (j + 2 < n) load_k(j + 2);
+                // Last chunk: every Q K^T of the tile has completed, so Q, the K stages and p_s take the next tile's
+                // first loads now.
+                if (j + 1 == n && more && ok && nm_elect_one()) load_tile_head(lc, tile_of(tile + (int)gridDim.x));
+                __syncwarp();
                 asm volatile("bar.sync %0, %1;" ::"r"(bar_pr), "n"(160) : "memory");   // P-ready(j)
-                if (ok && !wait(&bar_v_full[gi], v_cnt & 1u)) ok = false;
+                if (ok && !wait(&bar_v_full, v_cnt & 1u)) ok = false;
                 ++v_cnt;
                 if (ok) {
                     nm_tc_fence_after();
-                    const uint64_t pdesc = nm_smem_desc_sw128(nm_smem_u32(my_p));
-                    const uint32_t v_addr = nm_smem_u32(my_v);
+                    const uint32_t v_addr = nm_smem_u32(v_st);
                     if (nm_elect_one()) {
 #pragma unroll
-                        for (int k = 0; k < 4; ++k) {   // V rows (keys) 16k..16k+15: two groups of 8 rows, 1024 bytes apart
-                            const uint64_t vdesc = nm_smem_desc_sw128(v_addr + (uint32_t)(16 * k * ROWB));
-                            if constexpr (PT) mma_f16_a_tmem(my_tmem + O_OFF, tmem_p + (uint32_t)(8 * k), vdesc, IDESC_PV, (j | k) != 0);
-                            else nm_mma_f16(my_tmem + O_OFF, pdesc + 2 * k, vdesc, IDESC_PV, (j | k) != 0);
+                        for (int k = 0; k < 4 * P_TERMS; ++k) {   // V rows (keys) 16(k&3)..+15: two groups of 8 rows, 1024 bytes apart
+                            const uint64_t vdesc = nm_smem_desc_sw128(v_addr + (uint32_t)(16 * (k & 3) * ROWB));
+                            mma_f16_a_tmem(tmem_base + O_OFF, tmem_p + (uint32_t)(8 * k), vdesc, IDESC_PV, (j | k) != 0);
                         }
-                        nm_tc_commit(&bar_p_empty[gi]);
+                        nm_tc_commit(&bar_p_empty);
                     }
                     __syncwarp();
                 }
@@ -380,15 +358,15 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                 ++pv_cnt;
                 // the V stage is free once this P V has completed (nothing else to do until then): it takes the
                 // next chunk's V, or after the last chunk the next tile's first one
-                const bool next_v = j + 1 < half || (NG == 1 && more);
+                const bool next_v = j + 1 < n || more;
                 if (ok && next_v) {
-                    if (!wait(&bar_p_empty[gi], pv_par)) ok = false;
+                    if (!wait(&bar_p_empty, pv_par)) ok = false;
                     if (ok && nm_elect_one()) {
-                        if (j + 1 < half) {
-                            nm_mbar_expect_tx(&bar_v_full[gi], STAGE);
-                            nm_tma_load_3d(my_v, &tmV, g * HD, (gi + NG * (j + 1)) * CK, b, &bar_v_full[gi]);
+                        if (j + 1 < n) {
+                            nm_mbar_expect_tx(&bar_v_full, STAGE);
+                            nm_tma_load_3d(v_st, &tmV, g * HD, (j + 1) * CK, b, &bar_v_full);
                         } else {
-                            load_first_v(lc, tile_of(tile + (int)gridDim.x), gi);
+                            load_first_v(lc, tile_of(tile + (int)gridDim.x));
                         }
                     }
                     __syncwarp();
@@ -397,31 +375,26 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
         }
         if (!ok) {   // after an abort: let copies land and MMAs retire (bounded) before teardown
             if (nm_elect_one()) {
-                nm_tc_commit(&bar_drain[gi]);
+                nm_tc_commit(&bar_drain);
                 long long t0 = clock64();
-                while (!nm_mbar_try_wait(&bar_drain[gi], 0) && clock64() - t0 < 200000000LL) {}
+                while (!nm_mbar_try_wait(&bar_drain, 0) && clock64() - t0 < 200000000LL) {}
                 while (clock64() - t0 < 4000000LL) {}
             }
             __syncwarp();
         }
     } else {
         // ------------------------------------------------ softmax warps
-        // Warps 2-5 (group 0) take the even chunks, warps 6-9 (group 1) the odd ones; group g owns S
-        // buffer g, P buffer g and accumulator O_g, so the two groups form two independent pipelines.
-        // A warp never blocks on its group: it signals the control warp with bar.arrive.
+        // One row per thread.  A warp never blocks on the others: it signals the control warp with bar.arrive.
         const int q = warp & 3;
-        const int g2 = NG == 1 ? 0 : (warp - NG) >> 2;
         const int row = q * 32 + lane;
-        const uint32_t bar_sc = 2 + 2 * g2, bar_pr = 3 + 2 * g2, bar_oc = 6 + g2;
-        const uint32_t t_row = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)g2 * GRP_COLS;
-        const int cnt1 = (n128 - g2 + NG - 1) / NG;   // the group's 128-key chunks in sweep 1
+        const uint32_t bar_sc = 2, bar_pr = 3, bar_oc = 6;
+        const uint32_t t_row = tmem_base + ((uint32_t)(q * 32) << 16);
         const float inv_h = a.t_exp->inv_h, off = a.t_exp->off, nm1 = (float)(a.n_exp - 1);
         // this lane's copy of the replicated table, with the constant of the index trick folded in:
         // (bits << 7) = 0xA0000000 + s*128 (mod 2^32) for bits = 0x4B400000 + s
         const uint32_t rep_lane = nm_smem_u32(rep) + (uint32_t)(lane & 15) * 8u - 0xA0000000u;
         const uint64_t scale2 = nm_pack2(a.scale, a.scale), inv_h2 = nm_pack2(inv_h, inv_h), off2 = nm_pack2(off, off);
         const uint64_t magic2 = nm_pack2(12582912.0f, 12582912.0f);
-        const uint32_t prow = nm_smem_u32(p_s) + (uint32_t)(g2 * PBUF + row * ROWB);
         const uint32_t p_row = tmem_p + ((uint32_t)(q * 32) << 16);   // this warp's lane quarter of the P columns
         int ok = 1;
         // All lanes test the barrier; only when it is not yet complete does lane 0 poll (with sleeps).
@@ -435,27 +408,36 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                 if (ok) (void)nm_mbar_try_wait(bar, par);
             }
         };
-        // completions consumed so far: S products of this group, P V products of every group (the same count)
+        // completions consumed so far: S products, P V products
         uint32_t s_cnt = 0, pv_base = 0;
         for (int tile = (int)blockIdx.x; tile < n_tiles; tile += (int)gridDim.x) {
             const Tile t = tile_of(tile);
             const int qb = t.qb, g = t.g, b = t.b;
             const bool more = tile + (int)gridDim.x < n_tiles;
+            // RAGGED: a warp whose 32 queries all lie beyond the sequence waits and signals like the others, but
+            // computes nothing (its rows of the accumulator are never stored)
+            const bool live = !RAGGED || qb * BQ + q * 32 < L;
             // ---- sweep 1: the final row maximum
             float m = -INFINITY;
 #pragma unroll 1
-            for (int i = 0; i < cnt1; ++i) {
-                wait_all(&bar_s_full[g2], s_cnt & 1u);
+            for (int i = 0; i < n128; ++i) {
+                wait_all(&bar_s_full, s_cnt & 1u);
                 ++s_cnt;
-                if (ok) {
+                if (ok && live) {
                     nm_tc_fence_after();
 #pragma unroll
-                    for (int hh = 0; hh < 4; ++hh) {   // 128 keys: the scores span [S_g | O_g]
+                    for (int hh = 0; hh < 4; ++hh) {   // 128 keys: the scores span [S | O]
                         uint32_t r[32];
                         nm_tmem_ld32_sync(t_row + (uint32_t)(hh * 32), r);
                         if (hh == 3) {   // all of it is in registers: the control warp may overwrite S
                             nm_tc_fence_before();
                             asm volatile("bar.arrive %0, %1;" ::"r"(bar_sc), "n"(160) : "memory");
+                        }
+                        if (RAGGED && i == n128 - 1) {   // keys beyond L do not take part
+                            const int lim = L - i * 2 * CK - hh * 32;
+#pragma unroll
+                            for (int k = 0; k < 32; ++k)
+                                if (k >= lim) r[k] = 0xff800000u;   // -inf
                         }
                         float m0 = -INFINITY, m1 = -INFINITY;
 #pragma unroll
@@ -469,35 +451,37 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                     asm volatile("bar.arrive %0, %1;" ::"r"(bar_sc), "n"(160) : "memory");
                 }
             }
-            if constexpr (NG == 2) {   // the two groups saw different keys of the row
-                s_red[g2][row] = m;
-                asm volatile("bar.sync 1, %0;" ::"n"(NSOFT) : "memory");
-                m = fmaxf(s_red[0][row], s_red[1][row]);
-                asm volatile("bar.sync 1, %0;" ::"n"(NSOFT) : "memory");
-            }
             const float neg_ms = -(m * a.scale);
             const uint64_t neg_ms2 = nm_pack2(neg_ms, neg_ms);
             float sum0 = 0.f, sum1 = 0.f, sum2 = 0.f, sum3 = 0.f;
-            // ---- sweep 2: e = PWL_exp(s - m), row sum, P tiles
-#pragma unroll 1
-            for (int j = 0; j < half; ++j) {
-                wait_all(&bar_s_full[g2], s_cnt & 1u);
+            // ---- sweep 2: e = PWL_exp(s - m), row sum, P tiles.  LAST: the chunk that may hold keys beyond L; they
+            // take the maximum as their score (which keeps the table index in range) and the exponential 0.
+            auto chunk = [&](int j, auto last) {
+                constexpr bool LAST = decltype(last)::value;
+                wait_all(&bar_s_full, s_cnt & 1u);
                 ++s_cnt;
                 if (ok) nm_tc_fence_after();
 #pragma unroll
                 for (int hh = 0; hh < 2; ++hh) {
+                    const int lim = LAST ? L - j * CK - hh * 32 : 32;
                     uint32_t r[32];
-                    if (ok) {
+                    if (ok && live) {
                         nm_tmem_ld32_sync(t_row + (uint32_t)(hh * 32), r);
+                        if constexpr (LAST) {
+#pragma unroll
+                            for (int k = 0; k < 32; ++k)
+                                if (k >= lim) r[k] = __float_as_uint(m);
+                        }
                     }
                     if (hh == 1) {
                         nm_tc_fence_before();
                         asm volatile("bar.arrive %0, %1;" ::"r"(bar_sc), "n"(160) : "memory");
                     }
-                    uint32_t pk[16];   // the half's 32 exponentials, packed to 16 bits
-                    if (ok) {
+                    uint32_t pk[16];                       // the half's 32 exponentials, packed to 16 bits
+                    [[maybe_unused]] uint32_t pl[RAGGED ? 16 : 1];          // RAGGED: what the packing left, packed to 16 bits
+                    if (ok && live) {
 #pragma unroll
-                        for (int jj = 0; jj < 4; ++jj) {   // 8 keys = one 16-byte chunk of the P row
+                        for (int jj = 0; jj < 4; ++jj) {   // 8 keys
                             float e[8];
 #pragma unroll
                             for (int k = 0; k < 8; k += 2) {
@@ -527,89 +511,74 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                                 asm("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(k1), "=f"(c1) : "r"((__float_as_uint(f1) << 7) + rep_lane));
                                 e[k] = __fmaf_rn(k0, x0, c0);
                                 e[k + 1] = __fmaf_rn(k1, x1, c1);
+                                if constexpr (LAST) {
+                                    if (jj * 8 + k >= lim) e[k] = 0.f;
+                                    if (jj * 8 + k + 1 >= lim) e[k + 1] = 0.f;
+                                }
                             }
                             sum0 += e[0] + e[4];
                             sum1 += e[1] + e[5];
                             sum2 += e[2] + e[6];
                             sum3 += e[3] + e[7];
 #pragma unroll
-                            for (int k = 0; k < 4; ++k) pk[jj * 4 + k] = AT<T>::pack(e[2 * k], e[2 * k + 1]);
-                        }
-                    }
-                    // The stores wait until P V of the group's previous chunk has read the tile; that MMA was
-                    // issued just before this chunk began, so the first half's arithmetic runs ahead of it.
-                    if (hh == 0 && j >= 1) {
-                        wait_all(&bar_p_empty[g2], (pv_base + (uint32_t)(j - 1)) & 1u);
-                    }
-                    if (ok) {
-                        if constexpr (PT) {
-                            if (hh == 0 && j >= 1) nm_tc_fence_after();   // ordered after the P V that read the columns
-                            tmem_st16(p_row + (uint32_t)(hh * 16), pk);   // keys 32 hh .. 32 hh + 31 of this thread's row
-                        } else {
-#pragma unroll
-                            for (int jj = 0; jj < 4; ++jj) {
-                                // chunk index is XORed with the row (128-byte swizzle of the K-major P tile)
-                                const uint32_t addr = prow + (uint32_t)(((hh * 4 + jj) ^ (row & 7)) << 4);
-                                asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(addr), "r"(pk[jj * 4]), "r"(pk[jj * 4 + 1]),
-                                             "r"(pk[jj * 4 + 2]), "r"(pk[jj * 4 + 3])
-                                             : "memory");
+                            for (int k = 0; k < 4; ++k) {
+                                pk[jj * 4 + k] = AT<T>::pack(e[2 * k], e[2 * k + 1]);
+                                if constexpr (RAGGED) {
+                                    const float2 hi = AT<T>::unpack(pk[jj * 4 + k]);
+                                    pl[jj * 4 + k] = AT<T>::pack(e[2 * k] - hi.x, e[2 * k + 1] - hi.y);   // exact differences
+                                }
                             }
                         }
                     }
+                    // The stores wait until P V of the previous chunk has read the tile; that MMA was
+                    // issued just before this chunk began, so the first half's arithmetic runs ahead of it.
+                    if (hh == 0 && j >= 1) {
+                        wait_all(&bar_p_empty, (pv_base + (uint32_t)(j - 1)) & 1u);
+                    }
+                    if (ok && live) {
+                        if (hh == 0 && j >= 1) nm_tc_fence_after();   // ordered after the P V that read the columns
+                        tmem_st16(p_row + (uint32_t)(hh * 16), pk);   // keys 32 hh .. 32 hh + 31 of this thread's row
+                        if constexpr (RAGGED) tmem_st16(p_row + (uint32_t)(32 + hh * 16), pl);
+                    }
                 }
-                if constexpr (PT) {
-                    tmem_st_wait();          // the P columns are written
-                    nm_tc_fence_before();
-                } else {
-                    nm_fence_proxy_async();   // generic-proxy writes of P become visible to the tensor core
-                }
+                tmem_st_wait();          // the P columns are written
+                nm_tc_fence_before();
                 asm volatile("bar.arrive %0, %1;" ::"r"(bar_pr), "n"(160) : "memory");
-            }
-            float sum = (sum0 + sum1) + (sum2 + sum3);
-            if constexpr (NG == 2) {
-                s_red[g2][row] = sum;
-                asm volatile("bar.sync 1, %0;" ::"n"(NSOFT) : "memory");
-                sum = s_red[0][row] + s_red[1][row];
-            }
-            // ---- r = PWL_recip(sigma), then (O_0 + O_1) * r; each group stores 32 of the 64 channels
+            };
+#pragma unroll 1
+            for (int j = 0; j < (RAGGED ? n - 1 : n); ++j) chunk(j, std::false_type{});
+            if constexpr (RAGGED) chunk(n - 1, std::true_type{});
+            const float sum = (sum0 + sum1) + (sum2 + sum3);
+            // ---- r = PWL_recip(sigma), then O * r
             const int sr = nm_pwl_index(sum, a.t_rcp->inv_h, a.t_rcp->off, (float)(a.t_rcp->n - 1));
             const float2 kbr = a.t_rcp->kb[sr];
             const float rinv = __fmaf_rn(kbr.x, sum, kbr.y);
-#pragma unroll
-            for (int gg = 0; gg < NG; ++gg)   // the last P V of every group has completed
-                wait_all(&bar_p_empty[gg], (pv_base + (uint32_t)(half - 1)) & 1u);
-            pv_base += (uint32_t)half;
-            constexpr int CH = HD / NG;   // channels this warp stores
+            wait_all(&bar_p_empty, (pv_base + (uint32_t)(n - 1)) & 1u);   // the last P V has completed
+            pv_base += (uint32_t)n;
             if (ok) nm_tc_fence_after();
+            const bool store_row = !RAGGED || qb * BQ + row < L;
             T* orow = reinterpret_cast<T*>(a.out) + ((size_t)b * L + (size_t)qb * BQ + row) * ((size_t)a.heads * HD) +
-                      (size_t)g * HD + g2 * CH;
-            const uint32_t o_addr = tmem_base + ((uint32_t)(q * 32) << 16) + O_OFF + (uint32_t)(g2 * CH);
+                      (size_t)g * HD;
+            const uint32_t o_addr = t_row + O_OFF;
 #pragma unroll
-            for (int jj = 0; jj < CH / 16; ++jj) {   // 16 channels at a time, summed over the groups' accumulators
-                uint32_t r0[16], r1[16];
-                if (ok) {
-                    nm_tmem_ld16_sync(o_addr + (uint32_t)(jj * 16), r0);
-                    if constexpr (NG == 2) nm_tmem_ld16_sync(o_addr + GRP_COLS + (uint32_t)(jj * 16), r1);
-                }
-                if (jj == CH / 16 - 1 && more) {
-                    // all of O is in registers: the control warp may start the next tile's sweep 1 over [S_g | O_g]
+            for (int jj = 0; jj < HD / 16; ++jj) {   // 16 channels at a time
+                uint32_t r0[16];
+                if (ok && live) nm_tmem_ld16_sync(o_addr + (uint32_t)(jj * 16), r0);
+                if (jj == HD / 16 - 1 && more) {
+                    // all of O is in registers: the control warp may start the next tile's sweep 1 over [S | O]
                     nm_tc_fence_before();
                     asm volatile("bar.arrive %0, %1;" ::"r"(bar_oc), "n"(160) : "memory");
                 }
-                if (ok) {
+                if (ok && store_row) {
                     float v[16];
 #pragma unroll
-                    for (int k = 0; k < 16; ++k) {
-                        float x = __uint_as_float(r0[k]);
-                        if constexpr (NG == 2) x += __uint_as_float(r1[k]);
-                        v[k] = x * rinv;
-                    }
+                    for (int k = 0; k < 16; ++k) v[k] = __uint_as_float(r0[k]) * rinv;
                     if (a.out_q) {
                         int8_t code[16];
 #pragma unroll
                         for (int k = 0; k < 16; ++k) code[k] = nm_quant_i8(AT<T>::round(v[k]), a.q_inv_scale);
                         int8_t* qrow = a.out_q + ((size_t)b * L + (size_t)qb * BQ + row) * ((size_t)a.heads * HD) +
-                                       (size_t)g * HD + g2 * CH;
+                                       (size_t)g * HD;
                         reinterpret_cast<uint4*>(qrow)[jj] = *reinterpret_cast<const uint4*>(code);
                     } else {
                         uint32_t w[8];
@@ -625,11 +594,11 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
 
     nm_tc_fence_before();
     __syncthreads();
-    if (warp == NG - 1) {
+    if (warp == 0) {
         __syncwarp();
         nm_tc_fence_after();
         nm_tmem_dealloc(tmem_base, TMEM_COLS);
-        if constexpr (PT) nm_tmem_dealloc(tmem_p, P_COLS);
+        nm_tmem_dealloc(tmem_p, P_COLS);
     }
 }
 
@@ -652,7 +621,7 @@ nm_status make_map(nm_ctx* ctx, CUtensorMap* m, const void* ptr, nm_dtype dt, co
     return r == CUDA_SUCCESS ? NM_OK : NM_ERR_CUDA;
 }
 
-template <typename T, bool CLAMP_HI, int NG>
+template <typename T, bool CLAMP_HI, bool RAGGED>
 nm_status launch(nm_ctx* ctx, const nm_attn_desc* d, cudaStream_t st, int8_t* out_q, float q_inv_scale)
 {
     SArgs a;
@@ -664,33 +633,30 @@ nm_status launch(nm_ctx* ctx, const nm_attn_desc* d, cudaStream_t st, int8_t* ou
     a.n_exp = ctx->h_tables[d->exp_slot].n;
     a.out_q = out_q;
     a.q_inv_scale = q_inv_scale;
-    const size_t smem = (size_t)BQ * ROWB + NG * (3 * (size_t)STAGE + (size_t)PBUF) + (size_t)(a.n_exp + 1) * 16 * sizeof(float2) + 1024;
+    const size_t smem = (size_t)BQ * ROWB + 3 * (size_t)STAGE + (size_t)PBUF + (size_t)(a.n_exp + 1) * 16 * sizeof(float2) + 1024;
     if (smem > 227 * 1024 - 2048) return NM_ERR_UNSUPPORTED;   // an exp table too large to replicate
     CUtensorMap tmQ, tmK, tmV;
     nm_status s;
     if ((s = make_map(ctx, &tmQ, d->Q, d->dtype, d, BQ)) != NM_OK) return s;
     if ((s = make_map(ctx, &tmK, d->K, d->dtype, d, CK)) != NM_OK) return s;
     if ((s = make_map(ctx, &tmV, d->V, d->dtype, d, CK)) != NM_OK) return s;
-    auto kern = attention_stream_kernel<T, CLAMP_HI, NG>;
+    auto kern = attention_stream_kernel<T, CLAMP_HI, RAGGED>;
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
         return NM_ERR_CUDA;
-    const int64_t tiles = (int64_t)d->B * d->heads * (d->L / BQ);
+    const int64_t tiles = (int64_t)d->B * d->heads * ((d->L + BQ - 1) / BQ);
     if (tiles > 0x7fffffffLL) return NM_ERR_SHAPE;
-    int64_t grid = tiles;
-    if (NG == 1) {
-        // persistent: one resident wave of CTAs, each walking over tiles.  Three CTAs per SM by the launch bounds
-        // (registers) and by tensor memory (3 x 160 of 512 columns); fewer if the exp table makes the shared
-        // memory larger (233472 bytes per SM, 1 KB reserved per CTA).
-        int64_t per_sm = 233472 / (int64_t)(smem + 1024 + 1536);
-        if (per_sm > 3) per_sm = 3;
-        if (per_sm < 1) per_sm = 1;
-        const int64_t cap = (int64_t)ctx->sm_count * per_sm;
-        if (grid > cap) grid = cap;
-    }
+    // persistent: one resident wave of CTAs, each walking over tiles.  Three CTAs per SM (RAGGED: two) by the launch
+    // bounds (registers) and by tensor memory (3 x 160 or 2 x 192 of 512 columns); fewer if the exp table makes the
+    // shared memory larger (233472 bytes per SM, 1 KB reserved per CTA).
+    int64_t per_sm = 233472 / (int64_t)(smem + 1024 + 1536);
+    if (per_sm > (RAGGED ? 2 : 3)) per_sm = RAGGED ? 2 : 3;
+    if (per_sm < 1) per_sm = 1;
+    int64_t grid = (int64_t)ctx->sm_count * per_sm;
+    if (grid > tiles) grid = tiles;
     cudaLaunchConfig_t cfg;
     memset(&cfg, 0, sizeof(cfg));
     cfg.gridDim = dim3((unsigned)grid);
-    cfg.blockDim = dim3(160 * NG);
+    cfg.blockDim = dim3(160);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
@@ -707,9 +673,13 @@ nm_status launch(nm_ctx* ctx, const nm_attn_desc* d, cudaStream_t st, int8_t* ou
 
 bool nm_attention_stream_supported(const nm_attn_desc* d)
 {
+    return d->L % 128 == 0 && nm_attention_stream_any_length_supported(d);
+}
+
+bool nm_attention_stream_any_length_supported(const nm_attn_desc* d)
+{
     if (d->dtype != NM_BF16 && d->dtype != NM_F16) return false;
-    if (d->d != HD) return false;
-    if (d->L % 128 != 0 || d->L < 128) return false;
+    if (d->d != HD || d->L < 1) return false;
     if ((d->stride_t * 2) % 16 != 0 || (d->stride_b * 2) % 16 != 0) return false;
     return true;
 }
@@ -717,13 +687,16 @@ bool nm_attention_stream_supported(const nm_attn_desc* d)
 nm_status nm_launch_attention_stream(nm_ctx* ctx, const nm_attn_desc* d, cudaStream_t st, int8_t* out_q,
                                      float q_inv_scale)
 {
-    if (!nm_attention_stream_supported(d)) return NM_ERR_UNSUPPORTED;
+    if (!nm_attention_stream_any_length_supported(d)) return NM_ERR_UNSUPPORTED;
     // the softmax input is never positive: a table whose range reaches 0 needs no upper clamp
     const bool clamp_hi = ctx->h_tables[d->exp_slot].x_max < 0.0f;
-    // One softmax group per CTA: three persistent CTAs per SM with P through tensor memory.  (The kernel text
-    // still carries the two-group form, NG = 2, which splits the keys of a tile between two pipelines of one
-    // CTA; it measured slower at every length from 128 to 2048 once P left shared memory, and is not built.)
-    if (d->dtype == NM_BF16)
-        return clamp_hi ? launch<__nv_bfloat16, true, 1>(ctx, d, st, out_q, q_inv_scale) : launch<__nv_bfloat16, false, 1>(ctx, d, st, out_q, q_inv_scale);
-    return clamp_hi ? launch<__half, true, 1>(ctx, d, st, out_q, q_inv_scale) : launch<__half, false, 1>(ctx, d, st, out_q, q_inv_scale);
+    const bool ragged = d->L % 128 != 0;
+#define NM_ATTN_CASE(T)                                                                                               \
+    (clamp_hi ? (ragged ? launch<T, true, true>(ctx, d, st, out_q, q_inv_scale)                                       \
+                        : launch<T, true, false>(ctx, d, st, out_q, q_inv_scale))                                     \
+              : (ragged ? launch<T, false, true>(ctx, d, st, out_q, q_inv_scale)                                      \
+                        : launch<T, false, false>(ctx, d, st, out_q, q_inv_scale)))
+    if (d->dtype == NM_BF16) return NM_ATTN_CASE(__nv_bfloat16);
+    return NM_ATTN_CASE(__half);
+#undef NM_ATTN_CASE
 }

@@ -361,16 +361,15 @@ static nm_status attention_dispatch(nm_ctx* ctx, const nm_attn_desc* d, void* st
     if (!(d->scale > 0.0f) || !isfinite(d->scale)) return NM_ERR_INVALID_ARG;
     cudaStream_t st = (cudaStream_t)stream;
     if (d->algo == 1) return nm_launch_attention_simt(ctx, d, st);
-    // tensor-core kernels: the streaming one (several CTAs per SM, any L that is a multiple of 128) is the
+    // tensor-core kernels: the streaming one (several CTAs per SM; algo 2 takes multiples of 128 only) is the
     // default; algo 3 selects the one that keeps the whole score block in tensor memory (L <= 512)
     if (d->algo == 3) return nm_attention_tc_supported(d) ? nm_launch_attention_tc(ctx, d, st) : NM_ERR_UNSUPPORTED;
     if (d->algo == 0 && ctx->attn_resident && nm_attention_tc_supported(d)) {
         const nm_status s = nm_launch_attention_tc(ctx, d, st);
         if (s != NM_ERR_UNSUPPORTED) return s;
     }
-    const bool tc = nm_attention_stream_supported(d);
-    if (d->algo == 2) return tc ? nm_launch_attention_stream(ctx, d, st) : NM_ERR_UNSUPPORTED;
-    if (tc) {
+    if (d->algo == 2) return nm_attention_stream_supported(d) ? nm_launch_attention_stream(ctx, d, st) : NM_ERR_UNSUPPORTED;
+    if (nm_attention_stream_any_length_supported(d)) {
         const nm_status s = nm_launch_attention_stream(ctx, d, st, out_q, q_inv_scale);
         if (s != NM_ERR_UNSUPPORTED) {   // else: an exp table too large for shared memory
             if (fused && out_q && s == NM_OK) *fused = true;

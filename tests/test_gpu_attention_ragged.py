@@ -1,0 +1,81 @@
+"""GPU parity, attention at sequence lengths that are not a multiple of 128 (masked last chunk, probabilities as two
+16-bit terms)."""
+import numpy as np
+import pytest
+import torch
+
+import nm_inputs
+import oracle
+from util import load_tables_both, rms_rel, to_np
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ctx(nm):
+    c = nm.Context(0)
+    yield c
+    c.close()
+
+
+def run(ctx, dtype, B, L, h, seed, pad=0, n=64, exp_range=(-8.0, 0.0), score_shift=0.0):
+    tabs = load_tables_both(ctx, n, {"exp": exp_range, "recip": (max(L / 16.0, 0.5), float(max(L, 2)))})
+    H, td = h * 64, nm_inputs.torch_dtype(dtype)
+    qkv = nm_inputs.matrix((B * L, 3 * H), seed, dtype, 1.0)
+    qkv[:, :2 * H] *= 0.8
+    if score_shift:   # every score far below zero: a zero-filled key beyond L would be the row's largest
+        qkv[:, :H] += score_shift
+        qkv[:, H:2 * H] -= score_shift
+    qkv = nm_inputs.round_to(qkv, dtype)
+    buf = torch.zeros((B * L, 3 * H + pad), dtype=td, device="cuda")
+    buf[:, :3 * H] = torch.from_numpy(qkv).cuda().to(td)
+    out = torch.full((B * L + 1, H), float("nan"), dtype=td, device="cuda")
+    ctx.attention_pwl(buf[:, :3 * H], out, B, L, h, 64)
+    ctx.check_device_status()
+    assert torch.isnan(out[B * L:].float()).all()   # nothing is written beyond the last row
+    ref = oracle.attention(qkv, B, L, h, 64, tabs["exp"], tabs["recip"])
+    return to_np(out[:B * L]), ref
+
+
+def check(got, ref, dtype):
+    """The result's own rounding to the storage type is at most 2^-8 (bf16) or 2^-11 (fp16) of each element, its rms over
+    many elements at most 1/sqrt(3) of that; the probabilities add 2^-18 / 2^-22 and the fp32 sums less."""
+    half_ulp = {"bf16": 2.0 ** -8, "f16": 2.0 ** -11}[dtype]
+    assert np.all(np.isfinite(got))
+    rms = np.sqrt(np.mean(ref * ref))
+    assert np.all(np.abs(got - ref) <= half_ulp * 1.01 * np.abs(ref) + 2e-5 * rms + 2.0 ** -25), np.abs(got - ref).max()
+    if got.size >= 1024:
+        assert rms_rel(got, ref) <= half_ulp / np.sqrt(3.0)
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "f16"])
+@pytest.mark.parametrize("B,L,h,pad", [(1, 1, 1, 0), (2, 7, 2, 0), (1, 37, 12, 0), (3, 63, 1, 8), (1, 64, 2, 0), (2, 65, 3, 0),
+                                       (2, 96, 1, 0), (1, 127, 2, 16), (2, 129, 2, 0), (1, 191, 1, 0), (1, 193, 2, 0),
+                                       (2, 333, 3, 0), (1, 511, 2, 0), (1, 1000, 1, 0)])
+def test_lengths(ctx, dtype, B, L, h, pad):
+    check(*run(ctx, dtype, B, L, h, seed=L + h, pad=pad), dtype)
+
+
+def test_masked_keys_are_not_the_maximum(ctx):
+    got, ref = run(ctx, "bf16", 1, 70, 2, seed=5, score_shift=1.0)
+    check(got, ref, "bf16")
+
+
+@pytest.mark.parametrize("n,exp_range", [(16, (-8.0, 0.0)), (256, (-8.0, 0.0)), (64, (-6.0, -0.5))])
+def test_tables(ctx, n, exp_range):
+    """Small and large tables, and one whose range ends below zero (the upper clamp)."""
+    check(*run(ctx, "bf16", 2, 150, 2, seed=n, n=n, exp_range=exp_range), "bf16")
+
+
+def test_several_tiles_per_cta(ctx):
+    """More tiles than resident CTAs (two per SM): barrier phases run on from tile to tile, odd counts per tile."""
+    B, L, h = 12, 190, 16
+    assert B * h * 2 > 2 * torch.cuda.get_device_properties(0).multi_processor_count
+    check(*run(ctx, "bf16", B, L, h, seed=3), "bf16")
+
+
+def test_forced_streaming_kernel_still_takes_multiples_of_128_only(nm, ctx):
+    q = torch.zeros(100, 192, dtype=torch.bfloat16, device="cuda")
+    with pytest.raises(nm.NmError) as ei:
+        ctx.attention_pwl(q, torch.zeros(100, 64, dtype=torch.bfloat16, device="cuda"), 1, 100, 1, 64, algo=nm.ALGO_TC)
+    assert ei.value.code == 5
