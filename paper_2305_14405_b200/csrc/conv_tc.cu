@@ -1,8 +1,8 @@
 // Host side of the implicit-GEMM convolution: chooses the patch of output pixels a tile covers,
-// encodes the 4-D tensor maps over the NHWC tensors themselves and launches linear_tc_kernel in its
-// CONV form (linear_tc_kernel.cuh).  Section 3.1: a convolution is a matrix product whose dimensions
+// encodes the 4-D tensor maps over the NHWC tensors themselves and launches linear_tc_kernel
+// (linear_tc_kernel.cuh) or linear_split_kernel (linear_split_kernel.cuh) in its CONV form.  Section 3.1: a convolution is a matrix product whose dimensions
 // follow from width, height and channels; here the matrix is never written to memory.
-#include "linear_tc_kernel.cuh"
+#include "linear_split_kernel.cuh"
 
 using namespace nm_tc;
 
@@ -39,13 +39,11 @@ void choose_patch(int Wo, int Ho, int N, int* TW, int* TH, int* NB)
     }
 }
 
-template <typename T, bool TWO, int BN>
-nm_status launch(nm_ctx* ctx, const NmConvTc* c, cudaStream_t st)
+// Patch geometry and epilogue operands common to both kernels; returns the number of patches.
+int64_t fill_args(nm_ctx* ctx, const NmConvTc* c, TcArgs* a)
 {
-    constexpr int B_ROWS = TWO ? BN / 2 : BN;
-    TcArgs a;
-    memset(&a, 0, sizeof(a));
-    ConvDev& cv = a.cv;
+    memset(a, 0, sizeof(*a));
+    ConvDev& cv = a->cv;
     choose_patch(c->Wo, c->Ho, c->N, &cv.TW, &cv.TH, &cv.NB);
     cv.tiles_x = ceil_div(c->Wo, cv.TW);
     cv.tiles_y = ceil_div(c->Ho, cv.TH);
@@ -53,28 +51,63 @@ nm_status launch(nm_ctx* ctx, const NmConvTc* c, cudaStream_t st)
     cv.kw_eff = c->taps_x; cv.cblocks = c->cblocks;
     cv.Ho = c->Ho; cv.Nimg = c->N;
     cv.dw = c->depthwise;
-    const int64_t patches = (int64_t)cv.tiles_x * cv.tiles_y * ceil_div(c->N, cv.NB);
+    a->M = (int64_t)c->N * c->Ho * c->Wo; a->N = c->Cout; a->K = c->Ktot;
+    a->bias = c->bias;
+    a->has_res = c->residual ? 1 : 0;
+    a->res_first = c->res_first;
+    a->tab = c->slot == NM_SLOT_NONE ? nullptr : ctx->d_tables + c->slot;
+    a->n_seg = c->slot == NM_SLOT_NONE ? 0 : ctx->h_tables[c->slot].n;
+    a->status = ctx->d_status;
+    a->num_k_blocks = c->taps_y * c->taps_x * c->cblocks;
+    return (int64_t)cv.tiles_x * cv.tiles_y * ceil_div(c->N, cv.NB);
+}
+
+// A: one box per filter tap, strided like the convolution
+nm_status make_tmap_a(nm_ctx* ctx, CUtensorMap* m, const NmConvTc* c, const ConvDev& cv)
+{
+    const uint32_t abox[4] = {64u, (uint32_t)((cv.TW - 1) * cv.sw + 1), (uint32_t)((cv.TH - 1) * cv.sh + 1), (uint32_t)cv.NB};
+    const uint32_t aestr[4] = {1u, (uint32_t)cv.sw, (uint32_t)cv.sh, 1u};
+    if (abox[1] > 256 || abox[2] > 256) return NM_ERR_UNSUPPORTED;
+    return make_tmap4(ctx, m, c->a_base, c->dtype, c->a_dim, c->a_stride, abox, aestr);
+}
+
+template <typename T, int BN>
+nm_status launch_split(nm_ctx* ctx, const NmConvTc* c, int S, cudaStream_t st)
+{
+    SplitArgs s;
+    memset(&s, 0, sizeof(s));
+    const int64_t patches = fill_args(ctx, c, &s.t);
+    s.t.num_n_tiles = ceil_div(c->Cout, BN);
+    const int64_t tiles = patches * s.t.num_n_tiles;
+    s.S = S;
+    s.t.num_tiles = (int)tiles;
+    s.residual = c->residual; s.ldr = c->Cout;
+    s.out = c->out; s.ldo = c->Cout;
+    s.Wo = c->Wo;
+    CUtensorMap tmA, tmW;
+    nm_status e = make_tmap_a(ctx, &tmA, c, s.t.cv);
+    if (e != NM_OK) return e;
+    e = make_tmap(ctx, &tmW, c->w, c->dtype, c->depthwise ? 64 : c->Cout, c->Ktot, c->ldw, BN);
+    if (e != NM_OK) return e;
+    return launch_split_kernel<T, T, BN, true>(ctx, tmA, tmW, s, c->flops, st);
+}
+
+template <typename T, bool TWO, int BN>
+nm_status launch(nm_ctx* ctx, const NmConvTc* c, cudaStream_t st)
+{
+    constexpr int B_ROWS = TWO ? BN / 2 : BN;
+    TcArgs a;
+    const int64_t patches = fill_args(ctx, c, &a);
+    const ConvDev& cv = a.cv;
     const int64_t m_tiles = TWO ? (patches + 1) / 2 : patches;
-    a.M = (int64_t)c->N * c->Ho * c->Wo; a.N = c->Cout; a.K = c->Ktot;
-    a.bias = c->bias;
-    a.has_res = c->residual ? 1 : 0;
-    a.res_first = c->res_first;
-    a.tab = c->slot == NM_SLOT_NONE ? nullptr : ctx->d_tables + c->slot;
-    a.n_seg = c->slot == NM_SLOT_NONE ? 0 : ctx->h_tables[c->slot].n;
-    a.status = ctx->d_status;
     a.num_n_tiles = ceil_div(c->Cout, BN);
     if (m_tiles * a.num_n_tiles > 0x7fffffffLL) return NM_ERR_SHAPE;
     a.num_tiles = (int)(m_tiles * a.num_n_tiles);
-    a.num_k_blocks = c->taps_y * c->taps_x * c->cblocks;
     size_t smem = 0;
     if (!plan_smem<T, TWO, BN>(&a, c->bias != nullptr, &smem)) return NM_ERR_UNSUPPORTED;
 
     CUtensorMap tmA, tmW, tmO, tmR;
-    // A: one box per filter tap, strided like the convolution
-    const uint32_t abox[4] = {64u, (uint32_t)((cv.TW - 1) * cv.sw + 1), (uint32_t)((cv.TH - 1) * cv.sh + 1), (uint32_t)cv.NB};
-    const uint32_t aestr[4] = {1u, (uint32_t)cv.sw, (uint32_t)cv.sh, 1u};
-    if (abox[1] > 256 || abox[2] > 256) return NM_ERR_UNSUPPORTED;
-    nm_status s = make_tmap4(ctx, &tmA, c->a_base, c->dtype, c->a_dim, c->a_stride, abox, aestr);
+    nm_status s = make_tmap_a(ctx, &tmA, c, cv);
     if (s != NM_OK) return s;
     // (depthwise form: W is the one 64 x 64 matrix, whatever the number of output channels)
     s = make_tmap(ctx, &tmW, c->w, c->dtype, c->depthwise ? 64 : c->Cout, c->Ktot, c->ldw, B_ROWS);
@@ -94,19 +127,25 @@ nm_status launch(nm_ctx* ctx, const NmConvTc* c, cudaStream_t st)
     return launch_kernel<T, T, TWO, BN, true>(ctx, tmA, tmW, tmO, tmR, a, smem, c->flops, st);
 }
 
-template <typename T, int BN>
-nm_status launch_two(nm_ctx* ctx, const NmConvTc* c, cudaStream_t st)
-{
-    if (c->algo != 3 && (int64_t)c->N * c->Ho * c->Wo >= 256) return launch<T, true, BN>(ctx, c, st);
-    return launch<T, false, BN>(ctx, c, st);
-}
-
 template <typename T>
 nm_status launch_sel(nm_ctx* ctx, const NmConvTc* c, cudaStream_t st)
 {
-    if (c->Cout <= 64 || c->depthwise) return launch_two<T, 64>(ctx, c, st);
-    if (c->Cout <= 128) return launch_two<T, 128>(ctx, c, st);
-    return launch_two<T, 256>(ctx, c, st);
+    TileChoice t;
+    if (c->algo == 0) {
+        int tw, th, nb;
+        choose_patch(c->Wo, c->Ho, c->N, &tw, &th, &nb);
+        const int64_t patches = (int64_t)ceil_div(c->Wo, tw) * ceil_div(c->Ho, th) * ceil_div(c->N, nb);
+        t = choose_tile(patches, c->Cout, (int64_t)c->taps_y * c->taps_x * c->cblocks, true, c->slot != NM_SLOT_NONE,
+                        c->depthwise != 0, true, ctx->sm_count);
+    } else {
+        t.S = 0;
+        t.BN = c->Cout <= 64 || c->depthwise ? 64 : (c->Cout <= 128 ? 128 : 256);
+        t.two = c->algo != 3 && (int64_t)c->N * c->Ho * c->Wo >= 256;
+    }
+    if (t.S) return t.BN == 32 ? launch_split<T, 32>(ctx, c, t.S, st) : launch_split<T, 64>(ctx, c, t.S, st);
+    if (t.BN == 64) return t.two ? launch<T, true, 64>(ctx, c, st) : launch<T, false, 64>(ctx, c, st);
+    if (t.BN == 128) return t.two ? launch<T, true, 128>(ctx, c, st) : launch<T, false, 128>(ctx, c, st);
+    return t.two ? launch<T, true, 256>(ctx, c, st) : launch<T, false, 256>(ctx, c, st);
 }
 
 }  // namespace

@@ -1,0 +1,489 @@
+// The linear operator for problems whose tiles do not fill the GPU (a single request, a late convolution
+// stage): one 128 x BN output tile (BN = 64 or 32) per thread-block cluster, the K dimension split over the
+// cluster's CTAs.
+//
+//   out[m][j] = PWL( sum_c A[m][c]*W[j][c] * scale_j + bias[j] ) + residual[m][j]
+//
+// Such a launch is bound by latency: with the persistent kernel's 256-column tiles a BERT-base layer on 128
+// tokens keeps 3 to 12 SMs busy, each walking through the whole of K on its own.  Here every CTA multiplies
+// its share of the K-blocks (TMA ring, tcgen05.mma into tensor memory), writes its fp32 or int32 partial tile
+// to its own shared memory, and after one cluster barrier every CTA finishes every S-th row of the tile: it
+// reads the S partial rows over distributed shared memory, adds them in rank order (the sum does not depend
+// on timing), applies scale, bias, table and residual and stores whole row segments.
+//
+// CONV = true: the A operand is the NHWC activation, as in linear_tc_kernel (a tile's 128 rows are a patch of
+// output pixels and a K-block is one 4-D TMA box).
+#pragma once
+#include "linear_tc_kernel.cuh"
+
+namespace nm_tc {
+
+constexpr int SPLIT_THREADS = 256;
+constexpr int SPLIT_MAX_STAGES = 4;   // 96 KB at BN = 64: two CTAs per SM, so the next kernel's set-up can overlap
+
+struct SplitArgs {
+    TcArgs t;               // num_tiles, num_n_tiles, num_k_blocks, stages and the epilogue's operands
+    int S;                  // CTAs per cluster
+    const void* residual;
+    int64_t ldr, ldo;
+    void* out;
+    int Wo;                 // CONV: output pixels per row
+};
+
+// Words per row of a partial tile: 16-byte row stores and loads without bank conflicts.
+constexpr int part_pitch(int bn) { return bn + 4; }
+
+template <typename OutT> struct Quad;
+template <> struct Quad<float> {
+    using Raw = float4;
+    static __device__ __forceinline__ Raw fetch(const float* p) { return *reinterpret_cast<const float4*>(p); }
+    static __device__ __forceinline__ float4 widen(const Raw& w) { return w; }
+    static __device__ __forceinline__ void store(float* p, const float4& v, float) { *reinterpret_cast<float4*>(p) = v; }
+};
+template <> struct Quad<__nv_bfloat16> {
+    using Raw = uint2;
+    static __device__ __forceinline__ Raw fetch(const __nv_bfloat16* p) { return *reinterpret_cast<const uint2*>(p); }
+    static __device__ __forceinline__ float4 widen(const Raw& w)
+    {
+        const float2 a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&w.x));
+        const float2 b = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&w.y));
+        return make_float4(a.x, a.y, b.x, b.y);
+    }
+    static __device__ __forceinline__ void store(__nv_bfloat16* p, const float4& v, float)
+    {
+        const __nv_bfloat162 a = __floats2bfloat162_rn(v.x, v.y), b = __floats2bfloat162_rn(v.z, v.w);
+        *reinterpret_cast<uint2*>(p) = make_uint2(*reinterpret_cast<const uint32_t*>(&a), *reinterpret_cast<const uint32_t*>(&b));
+    }
+};
+template <> struct Quad<__half> {
+    using Raw = uint2;
+    static __device__ __forceinline__ Raw fetch(const __half* p) { return *reinterpret_cast<const uint2*>(p); }
+    static __device__ __forceinline__ float4 widen(const Raw& w)
+    {
+        const float2 a = __half22float2(*reinterpret_cast<const __half2*>(&w.x));
+        const float2 b = __half22float2(*reinterpret_cast<const __half2*>(&w.y));
+        return make_float4(a.x, a.y, b.x, b.y);
+    }
+    static __device__ __forceinline__ void store(__half* p, const float4& v, float)
+    {
+        const __half2 a = __floats2half2_rn(v.x, v.y), b = __floats2half2_rn(v.z, v.w);
+        *reinterpret_cast<uint2*>(p) = make_uint2(*reinterpret_cast<const uint32_t*>(&a), *reinterpret_cast<const uint32_t*>(&b));
+    }
+};
+template <> struct Quad<int8_t> {
+    using Raw = uint32_t;   // there is no int8 residual
+    static __device__ __forceinline__ Raw fetch(const int8_t*) { return 0u; }
+    static __device__ __forceinline__ float4 widen(const Raw&) { return make_float4(0.f, 0.f, 0.f, 0.f); }
+    static __device__ __forceinline__ void store(int8_t* p, const float4& v, float inv)
+    {
+        *reinterpret_cast<uint32_t*>(p) = nm_quant_i8x4(v.x, v.y, v.z, v.w, inv);
+    }
+};
+
+__device__ __forceinline__ uint4 ld_cluster_v4(uint32_t cluster_addr)
+{
+    uint4 v;
+    asm volatile("ld.shared::cluster.v4.b32 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+                 : "r"(cluster_addr));
+    return v;
+}
+
+// Final sum and epilogue of a cluster's tile: this CTA takes rows rank, rank + S, ... of the `rows` that exist and adds
+// the S partial tiles (one in each CTA's shared memory at `part`, part_pitch(BN) words per row) in rank order.  Four
+// columns per thread, whole row segments per group of BN / 4 threads.  Rows go in batches of up to FIN_U per thread, all
+// loads of a batch in flight together, and the vectors and the first batch's residual are fetched before the product
+// is even started: a row at a time cost a memory latency per row.
+constexpr int FIN_U = 4;
+
+template <bool INT, typename OutT, int BN, bool CONV, int THREADS>
+struct Finisher {
+    static constexpr int PITCH = part_pitch(BN);
+    static constexpr int QPR = BN / 4;            // 4-column groups per row
+    static constexpr int RPP = THREADS / QPR;     // rows per pass
+    const SplitArgs& s;
+    const int rank, mt, nt, rows;
+    const Patch pt;
+    const int qc;          // this thread's 4-column group in every pass
+    const int64_t col;
+    const bool col_ok;     // N is a multiple of 4
+    float4 bias, sc;
+    typename Quad<OutT>::Raw res[FIN_U];
+
+    __device__ __forceinline__ Finisher(const SplitArgs& s_, int rank_, int mt_, int nt_, int rows_, const Patch& pt_)
+        : s(s_), rank(rank_), mt(mt_), nt(nt_), rows(rows_), pt(pt_), qc((int)threadIdx.x % QPR),
+          col((int64_t)nt_ * BN + qc * 4), col_ok(col < s_.t.N)
+    {
+    }
+    // row of the output matrix that row r of the tile is, or -1
+    __device__ __forceinline__ int64_t out_row(int r) const
+    {
+        if (r >= rows) return -1;
+        if constexpr (CONV) {
+            const ConvDev& cv = s.t.cv;
+            const int ox = pt.ox0 + r % cv.TW, oy = pt.oy0 + (r / cv.TW) % cv.TH, img = pt.img0 + r / (cv.TW * cv.TH);
+            if (ox >= s.Wo || oy >= cv.Ho || img >= cv.Nimg) return -1;
+            return ((int64_t)img * cv.Ho + oy) * s.Wo + ox;
+        } else {
+            return (int64_t)mt * BM + r;
+        }
+    }
+    __device__ __forceinline__ int tile_row(int i) const { return ((int)threadIdx.x / QPR + i * RPP) * s.S + rank; }
+    __device__ __forceinline__ void load_res(int i0)
+    {
+        if (!s.residual || !col_ok) return;
+#pragma unroll
+        for (int u = 0; u < FIN_U; ++u) {
+            const int64_t g = out_row(tile_row(i0 + u));
+            if (g >= 0) res[u] = Quad<OutT>::fetch(reinterpret_cast<const OutT*>(s.residual) + g * s.ldr + col);
+        }
+    }
+    __device__ __forceinline__ void prefetch_vectors()
+    {
+        bias = make_float4(0.f, 0.f, 0.f, 0.f);
+        sc = bias;
+        if (col_ok) {
+            if (s.t.bias) bias = __ldg(reinterpret_cast<const float4*>(s.t.bias + col));
+            if constexpr (INT) {
+                const float4 ws = __ldg(reinterpret_cast<const float4*>(s.t.w_scale + col));
+                const float as = s.t.a_scale;
+                sc = make_float4(as * ws.x, as * ws.y, as * ws.z, as * ws.w);
+            }
+        }
+    }
+    __device__ __forceinline__ void run(const uint32_t* part, const float2* tab)
+    {
+        const int per_thread = (rows + s.S * RPP - 1) / (s.S * RPP);
+        if (per_thread <= 1) batches<1>(part, tab);
+        else if (per_thread <= 2) batches<2>(part, tab);
+        else batches<FIN_U>(part, tab);
+    }
+    template <int U>
+    __device__ __forceinline__ void batches(const uint32_t* part, const float2* tab)
+    {
+        const TcArgs& a = s.t;
+        const int S = s.S;
+        const bool has_tab = a.tab != nullptr;
+        const float inv_h = has_tab ? a.tab->inv_h : 0.f, off = has_tab ? a.tab->off : 0.f, nm1 = (float)(a.n_seg - 1);
+        const uint32_t part_u = nm_smem_u32(part);
+        for (int i0 = 0; tile_row(i0) < rows; i0 += U) {
+            if (i0 > 0) load_res(i0);
+            uint32_t acc[U][4];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                // (a row beyond the tile's last is read from the last and not used)
+                const int r = min(tile_row(i0 + u), BM - 1);
+                const uint32_t addr = part_u + (uint32_t)(r * PITCH + qc * 4) * 4u;
+                const uint4 p = S == 1 ? *reinterpret_cast<const uint4*>(part + (size_t)r * PITCH + qc * 4)
+                                       : ld_cluster_v4(nm_mapa(addr, 0));
+                acc[u][0] = p.x; acc[u][1] = p.y; acc[u][2] = p.z; acc[u][3] = p.w;
+            }
+#pragma unroll 2
+            for (int k = 1; k < S; ++k) {
+                uint4 o[U];
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const int r = min(tile_row(i0 + u), BM - 1);
+                    o[u] = ld_cluster_v4(nm_mapa(part_u + (uint32_t)(r * PITCH + qc * 4) * 4u, (uint32_t)k));
+                }
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const uint32_t w[4] = {o[u].x, o[u].y, o[u].z, o[u].w};
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        if constexpr (INT) acc[u][i] += w[i];
+                        else acc[u][i] = __float_as_uint(__uint_as_float(acc[u][i]) + __uint_as_float(w[i]));
+                    }
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int64_t grow = out_row(tile_row(i0 + u));
+                if (grow < 0 || !col_ok) continue;
+                float x[4];
+                const float bv[4] = {bias.x, bias.y, bias.z, bias.w}, sv[4] = {sc.x, sc.y, sc.z, sc.w};
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    if constexpr (INT) x[i] = __fmaf_rn((float)(int)acc[u][i], sv[i], bv[i]);
+                    else x[i] = __uint_as_float(acc[u][i]) + bv[i];
+                }
+                if constexpr (INT) {
+                    if (a.acc_dump)
+                        *reinterpret_cast<int4*>(a.acc_dump + grow * a.N + col) =
+                            make_int4((int)acc[u][0], (int)acc[u][1], (int)acc[u][2], (int)acc[u][3]);
+                }
+                float4 rv = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (s.residual) rv = Quad<OutT>::widen(res[u]);
+                if (s.residual && a.res_first) { x[0] += rv.x; x[1] += rv.y; x[2] += rv.z; x[3] += rv.w; }
+                int seg[4] = {-1, -1, -1, -1};
+                if (has_tab) {
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        seg[i] = nm_pwl_index(x[i], inv_h, off, nm1);
+                        const float2 t = tab[seg[i]];
+                        x[i] = __fmaf_rn(t.x, x[i], t.y);
+                    }
+                }
+                if (a.idx_dump) *reinterpret_cast<int4*>(a.idx_dump + grow * a.N + col) = make_int4(seg[0], seg[1], seg[2], seg[3]);
+                if (s.residual && !a.res_first) { x[0] += rv.x; x[1] += rv.y; x[2] += rv.z; x[3] += rv.w; }
+                Quad<OutT>::store(reinterpret_cast<OutT*>(s.out) + grow * s.ldo + col, make_float4(x[0], x[1], x[2], x[3]), a.inv_out_scale);
+            }
+        }
+    }
+};
+
+template <typename InT, typename OutT, int BN, bool CONV>
+__global__ void __launch_bounds__(SPLIT_THREADS, 2)
+linear_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmW, const SplitArgs s)
+{
+    const TcArgs& a = s.t;
+    constexpr bool INT = TcIn<InT>::is_int;
+    constexpr int B_BYTES = BN * ROW_BYTES;
+    constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
+    constexpr int BK_ELEMS = ROW_BYTES / (int)sizeof(InT);
+    constexpr uint32_t IDESC = nm_idesc(TcIn<InT>::c_fmt, TcIn<InT>::ab_fmt, 0, 0, BM, BN);
+    constexpr int PITCH = part_pitch(BN);
+
+    extern __shared__ uint8_t smem_raw[];
+    __shared__ uint64_t bar_full[SPLIT_MAX_STAGES], bar_empty[SPLIT_MAX_STAGES], bar_acc;
+    __shared__ uint32_t tmem_slot;
+    __shared__ int abort_flag;
+    __shared__ float2 s_tab[NM_MAX_SEGMENTS];
+
+    const int S = s.S;
+    const int rank = S > 1 ? (int)nm_cluster_ctarank() : 0;
+    const int tile = (int)blockIdx.x / S;
+    const int mt = tile / a.num_n_tiles, nt = tile % a.num_n_tiles;
+    const int kb0 = rank * a.num_k_blocks / S, kb1 = (rank + 1) * a.num_k_blocks / S;
+    const int stages = a.stages;
+    uint8_t* tiles = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+    uint32_t* part = reinterpret_cast<uint32_t*>(tiles);   // the partial tile takes the ring's place once K is done
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+
+    if (threadIdx.x == 0) {
+        abort_flag = 0;
+        nm_prefetch_tmap(&tmA);
+        nm_prefetch_tmap(&tmW);
+        for (int i = 0; i < stages; ++i) {
+            nm_mbar_init(&bar_full[i], 1);
+            nm_mbar_init(&bar_empty[i], 1);
+        }
+        nm_mbar_init(&bar_acc, 1);
+        nm_fence_barrier_init();
+    }
+    if (warp == 1) {
+        nm_tmem_alloc(&tmem_slot, BN);
+        nm_tmem_relinquish();
+    }
+    if (a.tab) {
+        for (int i = threadIdx.x; i < a.n_seg; i += SPLIT_THREADS) s_tab[i] = a.tab->kb[i];
+    }
+    nm_tc_fence_before();
+    __syncthreads();
+    nm_tc_fence_after();
+    const uint32_t tmem = tmem_slot;
+    volatile int* abortp = &abort_flag;
+    nm_grid_launch_dependents();
+
+    Patch pt = {0, 0, 0};
+    if constexpr (CONV) pt = patch_of(a.cv, mt);
+    const int rows = CONV ? BM : (int)(a.M - (int64_t)mt * BM < BM ? a.M - (int64_t)mt * BM : BM);
+    Finisher<INT, OutT, BN, CONV, SPLIT_THREADS> fin(s, rank, mt, nt, rows, pt);
+    bool ok = true;
+    nm_grid_dependency_wait();
+    fin.prefetch_vectors();
+    if (warp != 0) fin.load_res(0);
+    if (warp == 0) {
+        // ------------------------------------------------ TMA producer (all lanes run, one elected lane issues)
+        int stage = 0;
+        uint32_t phase = 0;
+        int tap = 0, cb = 0;
+        if constexpr (CONV) {
+            tap = kb0 / a.cv.cblocks;
+            cb = kb0 - tap * a.cv.cblocks;
+        }
+        for (int kb = kb0; kb < kb1; ++kb) {
+            if (!__all_sync(0xffffffffu, nm_mbar_wait(&bar_empty[stage], phase ^ 1u, abortp, a.status))) { ok = false; break; }
+            uint8_t* sa = tiles + (size_t)stage * STAGE_BYTES;
+            int c_c = 0, c_w = 0, c_h = 0, w_k = kb * BK_ELEMS, w_n = nt * BN;
+            if constexpr (CONV) {
+                const int ky = tap / a.cv.kw_eff, kx = tap - ky * a.cv.kw_eff;
+                c_c = cb * BK_ELEMS;
+                c_w = pt.ox0 * a.cv.sw - a.cv.pw + kx;
+                c_h = pt.oy0 * a.cv.sh - a.cv.ph + ky;
+                if (a.cv.dw) {   // pooling: channel block = column tile, one constant matrix for every tap and tile
+                    c_c = nt * BK_ELEMS;
+                    w_k = 0;
+                    w_n = 0;
+                }
+                if (++cb == a.cv.cblocks) { cb = 0; ++tap; }
+            }
+            if (nm_elect_one()) {
+                nm_mbar_expect_tx(&bar_full[stage], STAGE_BYTES);
+                if constexpr (CONV) nm_tma_load_4d(sa, &tmA, c_c, c_w, c_h, pt.img0, &bar_full[stage]);
+                else nm_tma_load_2d(sa, &tmA, kb * BK_ELEMS, mt * BM, &bar_full[stage]);
+                nm_tma_load_2d(sa + A_BYTES, &tmW, w_k, w_n, &bar_full[stage]);
+            }
+            __syncwarp();
+            if (++stage == stages) { stage = 0; phase ^= 1u; }
+        }
+        fin.load_res(0);
+        if (!ok) {
+            long long t0 = clock64();  // bounded pause: copies in flight land before teardown
+            while (clock64() - t0 < 4000000LL) {}
+        }
+    } else if (warp == 1) {
+        // ------------------------------------------------ MMA issuer
+        int stage = 0;
+        uint32_t phase = 0;
+        for (int kb = kb0; kb < kb1; ++kb) {
+            if (!__all_sync(0xffffffffu, nm_mbar_wait(&bar_full[stage], phase, abortp, a.status))) { ok = false; break; }
+            nm_tc_fence_after();
+            const uint32_t sa = nm_smem_u32(tiles + (size_t)stage * STAGE_BYTES);
+            const uint64_t adesc = nm_smem_desc_sw128(sa), bdesc = nm_smem_desc_sw128(sa + A_BYTES);
+            if (nm_elect_one()) {
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {  // 4 x 32 bytes of K per 128-byte row
+                    const uint32_t accum = (kb != kb0 || k != 0) ? 1u : 0u;
+                    if constexpr (INT) nm_mma_i8(tmem, adesc + 2 * k, bdesc + 2 * k, IDESC, accum);
+                    else nm_mma_f16(tmem, adesc + 2 * k, bdesc + 2 * k, IDESC, accum);
+                }
+                nm_tc_commit(&bar_empty[stage]);
+            }
+            __syncwarp();
+            if (++stage == stages) { stage = 0; phase ^= 1u; }
+        }
+        // After a timeout the commit still counts the MMAs that were issued, so that the wait below ends with them.
+        if (nm_elect_one()) nm_tc_commit(&bar_acc);
+        __syncwarp();
+    }
+    // Every warp waits for the accumulator: all MMAs have then read the ring, whose place the partial tile takes.
+    if (!nm_mbar_wait_relaxed<20>(&bar_acc, 0, abortp, a.status)) ok = false;
+    __syncwarp();
+    nm_tc_fence_after();
+    __syncthreads();
+    ok = ok && !abort_flag;
+    {   // two warps per tensor-memory lane quarter, each half of the columns
+        const int q = warp & 3, c0 = (warp >> 2) * (BN / 2);
+        uint32_t* my = part + (size_t)(q * 32 + lane) * PITCH + c0;
+        const uint32_t t_addr = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)c0;
+        if (q * 32 < rows) {
+#pragma unroll
+            for (int c = 0; c < BN / 2; c += 16) {
+                uint32_t r[16];
+                nm_tmem_ld16_sync(t_addr + (uint32_t)c, r);
+#pragma unroll
+                for (int i = 0; i < 16; i += 4)
+                    *reinterpret_cast<uint4*>(my + c + i) = make_uint4(r[i], r[i + 1], r[i + 2], r[i + 3]);
+            }
+        }
+    }
+    if (S > 1) nm_cluster_sync();
+    else __syncthreads();
+
+    if (ok) fin.run(part, s_tab);
+
+    // ---------------------------------------------------- teardown (all paths)
+    nm_tc_fence_before();
+    __syncthreads();
+    if (warp == 1) {
+        __syncwarp();
+        nm_tc_fence_after();
+        nm_tmem_dealloc(tmem, BN);
+    }
+    if (S > 1) nm_cluster_sync();   // a peer may still be reading this CTA's partial tile
+}
+
+// Launch attributes of a kernel in clusters of S CTAs; returns their number.
+inline unsigned split_launch_attrs(const nm_ctx* ctx, cudaLaunchAttribute* attr, int S)
+{
+    unsigned n = 0;
+    if (ctx->pdl) {
+        attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[n].val.programmaticStreamSerializationAllowed = 1;
+        ++n;
+    }
+    attr[n].id = cudaLaunchAttributeClusterDimension;
+    attr[n].val.clusterDim.x = (unsigned)S;
+    attr[n].val.clusterDim.y = 1;
+    attr[n].val.clusterDim.z = 1;
+    return n + 1;
+}
+
+// Which kernel and tile a problem of `m_tiles` blocks of 128 rows, N columns and `k_blocks` K-blocks gets: the least time
+// by a model of measured figures in us (chains of equal launches, 37 to 2331 rows, N 256 to 4096, K 256 to 4096, bf16 and
+// int8; it reproduces them to about 10 %).
+//   persistent kernel, r rounds of tiles: base + r * (k_blocks * per K-block), a round no shorter than its epilogue.  The
+//     K-block's time is its operands' way from L2 to one SM (50 bytes a clock), so a pair of CTAs and a wide tile need
+//     less of it per element, and a narrow tile makes better use of the last round.
+//   split kernel, n CTAs: 4.2 + the K-blocks beyond the three in flight at once, more when several CTAs share an SM, + the
+//     exchange over the cluster (0.4 / 1.0 / 1.8 for 2 / 4 / 8 CTAs) + the epilogue of four warps' worth per tile.
+// At 128 x 768 x 3072 one round of persistent tiles takes 17 us and the split over 8 CTAs 7.3; at 1024 x 768 x 768
+// 128 x 64 tiles take 6.7 and 256 x 256 pairs 9.8; at 16384 rows the widest tile wins.
+// `whole_chunks`: a row of the output is a multiple of 16 bytes.  The persistent kernel stores through a tensor map, which
+// writes whole 16-byte chunks and would reach beyond a row that is not; the split kernel stores four columns at a time.
+struct TileChoice {
+    int S;      // CTAs per cluster of the split kernel; 0: the persistent kernel
+    int BN;
+    bool two;   // persistent kernel: CTA pairs
+};
+
+inline TileChoice choose_tile(int64_t m_tiles, int64_t N, int64_t k_blocks, bool narrow_tiles, bool has_table, bool only64,
+                              bool whole_chunks, int sms)
+{
+    struct P { int BN; bool two; double base, kb; };
+    static const P persistent[6] = {{256, true, 4.6, 0.386}, {256, false, 5.1, 0.43}, {128, true, 4.2, 0.26},
+                                    {128, false, 3.6, 0.322}, {64, true, 3.6, 0.26},  {64, false, 3.2, 0.30}};
+    TileChoice best = {0, 0, false};
+    double best_t = 1e30;
+    for (const P& p : persistent) {
+        if (!whole_chunks || (!narrow_tiles && p.BN != 256) || (only64 && p.BN != 64) || (p.two && m_tiles < 2)) continue;
+        const int64_t tiles = (p.two ? (m_tiles + 1) / 2 : m_tiles) * ((N + p.BN - 1) / p.BN), slots = p.two ? sms / 2 : sms;
+        const double rounds = (double)((tiles + slots - 1) / slots);
+        const double epilogue = 3.6 * p.BN / 256, loop = p.kb * (double)k_blocks;
+        const double t = p.base + (has_table ? 1.8 * p.BN / 256 : 0.0) + rounds * (loop > epilogue ? loop : epilogue);
+        if (t < best_t * 0.97) { best_t = t; best = {0, p.BN, p.two}; }
+    }
+    for (int BN = 64; BN >= (only64 ? 64 : 32); BN /= 2) {
+        const int64_t tiles = m_tiles * ((N + BN - 1) / BN);
+        for (int S = 1; S <= 8 && S <= k_blocks; S *= 2) {
+            const int64_t n = tiles * S;
+            if (n > 2 * sms && (whole_chunks || S > 1 || n > 0x7fffffffLL)) break;
+            const double per = (double)((k_blocks + S - 1) / S), share = (double)n / sms;
+            const double t = 4.2 + (BN == 64 ? 0.32 : 0.24) * (per > 3 ? per - 3 : 0) * (share > 1 ? share : 1) +
+                             (S == 1 ? 0.0 : S == 2 ? 0.4 : S == 4 ? 1.0 : 1.8) + 0.5 * share * BN / 32 + (has_table ? 0.4 * BN / 64 : 0.0);
+            if (t < best_t * 0.97) { best_t = t; best = {S, BN, false}; }
+        }
+    }
+    return best;
+}
+
+template <typename InT, typename OutT, int BN, bool CONV>
+inline nm_status launch_split_kernel(nm_ctx* ctx, const CUtensorMap& tmA, const CUtensorMap& tmW, SplitArgs& s, double work,
+                                     cudaStream_t st)
+{
+    constexpr int STAGE_BYTES = A_BYTES + BN * ROW_BYTES;
+    const int per = (s.t.num_k_blocks + s.S - 1) / s.S;
+    constexpr int MIN_STAGES = (BM * part_pitch(BN) * 4 + STAGE_BYTES - 1) / STAGE_BYTES;   // the partial tile fits in the ring
+    static_assert(MIN_STAGES <= SPLIT_MAX_STAGES, "partial tile");
+    s.t.stages = per < MIN_STAGES ? MIN_STAGES : (per > SPLIT_MAX_STAGES ? SPLIT_MAX_STAGES : per);
+    const size_t smem = (size_t)s.t.stages * STAGE_BYTES + 1024;
+    auto kern = linear_split_kernel<InT, OutT, BN, CONV>;
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(SPLIT_MAX_STAGES * STAGE_BYTES + 1024)) !=
+        cudaSuccess)
+        return NM_ERR_CUDA;
+    cudaLaunchConfig_t cfg;
+    memset(&cfg, 0, sizeof(cfg));
+    cfg.gridDim = dim3((unsigned)(s.t.num_tiles * s.S));
+    cfg.blockDim = dim3(SPLIT_THREADS);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    cfg.attrs = attr;
+    cfg.numAttrs = split_launch_attrs(ctx, attr, s.S);
+    NmLaunchScope scope(ctx, NM_KERNEL_LINEAR_TC, work, st);
+    if (cudaLaunchKernelEx(&cfg, kern, tmA, tmW, s) != cudaSuccess) return NM_ERR_CUDA;
+    return cudaGetLastError() == cudaSuccess ? NM_OK : NM_ERR_CUDA;
+}
+
+}  // namespace nm_tc

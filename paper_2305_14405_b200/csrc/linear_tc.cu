@@ -1,10 +1,24 @@
-// Host side of the tensor-core linear operator: tile selection, tensor maps and launch of
-// linear_tc_kernel (linear_tc_kernel.cuh) for matrices in memory.
-#include "linear_tc_kernel.cuh"
+// Host side of the tensor-core linear operator: kernel and tile selection, tensor maps and launch of
+// linear_tc_kernel (linear_tc_kernel.cuh) or linear_split_kernel (linear_split_kernel.cuh) for matrices in memory.
+#include "linear_split_kernel.cuh"
 
 using namespace nm_tc;
 
 namespace {
+
+void fill_args(nm_ctx* ctx, const nm_linear_desc* d, TcArgs* a)
+{
+    memset(a, 0, sizeof(*a));
+    a->M = d->M; a->N = d->N; a->K = d->K;
+    a->bias = d->bias;
+    a->has_res = d->residual ? 1 : 0;
+    a->res_first = d->res_first;
+    a->tab = d->slot == NM_SLOT_NONE ? nullptr : ctx->d_tables + d->slot;
+    a->n_seg = d->slot == NM_SLOT_NONE ? 0 : ctx->h_tables[d->slot].n;
+    a->a_scale = d->a_scale; a->w_scale = d->w_scale; a->inv_out_scale = d->inv_out_scale;
+    a->acc_dump = d->acc_dump; a->idx_dump = d->idx_dump;
+    a->status = ctx->d_status;
+}
 
 template <typename InT, typename OutT, bool TWO, int BN>
 nm_status launch(nm_ctx* ctx, const nm_linear_desc* d, cudaStream_t st)
@@ -12,16 +26,7 @@ nm_status launch(nm_ctx* ctx, const nm_linear_desc* d, cudaStream_t st)
     constexpr int B_ROWS = TWO ? BN / 2 : BN;
     constexpr int TILE_M = TWO ? 2 * BM : BM;
     TcArgs a;
-    memset(&a, 0, sizeof(a));
-    a.M = d->M; a.N = d->N; a.K = d->K;
-    a.bias = d->bias;
-    a.has_res = d->residual ? 1 : 0;
-    a.res_first = d->res_first;
-    a.tab = d->slot == NM_SLOT_NONE ? nullptr : ctx->d_tables + d->slot;
-    a.n_seg = d->slot == NM_SLOT_NONE ? 0 : ctx->h_tables[d->slot].n;
-    a.a_scale = d->a_scale; a.w_scale = d->w_scale; a.inv_out_scale = d->inv_out_scale;
-    a.acc_dump = d->acc_dump; a.idx_dump = d->idx_dump;
-    a.status = ctx->d_status;
+    fill_args(ctx, d, &a);
     const int bk = ROW_BYTES / (int)sizeof(InT);
     const int64_t m_tiles = (d->M + TILE_M - 1) / TILE_M;
     a.num_n_tiles = (int)((d->N + BN - 1) / BN);
@@ -46,22 +51,48 @@ nm_status launch(nm_ctx* ctx, const nm_linear_desc* d, cudaStream_t st)
 }
 
 template <typename InT, typename OutT, int BN>
-nm_status launch_two(nm_ctx* ctx, const nm_linear_desc* d, cudaStream_t st)
+nm_status launch_split(nm_ctx* ctx, const nm_linear_desc* d, int S, cudaStream_t st)
 {
-    // algo 3 forces the one-CTA tile; otherwise problems with at least one 256-row tile use CTA pairs
-    if (d->algo != 3 && d->M >= 256) return launch<InT, OutT, true, BN>(ctx, d, st);
-    return launch<InT, OutT, false, BN>(ctx, d, st);
+    const int bk = ROW_BYTES / (int)sizeof(InT);
+    const int64_t k_blocks = (d->K + bk - 1) / bk, n_tiles = (d->N + BN - 1) / BN, tiles = (d->M + BM - 1) / BM * n_tiles;
+    SplitArgs s;
+    memset(&s, 0, sizeof(s));
+    s.S = S;
+    fill_args(ctx, d, &s.t);
+    s.t.num_n_tiles = (int)n_tiles;
+    s.t.num_tiles = (int)tiles;
+    s.t.num_k_blocks = (int)k_blocks;
+    s.residual = d->residual; s.ldr = d->ldr;
+    s.out = d->out; s.ldo = d->ldo;
+    CUtensorMap tmA, tmW;
+    nm_status e = make_tmap(ctx, &tmA, d->A, d->in_dtype, d->M, d->K, d->lda, BM);
+    if (e != NM_OK) return e;
+    e = make_tmap(ctx, &tmW, d->W, d->in_dtype, d->N, d->K, d->ldw, BN);
+    if (e != NM_OK) return e;
+    return launch_split_kernel<InT, OutT, BN, false>(ctx, tmA, tmW, s, 2.0 * (double)d->M * (double)d->N * (double)d->K, st);
 }
 
 template <typename InT, typename OutT>
 nm_status launch_sel(nm_ctx* ctx, const nm_linear_desc* d, cudaStream_t st)
 {
-    // narrow layers get a narrow tile (built for the 16-bit types)
-    if constexpr (!TcIn<InT>::is_int) {
-        if (d->N <= 64) return launch_two<InT, OutT, 64>(ctx, d, st);
-        if (d->N <= 128) return launch_two<InT, OutT, 128>(ctx, d, st);
+    constexpr bool NARROW = !TcIn<InT>::is_int;   // tiles of 64 and 128 columns are built for the 16-bit types
+    const int bk = ROW_BYTES / (int)sizeof(InT);
+    const int64_t m_tiles = (d->M + BM - 1) / BM, k_blocks = (d->K + bk - 1) / bk;
+    TileChoice c;
+    if (d->algo == 0) c = choose_tile(m_tiles, d->N, k_blocks, NARROW, d->slot != NM_SLOT_NONE, false, d->N * sizeof(OutT) % 16 == 0,
+                                      ctx->sm_count);
+    else {
+        // a forced kernel: by width alone; algo 3 asks for one CTA per tile, otherwise CTA pairs from one 256-row tile on
+        c.S = 0;
+        c.BN = NARROW && d->N <= 64 ? 64 : (NARROW && d->N <= 128 ? 128 : 256);
+        c.two = d->algo != 3 && d->M >= 256;
     }
-    return launch_two<InT, OutT, 256>(ctx, d, st);
+    if (c.S) return c.BN == 32 ? launch_split<InT, OutT, 32>(ctx, d, c.S, st) : launch_split<InT, OutT, 64>(ctx, d, c.S, st);
+    if constexpr (NARROW) {
+        if (c.BN == 64) return c.two ? launch<InT, OutT, true, 64>(ctx, d, st) : launch<InT, OutT, false, 64>(ctx, d, st);
+        if (c.BN == 128) return c.two ? launch<InT, OutT, true, 128>(ctx, d, st) : launch<InT, OutT, false, 128>(ctx, d, st);
+    }
+    return c.two ? launch<InT, OutT, true, 256>(ctx, d, st) : launch<InT, OutT, false, 256>(ctx, d, st);
 }
 
 }  // namespace
