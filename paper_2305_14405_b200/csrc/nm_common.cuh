@@ -48,6 +48,7 @@ struct nm_ctx {
     void* static_ws;           // device address of the library's fixed scratch array on this device (or null)
     void* d_pool_w;            // 64 x 64 matrix (1/HW on the diagonal) of the average pool run as a GEMM; 8 KB
     int pool_w_hw, pool_w_dtype;   // what d_pool_w currently holds (0 = nothing)
+    int f32_resident[9];       // clusters of 1..8 CTAs of the fp32 linear kernel the device holds; [0]: asked yet?
 };
 
 // Brackets one kernel launch with events when profiling is on; counts the launch always.
@@ -654,9 +655,13 @@ nm_status nm_launch_wait_selftest(nm_ctx* ctx, long long limit_cycles, cudaStrea
 nm_status nm_launch_quantize(nm_ctx* ctx, const void* x, nm_dtype dtype, int64_t count, float inv_scale,
                              int8_t* q, cudaStream_t st);
 nm_status nm_launch_linear_simt(nm_ctx* ctx, const nm_linear_desc* d, cudaStream_t st);
+nm_status nm_launch_linear_f32(nm_ctx* ctx, const nm_linear_desc* d, cudaStream_t st);
+bool nm_linear_f32_supported(const nm_linear_desc* d);   // fp32, N a multiple of 4; linear_simt takes the rest
 nm_status nm_launch_linear_tc(nm_ctx* ctx, const nm_linear_desc* d, cudaStream_t st);
 bool nm_linear_tc_supported(const nm_linear_desc* d);
 nm_status nm_launch_attention_simt(nm_ctx* ctx, const nm_attn_desc* d, cudaStream_t st);
+nm_status nm_launch_attention_f32(nm_ctx* ctx, const nm_attn_desc* d, cudaStream_t st);
+bool nm_attention_f32_supported(const nm_attn_desc* d);   // fp32, heads of 64 channels, scores that fit shared memory
 nm_status nm_launch_attention_tc(nm_ctx* ctx, const nm_attn_desc* d, cudaStream_t st);
 bool nm_attention_tc_supported(const nm_attn_desc* d);
 // out_q != nullptr: the output is written as int8 codes (of the value rounded to the storage type) to out_q
