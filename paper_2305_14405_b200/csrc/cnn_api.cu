@@ -92,6 +92,13 @@ size_t nm_conv2d_workspace_bytes(const nm_conv_desc* d)
 
 nm_status nm_conv2d_pwl(nm_ctx* ctx, const nm_conv_desc* d, void* workspace, size_t ws_bytes, void* stream)
 {
+    return nm_conv2d_dispatch(ctx, d, workspace, ws_bytes, (cudaStream_t)stream, NmChain());
+}
+
+}  // extern "C"
+
+nm_status nm_conv2d_dispatch(nm_ctx* ctx, const nm_conv_desc* d, void* workspace, size_t ws_bytes, cudaStream_t st, NmChain chain)
+{
     if (!ctx || !d) return NM_ERR_INVALID_ARG;
     ConvGeom g;
     if (!conv_geom(d, &g)) return NM_ERR_SHAPE;
@@ -106,7 +113,6 @@ nm_status nm_conv2d_pwl(nm_ctx* ctx, const nm_conv_desc* d, void* workspace, siz
         if (!workspace || ws_bytes < need) return NM_ERR_WORKSPACE;
         if (((uintptr_t)workspace & 255u) != 0) return NM_ERR_ALIGNMENT;
     }
-    cudaStream_t st = (cudaStream_t)stream;
     if (g.path == CONV_IMPLICIT || g.path == CONV_ROWTAP) {
         NmConvTc c;
         memset(&c, 0, sizeof(c));
@@ -141,7 +147,8 @@ nm_status nm_conv2d_pwl(nm_ctx* ctx, const nm_conv_desc* d, void* workspace, siz
             c.taps_y = d->kh; c.taps_x = 1; c.cblocks = 1;
             c.w = wp; c.ldw = (int64_t)d->kh * 64; c.Ktot = (int64_t)d->kh * 64;
         }
-        return nm_launch_conv_tc(ctx, &c, st);
+        if (g.path != CONV_IMPLICIT) chain.weights_ready = false;   // wp comes from a kernel just launched
+        return nm_launch_conv_tc(ctx, &c, st, chain);
     }
     const void* A = d->x;
     const void* Wm = d->w;
@@ -168,8 +175,11 @@ nm_status nm_conv2d_pwl(nm_ctx* ctx, const nm_conv_desc* d, void* workspace, siz
     ld.bias = d->bias; ld.residual = d->residual; ld.ldr = d->Cout;
     ld.slot = d->slot; ld.out = d->out; ld.ldo = d->Cout;
     ld.algo = d->algo; ld.res_first = d->res_first;
-    return nm_linear_pwl(ctx, &ld, stream);
+    if (g.path == CONV_GATHER && g.pad_w) chain.weights_ready = false;   // Wm comes from the kernel just launched
+    return nm_linear_dispatch(ctx, &ld, st, chain);
 }
+
+extern "C" {
 
 nm_status nm_maxpool2d(nm_ctx* ctx, const void* x, void* y, nm_dtype dtype, int32_t N, int32_t H, int32_t W, int32_t C,
                        int32_t ks, int32_t stride, int32_t pad, void* stream)
@@ -296,8 +306,13 @@ nm_status nm_resnet50_forward(nm_ctx* ctx, const nm_conv_params* convs, const vo
         d.x = in; d.w = convs[ci].w; d.bias = convs[ci].bias;
         d.residual = res; d.slot = cfg->relu_slot; d.res_first = res_first; d.out = out; d.algo = cfg->algo;
         ++ci;
-        return nm_conv2d_pwl(ctx, &d, gather_buf, gather, stream);
+        // the max-pool, launched without early start, lies between everything before this call and the convolutions behind it
+        NmChain chain;
+        chain.weights_ready = ci > 1;
+        return nm_conv2d_dispatch(ctx, &d, gather_buf, gather, (cudaStream_t)stream, chain);
     };
+    NmChain ready;
+    ready.weights_ready = true;
 
     // stem: 7x7/2 convolution + ReLU, 3x3/2 max-pool
     nm_status s = conv(x, 224, 224, 3, base, 7, 2, 3, nullptr, 0, buf[0]);
@@ -332,7 +347,7 @@ nm_status nm_resnet50_forward(nm_ctx* ctx, const nm_conv_params* convs, const vo
                 d.N = Nb; d.H = H; d.W = H; d.Cin = Cin; d.Cout = Cout; d.kh = 1; d.kw = 1; d.stride = stride; d.pad = 0;
                 d.dtype = cfg->dtype; d.x = buf[cur]; d.w = pd.w; d.bias = pd.bias; d.slot = NM_SLOT_NONE; d.out = sc;
                 d.algo = cfg->algo;
-                s = nm_conv2d_pwl(ctx, &d, gather_buf, gather, stream);
+                s = nm_conv2d_dispatch(ctx, &d, gather_buf, gather, (cudaStream_t)stream, ready);
                 if (s != NM_OK) return s;
                 shortcut = sc;
                 --ci;
@@ -343,7 +358,7 @@ nm_status nm_resnet50_forward(nm_ctx* ctx, const nm_conv_params* convs, const vo
                 d.N = Nb; d.H = Ho; d.W = Ho; d.Cin = width; d.Cout = Cout; d.kh = 1; d.kw = 1; d.stride = 1; d.pad = 0;
                 d.dtype = cfg->dtype; d.x = t2; d.w = pc.w; d.bias = pc.bias; d.residual = shortcut;
                 d.slot = cfg->relu_slot; d.res_first = 1; d.out = t1; d.algo = cfg->algo;
-                s = nm_conv2d_pwl(ctx, &d, gather_buf, gather, stream);
+                s = nm_conv2d_dispatch(ctx, &d, gather_buf, gather, (cudaStream_t)stream, ready);
                 if (s != NM_OK) return s;
             }
             ci += (b == 0) ? 2 : 1;
@@ -362,7 +377,7 @@ nm_status nm_resnet50_forward(nm_ctx* ctx, const nm_conv_params* convs, const vo
     ld.in_dtype = cfg->dtype; ld.out_dtype = cfg->dtype;
     ld.A = pool_buf; ld.lda = feat; ld.W = fc_w; ld.ldw = feat; ld.bias = fc_b;
     ld.slot = NM_SLOT_NONE; ld.out = logits; ld.ldo = cfg->num_classes; ld.algo = cfg->algo;
-    return nm_linear_pwl(ctx, &ld, stream);
+    return nm_linear_dispatch(ctx, &ld, (cudaStream_t)stream, ready);
 }
 
 nm_status nm_resnet50_forward_host_async(nm_ctx* ctx, const nm_conv_params* convs, const void* fc_w,

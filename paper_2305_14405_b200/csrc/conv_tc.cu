@@ -40,7 +40,7 @@ void choose_patch(int Wo, int Ho, int N, int* TW, int* TH, int* NB)
 }
 
 // Patch geometry and epilogue operands common to both kernels; returns the number of patches.
-int64_t fill_args(nm_ctx* ctx, const NmConvTc* c, TcArgs* a)
+int64_t fill_args(nm_ctx* ctx, const NmConvTc* c, NmChain chain, TcArgs* a)
 {
     memset(a, 0, sizeof(*a));
     ConvDev& cv = a->cv;
@@ -58,6 +58,8 @@ int64_t fill_args(nm_ctx* ctx, const NmConvTc* c, TcArgs* a)
     a->tab = c->slot == NM_SLOT_NONE ? nullptr : ctx->d_tables + c->slot;
     a->n_seg = c->slot == NM_SLOT_NONE ? 0 : ctx->h_tables[c->slot].n;
     a->status = ctx->d_status;
+    a->weights_ready = chain.weights_ready && !c->depthwise;
+    a->late_trigger = chain.late_trigger;
     a->num_k_blocks = c->taps_y * c->taps_x * c->cblocks;
     return (int64_t)cv.tiles_x * cv.tiles_y * ceil_div(c->N, cv.NB);
 }
@@ -72,11 +74,11 @@ nm_status make_tmap_a(nm_ctx* ctx, CUtensorMap* m, const NmConvTc* c, const Conv
 }
 
 template <typename T, int BN>
-nm_status launch_split(nm_ctx* ctx, const NmConvTc* c, int S, cudaStream_t st)
+nm_status launch_split(nm_ctx* ctx, const NmConvTc* c, int S, NmChain chain, cudaStream_t st)
 {
     SplitArgs s;
     memset(&s, 0, sizeof(s));
-    const int64_t patches = fill_args(ctx, c, &s.t);
+    const int64_t patches = fill_args(ctx, c, chain, &s.t);
     s.t.num_n_tiles = ceil_div(c->Cout, BN);
     const int64_t tiles = patches * s.t.num_n_tiles;
     s.S = S;
@@ -93,11 +95,11 @@ nm_status launch_split(nm_ctx* ctx, const NmConvTc* c, int S, cudaStream_t st)
 }
 
 template <typename T, bool TWO, int BN>
-nm_status launch(nm_ctx* ctx, const NmConvTc* c, cudaStream_t st)
+nm_status launch(nm_ctx* ctx, const NmConvTc* c, NmChain chain, cudaStream_t st)
 {
     constexpr int B_ROWS = TWO ? BN / 2 : BN;
     TcArgs a;
-    const int64_t patches = fill_args(ctx, c, &a);
+    const int64_t patches = fill_args(ctx, c, chain, &a);
     const ConvDev& cv = a.cv;
     const int64_t m_tiles = TWO ? (patches + 1) / 2 : patches;
     a.num_n_tiles = ceil_div(c->Cout, BN);
@@ -128,7 +130,7 @@ nm_status launch(nm_ctx* ctx, const NmConvTc* c, cudaStream_t st)
 }
 
 template <typename T>
-nm_status launch_sel(nm_ctx* ctx, const NmConvTc* c, cudaStream_t st)
+nm_status launch_sel(nm_ctx* ctx, const NmConvTc* c, NmChain chain, cudaStream_t st)
 {
     TileChoice t;
     if (c->algo == 0) {
@@ -142,17 +144,17 @@ nm_status launch_sel(nm_ctx* ctx, const NmConvTc* c, cudaStream_t st)
         t.BN = c->Cout <= 64 || c->depthwise ? 64 : (c->Cout <= 128 ? 128 : 256);
         t.two = c->algo != 3 && (int64_t)c->N * c->Ho * c->Wo >= 256;
     }
-    if (t.S) return t.BN == 32 ? launch_split<T, 32>(ctx, c, t.S, st) : launch_split<T, 64>(ctx, c, t.S, st);
-    if (t.BN == 64) return t.two ? launch<T, true, 64>(ctx, c, st) : launch<T, false, 64>(ctx, c, st);
-    if (t.BN == 128) return t.two ? launch<T, true, 128>(ctx, c, st) : launch<T, false, 128>(ctx, c, st);
-    return t.two ? launch<T, true, 256>(ctx, c, st) : launch<T, false, 256>(ctx, c, st);
+    if (t.S) return t.BN == 32 ? launch_split<T, 32>(ctx, c, t.S, chain, st) : launch_split<T, 64>(ctx, c, t.S, chain, st);
+    if (t.BN == 64) return t.two ? launch<T, true, 64>(ctx, c, chain, st) : launch<T, false, 64>(ctx, c, chain, st);
+    if (t.BN == 128) return t.two ? launch<T, true, 128>(ctx, c, chain, st) : launch<T, false, 128>(ctx, c, chain, st);
+    return t.two ? launch<T, true, 256>(ctx, c, chain, st) : launch<T, false, 256>(ctx, c, chain, st);
 }
 
 }  // namespace
 
-nm_status nm_launch_conv_tc(nm_ctx* ctx, const NmConvTc* c, cudaStream_t st)
+nm_status nm_launch_conv_tc(nm_ctx* ctx, const NmConvTc* c, cudaStream_t st, NmChain chain)
 {
-    if (c->dtype == NM_F16) return launch_sel<__half>(ctx, c, st);
-    if (c->dtype == NM_BF16) return launch_sel<__nv_bfloat16>(ctx, c, st);
+    if (c->dtype == NM_F16) return launch_sel<__half>(ctx, c, chain, st);
+    if (c->dtype == NM_BF16) return launch_sel<__nv_bfloat16>(ctx, c, chain, st);
     return NM_ERR_UNSUPPORTED;
 }

@@ -283,15 +283,30 @@ linear_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     nm_tc_fence_after();
     const uint32_t tmem = tmem_slot;
     volatile int* abortp = &abort_flag;
-    nm_grid_launch_dependents();
-
+    if (!a.late_trigger) nm_grid_launch_dependents();
+    // Weights that were complete before the previous kernel started need not wait for it: this CTA's share goes into the
+    // ring's stages and, beyond those, into L2 while that kernel still runs.
+    int early = 0;   // K-blocks whose W tile is on its way
+    if (a.weights_ready && warp == 0) {
+        early = kb1 - kb0 < stages ? kb1 - kb0 : stages;
+        if (nm_elect_one()) {
+            for (int i = 0; i < early; ++i) {
+                nm_mbar_expect_tx(&bar_full[i], STAGE_BYTES);
+                nm_tma_load_2d(tiles + (size_t)i * STAGE_BYTES + A_BYTES, &tmW, (kb0 + i) * BK_ELEMS, nt * BN, &bar_full[i]);
+            }
+            for (int kb = kb0 + early; kb < kb1; ++kb) nm_tma_prefetch_2d(&tmW, kb * BK_ELEMS, nt * BN);
+        }
+        __syncwarp();
+    }
     Patch pt = {0, 0, 0};
     if constexpr (CONV) pt = patch_of(a.cv, mt);
     const int rows = CONV ? BM : (int)(a.M - (int64_t)mt * BM < BM ? a.M - (int64_t)mt * BM : BM);
     Finisher<INT, OutT, BN, CONV, SPLIT_THREADS> fin(s, rank, mt, nt, rows, pt);
     bool ok = true;
+    if (a.weights_ready) fin.prefetch_vectors();
     nm_grid_dependency_wait();
-    fin.prefetch_vectors();
+    if (a.late_trigger) nm_grid_launch_dependents();
+    if (!a.weights_ready) fin.prefetch_vectors();
     if (warp != 0) fin.load_res(0);
     if (warp == 0) {
         // ------------------------------------------------ TMA producer (all lanes run, one elected lane issues)
@@ -319,10 +334,10 @@ linear_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                 if (++cb == a.cv.cblocks) { cb = 0; ++tap; }
             }
             if (nm_elect_one()) {
-                nm_mbar_expect_tx(&bar_full[stage], STAGE_BYTES);
+                if (kb - kb0 >= early) nm_mbar_expect_tx(&bar_full[stage], STAGE_BYTES);
                 if constexpr (CONV) nm_tma_load_4d(sa, &tmA, c_c, c_w, c_h, pt.img0, &bar_full[stage]);
                 else nm_tma_load_2d(sa, &tmA, kb * BK_ELEMS, mt * BM, &bar_full[stage]);
-                nm_tma_load_2d(sa + A_BYTES, &tmW, w_k, w_n, &bar_full[stage]);
+                if (kb - kb0 >= early) nm_tma_load_2d(sa + A_BYTES, &tmW, w_k, w_n, &bar_full[stage]);
             }
             __syncwarp();
             if (++stage == stages) { stage = 0; phase ^= 1u; }
@@ -438,6 +453,7 @@ inline TileChoice choose_tile(int64_t m_tiles, int64_t N, int64_t k_blocks, bool
     double best_t = 1e30;
     for (const P& p : persistent) {
         if (!whole_chunks || (!narrow_tiles && p.BN != 256) || (only64 && p.BN != 64) || (p.two && m_tiles < 2)) continue;
+        if (narrow_tiles && p.BN > 64 && N <= p.BN / 2) continue;   // half the tile would be padding
         const int64_t tiles = (p.two ? (m_tiles + 1) / 2 : m_tiles) * ((N + p.BN - 1) / p.BN), slots = p.two ? sms / 2 : sms;
         const double rounds = (double)((tiles + slots - 1) / slots);
         const double epilogue = 3.6 * p.BN / 256, loop = p.kb * (double)k_blocks;

@@ -6,7 +6,7 @@ using namespace nm_tc;
 
 namespace {
 
-void fill_args(nm_ctx* ctx, const nm_linear_desc* d, TcArgs* a)
+void fill_args(nm_ctx* ctx, const nm_linear_desc* d, NmChain chain, TcArgs* a)
 {
     memset(a, 0, sizeof(*a));
     a->M = d->M; a->N = d->N; a->K = d->K;
@@ -18,15 +18,17 @@ void fill_args(nm_ctx* ctx, const nm_linear_desc* d, TcArgs* a)
     a->a_scale = d->a_scale; a->w_scale = d->w_scale; a->inv_out_scale = d->inv_out_scale;
     a->acc_dump = d->acc_dump; a->idx_dump = d->idx_dump;
     a->status = ctx->d_status;
+    a->weights_ready = chain.weights_ready;
+    a->late_trigger = chain.late_trigger;
 }
 
 template <typename InT, typename OutT, bool TWO, int BN>
-nm_status launch(nm_ctx* ctx, const nm_linear_desc* d, cudaStream_t st)
+nm_status launch(nm_ctx* ctx, const nm_linear_desc* d, NmChain chain, cudaStream_t st)
 {
     constexpr int B_ROWS = TWO ? BN / 2 : BN;
     constexpr int TILE_M = TWO ? 2 * BM : BM;
     TcArgs a;
-    fill_args(ctx, d, &a);
+    fill_args(ctx, d, chain, &a);
     const int bk = ROW_BYTES / (int)sizeof(InT);
     const int64_t m_tiles = (d->M + TILE_M - 1) / TILE_M;
     a.num_n_tiles = (int)((d->N + BN - 1) / BN);
@@ -51,14 +53,14 @@ nm_status launch(nm_ctx* ctx, const nm_linear_desc* d, cudaStream_t st)
 }
 
 template <typename InT, typename OutT, int BN>
-nm_status launch_split(nm_ctx* ctx, const nm_linear_desc* d, int S, cudaStream_t st)
+nm_status launch_split(nm_ctx* ctx, const nm_linear_desc* d, int S, NmChain chain, cudaStream_t st)
 {
     const int bk = ROW_BYTES / (int)sizeof(InT);
     const int64_t k_blocks = (d->K + bk - 1) / bk, n_tiles = (d->N + BN - 1) / BN, tiles = (d->M + BM - 1) / BM * n_tiles;
     SplitArgs s;
     memset(&s, 0, sizeof(s));
     s.S = S;
-    fill_args(ctx, d, &s.t);
+    fill_args(ctx, d, chain, &s.t);
     s.t.num_n_tiles = (int)n_tiles;
     s.t.num_tiles = (int)tiles;
     s.t.num_k_blocks = (int)k_blocks;
@@ -73,7 +75,7 @@ nm_status launch_split(nm_ctx* ctx, const nm_linear_desc* d, int S, cudaStream_t
 }
 
 template <typename InT, typename OutT>
-nm_status launch_sel(nm_ctx* ctx, const nm_linear_desc* d, cudaStream_t st)
+nm_status launch_sel(nm_ctx* ctx, const nm_linear_desc* d, NmChain chain, cudaStream_t st)
 {
     constexpr bool NARROW = !TcIn<InT>::is_int;   // tiles of 64 and 128 columns are built for the 16-bit types
     const int bk = ROW_BYTES / (int)sizeof(InT);
@@ -87,12 +89,12 @@ nm_status launch_sel(nm_ctx* ctx, const nm_linear_desc* d, cudaStream_t st)
         c.BN = NARROW && d->N <= 64 ? 64 : (NARROW && d->N <= 128 ? 128 : 256);
         c.two = d->algo != 3 && d->M >= 256;
     }
-    if (c.S) return c.BN == 32 ? launch_split<InT, OutT, 32>(ctx, d, c.S, st) : launch_split<InT, OutT, 64>(ctx, d, c.S, st);
+    if (c.S) return c.BN == 32 ? launch_split<InT, OutT, 32>(ctx, d, c.S, chain, st) : launch_split<InT, OutT, 64>(ctx, d, c.S, chain, st);
     if constexpr (NARROW) {
-        if (c.BN == 64) return c.two ? launch<InT, OutT, true, 64>(ctx, d, st) : launch<InT, OutT, false, 64>(ctx, d, st);
-        if (c.BN == 128) return c.two ? launch<InT, OutT, true, 128>(ctx, d, st) : launch<InT, OutT, false, 128>(ctx, d, st);
+        if (c.BN == 64) return c.two ? launch<InT, OutT, true, 64>(ctx, d, chain, st) : launch<InT, OutT, false, 64>(ctx, d, chain, st);
+        if (c.BN == 128) return c.two ? launch<InT, OutT, true, 128>(ctx, d, chain, st) : launch<InT, OutT, false, 128>(ctx, d, chain, st);
     }
-    return c.two ? launch<InT, OutT, true, 256>(ctx, d, st) : launch<InT, OutT, false, 256>(ctx, d, st);
+    return c.two ? launch<InT, OutT, true, 256>(ctx, d, chain, st) : launch<InT, OutT, false, 256>(ctx, d, chain, st);
 }
 
 }  // namespace
@@ -108,16 +110,16 @@ bool nm_linear_tc_supported(const nm_linear_desc* d)
     return d->out_dtype == d->in_dtype;
 }
 
-nm_status nm_launch_linear_tc(nm_ctx* ctx, const nm_linear_desc* d, cudaStream_t st)
+nm_status nm_launch_linear_tc(nm_ctx* ctx, const nm_linear_desc* d, cudaStream_t st, NmChain chain)
 {
     if (!nm_linear_tc_supported(d)) return NM_ERR_UNSUPPORTED;
     switch (d->in_dtype) {
-    case NM_BF16: return launch_sel<__nv_bfloat16, __nv_bfloat16>(ctx, d, st);
-    case NM_F16: return launch_sel<__half, __half>(ctx, d, st);
+    case NM_BF16: return launch_sel<__nv_bfloat16, __nv_bfloat16>(ctx, d, chain, st);
+    case NM_F16: return launch_sel<__half, __half>(ctx, d, chain, st);
     case NM_I8:
-        if (d->out_dtype == NM_BF16) return launch_sel<int8_t, __nv_bfloat16>(ctx, d, st);
-        if (d->out_dtype == NM_F32) return launch_sel<int8_t, float>(ctx, d, st);
-        return launch_sel<int8_t, int8_t>(ctx, d, st);
+        if (d->out_dtype == NM_BF16) return launch_sel<int8_t, __nv_bfloat16>(ctx, d, chain, st);
+        if (d->out_dtype == NM_F32) return launch_sel<int8_t, float>(ctx, d, chain, st);
+        return launch_sel<int8_t, int8_t>(ctx, d, chain, st);
     default: return NM_ERR_UNSUPPORTED;
     }
 }

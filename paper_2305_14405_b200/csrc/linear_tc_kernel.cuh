@@ -71,6 +71,7 @@ struct TcArgs {
     int32_t* idx_dump;
     int* status;
     int num_n_tiles, num_tiles, num_k_blocks, stages, n_seg;
+    int weights_ready, late_trigger;   // NmChain
     ConvDev cv;
 };
 
@@ -260,8 +261,9 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     volatile int* abortp = &abort_flag;
     // set-up done: the next kernel in the stream may begin its own set-up; nothing produced by the
     // previous kernel has been touched yet, everything below may depend on it
-    nm_grid_launch_dependents();
+    if (!a.late_trigger) nm_grid_launch_dependents();
     nm_grid_dependency_wait();
+    if (a.late_trigger) nm_grid_launch_dependents();
 
     if (warp == 0) {
         // ------------------------------------------------ TMA producer

@@ -294,6 +294,13 @@ nm_status nm_pwl_apply(nm_ctx* ctx, int slot, const void* x, void* y, int64_t co
 
 nm_status nm_linear_pwl(nm_ctx* ctx, const nm_linear_desc* d, void* stream)
 {
+    return nm_linear_dispatch(ctx, d, (cudaStream_t)stream, NmChain());
+}
+
+}  // extern "C"
+
+nm_status nm_linear_dispatch(nm_ctx* ctx, const nm_linear_desc* d, cudaStream_t st, NmChain chain)
+{
     if (!ctx || !d) return NM_ERR_INVALID_ARG;
     if (d->M < 0 || d->N < 0 || d->K < 0) return NM_ERR_SHAPE;
     if (d->slot != NM_SLOT_NONE) {
@@ -321,15 +328,16 @@ nm_status nm_linear_pwl(nm_ctx* ctx, const nm_linear_desc* d, void* stream)
         if (d->out_dtype != d->in_dtype) return NM_ERR_UNSUPPORTED;
         if (d->acc_dump) return NM_ERR_UNSUPPORTED;
     }
-    cudaStream_t st = (cudaStream_t)stream;
     if (d->algo <= 1 && nm_linear_f32_supported(d)) return nm_launch_linear_f32(ctx, d, st);
     if (d->algo == 1) return nm_launch_linear_simt(ctx, d, st);
     const bool tc = nm_linear_tc_supported(d);
-    if (d->algo == 2 || d->algo == 3) return tc ? nm_launch_linear_tc(ctx, d, st) : NM_ERR_UNSUPPORTED;
+    if (d->algo == 2 || d->algo == 3) return tc ? nm_launch_linear_tc(ctx, d, st, chain) : NM_ERR_UNSUPPORTED;
     // (narrow matrices of more rows than the CUDA-core kernel's grid takes have always been refused)
     if (d->N < 64 && (d->M + 63) / 64 > 65535) return NM_ERR_SHAPE;
-    return tc ? nm_launch_linear_tc(ctx, d, st) : nm_launch_linear_simt(ctx, d, st);
+    return tc ? nm_launch_linear_tc(ctx, d, st, chain) : nm_launch_linear_simt(ctx, d, st);
 }
+
+extern "C" {
 
 // out_q != nullptr asks for the output as int8 codes in out_q instead of d->out; *fused tells whether the
 // kernel chosen could do that (the caller quantises d->out itself otherwise).
@@ -507,17 +515,17 @@ size_t nm_encoder_workspace_bytes(const nm_encoder_cfg* cfg)
 // layer's LN2 leaves those of the next (`next_a_x` > 0: the next layer's input scale).
 static nm_status encoder_layer_impl(nm_ctx* ctx, const nm_encoder_weights* w, const nm_encoder_cfg* c, const void* x,
                                     void* y, void* workspace, size_t ws_bytes, void* stream, bool in_codes_ready,
-                                    float next_a_x);
+                                    float next_a_x, bool first_of_call);
 
 nm_status nm_encoder_layer(nm_ctx* ctx, const nm_encoder_weights* w, const nm_encoder_cfg* c, const void* x, void* y,
                            void* workspace, size_t ws_bytes, void* stream)
 {
-    return encoder_layer_impl(ctx, w, c, x, y, workspace, ws_bytes, stream, false, 0.f);
+    return encoder_layer_impl(ctx, w, c, x, y, workspace, ws_bytes, stream, false, 0.f, true);
 }
 
 static nm_status encoder_layer_impl(nm_ctx* ctx, const nm_encoder_weights* w, const nm_encoder_cfg* c, const void* x,
                                     void* y, void* workspace, size_t ws_bytes, void* stream, bool in_codes_ready,
-                                    float next_a_x)
+                                    float next_a_x, bool first_of_call)
 {
     if (!ctx || !w || !c || !x || !y) return NM_ERR_INVALID_ARG;
     EncLayout lo;
@@ -538,6 +546,11 @@ static nm_status encoder_layer_impl(nm_ctx* ctx, const nm_encoder_weights* w, co
     void* g = ws + lo.g;
     int8_t* q8 = (int8_t*)(ws + lo.q8a);
     nm_status s;
+    // The first linear kernel of the call holds its successors back until what the caller enqueued before is complete;
+    // from the second on the weights may be fetched early.
+    NmChain chain;
+    chain.weights_ready = !first_of_call;
+    chain.late_trigger = first_of_call;
 
     auto linear = [&](const void* A, int64_t K, const void* W, int64_t N, const float* bias, const void* res,
                       int slot, void* out, nm_dtype out_dt, float a_scale, const float* w_scale,
@@ -552,7 +565,10 @@ static nm_status encoder_layer_impl(nm_ctx* ctx, const nm_encoder_weights* w, co
         ld.slot = slot; ld.out = out; ld.ldo = N;
         ld.a_scale = a_scale; ld.w_scale = w_scale; ld.inv_out_scale = inv_out_scale;
         ld.algo = c->algo;
-        return nm_linear_pwl(ctx, &ld, stream);
+        const nm_status e = nm_linear_dispatch(ctx, &ld, (cudaStream_t)stream, chain);
+        chain.weights_ready = true;
+        chain.late_trigger = false;
+        return e;
     };
 
     // qkv = x Wqkv^T + bqkv
@@ -604,9 +620,9 @@ static nm_status encoder_layer_impl(nm_ctx* ctx, const nm_encoder_weights* w, co
     // y = LN2(x1 + g W2^T + b2)
     s = linear(g, F, w->W2, H, w->b2, x1, NM_SLOT_NONE, z, act, w->a_g, w->s_w2, 0.f);
     if (s != NM_OK) return s;
-    const bool chain = i8 && next_a_x > 0.f;
-    return layernorm_checked(ctx, z, w->g2, w->be2, y, T, H, c->eps, c->rsqrt_slot, act, stream, chain ? q8 : nullptr,
-                             chain ? 1.0f / next_a_x : 0.f);
+    const bool next_codes = i8 && next_a_x > 0.f;
+    return layernorm_checked(ctx, z, w->g2, w->be2, y, T, H, c->eps, c->rsqrt_slot, act, stream, next_codes ? q8 : nullptr,
+                             next_codes ? 1.0f / next_a_x : 0.f);
 }
 
 nm_status nm_encoder_stack(nm_ctx* ctx, const nm_encoder_weights* layers, int32_t n_layers, const nm_encoder_cfg* c,
@@ -626,7 +642,8 @@ nm_status nm_encoder_stack(nm_ctx* ctx, const nm_encoder_weights* layers, int32_
         void* out = to_y ? y : pp;
         // int8: LN2 of layer l leaves the codes of layer l+1's input in the workspace
         const float next_a_x = (c->dtype == NM_I8 && l + 1 < n_layers) ? layers[l + 1].a_x : 0.f;
-        nm_status s = encoder_layer_impl(ctx, &layers[l], c, in, out, workspace, ws_bytes, stream, codes_ready, next_a_x);
+        nm_status s = encoder_layer_impl(ctx, &layers[l], c, in, out, workspace, ws_bytes, stream, codes_ready, next_a_x,
+                                         l == 0);
         codes_ready = next_a_x > 0.f;
         if (s != NM_OK) return s;
         in = out;

@@ -297,6 +297,12 @@ __device__ __forceinline__ void nm_tma_store_4d(const CUtensorMap* tmap, const v
     asm volatile("cp.async.bulk.commit_group;" ::: "memory");
 }
 
+// The same 2-D box brought into L2 only.
+__device__ __forceinline__ void nm_tma_prefetch_2d(const CUtensorMap* tmap, int c0, int c1)
+{
+    asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global [%0, {%1, %2}];" ::"l"(tmap), "r"(c0), "r"(c1) : "memory");
+}
+
 // TMA: 2-D tiled store shared -> global as one bulk group; parts of the box beyond the
 // tensor's extents are not written.  c0 (innermost) must be a multiple of 16 bytes.
 __device__ __forceinline__ void nm_tma_store_2d(const CUtensorMap* tmap, const void* smem_src, int c0, int c1)
@@ -657,7 +663,17 @@ nm_status nm_launch_quantize(nm_ctx* ctx, const void* x, nm_dtype dtype, int64_t
 nm_status nm_launch_linear_simt(nm_ctx* ctx, const nm_linear_desc* d, cudaStream_t st);
 nm_status nm_launch_linear_f32(nm_ctx* ctx, const nm_linear_desc* d, cudaStream_t st);
 bool nm_linear_f32_supported(const nm_linear_desc* d);   // fp32, N a multiple of 4; linear_simt takes the rest
-nm_status nm_launch_linear_tc(nm_ctx* ctx, const nm_linear_desc* d, cudaStream_t st);
+// What a caller that enqueues a whole chain of kernels knows about a launch's neighbours in the stream.
+//   weights_ready: everything the call was given (weights, biases, scales) was complete before the previous kernel
+//     started, so the kernel may fetch it before its grid-dependency wait; only the activation comes from that kernel.
+//   late_trigger: the first kernel of a chain.  Its successors may start only after its own wait has returned, so that
+//     what was enqueued before the chain is complete for all of them.
+struct NmChain {
+    bool weights_ready = false, late_trigger = false;
+};
+nm_status nm_launch_linear_tc(nm_ctx* ctx, const nm_linear_desc* d, cudaStream_t st, NmChain chain = NmChain());
+nm_status nm_linear_dispatch(nm_ctx* ctx, const nm_linear_desc* d, cudaStream_t st, NmChain chain);
+nm_status nm_conv2d_dispatch(nm_ctx* ctx, const nm_conv_desc* d, void* workspace, size_t ws_bytes, cudaStream_t st, NmChain chain);
 bool nm_linear_tc_supported(const nm_linear_desc* d);
 nm_status nm_launch_attention_simt(nm_ctx* ctx, const nm_attn_desc* d, cudaStream_t st);
 nm_status nm_launch_attention_f32(nm_ctx* ctx, const nm_attn_desc* d, cudaStream_t st);
@@ -693,7 +709,7 @@ struct NmConvTc {
     int depthwise;  // pooling as a GEMM: 64-channel column tile nt reads channel block nt; w is one constant 64 x 64 matrix
     double flops;   // 2 * pixels * Cout * (taps * Cin) of the convolution itself, for the launch records
 };
-nm_status nm_launch_conv_tc(nm_ctx* ctx, const NmConvTc* c, cudaStream_t st);
+nm_status nm_launch_conv_tc(nm_ctx* ctx, const NmConvTc* c, cudaStream_t st, NmChain chain = NmChain());
 // zero-padded copies that let a few-channel first layer run as an implicit GEMM: x [N,H,W,Cin] -> xp [N,Hp,Wp,8]
 // (border of `pad` pixels, channels Cin..7 zero) and w [Cout,kh,kw,Cin] -> wp [Cout,kh,8,8]
 nm_status nm_launch_pad_input(nm_ctx* ctx, const void* x, void* xp, nm_dtype dt, int Nb, int H, int W, int Cin, int pad,
