@@ -14,6 +14,8 @@ enum ConvPath {
     CONV_IMPLICIT,  // Cin a multiple of 64: implicit GEMM, one 4-D TMA box of the activation per filter tap
     CONV_ROWTAP,    // Cin <= 8, kw <= 8 (an RGB first layer): implicit GEMM over a zero-padded 8-channel copy of the
                     // input, one K-block per filter row: 8 taps x 8 channels = 64 contiguous elements
+    CONV_PAIRTAP,   // the same with stride 2 and Cin <= 4: image rows in pairs, a K-block is two filter rows of 8 taps x 4
+                    // channels (128 images of 224 x 224 x 3, 7 x 7: 279 us with one row per K-block, 179 so, copies included)
     CONV_GATHER     // anything else: explicit gather (im2col) into the workspace, then the GEMM
 };
 
@@ -22,7 +24,7 @@ struct ConvGeom {
     int64_t M;
     ConvPath path;
     bool pad_w;       // CONV_GATHER: weights need their rows padded to Kpad
-    int Hp, Wp;       // CONV_ROWTAP: extent of the padded input copy
+    int Hp, Wp;       // CONV_ROWTAP, CONV_PAIRTAP: extent of the padded input copy
     size_t a_bytes, w_bytes;
 };
 
@@ -44,6 +46,14 @@ bool conv_geom(const nm_conv_desc* d, ConvGeom* g)
         g->path = CONV_DIRECT;
     } else if (d->Cin % 64 == 0 && d->algo != 1) {
         g->path = CONV_IMPLICIT;
+    } else if (d->Cin <= 4 && d->kw <= 8 && d->stride == 2 && d->algo != 1) {
+        g->path = CONV_PAIRTAP;
+        // output row oy reads pair rows oy .. oy + pairs - 1, output pixel ox pixels 2 ox .. 2 ox + 7
+        const int pairs = (d->kh + 1) / 2;
+        g->Hp = g->Ho - 1 + pairs;
+        g->Wp = (g->Wo - 1) * 2 + 8;
+        g->a_bytes = align256((size_t)d->N * g->Hp * g->Wp * 8 * 2);
+        g->w_bytes = align256((size_t)d->Cout * pairs * 64 * 2);
     } else if (d->Cin <= 8 && d->kw <= 8 && d->algo != 1) {
         g->path = CONV_ROWTAP;
         // rows 0 .. (Ho-1)*s + kh - 1 and pixels 0 .. (Wo-1)*s + 7 of the padded copy are read
@@ -113,7 +123,7 @@ nm_status nm_conv2d_dispatch(nm_ctx* ctx, const nm_conv_desc* d, void* workspace
         if (!workspace || ws_bytes < need) return NM_ERR_WORKSPACE;
         if (((uintptr_t)workspace & 255u) != 0) return NM_ERR_ALIGNMENT;
     }
-    if (g.path == CONV_IMPLICIT || g.path == CONV_ROWTAP) {
+    if (g.path == CONV_IMPLICIT || g.path == CONV_ROWTAP || g.path == CONV_PAIRTAP) {
         NmConvTc c;
         memset(&c, 0, sizeof(c));
         c.dtype = d->dtype;
@@ -129,6 +139,21 @@ nm_status nm_conv2d_dispatch(nm_ctx* ctx, const nm_conv_desc* d, void* workspace
             c.sw = c.sh = d->stride; c.pw = c.ph = d->pad;
             c.taps_y = d->kh; c.taps_x = d->kw; c.cblocks = d->Cin / 64;
             c.w = d->w; c.ldw = g.K; c.Ktot = g.K;
+        } else if (g.path == CONV_PAIRTAP) {
+            void* xp = workspace;
+            void* wp = (uint8_t*)workspace + g.a_bytes;
+            const int pairs = (d->kh + 1) / 2;
+            const nm_status s = nm_launch_pad_pairs(ctx, d->x, xp, d->w, wp, d->dtype, d->N, d->H, d->W, d->Cin, d->pad, g.Hp, g.Wp,
+                                                    d->Cout, d->kh, d->kw, st);
+            if (s != NM_OK) return s;
+            c.a_base = xp;
+            c.a_dim[0] = 64; c.a_dim[1] = (uint64_t)g.Wo; c.a_dim[2] = (uint64_t)g.Hp; c.a_dim[3] = (uint64_t)d->N;
+            c.a_stride[0] = 2 * 8 * 2;                            // next output pixel: two pixels on
+            c.a_stride[1] = (uint64_t)g.Wp * 8 * 2;
+            c.a_stride[2] = (uint64_t)g.Hp * g.Wp * 8 * 2;
+            c.sw = c.sh = 1; c.pw = c.ph = 0;
+            c.taps_y = pairs; c.taps_x = 1; c.cblocks = 1;
+            c.w = wp; c.ldw = (int64_t)pairs * 64; c.Ktot = (int64_t)pairs * 64;
         } else {
             // the input with its border and five zero channels written out once (xp), the weights likewise (wp);
             // output pixel ox then reads the 64 contiguous elements of pixels ox*s .. ox*s + 7 of row oy*s + ky

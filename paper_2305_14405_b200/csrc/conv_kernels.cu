@@ -137,6 +137,53 @@ __global__ void pad_weight_kernel(const T* __restrict__ w, T* __restrict__ wp, i
     }
 }
 
+// The same for a stride-2 layer of at most four channels, two image rows to a row of the copy: x [N,H,W,Cin] ->
+// xp [N,Hp,Wp,2,4], pixel px of pair row r holding rows 2r - pad and 2r + 1 - pad of column px - pad.  Half the bytes of the
+// 8-channel copy, and a K-block of the convolution is two filter rows of 8 taps x 4 channels instead of one.  One thread
+// per 16-byte pixel pair.
+template <typename T>
+__global__ void __launch_bounds__(256) pad_input_pairs_kernel(const T* __restrict__ x, T* __restrict__ xp, int Nb, int H, int W,
+                                                              int Cin, int pad, int Hp, int Wp)
+{
+    const int px = (int)(blockIdx.x * 256 + threadIdx.x);
+    if (px >= Wp) return;
+    const int ix = px - pad;
+    for (int n = blockIdx.z; n < Nb; n += gridDim.z) {
+        for (int r = blockIdx.y; r < Hp; r += gridDim.y) {
+            T v[8];
+#pragma unroll
+            for (int c = 0; c < 8; ++c) v[c] = NmType<T>::from_f(0.f);
+            if (ix >= 0 && ix < W) {
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const int iy = 2 * r + h - pad;
+                    if (iy < 0 || iy >= H) continue;
+                    const T* src = x + (((int64_t)n * H + iy) * W + ix) * Cin;
+#pragma unroll
+                    for (int c = 0; c < 4; ++c)
+                        if (c < Cin) v[4 * h + c] = src[c];
+                }
+            }
+            *reinterpret_cast<uint4*>(xp + (((int64_t)n * Hp + r) * Wp + px) * 8) = *reinterpret_cast<const uint4*>(v);
+        }
+    }
+}
+
+// w [Cout,kh,kw,Cin] (kw <= 8, Cin <= 4) -> wp [Cout,pairs,8,2,4], zero where no filter row, tap or channel is
+template <typename T>
+__global__ void pad_weight_pairs_kernel(const T* __restrict__ w, T* __restrict__ wp, int Cout, int kh, int kw, int Cin)
+{
+    const int pairs = (kh + 1) / 2;
+    const int64_t total = (int64_t)Cout * pairs * 64;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
+        const int c = (int)(i & 3), h = (int)((i >> 2) & 1), kx = (int)((i >> 3) & 7);
+        const int64_t r = i >> 6;   // (co, pair)
+        const int64_t co = r / pairs;
+        const int ky = 2 * (int)(r - co * pairs) + h;
+        wp[i] = (ky < kh && kx < kw && c < Cin) ? w[((co * kh + ky) * kw + kx) * Cin + c] : NmType<T>::from_f(0.f);
+    }
+}
+
 __device__ __forceinline__ float2 unpack2(__half2 v) { return __half22float2(v); }
 __device__ __forceinline__ float2 unpack2(__nv_bfloat162 v) { return __bfloat1622float2(v); }
 template <typename T> struct Vec2;
@@ -324,6 +371,24 @@ nm_status nm_launch_pad_weight(nm_ctx* ctx, const void* w, void* wp, nm_dtype dt
     NmLaunchScope scope(ctx, NM_KERNEL_IM2COL, (double)total * 2.0 * nm_dtype_size(dt), st);
     if (dt == NM_F16) pad_weight_kernel<__half><<<grid_for(ctx, total), 256, 0, st>>>((const __half*)w, (__half*)wp, Cout, kh, kw, Cin);
     else pad_weight_kernel<__nv_bfloat16><<<grid_for(ctx, total), 256, 0, st>>>((const __nv_bfloat16*)w, (__nv_bfloat16*)wp, Cout, kh, kw, Cin);
+    return cudaGetLastError() == cudaSuccess ? NM_OK : NM_ERR_CUDA;
+}
+
+nm_status nm_launch_pad_pairs(nm_ctx* ctx, const void* x, void* xp, const void* w, void* wp, nm_dtype dt, int Nb, int H, int W,
+                              int Cin, int pad, int Hp, int Wp, int Cout, int kh, int kw, cudaStream_t st)
+{
+    const dim3 grid((unsigned)((Wp + 255) / 256), (unsigned)(Hp < 65535 ? Hp : 65535), (unsigned)(Nb < 65535 ? Nb : 65535));
+    const int64_t wtotal = (int64_t)Cout * ((kh + 1) / 2) * 64;
+    {
+        NmLaunchScope scope(ctx, NM_KERNEL_IM2COL, ((double)Nb * H * W * Cin + (double)Nb * Hp * Wp * 8) * nm_dtype_size(dt), st);
+        if (dt == NM_F16) pad_input_pairs_kernel<__half><<<grid, 256, 0, st>>>((const __half*)x, (__half*)xp, Nb, H, W, Cin, pad, Hp, Wp);
+        else pad_input_pairs_kernel<__nv_bfloat16><<<grid, 256, 0, st>>>((const __nv_bfloat16*)x, (__nv_bfloat16*)xp, Nb, H, W, Cin, pad, Hp, Wp);
+    }
+    {
+        NmLaunchScope scope(ctx, NM_KERNEL_IM2COL, (double)wtotal * 2.0 * nm_dtype_size(dt), st);
+        if (dt == NM_F16) pad_weight_pairs_kernel<__half><<<grid_for(ctx, wtotal), 256, 0, st>>>((const __half*)w, (__half*)wp, Cout, kh, kw, Cin);
+        else pad_weight_pairs_kernel<__nv_bfloat16><<<grid_for(ctx, wtotal), 256, 0, st>>>((const __nv_bfloat16*)w, (__nv_bfloat16*)wp, Cout, kh, kw, Cin);
+    }
     return cudaGetLastError() == cudaSuccess ? NM_OK : NM_ERR_CUDA;
 }
 

@@ -716,6 +716,9 @@ nm_status nm_launch_pad_input(nm_ctx* ctx, const void* x, void* xp, nm_dtype dt,
                               int Hp, int Wp, cudaStream_t st);
 nm_status nm_launch_pad_weight(nm_ctx* ctx, const void* w, void* wp, nm_dtype dt, int Cout, int kh, int kw, int Cin,
                                cudaStream_t st);
+// the same for a stride-2 layer of at most 4 channels, rows in pairs: xp [N,Hp,Wp,2,4], wp [Cout,(kh+1)/2,8,2,4]
+nm_status nm_launch_pad_pairs(nm_ctx* ctx, const void* x, void* xp, const void* w, void* wp, nm_dtype dt, int Nb, int H, int W,
+                              int Cin, int pad, int Hp, int Wp, int Cout, int kh, int kw, cudaStream_t st);
 nm_status nm_launch_im2col(nm_ctx* ctx, const void* x, void* A, nm_dtype dt, int Nb, int H, int W, int Cin, int kh,
                            int kw, int stride, int pad, int Ho, int Wo, int Kpad, cudaStream_t st);
 nm_status nm_launch_pad_rows(nm_ctx* ctx, const void* w, void* wp, nm_dtype dt, int rows, int K, int Kpad,
