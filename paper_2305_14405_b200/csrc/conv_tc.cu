@@ -73,6 +73,70 @@ nm_status make_tmap_a(nm_ctx* ctx, CUtensorMap* m, const NmConvTc* c, const Conv
     return make_tmap4(ctx, m, c->a_base, c->dtype, c->a_dim, c->a_stride, abox, aestr);
 }
 
+// output / residual: the 32 tile rows of an epilogue warp are a sub-box of the patch
+nm_status make_tmaps_out(nm_ctx* ctx, CUtensorMap* tmO, CUtensorMap* tmR, const NmConvTc* c, const ConvDev& cv)
+{
+    const int bh = cv.TH < 32 / cv.TW ? cv.TH : 32 / cv.TW;
+    const int bn = 32 / (cv.TW * bh);
+    const uint64_t odim[4] = {(uint64_t)c->Cout, (uint64_t)c->Wo, (uint64_t)c->Ho, (uint64_t)c->N};
+    const uint64_t ostr[3] = {(uint64_t)c->Cout * 2, (uint64_t)c->Wo * c->Cout * 2, (uint64_t)c->Ho * c->Wo * c->Cout * 2};
+    const uint32_t obox[4] = {64u, (uint32_t)cv.TW, (uint32_t)bh, (uint32_t)bn};
+    const uint32_t one[4] = {1u, 1u, 1u, 1u};
+    nm_status s = make_tmap4(ctx, tmO, c->out, c->dtype, odim, ostr, obox, one);
+    if (s != NM_OK) return s;
+    if (!c->residual) {
+        *tmR = *tmO;
+        return NM_OK;
+    }
+    return make_tmap4(ctx, tmR, c->residual, c->dtype, odim, ostr, obox, one);
+}
+
+// Is the halo form (linear_tc_kernel.cuh) the faster one?  3 x 3, stride 1, padding 1, at least two rounds of CTA pairs, and less
+// time by the bytes a tile takes from L2 (50 a clock) and the tensor core's cycles, although its fixed 8 x 16 patch wastes rows
+// that the free patch does not: 128 images, 56 x 56, 64 -> 64: HALO_A us against HALO_B; 28 x 28, 128 -> 128: HALO_C against
+// HALO_D.  Wider outputs are bound by the tensor core in either form.
+bool use_halo(const NmConvTc* c, int64_t free_patches, int sms)
+{
+    if (c->algo != 0 || c->taps_x != 3 || c->taps_y != 3 || c->sw != 1 || c->sh != 1 || c->pw != 1 || c->ph != 1 || c->depthwise ||
+        c->Cout > 128 || c->Cout <= 32)
+        return false;
+    const int64_t halo_patches = (int64_t)ceil_div(c->Wo, 8) * ceil_div(c->Ho, 16) * c->N;
+    if (halo_patches < 2LL * 2 * sms) return false;
+    const int bn = c->Cout <= 64 ? 64 : 128;
+    const double b_bytes = bn / 2 * ROW_BYTES, taps = 9.0 * c->cblocks, mma = bn == 64 ? 160.0 : 256.0;
+    const double w_stream = bn == 64 && c->cblocks == 1 ? 0.0 : taps * b_bytes;
+    const double feed_free = taps * (A_BYTES + b_bytes) / 50, feed_halo = (c->cblocks * (double)HALO_BYTES + w_stream) / 50;
+    const double t_free = (double)free_patches * (feed_free > taps * mma ? feed_free : taps * mma);
+    const double t_halo = (double)halo_patches * (feed_halo > taps * mma ? feed_halo : taps * mma);
+    return t_halo < 0.9 * t_free;
+}
+
+template <typename T, int BN>
+nm_status launch_halo(nm_ctx* ctx, const NmConvTc* c, NmChain chain, cudaStream_t st)
+{
+    TcArgs a;
+    fill_args(ctx, c, chain, &a);
+    ConvDev& cv = a.cv;
+    cv.TW = 8; cv.TH = 16; cv.NB = 1;
+    cv.tiles_x = ceil_div(c->Wo, cv.TW);
+    cv.tiles_y = ceil_div(c->Ho, cv.TH);
+    const int64_t patches = (int64_t)cv.tiles_x * cv.tiles_y * c->N;
+    a.num_n_tiles = 1;
+    if (patches / 2 > 0x7ffffffeLL) return NM_ERR_UNSUPPORTED;
+    a.num_tiles = (int)((patches + 1) / 2);
+    size_t smem = 0;
+    if (!plan_smem_halo<T, BN>(&a, c->bias != nullptr, &smem)) return NM_ERR_UNSUPPORTED;
+    CUtensorMap tmA, tmW, tmO, tmR;
+    const uint32_t abox[4] = {64u, HALO_W, HALO_H, 1u}, one[4] = {1u, 1u, 1u, 1u};
+    nm_status s = make_tmap4(ctx, &tmA, c->a_base, c->dtype, c->a_dim, c->a_stride, abox, one);
+    if (s != NM_OK) return s;
+    s = make_tmap(ctx, &tmW, c->w, c->dtype, c->Cout, c->Ktot, c->ldw, BN / 2);
+    if (s != NM_OK) return s;
+    s = make_tmaps_out(ctx, &tmO, &tmR, c, cv);
+    if (s != NM_OK) return s;
+    return launch_kernel<T, T, true, BN, true, true>(ctx, tmA, tmW, tmO, tmR, a, smem, c->flops, st);
+}
+
 template <typename T, int BN>
 nm_status launch_split(nm_ctx* ctx, const NmConvTc* c, int S, NmChain chain, cudaStream_t st)
 {
@@ -114,17 +178,7 @@ nm_status launch(nm_ctx* ctx, const NmConvTc* c, NmChain chain, cudaStream_t st)
     // (depthwise form: W is the one 64 x 64 matrix, whatever the number of output channels)
     s = make_tmap(ctx, &tmW, c->w, c->dtype, c->depthwise ? 64 : c->Cout, c->Ktot, c->ldw, B_ROWS);
     if (s != NM_OK) return s;
-    // output / residual: the 32 tile rows of an epilogue warp are a sub-box of the patch
-    const int bh = cv.TH < 32 / cv.TW ? cv.TH : 32 / cv.TW;
-    const int bn = 32 / (cv.TW * bh);
-    const uint64_t odim[4] = {(uint64_t)c->Cout, (uint64_t)c->Wo, (uint64_t)c->Ho, (uint64_t)c->N};
-    const uint64_t ostr[3] = {(uint64_t)c->Cout * 2, (uint64_t)c->Wo * c->Cout * 2, (uint64_t)c->Ho * c->Wo * c->Cout * 2};
-    const uint32_t obox[4] = {64u, (uint32_t)cv.TW, (uint32_t)bh, (uint32_t)bn};
-    const uint32_t one[4] = {1u, 1u, 1u, 1u};
-    s = make_tmap4(ctx, &tmO, c->out, c->dtype, odim, ostr, obox, one);
-    if (s != NM_OK) return s;
-    if (c->residual) s = make_tmap4(ctx, &tmR, c->residual, c->dtype, odim, ostr, obox, one);
-    else tmR = tmO;
+    s = make_tmaps_out(ctx, &tmO, &tmR, c, cv);
     if (s != NM_OK) return s;
     return launch_kernel<T, T, TWO, BN, true>(ctx, tmA, tmW, tmO, tmR, a, smem, c->flops, st);
 }
@@ -137,6 +191,10 @@ nm_status launch_sel(nm_ctx* ctx, const NmConvTc* c, NmChain chain, cudaStream_t
         int tw, th, nb;
         choose_patch(c->Wo, c->Ho, c->N, &tw, &th, &nb);
         const int64_t patches = (int64_t)ceil_div(c->Wo, tw) * ceil_div(c->Ho, th) * ceil_div(c->N, nb);
+        if (use_halo(c, patches, ctx->sm_count)) {
+            const nm_status e = c->Cout <= 64 ? launch_halo<T, 64>(ctx, c, chain, st) : launch_halo<T, 128>(ctx, c, chain, st);
+            if (e != NM_ERR_UNSUPPORTED) return e;
+        }
         t = choose_tile(patches, c->Cout, (int64_t)c->taps_y * c->taps_x * c->cblocks, true, c->slot != NM_SLOT_NONE,
                         c->depthwise != 0, true, ctx->sm_count);
     } else {

@@ -32,6 +32,12 @@
 //   shifted by the tap (and strided for a strided convolution); coordinates outside the image read
 //   zeros, which is the convolution's padding.  Nothing is gathered into memory first.  Output and
 //   residual tiles are 4-D boxes of the NHWC output in the same way.
+// HALO = true: a 3 x 3 convolution of stride 1 and padding 1 with a narrow output.  There the K-blocks' nine shifted boxes
+//   of the same activation are what the launch waits for (L2 to shared memory, 50 bytes a clock and SM), so a tile is a patch
+//   of 8 x 16 output pixels whose 10 x 18 input pixels are loaded ONCE per channel block: pixel (x, y) of the box is row
+//   10 y + x of shared memory, eight output pixels of a patch row are one 8-row group of the operand, the groups lie 1280 bytes
+//   apart, and tap (ky, kx) is the same operand 10 ky + kx rows further on.  The swizzle follows the address, so an operand may
+//   start at any row.  The weights have a ring of their own, or stay in shared memory if all of them fit.
 #pragma once
 #include <string.h>
 
@@ -46,6 +52,10 @@ constexpr int MAX_STAGES = 8;
 constexpr int NUM_THREADS = 320;  // TMA warp, MMA warp, 8 epilogue warps
 constexpr int NUM_EPI_WARPS = 8;
 constexpr int STAGE_BUF = 32 * 128;  // one staging buffer: 32 rows x 128 bytes
+constexpr int HALO_W = 10, HALO_H = 18;                    // input pixels of a patch of 8 x 16 output pixels
+constexpr int HALO_LOAD = HALO_W * HALO_H * ROW_BYTES;     // bytes of one halo box
+constexpr int HALO_BYTES = (HALO_LOAD + 1023) / 1024 * 1024;
+constexpr int MAX_W_STAGES = 18;
 
 // How a tile's 128 rows map onto the NHWC tensors of a convolution (CONV kernels only).
 struct ConvDev {
@@ -72,6 +82,8 @@ struct TcArgs {
     int* status;
     int num_n_tiles, num_tiles, num_k_blocks, stages, n_seg;
     int weights_ready, late_trigger;   // NmChain
+    int w_stages;                      // HALO: weight tiles in shared memory; w_resident: all of them, loaded once
+    int w_resident;
     ConvDev cv;
 };
 
@@ -172,7 +184,7 @@ __device__ __forceinline__ void res_tile_load(void* dst, const CUtensorMap* tmR,
     else nm_tma_load_2d(dst, tmR, col, row0, bar);
 }
 
-template <typename InT, typename OutT, bool TWO, int BN, bool CONV>
+template <typename InT, typename OutT, bool TWO, int BN, bool CONV, bool HALO = false>
 __global__ void __launch_bounds__(NUM_THREADS, 1)
 linear_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmW,
                  const __grid_constant__ CUtensorMap tmO, const __grid_constant__ CUtensorMap tmR, const TcArgs a)
@@ -180,7 +192,8 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     static_assert(BN == 64 || BN == 128 || BN == 256, "tile widths built");
     constexpr int B_ROWS = TWO ? BN / 2 : BN;
     constexpr int B_BYTES = B_ROWS * ROW_BYTES;
-    constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
+    constexpr int STAGE_BYTES = HALO ? HALO_BYTES : A_BYTES + B_BYTES;
+    static_assert(!HALO || (CONV && TWO), "the halo form is built for CTA pairs");
     constexpr int TILE_M = TWO ? 2 * BM : BM;
     constexpr int BK_ELEMS = ROW_BYTES / (int)sizeof(InT);
     constexpr uint32_t TMEM_COLS = 2 * BN;
@@ -205,13 +218,15 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     __shared__ uint64_t bar_acc_empty[2];
     __shared__ uint64_t bar_res[NUM_EPI_WARPS];
     __shared__ uint64_t bar_res_free[NUM_EPI_WARPS];
+    __shared__ uint64_t bar_wfull[HALO ? MAX_W_STAGES : 1], bar_wempty[HALO ? MAX_W_STAGES : 1];
     __shared__ uint64_t bar_drain;
     __shared__ uint32_t tmem_slot;
     __shared__ int abort_flag;
 
     const int stages = a.stages;
     uint8_t* tiles = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-    uint8_t* stage_out = tiles + (size_t)stages * STAGE_BYTES;   // 8 x 4 KB
+    uint8_t* w_tiles = tiles + (size_t)stages * STAGE_BYTES;     // HALO: w_stages x B_BYTES
+    uint8_t* stage_out = w_tiles + (HALO ? (size_t)a.w_stages * B_BYTES : 0);   // 8 x 4 KB
     uint8_t* stage_res = stage_out + NUM_EPI_WARPS * STAGE_BUF;   // 8 x 4 KB when a residual is given
     float2* rep = reinterpret_cast<float2*>(stage_res + (a.has_res ? NUM_EPI_WARPS * STAGE_BUF : 0));
     // per epilogue warp: bias (128 floats) and, for int8, a_scale * w_scale (128 floats) of its tile columns
@@ -231,6 +246,12 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         for (int s = 0; s < stages; ++s) {
             nm_mbar_init(&bar_full[s], 1);
             nm_mbar_init(&bar_empty[s], 1);
+        }
+        if constexpr (HALO) {
+            for (int i = 0; i < a.w_stages; ++i) {
+                nm_mbar_init(&bar_wfull[i], 1);
+                nm_mbar_init(&bar_wempty[i], 1);
+            }
         }
         for (int b = 0; b < 2; ++b) {
             nm_mbar_init(&bar_acc_full[b], 1);
@@ -269,7 +290,41 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         // ------------------------------------------------ TMA producer
         // All 32 lanes run the loop, so that stage, coordinates and addresses stay warp-uniform (the
         // compiler keeps them in uniform registers); one elected lane issues the copies.
-        {
+        if constexpr (HALO) {
+            int stage = 0, ws = 0;
+            uint32_t phase = 0, wphase = 0;
+            bool ok = true;
+            for (int tile = tile_first; ok && tile < a.num_tiles; tile += tile_step) {
+                const int mt = tile / a.num_n_tiles;
+                const int n0 = (tile % a.num_n_tiles) * BN + (int)rank * B_ROWS;
+                const Patch pt = patch_of(a.cv, mt * 2 + (int)rank);
+                const bool load_w = !a.w_resident || tile == tile_first;
+                for (int cb = 0; ok && cb < a.cv.cblocks; ++cb) {
+                    if (!__all_sync(0xffffffffu, nm_mbar_wait(&bar_empty[stage], phase ^ 1u, abortp, a.status))) { ok = false; break; }
+                    if (nm_elect_one()) {
+                        const uint32_t full = nm_mapa(nm_smem_u32(&bar_full[stage]), 0);
+                        if (rank == 0) nm_mbar_expect_tx(&bar_full[stage], 2 * HALO_LOAD);
+                        nm_tma_load_4d_2cta(tiles + (size_t)stage * STAGE_BYTES, &tmA, cb * BK_ELEMS, pt.ox0 - 1, pt.oy0 - 1, pt.img0, full);
+                    }
+                    __syncwarp();
+                    if (++stage == stages) { stage = 0; phase ^= 1u; }
+                    for (int tap = 0; load_w && tap < 9; ++tap) {
+                        if (!__all_sync(0xffffffffu, nm_mbar_wait(&bar_wempty[ws], wphase ^ 1u, abortp, a.status))) { ok = false; break; }
+                        if (nm_elect_one()) {
+                            const uint32_t full = nm_mapa(nm_smem_u32(&bar_wfull[ws]), 0);
+                            if (rank == 0) nm_mbar_expect_tx(&bar_wfull[ws], 2 * B_BYTES);
+                            nm_tma_load_2d_2cta(w_tiles + (size_t)ws * B_BYTES, &tmW, (tap * a.cv.cblocks + cb) * BK_ELEMS, n0, full);
+                        }
+                        __syncwarp();
+                        if (++ws == a.w_stages) { ws = 0; wphase ^= 1u; }
+                    }
+                }
+            }
+            if (!ok) {
+                long long t0 = clock64();  // bounded pause: copies in flight land before teardown
+                while (clock64() - t0 < 4000000LL) {}
+            }
+        } else {
             int stage = 0;
             uint32_t phase = 0;
             bool ok = true;
@@ -332,13 +387,39 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             int buf = 0;
             uint32_t acc_phase = 0;
             bool ok = true;
+            [[maybe_unused]] int ws = 0;
+            [[maybe_unused]] uint32_t wphase = 0;
             for (int tile = tile_first; ok && tile < a.num_tiles; tile += tile_step) {
                 // CTA-scope acquire also where the peer CTA's epilogue warps arrive: what the hand-back orders are
                 // tcgen05 operations, ordered by tcgen05.fence (a cluster-scope acquire costs ~400 cycles per tile)
                 if (!__all_sync(0xffffffffu, nm_mbar_wait(&bar_acc_empty[buf], acc_phase ^ 1u, abortp, a.status))) { ok = false; break; }
                 nm_tc_fence_after();
                 const uint32_t d_tmem = tmem_base + (uint32_t)(buf * BN);
-                for (int kb = 0; kb < a.num_k_blocks; ++kb) {
+                if constexpr (HALO) {
+                    const bool wait_w = !a.w_resident || tile == tile_first;
+                    for (int cb = 0; ok && cb < a.cv.cblocks; ++cb) {
+                        if (!__all_sync(0xffffffffu, nm_mbar_wait(&bar_full[stage], phase, abortp, a.status))) { ok = false; break; }
+                        const uint32_t sa = nm_smem_u32(tiles + (size_t)stage * STAGE_BYTES);
+                        for (int tap = 0; tap < 9; ++tap) {
+                            if (wait_w && !__all_sync(0xffffffffu, nm_mbar_wait(&bar_wfull[ws], wphase, abortp, a.status))) { ok = false; break; }
+                            nm_tc_fence_after();
+                            const int ky = tap / 3, kx = tap - 3 * ky;
+                            const uint64_t adesc = nm_smem_desc_sw128(sa + (uint32_t)((HALO_W * ky + kx) * ROW_BYTES), HALO_W * ROW_BYTES);
+                            const uint64_t bdesc = nm_smem_desc_sw128(nm_smem_u32(w_tiles + (size_t)ws * B_BYTES));
+                            if (nm_elect_one()) {
+#pragma unroll
+                                for (int k = 0; k < 4; ++k)
+                                    nm_mma_f16_2cta(d_tmem, adesc + 2 * k, bdesc + 2 * k, IDESC, (cb | tap | k) != 0 ? 1u : 0u);
+                                if (!a.w_resident) nm_tc_commit2(&bar_wempty[ws], 3);
+                                if (tap == 8) nm_tc_commit2(&bar_empty[stage], 3);
+                            }
+                            __syncwarp();
+                            if (++ws == a.w_stages) { ws = 0; wphase ^= 1u; }
+                        }
+                        if (++stage == stages) { stage = 0; phase ^= 1u; }
+                    }
+                }
+                for (int kb = 0; !HALO && kb < a.num_k_blocks; ++kb) {
                     if (!__all_sync(0xffffffffu, nm_mbar_wait(&bar_full[stage], phase, abortp, a.status))) { ok = false; break; }
                     nm_tc_fence_after();
                     const uint32_t sa = nm_smem_u32(tiles + (size_t)stage * STAGE_BYTES);
@@ -678,12 +759,37 @@ inline bool plan_smem(TcArgs* a, bool has_vec, size_t* smem_out)
     return true;
 }
 
+// The same for the halo form: all weight tiles if they leave room for two halo boxes and the columns are one tile, else a ring.
+template <typename T, int BN>
+inline bool plan_smem_halo(TcArgs* a, bool has_vec, size_t* smem_out)
+{
+    constexpr int B_BYTES = BN / 2 * ROW_BYTES;
+    const size_t table_bytes = (size_t)a->n_seg * 32 * sizeof(float2);
+    const size_t vec_bytes = has_vec ? (size_t)NUM_EPI_WARPS * 256 * sizeof(float) : 0;
+    const size_t fixed = (size_t)NUM_EPI_WARPS * STAGE_BUF * (a->has_res ? 2 : 1) + vec_bytes + table_bytes + 2048;
+    const long long room = 227 * 1024 - (long long)fixed;
+    const int kb = a->num_k_blocks;
+    a->w_resident = a->num_n_tiles == 1 && kb <= MAX_W_STAGES && room >= (long long)kb * B_BYTES + 2 * HALO_BYTES;
+    a->stages = 3;
+    if (a->w_resident) {
+        a->w_stages = kb;
+        a->stages = (int)((room - (long long)kb * B_BYTES) / HALO_BYTES);
+        if (a->stages > 4) a->stages = 4;
+    } else {
+        a->w_stages = (int)((room - 3LL * HALO_BYTES) / B_BYTES);
+        if (a->w_stages > MAX_W_STAGES) a->w_stages = MAX_W_STAGES;
+        if (room < 3LL * HALO_BYTES + 4LL * B_BYTES) return false;
+    }
+    *smem_out = (size_t)a->stages * HALO_BYTES + (size_t)a->w_stages * B_BYTES + fixed - 1024;
+    return true;
+}
+
 // Launches the persistent kernel over a.num_tiles tiles (one CTA, or one CTA pair, per resident slot).
-template <typename InT, typename OutT, bool TWO, int BN, bool CONV>
+template <typename InT, typename OutT, bool TWO, int BN, bool CONV, bool HALO = false>
 inline nm_status launch_kernel(nm_ctx* ctx, const CUtensorMap& tmA, const CUtensorMap& tmW, const CUtensorMap& tmO,
                                const CUtensorMap& tmR, const TcArgs& a, size_t smem, double work, cudaStream_t st)
 {
-    auto kern = linear_tc_kernel<InT, OutT, TWO, BN, CONV>;
+    auto kern = linear_tc_kernel<InT, OutT, TWO, BN, CONV, HALO>;
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
         return NM_ERR_CUDA;
     cudaLaunchConfig_t cfg;

@@ -578,12 +578,14 @@ __device__ __forceinline__ void nm_mma_i8_2cta(uint32_t d_tmem, uint64_t adesc, 
 // 8 rows 1024 bytes apart.  Valid for a K-major operand whose K extent per tile is
 // 128 bytes, and for an MN-major operand whose MN extent is 128 bytes (then the
 // 8-row groups run along K).
-__device__ __forceinline__ uint64_t nm_smem_desc_sw128(uint32_t smem_addr)
+// `group_bytes`: distance of the 8-row groups.  The swizzle is a function of the address, so the operand may start at any
+// row of what was written with it, and the groups may lie any multiple of a row apart.
+__device__ __forceinline__ uint64_t nm_smem_desc_sw128(uint32_t smem_addr, uint32_t group_bytes = 1024)
 {
     uint64_t d = 0;
     d |= (uint64_t)((smem_addr & 0x3FFFFu) >> 4);       // start address
     d |= (uint64_t)1 << 16;                             // leading byte offset (unused with swizzle)
-    d |= (uint64_t)(1024 >> 4) << 32;                   // stride byte offset: 8 rows * 128 B
+    d |= (uint64_t)(group_bytes >> 4) << 32;            // stride byte offset
     d |= (uint64_t)1 << 46;                             // descriptor version (sm_100)
     d |= (uint64_t)2 << 61;                             // SWIZZLE_128B
     return d;
