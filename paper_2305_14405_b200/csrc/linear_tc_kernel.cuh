@@ -210,6 +210,13 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     constexpr int GROUP_COLS = 32 * GC;
     constexpr int WPC = 32 / GC;  // packed words per chunk
     constexpr int EPI_STEP = ALT ? 2 : 1;   // a warp works on every EPI_STEP-th tile of its CTA
+    // The producer's and the MMA issuer's loops run in one elected lane for narrow tiles.  A K-block of those is bound by the
+    // loop and not by the tensor core: 4 MMAs of 64 columns take 192 cycles to issue; with a wait by all lanes and its vote, an
+    // election and the commit that was 393, with one lane, which looks at the next stage's barrier before it issues this
+    // one's MMAs, 281 and less (128 images, 28 x 28, 128 -> 128, 3 x 3: 45.6 -> 39.2 us).  With 256 columns the tensor core
+    // covers it, and all lanes, whose stage numbers and descriptors stay in uniform registers, are 1 % faster.
+    constexpr bool ONE_LANE = BN < 256;
+    auto vote = [](bool done) { return ONE_LANE ? done : __all_sync(0xffffffffu, done) != 0; };
 
     extern __shared__ uint8_t smem_raw[];
     __shared__ uint64_t bar_full[MAX_STAGES];
@@ -288,144 +295,143 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
 
     if (warp == 0) {
         // ------------------------------------------------ TMA producer
-        // All 32 lanes run the loop, so that stage, coordinates and addresses stay warp-uniform (the
-        // compiler keeps them in uniform registers); one elected lane issues the copies.
-        if constexpr (HALO) {
-            int stage = 0, ws = 0;
-            uint32_t phase = 0, wphase = 0;
-            bool ok = true;
-            for (int tile = tile_first; ok && tile < a.num_tiles; tile += tile_step) {
-                const int mt = tile / a.num_n_tiles;
-                const int n0 = (tile % a.num_n_tiles) * BN + (int)rank * B_ROWS;
-                const Patch pt = patch_of(a.cv, mt * 2 + (int)rank);
-                const bool load_w = !a.w_resident || tile == tile_first;
-                for (int cb = 0; ok && cb < a.cv.cblocks; ++cb) {
-                    if (!__all_sync(0xffffffffu, nm_mbar_wait(&bar_empty[stage], phase ^ 1u, abortp, a.status))) { ok = false; break; }
-                    if (nm_elect_one()) {
+        if (!ONE_LANE || nm_elect_one()) {
+            if constexpr (HALO) {
+                int stage = 0, ws = 0;
+                uint32_t phase = 0, wphase = 0;
+                bool ok = true;
+                for (int tile = tile_first; ok && tile < a.num_tiles; tile += tile_step) {
+                    const int mt = tile / a.num_n_tiles;
+                    const int n0 = (tile % a.num_n_tiles) * BN + (int)rank * B_ROWS;
+                    const Patch pt = patch_of(a.cv, mt * 2 + (int)rank);
+                    const bool load_w = !a.w_resident || tile == tile_first;
+                    for (int cb = 0; ok && cb < a.cv.cblocks; ++cb) {
+                        if (!nm_mbar_wait(&bar_empty[stage], phase ^ 1u, abortp, a.status)) { ok = false; break; }
                         const uint32_t full = nm_mapa(nm_smem_u32(&bar_full[stage]), 0);
                         if (rank == 0) nm_mbar_expect_tx(&bar_full[stage], 2 * HALO_LOAD);
                         nm_tma_load_4d_2cta(tiles + (size_t)stage * STAGE_BYTES, &tmA, cb * BK_ELEMS, pt.ox0 - 1, pt.oy0 - 1, pt.img0, full);
-                    }
-                    __syncwarp();
-                    if (++stage == stages) { stage = 0; phase ^= 1u; }
-                    for (int tap = 0; load_w && tap < 9; ++tap) {
-                        if (!__all_sync(0xffffffffu, nm_mbar_wait(&bar_wempty[ws], wphase ^ 1u, abortp, a.status))) { ok = false; break; }
-                        if (nm_elect_one()) {
+                        if (++stage == stages) { stage = 0; phase ^= 1u; }
+                        for (int tap = 0; load_w && tap < 9; ++tap) {
+                            if (!nm_mbar_wait(&bar_wempty[ws], wphase ^ 1u, abortp, a.status)) { ok = false; break; }
                             const uint32_t full = nm_mapa(nm_smem_u32(&bar_wfull[ws]), 0);
                             if (rank == 0) nm_mbar_expect_tx(&bar_wfull[ws], 2 * B_BYTES);
                             nm_tma_load_2d_2cta(w_tiles + (size_t)ws * B_BYTES, &tmW, (tap * a.cv.cblocks + cb) * BK_ELEMS, n0, full);
+                            if (++ws == a.w_stages) { ws = 0; wphase ^= 1u; }
                         }
-                        __syncwarp();
-                        if (++ws == a.w_stages) { ws = 0; wphase ^= 1u; }
                     }
                 }
-            }
-            if (!ok) {
-                long long t0 = clock64();  // bounded pause: copies in flight land before teardown
-                while (clock64() - t0 < 4000000LL) {}
-            }
-        } else {
-            int stage = 0;
-            uint32_t phase = 0;
-            bool ok = true;
-            for (int tile = tile_first; ok && tile < a.num_tiles; tile += tile_step) {
-                const int mt = tile / a.num_n_tiles;
-                const int m0 = mt * TILE_M + (int)rank * BM;
-                const int n0 = (tile % a.num_n_tiles) * BN + (int)rank * B_ROWS;
-                Patch pt = {0, 0, 0};
-                if constexpr (CONV) pt = patch_of(a.cv, mt * (TWO ? 2 : 1) + (int)rank);
-                int tap = 0, cb = 0;   // CONV: K-block = (tap, channel block)
-                for (int kb = 0; kb < a.num_k_blocks; ++kb) {
-                    if (!__all_sync(0xffffffffu, nm_mbar_wait(&bar_empty[stage], phase ^ 1u, abortp, a.status))) { ok = false; break; }
-                    uint8_t* sa = tiles + (size_t)stage * STAGE_BYTES;
-                    int c_c = 0, c_w = 0, c_h = 0, w_k = kb * BK_ELEMS, w_n = n0;
-                    if constexpr (CONV) {
-                        const int ky = tap / a.cv.kw_eff, kx = tap - ky * a.cv.kw_eff;
-                        c_c = cb * BK_ELEMS;
-                        c_w = pt.ox0 * a.cv.sw - a.cv.pw + kx;
-                        c_h = pt.oy0 * a.cv.sh - a.cv.ph + ky;
-                        if (a.cv.dw) {   // pooling: channel block = column tile, one constant matrix for every tap and tile
-                            c_c = (tile % a.num_n_tiles) * BK_ELEMS;
-                            w_k = 0;
-                            w_n = (int)rank * B_ROWS;
-                        }
-                    }
-                    if (nm_elect_one()) {
-                        if constexpr (TWO) {
-                            // both CTAs' copies are counted on the leader's barrier
-                            const uint32_t full = nm_mapa(nm_smem_u32(&bar_full[stage]), 0);
-                            if (rank == 0) nm_mbar_expect_tx(&bar_full[stage], 2 * STAGE_BYTES);
-                            if constexpr (CONV) nm_tma_load_4d_2cta(sa, &tmA, c_c, c_w, c_h, pt.img0, full);
-                            else nm_tma_load_2d_2cta(sa, &tmA, kb * BK_ELEMS, m0, full);
-                            nm_tma_load_2d_2cta(sa + A_BYTES, &tmW, w_k, w_n, full);
-                        } else {
-                            nm_mbar_expect_tx(&bar_full[stage], STAGE_BYTES);
-                            if constexpr (CONV) nm_tma_load_4d(sa, &tmA, c_c, c_w, c_h, pt.img0, &bar_full[stage]);
-                            else nm_tma_load_2d(sa, &tmA, kb * BK_ELEMS, m0, &bar_full[stage]);
-                            nm_tma_load_2d(sa + A_BYTES, &tmW, w_k, w_n, &bar_full[stage]);
-                        }
-                    }
-                    __syncwarp();
-                    if constexpr (CONV) {
-                        if (++cb == a.cv.cblocks) { cb = 0; ++tap; }
-                    }
-                    if (++stage == stages) { stage = 0; phase ^= 1u; }
+                if (!ok) {
+                    long long t0 = clock64();  // bounded pause: copies in flight land before teardown
+                    while (clock64() - t0 < 4000000LL) {}
                 }
-            }
-            if (!ok) {
-                long long t0 = clock64();  // bounded pause: copies in flight land before teardown
-                while (clock64() - t0 < 4000000LL) {}
+            } else {
+                int stage = 0;
+                uint32_t phase = 0;
+                bool ok = true;
+                for (int tile = tile_first; ok && tile < a.num_tiles; tile += tile_step) {
+                    const int mt = tile / a.num_n_tiles;
+                    const int m0 = mt * TILE_M + (int)rank * BM;
+                    const int n0 = (tile % a.num_n_tiles) * BN + (int)rank * B_ROWS;
+                    Patch pt = {0, 0, 0};
+                    if constexpr (CONV) pt = patch_of(a.cv, mt * (TWO ? 2 : 1) + (int)rank);
+                    int kx = 0, ky = 0, cb = 0;   // CONV: K-block = (filter row, tap, channel block)
+                    for (int kb = 0; kb < a.num_k_blocks; ++kb) {
+                        if (!vote(nm_mbar_wait(&bar_empty[stage], phase ^ 1u, abortp, a.status))) { ok = false; break; }
+                        uint8_t* sa = tiles + (size_t)stage * STAGE_BYTES;
+                        int c_c = 0, c_w = 0, c_h = 0, w_k = kb * BK_ELEMS, w_n = n0;
+                        if constexpr (CONV) {
+                            c_c = cb * BK_ELEMS;
+                            c_w = pt.ox0 * a.cv.sw - a.cv.pw + kx;
+                            c_h = pt.oy0 * a.cv.sh - a.cv.ph + ky;
+                            if (a.cv.dw) {   // pooling: channel block = column tile, one constant matrix for every tap and tile
+                                c_c = (tile % a.num_n_tiles) * BK_ELEMS;
+                                w_k = 0;
+                                w_n = (int)rank * B_ROWS;
+                            }
+                        }
+                        if (ONE_LANE || nm_elect_one()) {
+                            if constexpr (TWO) {
+                                // both CTAs' copies are counted on the leader's barrier
+                                const uint32_t full = nm_mapa(nm_smem_u32(&bar_full[stage]), 0);
+                                if (rank == 0) nm_mbar_expect_tx(&bar_full[stage], 2 * STAGE_BYTES);
+                                if constexpr (CONV) nm_tma_load_4d_2cta(sa, &tmA, c_c, c_w, c_h, pt.img0, full);
+                                else nm_tma_load_2d_2cta(sa, &tmA, kb * BK_ELEMS, m0, full);
+                                nm_tma_load_2d_2cta(sa + A_BYTES, &tmW, w_k, w_n, full);
+                            } else {
+                                nm_mbar_expect_tx(&bar_full[stage], STAGE_BYTES);
+                                if constexpr (CONV) nm_tma_load_4d(sa, &tmA, c_c, c_w, c_h, pt.img0, &bar_full[stage]);
+                                else nm_tma_load_2d(sa, &tmA, kb * BK_ELEMS, m0, &bar_full[stage]);
+                                nm_tma_load_2d(sa + A_BYTES, &tmW, w_k, w_n, &bar_full[stage]);
+                            }
+                        }
+                        if constexpr (!ONE_LANE) __syncwarp();
+                        if constexpr (CONV) {
+                            if (++cb == a.cv.cblocks) {
+                                cb = 0;
+                                if (++kx == a.cv.kw_eff) { kx = 0; ++ky; }
+                            }
+                        }
+                        if (++stage == stages) { stage = 0; phase ^= 1u; }
+                    }
+                }
+                if (!ok) {
+                    long long t0 = clock64();  // bounded pause: copies in flight land before teardown
+                    while (clock64() - t0 < 4000000LL) {}
+                }
             }
         }
+        __syncwarp();
     } else if (warp == 1) {
         // ------------------------------------------------ MMA issuer (the leader CTA of a pair)
-        // All 32 lanes run the loop (waits, counters and descriptors stay warp-uniform); one elected
-        // lane, always the same, issues the tcgen05 instructions and their commits.
-        if (rank == 0) {
+        if (rank == 0 && (!ONE_LANE || nm_elect_one())) {
             int stage = 0;
             uint32_t phase = 0;
             int buf = 0;
             uint32_t acc_phase = 0;
             bool ok = true;
+            bool ready = false;   // the stage about to be used was seen complete
             [[maybe_unused]] int ws = 0;
             [[maybe_unused]] uint32_t wphase = 0;
             for (int tile = tile_first; ok && tile < a.num_tiles; tile += tile_step) {
                 // CTA-scope acquire also where the peer CTA's epilogue warps arrive: what the hand-back orders are
                 // tcgen05 operations, ordered by tcgen05.fence (a cluster-scope acquire costs ~400 cycles per tile)
-                if (!__all_sync(0xffffffffu, nm_mbar_wait(&bar_acc_empty[buf], acc_phase ^ 1u, abortp, a.status))) { ok = false; break; }
+                if (!vote(nm_mbar_wait(&bar_acc_empty[buf], acc_phase ^ 1u, abortp, a.status))) { ok = false; break; }
                 nm_tc_fence_after();
                 const uint32_t d_tmem = tmem_base + (uint32_t)(buf * BN);
                 if constexpr (HALO) {
                     const bool wait_w = !a.w_resident || tile == tile_first;
                     for (int cb = 0; ok && cb < a.cv.cblocks; ++cb) {
-                        if (!__all_sync(0xffffffffu, nm_mbar_wait(&bar_full[stage], phase, abortp, a.status))) { ok = false; break; }
+                        if (!ready && !nm_mbar_wait(&bar_full[stage], phase, abortp, a.status)) { ok = false; break; }
+                        const int nxt = stage + 1 == stages ? 0 : stage + 1;
+                        ready = nm_mbar_test_wait(&bar_full[nxt], nxt == 0 ? phase ^ 1u : phase);
                         const uint32_t sa = nm_smem_u32(tiles + (size_t)stage * STAGE_BYTES);
                         for (int tap = 0; tap < 9; ++tap) {
-                            if (wait_w && !__all_sync(0xffffffffu, nm_mbar_wait(&bar_wfull[ws], wphase, abortp, a.status))) { ok = false; break; }
+                            if (wait_w && !nm_mbar_wait(&bar_wfull[ws], wphase, abortp, a.status)) { ok = false; break; }
                             nm_tc_fence_after();
                             const int ky = tap / 3, kx = tap - 3 * ky;
                             const uint64_t adesc = nm_smem_desc_sw128(sa + (uint32_t)((HALO_W * ky + kx) * ROW_BYTES), HALO_W * ROW_BYTES);
                             const uint64_t bdesc = nm_smem_desc_sw128(nm_smem_u32(w_tiles + (size_t)ws * B_BYTES));
-                            if (nm_elect_one()) {
 #pragma unroll
-                                for (int k = 0; k < 4; ++k)
-                                    nm_mma_f16_2cta(d_tmem, adesc + 2 * k, bdesc + 2 * k, IDESC, (cb | tap | k) != 0 ? 1u : 0u);
-                                if (!a.w_resident) nm_tc_commit2(&bar_wempty[ws], 3);
-                                if (tap == 8) nm_tc_commit2(&bar_empty[stage], 3);
-                            }
-                            __syncwarp();
+                            for (int k = 0; k < 4; ++k)
+                                nm_mma_f16_2cta(d_tmem, adesc + 2 * k, bdesc + 2 * k, IDESC, (cb | tap | k) != 0 ? 1u : 0u);
+                            if (!a.w_resident) nm_tc_commit2(&bar_wempty[ws], 3);
+                            if (tap == 8) nm_tc_commit2(&bar_empty[stage], 3);
                             if (++ws == a.w_stages) { ws = 0; wphase ^= 1u; }
                         }
                         if (++stage == stages) { stage = 0; phase ^= 1u; }
                     }
                 }
                 for (int kb = 0; !HALO && kb < a.num_k_blocks; ++kb) {
-                    if (!__all_sync(0xffffffffu, nm_mbar_wait(&bar_full[stage], phase, abortp, a.status))) { ok = false; break; }
+                    if (!ready && !vote(nm_mbar_wait(&bar_full[stage], phase, abortp, a.status))) { ok = false; break; }
+                    if constexpr (ONE_LANE) {
+                        const int nxt = stage + 1 == stages ? 0 : stage + 1;
+                        ready = nm_mbar_test_wait(&bar_full[nxt], nxt == 0 ? phase ^ 1u : phase);
+                    }
                     nm_tc_fence_after();
                     const uint32_t sa = nm_smem_u32(tiles + (size_t)stage * STAGE_BYTES);
                     const uint64_t adesc = nm_smem_desc_sw128(sa);
                     const uint64_t bdesc = nm_smem_desc_sw128(sa + A_BYTES);
-                    if (nm_elect_one()) {
+                    if (ONE_LANE || nm_elect_one()) {
 #pragma unroll
                         for (int k = 0; k < 4; ++k) {  // 4 x 32 bytes of K per 128-byte row
                             const uint32_t accum = (kb | k) != 0 ? 1u : 0u;
@@ -441,28 +447,26 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                         if constexpr (TWO) nm_tc_commit2(&bar_empty[stage], 3);
                         else nm_tc_commit(&bar_empty[stage]);
                     }
-                    __syncwarp();
+                    if constexpr (!ONE_LANE) __syncwarp();
                     if (++stage == stages) { stage = 0; phase ^= 1u; }
                 }
                 if (!ok) break;
-                if (nm_elect_one()) {
+                if (ONE_LANE || nm_elect_one()) {
                     if constexpr (TWO) nm_tc_commit2(&bar_acc_full[buf], 3);
                     else nm_tc_commit(&bar_acc_full[buf]);
                 }
-                __syncwarp();
+                if constexpr (!ONE_LANE) __syncwarp();
                 buf ^= 1;
                 if (buf == 0) acc_phase ^= 1u;
             }
-            if (!ok) {
-                if (nm_elect_one()) {
-                    if constexpr (TWO) nm_tc_commit2(&bar_drain, 1);
-                    else nm_tc_commit(&bar_drain);
-                    long long t0 = clock64();
-                    while (!nm_mbar_try_wait(&bar_drain, 0) && clock64() - t0 < 200000000LL) {}
-                }
-                __syncwarp();
+            if (!ok && (ONE_LANE || nm_elect_one())) {
+                if constexpr (TWO) nm_tc_commit2(&bar_drain, 1);
+                else nm_tc_commit(&bar_drain);
+                long long t0 = clock64();
+                while (!nm_mbar_try_wait(&bar_drain, 0) && clock64() - t0 < 200000000LL) {}
             }
         }
+        __syncwarp();
     } else {
         // ------------------------------------------------ epilogue (warps 2..9)
         const int e = warp - 2;   // epilogue warp index
