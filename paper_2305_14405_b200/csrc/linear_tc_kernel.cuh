@@ -485,6 +485,8 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         const float inv_h = has_tab ? a.tab->inv_h : 0.f;
         const float off = has_tab ? a.tab->off : 0.f;
         const float nm1 = (float)(a.n_seg - 1);
+        const bool two_seg = BN < 256 && has_tab && a.n_seg == 2;   // (the code costs 256-wide tiles registers, and they are not bound here)
+        const float2 seg0 = two_seg ? a.tab->kb[0] : make_float2(0.f, 0.f), seg1 = two_seg ? a.tab->kb[1] : seg0;
         // the tiles this warp works on: every EPI_STEP-th of the CTA's, starting with its wsel-th
         const int my_first = tile_first + (ALT ? wsel * tile_step : 0);
         const int my_step = tile_step * EPI_STEP;
@@ -671,8 +673,13 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                             }
                         } else {
                             const uint64_t inv_h2 = nm_pack2(inv_h, inv_h), off2 = nm_pack2(off, off);
+                            if (BN < 256 && two_seg) {
 #pragma unroll
-                            for (int i = 0; i < 32; i += 2) nm_pwl_fast2(rep_lane, v[i], v[i + 1], inv_h2, off2, nm1);
+                                for (int i = 0; i < 32; i += 2) nm_pwl_two2(seg0, seg1, v[i], v[i + 1], inv_h2, off2);
+                            } else {
+#pragma unroll
+                                for (int i = 0; i < 32; i += 2) nm_pwl_fast2(rep_lane, v[i], v[i + 1], inv_h2, off2, nm1);
+                            }
                         }
                     } else if (a.idx_dump) {
 #pragma unroll

@@ -372,6 +372,22 @@ __device__ __forceinline__ void nm_pwl_fast2(uint32_t rep_lane, float& x0, float
     x1 = __fmaf_rn(k1, x1, c1);
 }
 
+// The same for a table of two segments held in registers (ReLU): floor(clamp(u, 0, 1)) is 1 exactly where u >= 1 (NaN: 0),
+// so the lookup is a comparison and two selections.
+__device__ __forceinline__ void nm_pwl_two2(float2 kb0, float2 kb1, float& x0, float& x1, uint64_t inv_h2, uint64_t off2)
+{
+    uint64_t u2, y2;
+    const uint64_t x2 = nm_pack2(x0, x1);
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(u2) : "l"(x2), "l"(inv_h2), "l"(off2));
+    float u0, u1;
+    nm_unpack2(u2, u0, u1);
+    const bool p0 = u0 >= 1.0f, p1 = u1 >= 1.0f;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;"
+        : "=l"(y2)
+        : "l"(nm_pack2(p0 ? kb1.x : kb0.x, p1 ? kb1.x : kb0.x)), "l"(x2), "l"(nm_pack2(p0 ? kb1.y : kb0.y, p1 ? kb1.y : kb0.y)));
+    nm_unpack2(y2, x0, x1);
+}
+
 __device__ __forceinline__ void nm_prefetch_tmap(const CUtensorMap* tmap)
 {
     asm volatile("prefetch.tensormap [%0];" ::"l"(tmap) : "memory");
