@@ -419,7 +419,7 @@ nm_status nm_attention_pwl_i8(nm_ctx* ctx, const nm_attn_i8_desc* d, void* strea
 // q != nullptr: the kernel also writes the int8 codes of its (rounded) output, scale 1/q_inv_scale
 static nm_status layernorm_checked(nm_ctx* ctx, const void* x, const float* gamma, const float* beta, void* y,
                                    int64_t rows, int32_t H, float eps, int32_t rsqrt_slot, nm_dtype dtype, void* stream,
-                                   int8_t* q, float q_inv_scale)
+                                   int8_t* q, float q_inv_scale, bool early)
 {
     if (!ctx) return NM_ERR_INVALID_ARG;
     if (rows < 0 || H < 0) return NM_ERR_SHAPE;
@@ -430,13 +430,13 @@ static nm_status layernorm_checked(nm_ctx* ctx, const void* x, const float* gamm
     if (H % 8 != 0) return NM_ERR_SHAPE;
     if (!nm_aligned16(x) || !nm_aligned16(y) || !nm_aligned16(gamma) || !nm_aligned16(beta)) return NM_ERR_ALIGNMENT;
     return nm_launch_layernorm(ctx, x, gamma, beta, y, rows, H, eps, rsqrt_slot, NM_SLOT_NONE, dtype, (cudaStream_t)stream,
-                               q, q_inv_scale);
+                               q, q_inv_scale, early);
 }
 
 nm_status nm_layernorm_pwl(nm_ctx* ctx, const void* x, const float* gamma, const float* beta, void* y,
                            int64_t rows, int32_t H, float eps, int32_t rsqrt_slot, nm_dtype dtype, void* stream)
 {
-    return layernorm_checked(ctx, x, gamma, beta, y, rows, H, eps, rsqrt_slot, dtype, stream, nullptr, 0.f);
+    return layernorm_checked(ctx, x, gamma, beta, y, rows, H, eps, rsqrt_slot, dtype, stream, nullptr, 0.f, false);
 }
 
 nm_status nm_layernorm_pwl_sqrt_recip(nm_ctx* ctx, const void* x, const float* gamma, const float* beta, void* y,
@@ -608,7 +608,7 @@ static nm_status encoder_layer_impl(nm_ctx* ctx, const nm_encoder_weights* w, co
     s = linear(a_in, H, w->Wo, H, w->bo, x, NM_SLOT_NONE, z, act, w->a_attn, w->s_wo, 0.f);
     if (s != NM_OK) return s;
     s = layernorm_checked(ctx, z, w->g1, w->be1, x1, T, H, c->eps, c->rsqrt_slot, act, stream, i8 ? q8 : nullptr,
-                          i8 ? 1.0f / w->a_x1 : 0.f);
+                          i8 ? 1.0f / w->a_x1 : 0.f, act != NM_F32);
     if (s != NM_OK) return s;
 
     // g = PWLgelu(x1 W1^T + b1)   (int8 path: requantised in the epilogue with the scale of g)
@@ -622,7 +622,7 @@ static nm_status encoder_layer_impl(nm_ctx* ctx, const nm_encoder_weights* w, co
     if (s != NM_OK) return s;
     const bool next_codes = i8 && next_a_x > 0.f;
     return layernorm_checked(ctx, z, w->g2, w->be2, y, T, H, c->eps, c->rsqrt_slot, act, stream, next_codes ? q8 : nullptr,
-                             next_codes ? 1.0f / next_a_x : 0.f);
+                             next_codes ? 1.0f / next_a_x : 0.f, act != NM_F32);
 }
 
 nm_status nm_encoder_stack(nm_ctx* ctx, const nm_encoder_weights* layers, int32_t n_layers, const nm_encoder_cfg* c,

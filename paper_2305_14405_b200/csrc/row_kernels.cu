@@ -78,13 +78,16 @@ __global__ void __launch_bounds__(256) pwl_apply_kernel(const NmTable* __restric
 // GB_REGS: the lane's gamma and beta values stay in registers for all of the warp's rows (2 x ITERS x N
 // registers: rows up to 32 x 3 vectors, two blocks per SM).  Otherwise they are fetched per row through L1,
 // which then carries four times the bytes of the row itself and ~700 exposed cycles per row.
-template <typename T, int ITERS, bool GB_REGS>
-__global__ void __launch_bounds__(256, GB_REGS ? 2 : 1) layernorm_kernel(const NmTable* __restrict__ tab,
+// ONE_ROW: no warp has more than one row; gamma and beta stay in registers at any width (one block per SM is enough then),
+// the rsqrt table comes from shared memory, and where the caller knows them complete (`early`) all three are fetched while
+// the previous kernel still runs.
+template <typename T, int ITERS, bool GB_REGS, bool ONE_ROW>
+__global__ void __launch_bounds__(256, GB_REGS && !ONE_ROW ? 2 : 1) layernorm_kernel(const NmTable* __restrict__ tab,
                                                         const NmTable* __restrict__ tab2, const T* __restrict__ x,
                                                         const float* __restrict__ gamma,
                                                         const float* __restrict__ beta, T* __restrict__ y,
                                                         int64_t rows, int H, float eps, int8_t* __restrict__ q,
-                                                        float q_inv_scale)
+                                                        float q_inv_scale, int early)
 {
     // A warp walks over rows with a grid-wide stride; the raw 16-byte vectors of its NEXT row are
     // already in flight while the current row is reduced and written, so every SM keeps several
@@ -96,6 +99,28 @@ __global__ void __launch_bounds__(256, GB_REGS ? 2 : 1) layernorm_kernel(const N
     const int nvec = H / N;  // H is a multiple of N
     const float inv_h = tab->inv_h, off = tab->off, nm1 = (float)(tab->n - 1);
     nm_grid_launch_dependents();   // the next kernel may start its set-up
+    __shared__ float2 s_tab[ONE_ROW ? NM_MAX_SEGMENTS : 1];
+    float rg[GB_REGS ? ITERS : 1][N], rb[GB_REGS ? ITERS : 1][N];
+    auto fetch_gb = [&]() {
+        if constexpr (GB_REGS) {
+#pragma unroll
+            for (int it = 0; it < ITERS; ++it) {
+                const int v = it * 32 + lane;
+                if (v < nvec) {
+#pragma unroll
+                    for (int i = 0; i < N; i += 4) {
+                        *reinterpret_cast<float4*>(&rg[it][i]) = __ldg(reinterpret_cast<const float4*>(gamma + v * N + i));
+                        *reinterpret_cast<float4*>(&rb[it][i]) = __ldg(reinterpret_cast<const float4*>(beta + v * N + i));
+                    }
+                }
+            }
+        }
+    };
+    if constexpr (ONE_ROW) {
+        for (int i = threadIdx.x; i < tab->n; i += blockDim.x) s_tab[i] = tab->kb[i];
+        if (early) fetch_gb();
+        __syncthreads();
+    }
     nm_grid_dependency_wait();     // x comes from the previous kernel
     uint4 nxt[ITERS];
     if (warp0 < rows) {
@@ -105,20 +130,7 @@ __global__ void __launch_bounds__(256, GB_REGS ? 2 : 1) layernorm_kernel(const N
             if (v < nvec) nxt[it] = *reinterpret_cast<const uint4*>(x + warp0 * H + v * N);
         }
     }
-    float rg[GB_REGS ? ITERS : 1][N], rb[GB_REGS ? ITERS : 1][N];
-    if constexpr (GB_REGS) {
-#pragma unroll
-        for (int it = 0; it < ITERS; ++it) {
-            const int v = it * 32 + lane;
-            if (v < nvec) {
-#pragma unroll
-                for (int i = 0; i < N; i += 4) {
-                    *reinterpret_cast<float4*>(&rg[it][i]) = __ldg(reinterpret_cast<const float4*>(gamma + v * N + i));
-                    *reinterpret_cast<float4*>(&rb[it][i]) = __ldg(reinterpret_cast<const float4*>(beta + v * N + i));
-                }
-            }
-        }
-    }
+    if (!ONE_ROW || !early) fetch_gb();
     for (int64_t row = warp0; row < rows; row += nwarps) {
         float f[ITERS][N];
         float sum = 0.f;
@@ -135,7 +147,7 @@ __global__ void __launch_bounds__(256, GB_REGS ? 2 : 1) layernorm_kernel(const N
             }
         }
         const int64_t nrow = row + nwarps;
-        if (nrow < rows) {
+        if (!ONE_ROW && nrow < rows) {
 #pragma unroll
             for (int it = 0; it < ITERS; ++it) {
                 const int v = it * 32 + lane;
@@ -162,7 +174,7 @@ __global__ void __launch_bounds__(256, GB_REGS ? 2 : 1) layernorm_kernel(const N
         for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
         const float var = sq / (float)H + eps;
         const int s = nm_pwl_index(var, inv_h, off, nm1);
-        const float2 kb = tab->kb[s];
+        const float2 kb = ONE_ROW ? s_tab[s] : tab->kb[s];
         float r = __fmaf_rn(kb.x, var, kb.y);
         if (tab2) {   // two-table form: `tab` gave sqrt(v + eps), `tab2` takes its reciprocal
             const int s2 = nm_pwl_index(r, tab2->inv_h, tab2->off, (float)(tab2->n - 1));
@@ -252,7 +264,7 @@ __global__ void wait_selftest_kernel(int* status, long long limit_cycles, int* r
 
 template <typename T>
 nm_status launch_ln(nm_ctx* ctx, const NmTable* tab, const NmTable* tab2, const void* x, const float* gamma, const float* beta, void* y,
-                    int64_t rows, int H, float eps, int8_t* q, float q_inv_scale, cudaStream_t st)
+                    int64_t rows, int H, float eps, int8_t* q, float q_inv_scale, bool early, cudaStream_t st)
 {
     constexpr int N = VecOf<T>::N;
     const int nvec = H / N;
@@ -263,6 +275,9 @@ nm_status launch_ln(nm_ctx* ctx, const NmTable* tab, const NmTable* tab2, const 
     // bandwidth-bound and want more warps per SM: the per-row fetch of gamma and beta, 6 blocks of 8 warps per SM
     // (5.5 instead of 4.9 TB/s at 2^19 x 768).
     const bool small = (double)rows * H * sizeof(T) <= 48e6 && iters <= 3;
+    // At most one row per warp of one block per SM: bound by latency alone (128 x 1024 bf16 with int8 codes: 4.6 us per
+    // launch in a chain, 2.8 so; 37 x 768: 3.2 and 2.3).
+    const bool one_row = rows <= (int64_t)ctx->sm_count * (threads / 32) && iters * N <= 32;
     int64_t blocks = (rows + 7) / 8;
  NmLaunchScope scope(ctx, NM_KERNEL_LAYERNORM, 2.0 * (double)rows * H * sizeof(T), st);
     cudaLaunchConfig_t cfg;
@@ -277,27 +292,35 @@ nm_status launch_ln(nm_ctx* ctx, const NmTable* tab, const NmTable* tab2, const 
     cfg.numAttrs = ctx->pdl ? 1 : 0;
     const T* xt = (const T*)x;
     T* yt = (T*)y;
-#define NM_LN_CASE(I, GB)                                                                                     \
+#define NM_LN_CASE(I, GB, ONE)                                                                                \
     do {                                                                                                      \
         static int resident = 0;   /* blocks per SM that this instantiation's registers allow */              \
         if (GB && resident == 0 &&                                                                            \
-            (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, layernorm_kernel<T, I, GB>, threads, 0) != \
+            (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, layernorm_kernel<T, I, GB, ONE>, threads, 0) != \
                  cudaSuccess || resident < 1))                                                                \
             resident = 2;                                                                                     \
         const int64_t cap = (int64_t)ctx->sm_count * (GB ? resident : 6);                                     \
         cfg.gridDim = dim3((unsigned)(blocks > cap ? cap : blocks));                                          \
-        cudaLaunchKernelEx(&cfg, layernorm_kernel<T, I, GB>, tab, tab2, xt, gamma, beta, yt, rows, H, eps, q,  \
-                           q_inv_scale);                                                                      \
+        cudaLaunchKernelEx(&cfg, layernorm_kernel<T, I, GB, ONE>, tab, tab2, xt, gamma, beta, yt, rows, H,     \
+                           eps, q, q_inv_scale, early ? 1 : 0);                                               \
     } while (0)
-    if (small && iters <= 1) NM_LN_CASE(1, true);
-    else if (small && iters <= 2) NM_LN_CASE(2, true);
-    else if (small && iters <= 3) NM_LN_CASE(3, true);
-    else if (iters <= 1) NM_LN_CASE(1, false);
-    else if (iters <= 2) NM_LN_CASE(2, false);
-    else if (iters <= 3) NM_LN_CASE(3, false);
-    else if (iters <= 4) NM_LN_CASE(4, false);
-    else if (iters <= 8) NM_LN_CASE(8, false);
-    else if (iters <= 16) NM_LN_CASE(16, false);
+    if constexpr (N == 4) {
+        if (one_row && iters <= 4) NM_LN_CASE(4, true, true);
+        else if (one_row) NM_LN_CASE(8, true, true);
+    }
+    if (one_row && N == 4) {}
+    else if (one_row && iters <= 2) NM_LN_CASE(2, true, true);
+    else if (one_row && iters <= 3) NM_LN_CASE(3, true, true);
+    else if (one_row) NM_LN_CASE(4, true, true);
+    else if (small && iters <= 1) NM_LN_CASE(1, true, false);
+    else if (small && iters <= 2) NM_LN_CASE(2, true, false);
+    else if (small && iters <= 3) NM_LN_CASE(3, true, false);
+    else if (iters <= 1) NM_LN_CASE(1, false, false);
+    else if (iters <= 2) NM_LN_CASE(2, false, false);
+    else if (iters <= 3) NM_LN_CASE(3, false, false);
+    else if (iters <= 4) NM_LN_CASE(4, false, false);
+    else if (iters <= 8) NM_LN_CASE(8, false, false);
+    else if (iters <= 16) NM_LN_CASE(16, false, false);
     else return NM_ERR_UNSUPPORTED;
 #undef NM_LN_CASE
     return cudaGetLastError() == cudaSuccess ? NM_OK : NM_ERR_CUDA;
@@ -336,14 +359,14 @@ nm_status nm_launch_pwl_apply(nm_ctx* ctx, int slot, const void* x, void* y, int
 
 nm_status nm_launch_layernorm(nm_ctx* ctx, const void* x, const float* gamma, const float* beta, void* y,
                               int64_t rows, int32_t H, float eps, int32_t slot, int32_t slot2, nm_dtype dtype,
-                              cudaStream_t st, int8_t* q, float q_inv_scale)
+                              cudaStream_t st, int8_t* q, float q_inv_scale, bool early)
 {
     const NmTable* tab = ctx->d_tables + slot;
     const NmTable* tab2 = slot2 == NM_SLOT_NONE ? nullptr : ctx->d_tables + slot2;
     switch (dtype) {
-    case NM_F32: return launch_ln<float>(ctx, tab, tab2, x, gamma, beta, y, rows, H, eps, q, q_inv_scale, st);
-    case NM_BF16: return launch_ln<__nv_bfloat16>(ctx, tab, tab2, x, gamma, beta, y, rows, H, eps, q, q_inv_scale, st);
-    case NM_F16: return launch_ln<__half>(ctx, tab, tab2, x, gamma, beta, y, rows, H, eps, q, q_inv_scale, st);
+    case NM_F32: return launch_ln<float>(ctx, tab, tab2, x, gamma, beta, y, rows, H, eps, q, q_inv_scale, early, st);
+    case NM_BF16: return launch_ln<__nv_bfloat16>(ctx, tab, tab2, x, gamma, beta, y, rows, H, eps, q, q_inv_scale, early, st);
+    case NM_F16: return launch_ln<__half>(ctx, tab, tab2, x, gamma, beta, y, rows, H, eps, q, q_inv_scale, early, st);
     default: return NM_ERR_UNSUPPORTED;
     }
 }
