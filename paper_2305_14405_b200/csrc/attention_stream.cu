@@ -30,6 +30,11 @@
 // The second term's 32 columns make it two CTAs per SM instead of three.  B 7, L 333, 12 heads: 2368 us on the CUDA
 // cores, 21.3 us here; B 1, L 37: 13.4 and 7.0 us.
 //
+// ONE form (L <= 128, a single 128-key chunk): the scores and the accumulator do not share columns (128 | 64, and P behind
+// them: 256 columns, two CTAs per SM), so the one Q K^T of sweep 1 serves sweep 2 as well, and nothing is fetched or
+// multiplied twice in what is then a latency-bound kernel (B 1, L 128, 16 heads: 6.4 -> 4.9 us; B 32, L 100, 12 heads:
+// 19.0 -> 16.7).
+//
 //   warp 0            control: TMA loads (K chunks through two stages, V chunks through one) and the tcgen05.mma
 //                     for S = Q K_c^T and O += P_c V_c (V as an MN-major operand).  It sleeps in a named barrier
 //                     (bar.sync) that the softmax warps signal with bar.arrive, so hand-offs cost no polling.
@@ -162,16 +167,17 @@ __device__ __forceinline__ void load_first_v(const LoadCtx& c, const Tile& t)
     nm_tma_load_3d(c.v_st, c.tmV, t.g * HD, 0, t.b, c.bar_v_full);
 }
 
-template <typename T, bool CLAMP_HI, bool RAGGED>
-__global__ void __launch_bounds__(160, RAGGED ? 2 : 3)
+template <typename T, bool CLAMP_HI, bool RAGGED, bool ONE>
+__global__ void __launch_bounds__(160, RAGGED || ONE ? 2 : 3)
 attention_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                         const __grid_constant__ CUtensorMap tmV, const SArgs a)
 {
     constexpr uint32_t IDESC_QK = nm_idesc(1, AT<T>::fmt, 0, 0, BQ, CK);   // S chunk: 128 x 64
     constexpr uint32_t IDESC_PV = nm_idesc(1, AT<T>::fmt, 0, 1, BQ, HD);   // O: 128 x 64, V MN-major
     constexpr uint32_t IDESC_QK1 = nm_idesc(1, AT<T>::fmt, 0, 0, BQ, 2 * CK);   // sweep 1: 128 x 128
-    constexpr uint32_t TMEM_COLS = 128;   // S | O; sweep 1 writes 128 keys over [S | O]
-    constexpr uint32_t O_OFF = 64;
+    // S | O, sweep 1 writes 128 keys over [S | O]; ONE: S of 128 keys | O | P
+    constexpr uint32_t TMEM_COLS = ONE ? 256 : 128;
+    constexpr uint32_t O_OFF = ONE ? 128 : 64;
     // The 16-bit P tile goes through a second allocation of 32 columns (64 keys, two per column) and is the A operand
     // of P V from there; three CTAs hold 3 x (128 + 32) of the SM's 512 columns.  RAGGED: 32 more for the low terms.
     constexpr uint32_t P_COLS = RAGGED ? 64 : 32;
@@ -185,7 +191,7 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
 
     const int L = a.L;
     const int n = RAGGED ? (L + CK - 1) / CK : L / CK;                    // 64-key chunks of sweep 2
-    const int n128 = RAGGED ? (L + 2 * CK - 1) / (2 * CK) : L / (2 * CK);   // 128-key chunks of sweep 1
+    const int n128 = ONE ? 1 : RAGGED ? (L + 2 * CK - 1) / (2 * CK) : L / (2 * CK);   // 128-key chunks of sweep 1
     uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     uint8_t* q_s = base;                       // 16 KB
     uint8_t* k_st = q_s + BQ * ROWB;           // 2 x 8 KB
@@ -234,7 +240,7 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
     }
     if (warp == 0) {
         nm_tmem_alloc(&tmem_slot, TMEM_COLS);
-        nm_tmem_alloc(&tmem_slot_p, P_COLS);
+        if constexpr (!ONE) nm_tmem_alloc(&tmem_slot_p, P_COLS);
         nm_tmem_relinquish();
     } else {
         // 16-way replicated exp table: entry s, copy c at rep[s*16 + c].  A 64-bit warp load is served
@@ -247,7 +253,7 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
     __syncthreads();
     nm_tc_fence_after();
     const uint32_t tmem_base = tmem_slot;
-    const uint32_t tmem_p = tmem_slot_p;
+    const uint32_t tmem_p = ONE ? tmem_base + 192u : tmem_slot_p;
     volatile int* abortp = &abort_flag;
     nm_grid_launch_dependents();   // the next kernel may start its set-up
     nm_grid_dependency_wait();     // Q, K, V come from the previous kernel
@@ -267,7 +273,7 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
         bool ok = true;
         const uint64_t qdesc = nm_smem_desc_sw128(nm_smem_u32(q_s));
         // completions consumed so far on each barrier (they run on from tile to tile)
-        uint32_t q_cnt = 0, k1_cnt0 = 0, k1_cnt1 = 0, k_cnt0 = 0, k_n128 = 0, v_cnt = 0, pv_cnt = 0;
+        uint32_t q_cnt = 0, k1_cnt0 = 0, k1_cnt1 = 0, k_cnt0 = 0, k_cnt1 = 0, v_cnt = 0, pv_cnt = 0;
         for (int tile = (int)blockIdx.x, ti = 0; tile < n_tiles; tile += (int)gridDim.x, ++ti) {
             const Tile t = tile_of(tile);
             const int g = t.g, b = t.b;
@@ -293,7 +299,7 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                 __syncwarp();
             };
             if (n128 > 0) issue_qk1(0);
-            for (int i = 0; i < n128; ++i) {
+            for (int i = 0; !ONE && i < n128; ++i) {
                 asm volatile("bar.sync %0, %1;" ::"r"(bar_sc), "n"(160) : "memory");   // S-consumed: chunk i is in registers
                 if (i + 1 < n128) issue_qk1(i + 1);
                 if (ok && i + 2 < n128 && nm_elect_one()) {   // its MMAs are complete: the stage takes the chunk after next
@@ -314,8 +320,8 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                 __syncwarp();
             };
             auto issue_qk = [&](int j) {   // S = Q K^T
-                const uint32_t par = ((j & 1) ? k_n128 : k_cnt0) & 1u;
-                if (j & 1) ++k_n128; else ++k_cnt0;
+                const uint32_t par = ((j & 1) ? k_cnt1 : k_cnt0) & 1u;
+                if (j & 1) ++k_cnt1; else ++k_cnt0;
                 if (!ok) return;
                 if (!wait(&bar_k_full[j & 1], par)) { ok = false; return; }
                 nm_tc_fence_after();
@@ -327,13 +333,19 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                 }
                 __syncwarp();
             };
-            load_k(0);   // every MMA of sweep 1 has completed: the K stages are free
-            if (n > 1) load_k(1);
-            issue_qk(0);
+            if constexpr (!ONE) {
+                load_k(0);   // every MMA of sweep 1 has completed: the K stages are free
+                if (n > 1) load_k(1);
+                issue_qk(0);
+            }
             for (int j = 0; j < n; ++j) {
-                asm volatile("bar.sync %0, %1;" ::"r"(bar_sc), "n"(160) : "memory");   // S-consumed(j)
-                if (j + 1 < n) issue_qk(j + 1);
-                if (j + 2 < n) load_k(j + 2);
+                if constexpr (!ONE) {
+                    asm volatile("bar.sync %0, %1;" ::"r"(bar_sc), "n"(160) : "memory");   // S-consumed(j)
+                    if (j + 1 < n) issue_qk(j + 1);
+                    if (j + 2 < n) load_k(j + 2);
+                } else if (j + 1 == n && more && ok) {
+                    if (!wait(&bar_s_full, (uint32_t)ti & 1u)) ok = false;   // the tile's one product has read Q and K
+                }
                 // Last chunk: every Q K^T of the tile has completed, so Q, the K stages and p_s take the next tile's
                 // first loads now.
                 if (j + 1 == n && more && ok && nm_elect_one()) load_tile_head(lc, tile_of(tile + (int)gridDim.x));
@@ -410,6 +422,12 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
         };
         // completions consumed so far: S products, P V products
         uint32_t s_cnt = 0, pv_base = 0;
+        float r_inv_h = 0.f, r_off = 0.f, r_nm1 = 0.f;   // fetched early where latency counts and registers do not
+        if constexpr (ONE) {
+            r_inv_h = a.t_rcp->inv_h;
+            r_off = a.t_rcp->off;
+            r_nm1 = (float)(a.t_rcp->n - 1);
+        }
         for (int tile = (int)blockIdx.x; tile < n_tiles; tile += (int)gridDim.x) {
             const Tile t = tile_of(tile);
             const int qb = t.qb, g = t.g, b = t.b;
@@ -428,8 +446,9 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
 #pragma unroll
                     for (int hh = 0; hh < 4; ++hh) {   // 128 keys: the scores span [S | O]
                         uint32_t r[32];
+                        if (ONE && hh * 32 >= L) continue;   // no keys there
                         nm_tmem_ld32_sync(t_row + (uint32_t)(hh * 32), r);
-                        if (hh == 3) {   // all of it is in registers: the control warp may overwrite S
+                        if (!ONE && hh == 3) {   // all of it is in registers: the control warp may overwrite S
                             nm_tc_fence_before();
                             asm volatile("bar.arrive %0, %1;" ::"r"(bar_sc), "n"(160) : "memory");
                         }
@@ -447,7 +466,7 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                         }
                         m = max3f(m, m0, m1);
                     }
-                } else {
+                } else if (!ONE) {
                     asm volatile("bar.arrive %0, %1;" ::"r"(bar_sc), "n"(160) : "memory");
                 }
             }
@@ -458,22 +477,24 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
             // take the maximum as their score (which keeps the table index in range) and the exponential 0.
             auto chunk = [&](int j, auto last) {
                 constexpr bool LAST = decltype(last)::value;
-                wait_all(&bar_s_full, s_cnt & 1u);
-                ++s_cnt;
-                if (ok) nm_tc_fence_after();
+                if constexpr (!ONE) {
+                    wait_all(&bar_s_full, s_cnt & 1u);
+                    ++s_cnt;
+                    if (ok) nm_tc_fence_after();
+                }
 #pragma unroll
                 for (int hh = 0; hh < 2; ++hh) {
                     const int lim = LAST ? L - j * CK - hh * 32 : 32;
                     uint32_t r[32];
                     if (ok && live) {
-                        nm_tmem_ld32_sync(t_row + (uint32_t)(hh * 32), r);
+                        nm_tmem_ld32_sync(t_row + (uint32_t)((ONE ? j * CK : 0) + hh * 32), r);
                         if constexpr (LAST) {
 #pragma unroll
                             for (int k = 0; k < 32; ++k)
                                 if (k >= lim) r[k] = __float_as_uint(m);
                         }
                     }
-                    if (hh == 1) {
+                    if (!ONE && hh == 1) {
                         nm_tc_fence_before();
                         asm volatile("bar.arrive %0, %1;" ::"r"(bar_sc), "n"(160) : "memory");
                     }
@@ -550,7 +571,8 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
             if constexpr (RAGGED) chunk(n - 1, std::true_type{});
             const float sum = (sum0 + sum1) + (sum2 + sum3);
             // ---- r = PWL_recip(sigma), then O * r
-            const int sr = nm_pwl_index(sum, a.t_rcp->inv_h, a.t_rcp->off, (float)(a.t_rcp->n - 1));
+            const int sr = ONE ? nm_pwl_index(sum, r_inv_h, r_off, r_nm1)
+                               : nm_pwl_index(sum, a.t_rcp->inv_h, a.t_rcp->off, (float)(a.t_rcp->n - 1));
             const float2 kbr = a.t_rcp->kb[sr];
             const float rinv = __fmaf_rn(kbr.x, sum, kbr.y);
             wait_all(&bar_p_empty, (pv_base + (uint32_t)(n - 1)) & 1u);   // the last P V has completed
@@ -598,7 +620,7 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
         __syncwarp();
         nm_tc_fence_after();
         nm_tmem_dealloc(tmem_base, TMEM_COLS);
-        nm_tmem_dealloc(tmem_p, P_COLS);
+        if constexpr (!ONE) nm_tmem_dealloc(tmem_p, P_COLS);
     }
 }
 
@@ -621,7 +643,7 @@ nm_status make_map(nm_ctx* ctx, CUtensorMap* m, const void* ptr, nm_dtype dt, co
     return r == CUDA_SUCCESS ? NM_OK : NM_ERR_CUDA;
 }
 
-template <typename T, bool CLAMP_HI, bool RAGGED>
+template <typename T, bool CLAMP_HI, bool RAGGED, bool ONE>
 nm_status launch(nm_ctx* ctx, const nm_attn_desc* d, cudaStream_t st, int8_t* out_q, float q_inv_scale)
 {
     SArgs a;
@@ -640,16 +662,16 @@ nm_status launch(nm_ctx* ctx, const nm_attn_desc* d, cudaStream_t st, int8_t* ou
     if ((s = make_map(ctx, &tmQ, d->Q, d->dtype, d, BQ)) != NM_OK) return s;
     if ((s = make_map(ctx, &tmK, d->K, d->dtype, d, CK)) != NM_OK) return s;
     if ((s = make_map(ctx, &tmV, d->V, d->dtype, d, CK)) != NM_OK) return s;
-    auto kern = attention_stream_kernel<T, CLAMP_HI, RAGGED>;
+    auto kern = attention_stream_kernel<T, CLAMP_HI, RAGGED, ONE>;
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
         return NM_ERR_CUDA;
     const int64_t tiles = (int64_t)d->B * d->heads * ((d->L + BQ - 1) / BQ);
     if (tiles > 0x7fffffffLL) return NM_ERR_SHAPE;
-    // persistent: one resident wave of CTAs, each walking over tiles.  Three CTAs per SM (RAGGED: two) by the launch
-    // bounds (registers) and by tensor memory (3 x 160 or 2 x 192 of 512 columns); fewer if the exp table makes the
+    // persistent: one resident wave of CTAs, each walking over tiles.  Three CTAs per SM (RAGGED, ONE: two) by the launch
+    // bounds (registers) and by tensor memory (3 x 160, 2 x 192 or 2 x 256 of 512 columns); fewer if the exp table makes the
     // shared memory larger (233472 bytes per SM, 1 KB reserved per CTA).
     int64_t per_sm = 233472 / (int64_t)(smem + 1024 + 1536);
-    if (per_sm > (RAGGED ? 2 : 3)) per_sm = RAGGED ? 2 : 3;
+    if (per_sm > (RAGGED || ONE ? 2 : 3)) per_sm = RAGGED || ONE ? 2 : 3;
     if (per_sm < 1) per_sm = 1;
     int64_t grid = (int64_t)ctx->sm_count * per_sm;
     if (grid > tiles) grid = tiles;
@@ -690,13 +712,15 @@ nm_status nm_launch_attention_stream(nm_ctx* ctx, const nm_attn_desc* d, cudaStr
     if (!nm_attention_stream_any_length_supported(d)) return NM_ERR_UNSUPPORTED;
     // the softmax input is never positive: a table whose range reaches 0 needs no upper clamp
     const bool clamp_hi = ctx->h_tables[d->exp_slot].x_max < 0.0f;
-    const bool ragged = d->L % 128 != 0;
-#define NM_ATTN_CASE(T)                                                                                               \
-    (clamp_hi ? (ragged ? launch<T, true, true>(ctx, d, st, out_q, q_inv_scale)                                       \
-                        : launch<T, true, false>(ctx, d, st, out_q, q_inv_scale))                                     \
-              : (ragged ? launch<T, false, true>(ctx, d, st, out_q, q_inv_scale)                                      \
-                        : launch<T, false, false>(ctx, d, st, out_q, q_inv_scale)))
+    const bool ragged = d->L % 128 != 0, one = d->L <= 128;
+#define NM_ATTN_FORM(T, CH)                                                                                           \
+    (one ? (ragged ? launch<T, CH, true, true>(ctx, d, st, out_q, q_inv_scale)                                        \
+                   : launch<T, CH, false, true>(ctx, d, st, out_q, q_inv_scale))                                      \
+         : (ragged ? launch<T, CH, true, false>(ctx, d, st, out_q, q_inv_scale)                                       \
+                   : launch<T, CH, false, false>(ctx, d, st, out_q, q_inv_scale)))
+#define NM_ATTN_CASE(T) (clamp_hi ? NM_ATTN_FORM(T, true) : NM_ATTN_FORM(T, false))
     if (d->dtype == NM_BF16) return NM_ATTN_CASE(__nv_bfloat16);
     return NM_ATTN_CASE(__half);
 #undef NM_ATTN_CASE
+#undef NM_ATTN_FORM
 }
