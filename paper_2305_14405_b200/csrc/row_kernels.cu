@@ -75,14 +75,17 @@ __global__ void __launch_bounds__(256) pwl_apply_kernel(const NmTable* __restric
 
 // ---- LayerNorm with PWL rsqrt: one warp per row, the row kept in registers ------
 //   mu = mean(z); v = mean((z-mu)^2); r = PWL_rsqrt(v + eps); y = (z-mu)*r*gamma + beta
-// GB_REGS: the lane's gamma and beta values stay in registers for all of the warp's rows (2 x ITERS x N
-// registers: rows up to 32 x 3 vectors, two blocks per SM).  Otherwise they are fetched per row through L1,
-// which then carries four times the bytes of the row itself and ~700 exposed cycles per row.
-// ONE_ROW: no warp has more than one row; gamma and beta stay in registers at any width (one block per SM is enough then),
-// the rsqrt table comes from shared memory, and where the caller knows them complete (`early`) all three are fetched while
-// the previous kernel still runs.
-template <typename T, int ITERS, bool GB_REGS, bool ONE_ROW>
-__global__ void __launch_bounds__(256, GB_REGS && !ONE_ROW ? 2 : 1) layernorm_kernel(const NmTable* __restrict__ tab,
+// A row is a chain of its load, two shuffle trees, two divisions and a table lookup, about 1.9k cycles whatever its loads do.
+// Where gamma and beta are for that time:
+//   LN_SMEM     in shared memory as the lanes read them (16-byte groups of consecutive lanes side by side), MINB blocks of 8
+//               warps per SM: tensors beyond the L2, which want many warps, and rows too wide for the registers (fetched per
+//               row through L1 they carried four times the row's bytes).
+//   LN_REGS     in the lane's registers for all of the warp's rows (rows up to 32 x 3 vectors, two blocks per SM).
+//   LN_ONE_ROW  likewise at any width, no warp having more than one row, one block per SM; where the caller knows them complete
+//               (`early`) they are fetched while the previous kernel still runs.
+enum { LN_SMEM, LN_REGS, LN_ONE_ROW };
+template <typename T, int ITERS, int MODE, int MINB>
+__global__ void __launch_bounds__(256, MINB) layernorm_kernel(const NmTable* __restrict__ tab,
                                                         const NmTable* __restrict__ tab2, const T* __restrict__ x,
                                                         const float* __restrict__ gamma,
                                                         const float* __restrict__ beta, T* __restrict__ y,
@@ -99,7 +102,10 @@ __global__ void __launch_bounds__(256, GB_REGS && !ONE_ROW ? 2 : 1) layernorm_ke
     const int nvec = H / N;  // H is a multiple of N
     const float inv_h = tab->inv_h, off = tab->off, nm1 = (float)(tab->n - 1);
     nm_grid_launch_dependents();   // the next kernel may start its set-up
-    __shared__ float2 s_tab[ONE_ROW ? NM_MAX_SEGMENTS : 1];
+    constexpr bool GB_REGS = MODE != LN_SMEM, ONE_ROW = MODE == LN_ONE_ROW;
+    constexpr int Q = N / 4;           // 16-byte groups of gamma (and of beta) per vector
+    extern __shared__ float4 s_gb[];   // LN_SMEM: gamma, then beta: [ITERS][Q][32]
+    __shared__ float2 s_tab[MODE != LN_REGS ? NM_MAX_SEGMENTS : 1];
     float rg[GB_REGS ? ITERS : 1][N], rb[GB_REGS ? ITERS : 1][N];
     auto fetch_gb = [&]() {
         if constexpr (GB_REGS) {
@@ -116,8 +122,10 @@ __global__ void __launch_bounds__(256, GB_REGS && !ONE_ROW ? 2 : 1) layernorm_ke
             }
         }
     };
-    if constexpr (ONE_ROW) {
+    if constexpr (MODE != LN_REGS) {
         for (int i = threadIdx.x; i < tab->n; i += blockDim.x) s_tab[i] = tab->kb[i];
+    }
+    if constexpr (ONE_ROW) {
         if (early) fetch_gb();
         __syncthreads();
     }
@@ -131,6 +139,14 @@ __global__ void __launch_bounds__(256, GB_REGS && !ONE_ROW ? 2 : 1) layernorm_ke
         }
     }
     if (!ONE_ROW || !early) fetch_gb();
+    if constexpr (MODE == LN_SMEM) {
+        for (int i = threadIdx.x; i < nvec * Q; i += blockDim.x) {   // group i: the (i % Q)-th four of vector i / Q
+            const int v = i / Q, at = ((v >> 5) * Q + i % Q) * 32 + (v & 31);
+            s_gb[at] = __ldg(reinterpret_cast<const float4*>(gamma) + i);
+            s_gb[ITERS * Q * 32 + at] = __ldg(reinterpret_cast<const float4*>(beta) + i);
+        }
+        __syncthreads();
+    }
     for (int64_t row = warp0; row < rows; row += nwarps) {
         float f[ITERS][N];
         float sum = 0.f;
@@ -174,7 +190,7 @@ __global__ void __launch_bounds__(256, GB_REGS && !ONE_ROW ? 2 : 1) layernorm_ke
         for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
         const float var = sq / (float)H + eps;
         const int s = nm_pwl_index(var, inv_h, off, nm1);
-        const float2 kb = ONE_ROW ? s_tab[s] : tab->kb[s];
+        const float2 kb = MODE != LN_REGS ? s_tab[s] : tab->kb[s];
         float r = __fmaf_rn(kb.x, var, kb.y);
         if (tab2) {   // two-table form: `tab` gave sqrt(v + eps), `tab2` takes its reciprocal
             const int s2 = nm_pwl_index(r, tab2->inv_h, tab2->off, (float)(tab2->n - 1));
@@ -195,9 +211,9 @@ __global__ void __launch_bounds__(256, GB_REGS && !ONE_ROW ? 2 : 1) layernorm_ke
                     }
                 } else {
 #pragma unroll
-                    for (int i = 0; i < N; i += 4) {
-                        *reinterpret_cast<float4*>(&g[i]) = __ldg(reinterpret_cast<const float4*>(gamma + v * N + i));
-                        *reinterpret_cast<float4*>(&b[i]) = __ldg(reinterpret_cast<const float4*>(beta + v * N + i));
+                    for (int i = 0; i < Q; ++i) {
+                        *reinterpret_cast<float4*>(&g[4 * i]) = s_gb[(it * Q + i) * 32 + lane];
+                        *reinterpret_cast<float4*>(&b[4 * i]) = s_gb[(ITERS * Q + it * Q + i) * 32 + lane];
                     }
                 }
 #pragma unroll
@@ -270,10 +286,10 @@ nm_status launch_ln(nm_ctx* ctx, const NmTable* tab, const NmTable* tab2, const 
     const int nvec = H / N;
     const int iters = (nvec + 31) / 32;
     const int threads = 256;
-    // Tensors that fit the L2 (the encoder's: 16384 x 768 is 25 MB) are latency-bound: gamma and beta in registers,
-    // one resident wave of 2 blocks per SM, 9.9 instead of 13.3 us for that shape.  Tensors far beyond the L2 are
-    // bandwidth-bound and want more warps per SM: the per-row fetch of gamma and beta, 6 blocks of 8 warps per SM
-    // (5.5 instead of 4.9 TB/s at 2^19 x 768).
+    // Tensors that fit the L2 (the encoder's: 16384 x 768 is 25 MB) are latency-bound: gamma and beta in registers, one resident
+    // wave of 2 blocks per SM, 12.8 us for that shape as with 4 blocks and shared memory, and 3.2 against 3.8 for 2331 rows,
+    // which pay for filling it.  Tensors far beyond the L2 want more warps per SM: 284 us at 2^19 x 768 (5.68 TB/s; 291 with
+    // per-row fetches), 182 at 2^18 x 1024 (196); 8192 x 1024: 9.7 (12.4).
     const bool small = (double)rows * H * sizeof(T) <= 48e6 && iters <= 3;
     // At most one row per warp of one block per SM: bound by latency alone (128 x 1024 bf16 with int8 codes: 4.6 us per
     // launch in a chain, 2.8 so; 37 x 768: 3.2 and 2.3).
@@ -292,35 +308,31 @@ nm_status launch_ln(nm_ctx* ctx, const NmTable* tab, const NmTable* tab2, const 
     cfg.numAttrs = ctx->pdl ? 1 : 0;
     const T* xt = (const T*)x;
     T* yt = (T*)y;
-#define NM_LN_CASE(I, GB, ONE)                                                                                \
+#define NM_LN_CASE(I, MODE, MINB)                                                                             \
     do {                                                                                                      \
-        static int resident = 0;   /* blocks per SM that this instantiation's registers allow */              \
-        if (GB && resident == 0 &&                                                                            \
-            (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, layernorm_kernel<T, I, GB, ONE>, threads, 0) != \
-                 cudaSuccess || resident < 1))                                                                \
-            resident = 2;                                                                                     \
-        const int64_t cap = (int64_t)ctx->sm_count * (GB ? resident : 6);                                     \
+        const int64_t cap = (int64_t)ctx->sm_count * MINB;                                                    \
         cfg.gridDim = dim3((unsigned)(blocks > cap ? cap : blocks));                                          \
-        cudaLaunchKernelEx(&cfg, layernorm_kernel<T, I, GB, ONE>, tab, tab2, xt, gamma, beta, yt, rows, H,     \
+        cfg.dynamicSmemBytes = MODE == LN_SMEM ? (size_t)I * 32 * N * 2 * sizeof(float) : 0;                  \
+        cudaLaunchKernelEx(&cfg, layernorm_kernel<T, I, MODE, MINB>, tab, tab2, xt, gamma, beta, yt, rows, H,  \
                            eps, q, q_inv_scale, early ? 1 : 0);                                               \
     } while (0)
     if constexpr (N == 4) {
-        if (one_row && iters <= 4) NM_LN_CASE(4, true, true);
-        else if (one_row) NM_LN_CASE(8, true, true);
+        if (one_row && iters <= 4) NM_LN_CASE(4, LN_ONE_ROW, 1);
+        else if (one_row) NM_LN_CASE(8, LN_ONE_ROW, 1);
     }
     if (one_row && N == 4) {}
-    else if (one_row && iters <= 2) NM_LN_CASE(2, true, true);
-    else if (one_row && iters <= 3) NM_LN_CASE(3, true, true);
-    else if (one_row) NM_LN_CASE(4, true, true);
-    else if (small && iters <= 1) NM_LN_CASE(1, true, false);
-    else if (small && iters <= 2) NM_LN_CASE(2, true, false);
-    else if (small && iters <= 3) NM_LN_CASE(3, true, false);
-    else if (iters <= 1) NM_LN_CASE(1, false, false);
-    else if (iters <= 2) NM_LN_CASE(2, false, false);
-    else if (iters <= 3) NM_LN_CASE(3, false, false);
-    else if (iters <= 4) NM_LN_CASE(4, false, false);
-    else if (iters <= 8) NM_LN_CASE(8, false, false);
-    else if (iters <= 16) NM_LN_CASE(16, false, false);
+    else if (one_row && iters <= 2) NM_LN_CASE(2, LN_ONE_ROW, 1);
+    else if (one_row && iters <= 3) NM_LN_CASE(3, LN_ONE_ROW, 1);
+    else if (one_row) NM_LN_CASE(4, LN_ONE_ROW, 1);
+    else if (small && iters <= 1) NM_LN_CASE(1, LN_REGS, 2);
+    else if (small && iters <= 2) NM_LN_CASE(2, LN_REGS, 2);
+    else if (small && iters <= 3) NM_LN_CASE(3, LN_REGS, 2);
+    else if (iters <= 1) NM_LN_CASE(1, LN_SMEM, 4);
+    else if (iters <= 2) NM_LN_CASE(2, LN_SMEM, 4);
+    else if (iters <= 3) NM_LN_CASE(3, LN_SMEM, 4);
+    else if (iters <= 4) NM_LN_CASE(4, LN_SMEM, 3);
+    else if (iters <= 8) NM_LN_CASE(8, LN_SMEM, 2);
+    else if (iters <= 16) NM_LN_CASE(16, LN_SMEM, 1);
     else return NM_ERR_UNSUPPORTED;
 #undef NM_LN_CASE
     return cudaGetLastError() == cudaSuccess ? NM_OK : NM_ERR_CUDA;
