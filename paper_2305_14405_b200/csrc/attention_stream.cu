@@ -28,7 +28,7 @@
 // probabilities in fp32, so this form does not round them to 16 bits: e = hi + lo, two 16-bit terms (the error of
 // the pair is at most 2^-18 e in bf16, against the 2^-9 of the result's own rounding), and P V runs once per term.
 // The second term's 32 columns make it two CTAs per SM instead of three.  B 7, L 333, 12 heads: 2368 us on the CUDA
-// cores, 21.3 us here; B 1, L 37: 13.4 and 7.0 us.
+// cores, 20.3 us here; B 1, L 37: 13.4 and 5.4 us.
 //
 // ONE form (L <= 128, a single 128-key chunk): the scores and the accumulator do not share columns (128 | 64, and P behind
 // them: 256 columns, two CTAs per SM), so the one Q K^T of sweep 1 serves sweep 2 as well, and nothing is fetched or
@@ -102,6 +102,12 @@ __device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t* r)
         "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]),
         "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
         : "memory");
+}
+__device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t* r)
+{
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"r"(taddr), "r"(r[0]), "r"(r[1]),
+                 "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7])
+                 : "memory");
 }
 __device__ __forceinline__ void tmem_st_wait()
 {
@@ -477,32 +483,34 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
             // take the maximum as their score (which keeps the table index in range) and the exponential 0.
             auto chunk = [&](int j, auto last) {
                 constexpr bool LAST = decltype(last)::value;
+                constexpr int W = RAGGED ? 16 : 32;   // (with two terms of P, 32 keys at a time spill: 129 us at B 32, L 500, 12 heads, 114 so)
                 if constexpr (!ONE) {
                     wait_all(&bar_s_full, s_cnt & 1u);
                     ++s_cnt;
                     if (ok) nm_tc_fence_after();
                 }
 #pragma unroll
-                for (int hh = 0; hh < 2; ++hh) {
-                    const int lim = LAST ? L - j * CK - hh * 32 : 32;
-                    uint32_t r[32];
+                for (int hh = 0; hh < CK / W; ++hh) {   // W keys at a time
+                    const int lim = LAST ? L - j * CK - hh * W : W;
+                    uint32_t r[W];
                     if (ok && live) {
-                        nm_tmem_ld32_sync(t_row + (uint32_t)((ONE ? j * CK : 0) + hh * 32), r);
+                        if constexpr (W == 32) nm_tmem_ld32_sync(t_row + (uint32_t)((ONE ? j * CK : 0) + hh * 32), r);
+                        else nm_tmem_ld16_sync(t_row + (uint32_t)((ONE ? j * CK : 0) + hh * 16), r);
                         if constexpr (LAST) {
 #pragma unroll
-                            for (int k = 0; k < 32; ++k)
+                            for (int k = 0; k < W; ++k)
                                 if (k >= lim) r[k] = __float_as_uint(m);
                         }
                     }
-                    if (!ONE && hh == 1) {
+                    if (!ONE && hh == CK / W - 1) {
                         nm_tc_fence_before();
                         asm volatile("bar.arrive %0, %1;" ::"r"(bar_sc), "n"(160) : "memory");
                     }
-                    uint32_t pk[16];                       // the half's 32 exponentials, packed to 16 bits
-                    [[maybe_unused]] uint32_t pl[RAGGED ? 16 : 1];          // RAGGED: what the packing left, packed to 16 bits
+                    uint32_t pk[W / 2];                    // the exponentials, packed to 16 bits
+                    [[maybe_unused]] uint32_t pl[RAGGED ? W / 2 : 1];          // RAGGED: what the packing left, packed to 16 bits
                     if (ok && live) {
 #pragma unroll
-                        for (int jj = 0; jj < 4; ++jj) {   // 8 keys
+                        for (int jj = 0; jj < W / 8; ++jj) {   // 8 keys
                             float e[8];
 #pragma unroll
                             for (int k = 0; k < 8; k += 2) {
@@ -558,8 +566,12 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                     }
                     if (ok && live) {
                         if (hh == 0 && j >= 1) nm_tc_fence_after();   // ordered after the P V that read the columns
-                        tmem_st16(p_row + (uint32_t)(hh * 16), pk);   // keys 32 hh .. 32 hh + 31 of this thread's row
-                        if constexpr (RAGGED) tmem_st16(p_row + (uint32_t)(32 + hh * 16), pl);
+                        if constexpr (RAGGED) {   // keys 16 hh .. 16 hh + 15 of this thread's row
+                            tmem_st8(p_row + (uint32_t)(hh * 8), pk);
+                            tmem_st8(p_row + (uint32_t)(32 + hh * 8), pl);
+                        } else {
+                            tmem_st16(p_row + (uint32_t)(hh * 16), pk);   // keys 32 hh .. 32 hh + 31
+                        }
                     }
                 }
                 tmem_st_wait();          // the P columns are written
