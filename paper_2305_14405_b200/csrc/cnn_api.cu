@@ -334,10 +334,11 @@ nm_status nm_resnet50_forward(nm_ctx* ctx, const nm_conv_params* convs, const vo
         // the max-pool, launched without early start, lies between everything before this call and the convolutions behind it
         NmChain chain;
         chain.weights_ready = ci > 1;
+        chain.back_to_back = true;
         return nm_conv2d_dispatch(ctx, &d, gather_buf, gather, (cudaStream_t)stream, chain);
     };
     NmChain ready;
-    ready.weights_ready = true;
+    ready.weights_ready = ready.back_to_back = true;
 
     // stem: 7x7/2 convolution + ReLU, 3x3/2 max-pool
     nm_status s = conv(x, 224, 224, 3, base, 7, 2, 3, nullptr, 0, buf[0]);

@@ -93,8 +93,8 @@ nm_status make_tmaps_out(nm_ctx* ctx, CUtensorMap* tmO, CUtensorMap* tmR, const 
 
 // Is the halo form (linear_tc_kernel.cuh) the faster one?  3 x 3, stride 1, padding 1, at least two rounds of CTA pairs, and less
 // time by the bytes a tile takes from L2 (50 a clock) and the tensor core's cycles, although its fixed 8 x 16 patch wastes rows
-// that the free patch does not: 128 images, 56 x 56, 64 -> 64: 60 us against 77; 28 x 28, 128 -> 128: 45.6 against
-// 44.8, and not taken.  Wider outputs are bound by the tensor core in either form.
+// that the free patch does not: 128 images, 56 x 56, 64 -> 64: 52 us against 77; 28 x 28, 128 -> 128: 39.2 against
+// 44.8.  Wider outputs are bound by the tensor core in either form.
 bool use_halo(const NmConvTc* c, int64_t free_patches, int sms)
 {
     if (c->algo != 0 || c->taps_x != 3 || c->taps_y != 3 || c->sw != 1 || c->sh != 1 || c->pw != 1 || c->ph != 1 || c->depthwise ||
@@ -155,7 +155,7 @@ nm_status launch_split(nm_ctx* ctx, const NmConvTc* c, int S, NmChain chain, cud
     if (e != NM_OK) return e;
     e = make_tmap(ctx, &tmW, c->w, c->dtype, c->depthwise ? 64 : c->Cout, c->Ktot, c->ldw, BN);
     if (e != NM_OK) return e;
-    return launch_split_kernel<T, T, BN, true>(ctx, tmA, tmW, s, c->flops, st);
+    return launch_split_kernel<T, T, BN, true>(ctx, tmA, tmW, s, chain.back_to_back, c->flops, st);
 }
 
 template <typename T, bool TWO, int BN>
@@ -195,8 +195,8 @@ nm_status launch_sel(nm_ctx* ctx, const NmConvTc* c, NmChain chain, cudaStream_t
             const nm_status e = c->Cout <= 64 ? launch_halo<T, 64>(ctx, c, chain, st) : launch_halo<T, 128>(ctx, c, chain, st);
             if (e != NM_ERR_UNSUPPORTED) return e;
         }
-        t = choose_tile(patches, c->Cout, (int64_t)c->taps_y * c->taps_x * c->cblocks, true, c->slot != NM_SLOT_NONE,
-                        c->depthwise != 0, true, ctx->sm_count);
+        t = choose_tile((int64_t)c->N * c->Ho * c->Wo, patches, c->Cout, (int64_t)c->taps_y * c->taps_x * c->cblocks, true, c->slot != NM_SLOT_NONE,
+                        c->depthwise != 0, true, chain, ctx->sm_count);
     } else {
         t.S = 0;
         t.BN = c->Cout <= 64 || c->depthwise ? 64 : (c->Cout <= 128 ? 128 : 256);

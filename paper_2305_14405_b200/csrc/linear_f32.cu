@@ -145,7 +145,7 @@ linear_f32_kernel(const float* __restrict__ A, const float* __restrict__ W, int6
         *reinterpret_cast<float4*>(p) = v;
     }
     const int rows = (int)(a.M - m0 < FBM ? a.M - m0 : FBM);
-    Finisher<false, float, FBN, false, F_THREADS> fin(s, rank, mt, nt, rows, Patch{0, 0, 0});
+    Finisher<false, float, FBN, false, F_THREADS, false> fin(s, rank, mt, nt, rows, Patch{0, 0, 0});
     fin.prefetch_vectors();
     fin.load_res(0);
     if (S > 1) nm_cluster_sync();

@@ -6,10 +6,15 @@
 //
 // Such a launch is bound by latency: with the persistent kernel's 256-column tiles a BERT-base layer on 128
 // tokens keeps 3 to 12 SMs busy, each walking through the whole of K on its own.  Here every CTA multiplies
-// its share of the K-blocks (TMA ring, tcgen05.mma into tensor memory), writes its fp32 or int32 partial tile
-// to its own shared memory, and after one cluster barrier every CTA finishes every S-th row of the tile: it
-// reads the S partial rows over distributed shared memory, adds them in rank order (the sum does not depend
-// on timing), applies scale, bias, table and residual and stores whole row segments.
+// its share of the K-blocks (TMA ring, tcgen05.mma into tensor memory) and finishes every S-th row of the tile.
+// It sends its fp32 or int32 partial rows straight from registers to the CTAs that own them (st.async over
+// distributed shared memory, counted on the owner's mbarrier), waits for the rows sent to it, adds the S
+// partial rows in rank order (the sum does not depend on timing), applies scale, bias, table and residual and
+// stores whole row segments.  Nobody reads another CTA's memory and no CTA waits for a cluster barrier: with
+// the partial tiles left where they were made, the barrier before the remote reads, the reads and the barrier
+// before the exit took 1300 + 1300 to 3000 + 1300 cycles of a launch of 8 to 12 thousand (12 layers, 37 tokens: 470 us
+// then, 417 so).  S is a template parameter: a launch runs its code once, from a cold instruction cache, and what it does not
+// need is in its way (37 tokens: 403 -> 391 us, ResNet-50 batch 1: 373 -> 357).
 //
 // CONV = true: the A operand is the NHWC activation, as in linear_tc_kernel (a tile's 128 rows are a patch of
 // output pixels and a K-block is one 4-D TMA box).
@@ -19,7 +24,7 @@
 namespace nm_tc {
 
 constexpr int SPLIT_THREADS = 256;
-constexpr int SPLIT_MAX_STAGES = 4;   // 96 KB at BN = 64: two CTAs per SM, so the next kernel's set-up can overlap
+constexpr int SPLIT_MAX_STAGES = 6;
 
 struct SplitArgs {
     TcArgs t;               // num_tiles, num_n_tiles, num_k_blocks, stages and the epilogue's operands
@@ -80,6 +85,13 @@ template <> struct Quad<int8_t> {
     }
 };
 
+// 16 bytes into the shared memory of a CTA of the cluster, counted on that CTA's mbarrier
+__device__ __forceinline__ void st_async_v4(uint32_t cluster_addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d, uint32_t cluster_bar)
+{
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1,%2,%3,%4}, [%5];" ::"r"(cluster_addr),
+                 "r"(a), "r"(b), "r"(c), "r"(d), "r"(cluster_bar)
+                 : "memory");
+}
 __device__ __forceinline__ uint4 ld_cluster_v4(uint32_t cluster_addr)
 {
     uint4 v;
@@ -90,13 +102,14 @@ __device__ __forceinline__ uint4 ld_cluster_v4(uint32_t cluster_addr)
 }
 
 // Final sum and epilogue of a cluster's tile: this CTA takes rows rank, rank + S, ... of the `rows` that exist and adds
-// the S partial tiles (one in each CTA's shared memory at `part`, part_pitch(BN) words per row) in rank order.  Four
-// columns per thread, whole row segments per group of BN / 4 threads.  Rows go in batches of up to FIN_U per thread, all
-// loads of a batch in flight together, and the vectors and the first batch's residual are fetched before the product
-// is even started: a row at a time cost a memory latency per row.
+// the S partial rows in rank order, part_pitch(BN) words per row.  PUSHED: they are in this CTA's shared memory, row r of
+// CTA k at row k * (BM / S) + r / S of `part`; otherwise in each CTA's own, row r at row r of its `part`.  Four columns
+// per thread, whole row segments per group of BN / 4 threads.  Rows go in batches of up to FIN_U per thread, all loads
+// of a batch in flight together, and the vectors and the first batch's residual are fetched before the product is even
+// started: a row at a time cost a memory latency per row.  CTAS: S, or 0 where it is not known at compile time.
 constexpr int FIN_U = 4;
 
-template <bool INT, typename OutT, int BN, bool CONV, int THREADS>
+template <bool INT, typename OutT, int BN, bool CONV, int THREADS, bool PUSHED, int CTAS = 0>
 struct Finisher {
     static constexpr int PITCH = part_pitch(BN);
     static constexpr int QPR = BN / 4;            // 4-column groups per row
@@ -128,7 +141,8 @@ struct Finisher {
             return (int64_t)mt * BM + r;
         }
     }
-    __device__ __forceinline__ int tile_row(int i) const { return ((int)threadIdx.x / QPR + i * RPP) * s.S + rank; }
+    __device__ __forceinline__ int tile_row(int i) const { return ((int)threadIdx.x / QPR + i * RPP) * ctas() + rank; }
+    __device__ __forceinline__ int ctas() const { return CTAS ? CTAS : s.S; }
     __device__ __forceinline__ void load_res(int i0)
     {
         if (!s.residual || !col_ok) return;
@@ -153,7 +167,7 @@ struct Finisher {
     }
     __device__ __forceinline__ void run(const uint32_t* part, const float2* tab)
     {
-        const int per_thread = (rows + s.S * RPP - 1) / (s.S * RPP);
+        const int per_thread = (rows + ctas() * RPP - 1) / (ctas() * RPP);
         if (per_thread <= 1) batches<1>(part, tab);
         else if (per_thread <= 2) batches<2>(part, tab);
         else batches<FIN_U>(part, tab);
@@ -162,30 +176,30 @@ struct Finisher {
     __device__ __forceinline__ void batches(const uint32_t* part, const float2* tab)
     {
         const TcArgs& a = s.t;
-        const int S = s.S;
+        const int S = ctas();
         const bool has_tab = a.tab != nullptr;
         const float inv_h = has_tab ? a.tab->inv_h : 0.f, off = has_tab ? a.tab->off : 0.f, nm1 = (float)(a.n_seg - 1);
         const uint32_t part_u = nm_smem_u32(part);
+        const int slot = PUSHED ? BM / S : 0, lg = 31 - __clz(S);   // slot: rows between the partial rows of two CTAs; S is 1, 2, 4, 8
+        auto partial = [&](int r, int k) {
+            if constexpr (PUSHED) return *reinterpret_cast<const uint4*>(part + (k * slot + (r >> lg)) * PITCH + qc * 4);
+            else return S == 1 ? *reinterpret_cast<const uint4*>(part + (size_t)r * PITCH + qc * 4)
+                               : ld_cluster_v4(nm_mapa(part_u + (uint32_t)(r * PITCH + qc * 4) * 4u, (uint32_t)k));
+        };
         for (int i0 = 0; tile_row(i0) < rows; i0 += U) {
             if (i0 > 0) load_res(i0);
             uint32_t acc[U][4];
 #pragma unroll
             for (int u = 0; u < U; ++u) {
                 // (a row beyond the tile's last is read from the last and not used)
-                const int r = min(tile_row(i0 + u), BM - 1);
-                const uint32_t addr = part_u + (uint32_t)(r * PITCH + qc * 4) * 4u;
-                const uint4 p = S == 1 ? *reinterpret_cast<const uint4*>(part + (size_t)r * PITCH + qc * 4)
-                                       : ld_cluster_v4(nm_mapa(addr, 0));
+                const uint4 p = partial(min(tile_row(i0 + u), BM - 1), 0);
                 acc[u][0] = p.x; acc[u][1] = p.y; acc[u][2] = p.z; acc[u][3] = p.w;
             }
 #pragma unroll 2
             for (int k = 1; k < S; ++k) {
                 uint4 o[U];
 #pragma unroll
-                for (int u = 0; u < U; ++u) {
-                    const int r = min(tile_row(i0 + u), BM - 1);
-                    o[u] = ld_cluster_v4(nm_mapa(part_u + (uint32_t)(r * PITCH + qc * 4) * 4u, (uint32_t)k));
-                }
+                for (int u = 0; u < U; ++u) o[u] = partial(min(tile_row(i0 + u), BM - 1), k);
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
                     const uint32_t w[4] = {o[u].x, o[u].y, o[u].z, o[u].w};
@@ -232,7 +246,7 @@ struct Finisher {
     }
 };
 
-template <typename InT, typename OutT, int BN, bool CONV>
+template <typename InT, typename OutT, int BN, bool CONV, int S>
 __global__ void __launch_bounds__(SPLIT_THREADS, 2)
 linear_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmW, const SplitArgs s)
 {
@@ -245,19 +259,21 @@ linear_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     constexpr int PITCH = part_pitch(BN);
 
     extern __shared__ uint8_t smem_raw[];
-    __shared__ uint64_t bar_full[SPLIT_MAX_STAGES], bar_empty[SPLIT_MAX_STAGES], bar_acc;
+    __shared__ uint64_t bar_full[SPLIT_MAX_STAGES], bar_empty[SPLIT_MAX_STAGES], bar_acc, bar_part;
     __shared__ uint32_t tmem_slot;
     __shared__ int abort_flag;
     __shared__ float2 s_tab[NM_MAX_SEGMENTS];
 
-    const int S = s.S;
     const int rank = S > 1 ? (int)nm_cluster_ctarank() : 0;
     const int tile = (int)blockIdx.x / S;
     const int mt = tile / a.num_n_tiles, nt = tile % a.num_n_tiles;
     const int kb0 = rank * a.num_k_blocks / S, kb1 = (rank + 1) * a.num_k_blocks / S;
     const int stages = a.stages;
     uint8_t* tiles = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-    uint32_t* part = reinterpret_cast<uint32_t*>(tiles);   // the partial tile takes the ring's place once K is done
+    // The partial rows: without a split they take the ring's place once K is done; with one they arrive while the ring may
+    // still be in use.
+    uint32_t* part = reinterpret_cast<uint32_t*>(tiles + (S > 1 ? (size_t)stages * STAGE_BYTES : 0));
+    const int rows = CONV ? BM : (int)(a.M - (int64_t)mt * BM < BM ? a.M - (int64_t)mt * BM : BM);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
     if (threadIdx.x == 0) {
@@ -269,7 +285,10 @@ linear_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
             nm_mbar_init(&bar_empty[i], 1);
         }
         nm_mbar_init(&bar_acc, 1);
+        nm_mbar_init(&bar_part, 1);
         nm_fence_barrier_init();
+        // what the others will send: their columns of each of this CTA's rows
+        if (S > 1) nm_mbar_expect_tx(&bar_part, (uint32_t)((rows - rank + S - 1) / S) * (uint32_t)(S - 1) * BN * 4u);
     }
     if (warp == 1) {
         nm_tmem_alloc(&tmem_slot, BN);
@@ -281,6 +300,7 @@ linear_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     nm_tc_fence_before();
     __syncthreads();
     nm_tc_fence_after();
+    if (S > 1) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");   // this CTA's barrier may be sent to
     const uint32_t tmem = tmem_slot;
     volatile int* abortp = &abort_flag;
     if (!a.late_trigger) nm_grid_launch_dependents();
@@ -294,14 +314,13 @@ linear_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                 nm_mbar_expect_tx(&bar_full[i], STAGE_BYTES);
                 nm_tma_load_2d(tiles + (size_t)i * STAGE_BYTES + A_BYTES, &tmW, (kb0 + i) * BK_ELEMS, nt * BN, &bar_full[i]);
             }
-            for (int kb = kb0 + early; kb < kb1; ++kb) nm_tma_prefetch_2d(&tmW, kb * BK_ELEMS, nt * BN);
+            for (int kb = kb0 + early; kb < kb1 && mt == 0; ++kb) nm_tma_prefetch_2d(&tmW, kb * BK_ELEMS, nt * BN);
         }
         __syncwarp();
     }
     Patch pt = {0, 0, 0};
     if constexpr (CONV) pt = patch_of(a.cv, mt);
-    const int rows = CONV ? BM : (int)(a.M - (int64_t)mt * BM < BM ? a.M - (int64_t)mt * BM : BM);
-    Finisher<INT, OutT, BN, CONV, SPLIT_THREADS> fin(s, rank, mt, nt, rows, pt);
+    Finisher<INT, OutT, BN, CONV, SPLIT_THREADS, true, S> fin(s, rank, mt, nt, rows, pt);
     // One lane runs the producer's and the issuer's loops for the 16-bit types (12 layers, 37 tokens: 547 -> 537 us); for int8 all
     // lanes do, with one elected to issue (24 layers, 128 tokens: 1215 us against 1230).
     constexpr bool ONE_LANE = !INT;
@@ -396,23 +415,31 @@ linear_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     nm_tc_fence_after();
     __syncthreads();
     ok = ok && !abort_flag;
+    if (S > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");   // (long complete: it was reached before K)
     {   // two warps per tensor-memory lane quarter, each half of the columns
-        const int q = warp & 3, c0 = (warp >> 2) * (BN / 2);
-        uint32_t* my = part + (size_t)(q * 32 + lane) * PITCH + c0;
+        const int q = warp & 3, c0 = (warp >> 2) * (BN / 2), row = q * 32 + lane, owner = row & (S - 1);
+        uint32_t* mine = part + (((rank * BM + row) >> (31 - __clz(S))) * PITCH + c0);   // the row's place, in the owner
         const uint32_t t_addr = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)c0;
-        if (q * 32 < rows) {
+        const uint32_t dst = nm_mapa(nm_smem_u32(mine), (uint32_t)owner), bar = nm_mapa(nm_smem_u32(&bar_part), (uint32_t)owner);
+        if (ok && q * 32 < rows) {
 #pragma unroll
             for (int c = 0; c < BN / 2; c += 16) {
                 uint32_t r[16];
                 nm_tmem_ld16_sync(t_addr + (uint32_t)c, r);
+                if (row >= rows) continue;
+                if (owner == rank) {
 #pragma unroll
-                for (int i = 0; i < 16; i += 4)
-                    *reinterpret_cast<uint4*>(my + c + i) = make_uint4(r[i], r[i + 1], r[i + 2], r[i + 3]);
+                    for (int i = 0; i < 16; i += 4)
+                        *reinterpret_cast<uint4*>(mine + c + i) = make_uint4(r[i], r[i + 1], r[i + 2], r[i + 3]);
+                } else {
+#pragma unroll
+                    for (int i = 0; i < 16; i += 4) st_async_v4(dst + (uint32_t)(c + i) * 4u, r[i], r[i + 1], r[i + 2], r[i + 3], bar);
+                }
             }
         }
     }
-    if (S > 1) nm_cluster_sync();
-    else __syncthreads();
+    __syncthreads();
+    if (S > 1 && ok && !nm_mbar_wait(&bar_part, 0, abortp, a.status)) ok = false;
 
     if (ok) fin.run(part, s_tab);
 
@@ -424,7 +451,9 @@ linear_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         nm_tc_fence_after();
         nm_tmem_dealloc(tmem, BN);
     }
-    if (S > 1) nm_cluster_sync();   // a peer may still be reading this CTA's partial tile
+    // Every row sent to this CTA has arrived before it gets here, unless something timed out: then it stays until the others,
+    // who may still be sending, have got as far or are gone.
+    if (S > 1 && __syncthreads_or(ok ? 0 : 1)) nm_cluster_sync();
 }
 
 // Launch attributes of a kernel in clusters of S CTAs; returns their number.
@@ -443,16 +472,22 @@ inline unsigned split_launch_attrs(const nm_ctx* ctx, cudaLaunchAttribute* attr,
     return n + 1;
 }
 
-// Which kernel and tile a problem of `m_tiles` blocks of 128 rows, N columns and `k_blocks` K-blocks gets: the least time
-// by a model of measured figures in us (chains of equal launches, 37 to 2331 rows, N 256 to 4096, K 256 to 4096, bf16 and
-// int8; it reproduces them to about 10 %).
-//   persistent kernel, r rounds of tiles: base + r * (k_blocks * per K-block), a round no shorter than its epilogue.  The
-//     K-block's time is its operands' way from L2 to one SM (50 bytes a clock), so a pair of CTAs and a wide tile need
-//     less of it per element, and a narrow tile makes better use of the last round.
-//   split kernel, n CTAs: 4.2 + the K-blocks beyond the three in flight at once, more when several CTAs share an SM, + the
-//     exchange over the cluster (0.4 / 1.0 / 1.8 for 2 / 4 / 8 CTAs) + the epilogue of four warps' worth per tile.
-// At 128 x 768 x 3072 one round of persistent tiles takes 17 us and the split over 8 CTAs 7.3; at 1024 x 768 x 768
-// 128 x 64 tiles take 6.7 and 256 x 256 pairs 9.8; at 16384 rows the widest tile wins.
+// Which kernel and tile a problem of `rows` rows (`m_tiles` blocks of 128), N columns and `k_blocks` K-blocks gets: the least
+// time by a model fitted to measured times in us: chains of equal launches at 72 problems, 37 to 4096 rows, N 256 to 4096,
+// K 256 to 4096, bf16 and int8, every kernel and tile.  It is 9 % off on the average, and the tile it picks 1 % behind the
+// best; at 16384 rows it predicts 47, 22, 64 and 67 us for the BERT-base projections (44, 22, 62 and 64 measured).
+//   persistent kernel, r rounds of tiles: base + r * k_blocks * (per K-block).  With most SMs busy a K-block takes at least
+//     its operands' way from L2 (97 KB a us and SM).  From the third round on a round takes at least its epilogue, by the
+//     short-K convolutions (64 -> 256 channels: 98 us with 256-column tiles, 79 with 128).
+//   split kernel, n CTAs: base with the epilogue of the rows that exist + the K-blocks beyond those in flight at once (more when
+//     CTAs share an SM) + the exchange.
+//   Between kernels that are no matrix products the persistent kernel's longer set-up and tail overlap less, 0.4 us (11 layers, 128
+//   tokens: 497 us without it, 437 with).  A CNN's launches stand back to back and begin while their predecessor drains: there every
+//   round counts with its epilogue and narrow tiles do better than alone, so they have a row of parameters of their own (ResNet-50 batch
+//   13: 624 us, 657 with the other row; batch 23: 747 and 782).  There, and among the split kernel's widths, the wider tile wins
+//   within 3 %: it leaves more SMs to the neighbours.
+// E.g. 128 x 768 x 3072: 13.4 us in one round of the best persistent tile, 7.0 split over 8; 1024 x 768 x 768: 5.9 with 128 x 64
+// tiles, 9.8 with 256 x 256 pairs.
 // `whole_chunks`: a row of the output is a multiple of 16 bytes.  The persistent kernel stores through a tensor map, which
 // writes whole 16-byte chunks and would reach beyond a row that is not; the split kernel stores four columns at a time.
 struct TileChoice {
@@ -461,49 +496,78 @@ struct TileChoice {
     bool two;   // persistent kernel: CTA pairs
 };
 
-inline TileChoice choose_tile(int64_t m_tiles, int64_t N, int64_t k_blocks, bool narrow_tiles, bool has_table, bool only64,
-                              bool whole_chunks, int sms)
+// A cluster's CTAs share a GPC, so not every SM is in one: the CTAs, in clusters of S, that certainly find an SM each.
+inline bool split_alone(int S, int64_t ctas, int sms) { return ctas <= (S == 8 ? sms * 3 / 4 : sms * 7 / 8); }
+
+// K-blocks in flight per CTA.  One CTA per SM: six stages, or five with 64 columns (12 layers, 37 tokens: 416 us, 436 with the
+// shallow ring); more CTAs, or neighbours in the stream of the same kind, whose set-up should overlap: what lets two share an SM
+// (ResNet-50 batch 1: 381 us, 430 with the deep ring).  Clusters of 8 fill fewer SMs: 128 CTAs with deep rings ran as two waves
+// (48 x 1024 x 4096: 12.4 us against 7.5).
+inline int split_stages(int BN, int S, int64_t ctas, int sms, bool back_to_back)
 {
-    struct P { int BN; bool two; double base, kb; };
-    static const P persistent[6] = {{256, true, 4.6, 0.386}, {256, false, 5.1, 0.43}, {128, true, 4.2, 0.26},
-                                    {128, false, 3.6, 0.322}, {64, true, 3.6, 0.26},  {64, false, 3.2, 0.30}};
+    if (S == 1) return 4;
+    if (back_to_back) return BN == 64 ? 3 : 4;
+    return BN == 64 ? (split_alone(S, ctas, sms) ? 5 : 3) : (split_alone(S, ctas, sms) ? 6 : 4);
+}
+
+inline TileChoice choose_tile(int64_t rows, int64_t m_tiles, int64_t N, int64_t k_blocks, bool narrow_tiles, bool has_table, bool only64,
+                              bool whole_chunks, NmChain chain, int sms)
+{
+    struct P { int BN; bool two; double base, kb, round; };
+    static const P apart[6] = {{256, true, 5.56, 0.420, 4.4}, {256, false, 4.72, 0.461, 4.8}, {128, true, 4.07, 0.233, 1.8},
+                               {128, false, 2.94, 0.315, 1.95}, {64, true, 3.19, 0.251, 1.15}, {64, false, 3.00, 0.218, 1.25}};
+    static const P joined[6] = {{256, true, 4.9, 0.386, 3.6}, {256, false, 5.4, 0.43, 3.6}, {128, true, 4.5, 0.26, 1.8},
+                                {128, false, 3.9, 0.322, 1.8}, {64, true, 3.9, 0.26, 0.9}, {64, false, 3.5, 0.30, 0.9}};
+    const bool in_cnn = chain.back_to_back;
     TileChoice best = {0, 0, false};
     double best_t = 1e30;
-    for (const P& p : persistent) {
+    for (int i = 0; i < 6; ++i) {
+        const P& p = in_cnn ? joined[i] : apart[i];
         if (!whole_chunks || (!narrow_tiles && p.BN != 256) || (only64 && p.BN != 64) || (p.two && m_tiles < 2)) continue;
         if (narrow_tiles && p.BN > 64 && N <= p.BN / 2) continue;   // half the tile would be padding
         const int64_t tiles = (p.two ? (m_tiles + 1) / 2 : m_tiles) * ((N + p.BN - 1) / p.BN), slots = p.two ? sms / 2 : sms;
-        const double rounds = (double)((tiles + slots - 1) / slots);
-        const double epilogue = 3.6 * p.BN / 256, loop = p.kb * (double)k_blocks;
-        const double t = p.base + (has_table ? 1.8 * p.BN / 256 : 0.0) + rounds * (loop > epilogue ? loop : epilogue);
-        if (t < best_t * 0.97) { best_t = t; best = {0, p.BN, p.two}; }
+        const int64_t rounds = (tiles + slots - 1) / slots;
+        const double share = tiles < slots ? (double)tiles / slots : 1.0;
+        const double feed = (A_BYTES + (p.two ? p.BN / 2 : p.BN) * ROW_BYTES) / 96.6e3;
+        double loop = (double)k_blocks * (!in_cnn && share >= 0.8 && feed > p.kb ? feed : p.kb);
+        if ((in_cnn || rounds > 2) && loop < p.round) loop = p.round;
+        const double t = p.base + (double)rounds * loop + (in_cnn ? 0.0 : (chain.weights_ready ? 0.4 : 0.0) + 0.32 * share * p.BN / 64) +
+                         (has_table ? (in_cnn ? 1.8 : 1.5) * p.BN / 256 : 0.0);
+        if (t < best_t * (in_cnn ? 0.97 : 1.0)) { best_t = t; best = {0, p.BN, p.two}; }
     }
+    const double tile_rows = (rows < BM ? (double)rows : (double)BM) / BM;
     for (int BN = 64; BN >= (only64 ? 64 : 32); BN /= 2) {
         const int64_t tiles = m_tiles * ((N + BN - 1) / BN);
         for (int S = 1; S <= 8 && S <= k_blocks; S *= 2) {
             const int64_t n = tiles * S;
             if (n > 2 * sms && (whole_chunks || S > 1 || n > 0x7fffffffLL)) break;
-            const double per = (double)((k_blocks + S - 1) / S), share = (double)n / sms;
-            const double t = 4.2 + (BN == 64 ? 0.32 : 0.24) * (per > 3 ? per - 3 : 0) * (share > 1 ? share : 1) +
-                             (S == 1 ? 0.0 : S == 2 ? 0.4 : S == 4 ? 1.0 : 1.8) + 0.5 * share * BN / 32 + (has_table ? 0.4 * BN / 64 : 0.0);
-            if (t < best_t * 0.97) { best_t = t; best = {S, BN, false}; }
+            const double per = (double)((k_blocks + S - 1) / S), share = (double)n / sms, beyond = per - split_stages(BN, S, n, sms, in_cnn);
+            const double t = 4.29 + 0.73 * tile_rows * BN / 64 + 0.038 * per +
+                             (BN == 64 ? 0.235 : 0.179) * (beyond > 0 ? beyond : 0) * (share > 1 ? share : 1) +
+                             (S == 1 ? 0.0 : S == 2 ? 0.21 : S == 4 ? 0.26 : 0.56) +
+                             (0.35 * (share < 1 ? share : 1) + 0.85 * (share > 1 ? share - 1 : 0)) * BN / 32 + (has_table ? 0.42 * BN / 64 : 0.0);
+            if (t < best_t * (in_cnn || best.S ? 0.97 : 1.0)) { best_t = t; best = {S, BN, false}; }
         }
     }
     return best;
 }
 
 template <typename InT, typename OutT, int BN, bool CONV>
-inline nm_status launch_split_kernel(nm_ctx* ctx, const CUtensorMap& tmA, const CUtensorMap& tmW, SplitArgs& s, double work,
-                                     cudaStream_t st)
+inline nm_status launch_split_kernel(nm_ctx* ctx, const CUtensorMap& tmA, const CUtensorMap& tmW, SplitArgs& s, bool back_to_back,
+                                     double work, cudaStream_t st)
 {
     constexpr int STAGE_BYTES = A_BYTES + BN * ROW_BYTES;
-    const int per = (s.t.num_k_blocks + s.S - 1) / s.S;
-    constexpr int MIN_STAGES = (BM * part_pitch(BN) * 4 + STAGE_BYTES - 1) / STAGE_BYTES;   // the partial tile fits in the ring
-    static_assert(MIN_STAGES <= SPLIT_MAX_STAGES, "partial tile");
-    s.t.stages = per < MIN_STAGES ? MIN_STAGES : (per > SPLIT_MAX_STAGES ? SPLIT_MAX_STAGES : per);
-    const size_t smem = (size_t)s.t.stages * STAGE_BYTES + 1024;
-    auto kern = linear_split_kernel<InT, OutT, BN, CONV>;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(SPLIT_MAX_STAGES * STAGE_BYTES + 1024)) !=
+    constexpr int PART_BYTES = BM * part_pitch(BN) * 4;   // without a split it takes the ring's place and must fit in it
+    constexpr int MIN_STAGES = (PART_BYTES + STAGE_BYTES - 1) / STAGE_BYTES;
+    static_assert(MIN_STAGES <= 3, "partial tile");
+    const int per = (s.t.num_k_blocks + s.S - 1) / s.S, most = split_stages(BN, s.S, (int64_t)s.t.num_tiles * s.S, ctx->sm_count, back_to_back);
+    s.t.stages = per < MIN_STAGES ? MIN_STAGES : (per > most ? most : per);
+    const size_t smem = (size_t)s.t.stages * STAGE_BYTES + (s.S > 1 ? PART_BYTES : 0) + 1024;
+    auto kern = s.S == 1   ? linear_split_kernel<InT, OutT, BN, CONV, 1>
+                : s.S == 2 ? linear_split_kernel<InT, OutT, BN, CONV, 2>
+                : s.S == 4 ? linear_split_kernel<InT, OutT, BN, CONV, 4>
+                           : linear_split_kernel<InT, OutT, BN, CONV, 8>;
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(SPLIT_MAX_STAGES * STAGE_BYTES + PART_BYTES + 1024)) !=
         cudaSuccess)
         return NM_ERR_CUDA;
     cudaLaunchConfig_t cfg;

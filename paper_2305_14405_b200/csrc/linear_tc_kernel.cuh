@@ -82,6 +82,7 @@ struct TcArgs {
     int* status;
     int num_n_tiles, num_tiles, num_k_blocks, stages, n_seg;
     int weights_ready, late_trigger;   // NmChain
+    int prefetch_w;                    // persistent kernel: bring W into L2 before the dependency wait
     int w_stages;                      // HALO: weight tiles in shared memory; w_resident: all of them, loaded once
     int w_resident;
     ConvDev cv;
@@ -290,6 +291,15 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     // set-up done: the next kernel in the stream may begin its own set-up; nothing produced by the
     // previous kernel has been touched yet, everything below may depend on it
     if (!a.late_trigger) nm_grid_launch_dependents();
+    if constexpr (!CONV) {
+        // A launch of one round whose weights were complete before the previous kernel started: the first row of tiles brings
+        // them into L2 meanwhile.
+        if (a.prefetch_w && warp == 0 && tile_first < a.num_n_tiles && tile_first + tile_step >= a.num_tiles && nm_elect_one()) {
+            const int n0 = tile_first * BN + (int)rank * B_ROWS;
+            for (int kb = 0; kb < a.num_k_blocks; ++kb) nm_tma_prefetch_2d(&tmW, kb * BK_ELEMS, n0);
+        }
+        __syncwarp();
+    }
     nm_grid_dependency_wait();
     if (a.late_trigger) nm_grid_launch_dependents();
 

@@ -687,8 +687,9 @@ bool nm_linear_f32_supported(const nm_linear_desc* d);   // fp32, N a multiple o
 //     started, so the kernel may fetch it before its grid-dependency wait; only the activation comes from that kernel.
 //   late_trigger: the first kernel of a chain.  Its successors may start only after its own wait has returned, so that
 //     what was enqueued before the chain is complete for all of them.
+//   back_to_back: the neighbours are matrix kernels too (a convolutional network).
 struct NmChain {
-    bool weights_ready = false, late_trigger = false;
+    bool weights_ready = false, late_trigger = false, back_to_back = false;
 };
 nm_status nm_launch_linear_tc(nm_ctx* ctx, const nm_linear_desc* d, cudaStream_t st, NmChain chain = NmChain());
 nm_status nm_linear_dispatch(nm_ctx* ctx, const nm_linear_desc* d, cudaStream_t st, NmChain chain);

@@ -119,3 +119,10 @@ def test_convolution(nm, ctx, N, H, Cin, Cout, k, stride, pad, res):
     # fp32 sums in another order, then one rounding each to fp16: at most one unit in the last place apart
     assert np.all(np.abs(outs[0] - outs[1]) <= 2.0 ** -10 * np.abs(outs[1]) + 1e-5), np.abs(outs[0] - outs[1]).max()
     assert rms_rel(outs[0], outs[1]) <= 2.0 ** -11
+
+
+@pytest.mark.parametrize("M", [1, 3, 7, 37, 127, 130])
+@pytest.mark.parametrize("N,K", [(36, 640), (64, 1024), (768, 3072), (1024, 4096)])
+def test_rows_of_a_cluster(nm, ctx, M, N, K):
+    """Fewer rows than CTAs in a cluster, row counts that do not divide among them, every cluster size."""
+    test_16_bit(nm, ctx, "bf16", M, N, K, "bias_res")
