@@ -554,7 +554,11 @@ nm_status launch(nm_ctx* ctx, const nm_attn_i8_desc* d, cudaStream_t st)
 
 nm_status nm_launch_attention_i8(nm_ctx* ctx, const nm_attn_i8_desc* d, cudaStream_t st)
 {
-    const bool clamp_hi = ctx->h_tables[d->exp_slot].x_max < 0.0f;
+    // A table whose range reaches 0 needs no upper clamp as long as the input, fma(acc, sc, -(m * sc)) and so at most half an ulp
+    // of m * sc above 0, is less than one segment above it: the replicated table has one spare entry.  |m| < 64 * 127^2 < 2^20.
+    const NmTable& t = ctx->h_tables[d->exp_slot];
+    const float sc = (d->s_q * d->s_k) * d->scale;
+    const bool clamp_hi = t.x_max < 0.0f || !(0x1p20f * 0x1p-24f * sc * t.inv_h < 0.5f);
     if (d->out_dtype == NM_F32)
         return clamp_hi ? launch<float, true>(ctx, d, st) : launch<float, false>(ctx, d, st);
     return clamp_hi ? launch<__nv_bfloat16, true>(ctx, d, st) : launch<__nv_bfloat16, false>(ctx, d, st);

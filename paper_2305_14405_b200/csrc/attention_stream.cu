@@ -476,7 +476,11 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                     asm volatile("bar.arrive %0, %1;" ::"r"(bar_sc), "n"(160) : "memory");
                 }
             }
-            const float neg_ms = -(m * a.scale);
+            // RAGGED: the scores are scaled and rounded before the maximum is subtracted, and the segment number is clamped on
+            // both sides, as on the CUDA cores.  Otherwise one FMA does both, and its result must not lie above 0, which is what
+            // bounds the segment number there: the product is rounded up.  Rounded to nearest, fma(m, scale, -m scale) lies up
+            // to half an ulp of m * scale above 0 for a scale that is no power of two, past the table's spare entry from 1e6 on.
+            const float neg_ms = RAGGED ? -__fmul_rn(m, a.scale) : -__fmul_ru(m, a.scale);
             const uint64_t neg_ms2 = nm_pack2(neg_ms, neg_ms);
             float sum0 = 0.f, sum1 = 0.f, sum2 = 0.f, sum3 = 0.f;
             // ---- sweep 2: e = PWL_exp(s - m), row sum, P tiles.  LAST: the chunk that may hold keys beyond L; they
@@ -517,10 +521,12 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                                 // two scores at a time on the packed fp32 instructions: each half is the same correctly
                                 // rounded operation as the scalar form
                                 uint64_t x2, u2, b2;
-                                asm("fma.rn.f32x2 %0, %1, %2, %3;"
-                                    : "=l"(x2)
-                                    : "l"(nm_pack2(__uint_as_float(r[jj * 8 + k]), __uint_as_float(r[jj * 8 + k + 1]))), "l"(scale2),
-                                      "l"(neg_ms2));
+                                const float s0 = __uint_as_float(r[jj * 8 + k]), s1 = __uint_as_float(r[jj * 8 + k + 1]);
+                                if constexpr (RAGGED) {   // (the packed mul and add would be contracted into an FMA)
+                                    x2 = nm_pack2(__fadd_rn(__fmul_rn(s0, a.scale), neg_ms), __fadd_rn(__fmul_rn(s1, a.scale), neg_ms));
+                                } else {
+                                    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(x2) : "l"(nm_pack2(s0, s1)), "l"(scale2), "l"(neg_ms2));
+                                }
                                 asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(u2) : "l"(x2), "l"(inv_h2), "l"(off2));
                                 float x0, x1, u0, u1;
                                 nm_unpack2(x2, x0, x1);
@@ -722,15 +728,12 @@ nm_status nm_launch_attention_stream(nm_ctx* ctx, const nm_attn_desc* d, cudaStr
                                      float q_inv_scale)
 {
     if (!nm_attention_stream_any_length_supported(d)) return NM_ERR_UNSUPPORTED;
-    // the softmax input is never positive: a table whose range reaches 0 needs no upper clamp
+    // the unmasked forms' softmax input is never above 0: a table whose range reaches 0 needs no upper clamp there
     const bool clamp_hi = ctx->h_tables[d->exp_slot].x_max < 0.0f;
     const bool ragged = d->L % 128 != 0, one = d->L <= 128;
-#define NM_ATTN_FORM(T, CH)                                                                                           \
-    (one ? (ragged ? launch<T, CH, true, true>(ctx, d, st, out_q, q_inv_scale)                                        \
-                   : launch<T, CH, false, true>(ctx, d, st, out_q, q_inv_scale))                                      \
-         : (ragged ? launch<T, CH, true, false>(ctx, d, st, out_q, q_inv_scale)                                       \
-                   : launch<T, CH, false, false>(ctx, d, st, out_q, q_inv_scale)))
-#define NM_ATTN_CASE(T) (clamp_hi ? NM_ATTN_FORM(T, true) : NM_ATTN_FORM(T, false))
+#define NM_ATTN_FORM(T, CH, RG)                                                                                       \
+    (one ? launch<T, CH, RG, true>(ctx, d, st, out_q, q_inv_scale) : launch<T, CH, RG, false>(ctx, d, st, out_q, q_inv_scale))
+#define NM_ATTN_CASE(T) (ragged ? NM_ATTN_FORM(T, true, true) : clamp_hi ? NM_ATTN_FORM(T, true, false) : NM_ATTN_FORM(T, false, false))
     if (d->dtype == NM_BF16) return NM_ATTN_CASE(__nv_bfloat16);
     return NM_ATTN_CASE(__half);
 #undef NM_ATTN_CASE

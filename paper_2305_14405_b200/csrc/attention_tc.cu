@@ -235,7 +235,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
 #pragma unroll
         for (int i = 0; i < NH; ++i) m = fmaxf(m, s_red[i][row]);  // the FINAL row maximum
         asm volatile("bar.sync 1, %0;" ::"n"(NSOFT) : "memory");
-        const float neg_ms = -(m * a.scale);
+        const float neg_ms = -__fmul_ru(m, a.scale);   // rounded up: the table's input is then never above 0
         float sum0 = 0.f, sum1 = 0.f, sum2 = 0.f, sum3 = 0.f;
         if (ok) {
             // ---- pass 2: e = PWL_exp(s - m), row sum, P tiles for the second MMA
@@ -394,7 +394,7 @@ nm_status launch(nm_ctx* ctx, const nm_attn_desc* d, cudaStream_t st)
 template <typename T>
 nm_status launch_sel(nm_ctx* ctx, const nm_attn_desc* d, cudaStream_t st)
 {
-    // the softmax input is never positive: a table whose range reaches 0 needs no upper clamp
+    // the softmax input is never above 0 (the kernel sees to it): a table whose range reaches 0 needs no upper clamp
     const bool clamp_hi = ctx->h_tables[d->exp_slot].x_max < 0.0f;
     if (d->L >= 256) return clamp_hi ? launch<T, 4, true>(ctx, d, st) : launch<T, 4, false>(ctx, d, st);
     return clamp_hi ? launch<T, 2, true>(ctx, d, st) : launch<T, 2, false>(ctx, d, st);

@@ -82,6 +82,55 @@ def test_attention_bf16_segment_counts(nm, ctx, n):
     assert_close_bf16(got, ref, "attention n=%d" % n)
 
 
+def scaled_scores(qkv, B, L, h, scale, tabs, two_roundings):
+    """float64 attention whose table input is rounded as the kernels round it (the integer products are exact): scale, then
+    subtract the maximum, or both in one FMA whose maximum is rounded up.  Returns the output and sum_j |e_j v_j| * |r|."""
+    q, k, v = [t.reshape(B, L, h, 64).transpose(0, 2, 1, 3) for t in np.split(qkv.astype(np.float64), 3, 1)]
+    s = q @ k.transpose(0, 1, 3, 2)
+    sc = np.float64(np.float32(scale))
+    if two_roundings:
+        t = (s * sc).astype(np.float32)
+        x = t - t.max(-1, keepdims=True)
+    else:
+        m = s.max(-1, keepdims=True) * sc
+        up = m.astype(np.float32)
+        up = np.where(up < m, np.nextafter(up, np.float32(np.inf)), up)
+        x = (s * sc - up).astype(np.float32)
+    assert x.max() <= 0
+    t = tabs["exp"]
+    i = np.clip(np.floor((x.astype(np.float64) - t.x_min) * (t.n / (t.x_max - t.x_min))), 0, t.n - 1).astype(int)
+    e = t.k.astype(np.float64)[i] * x + t.b.astype(np.float64)[i]
+    sigma = e.sum(-1, keepdims=True)
+    t = tabs["recip"]
+    i = np.clip(np.floor((sigma - t.x_min) * (t.n / (t.x_max - t.x_min))), 0, t.n - 1).astype(int)
+    r = t.k.astype(np.float64)[i] * sigma + t.b.astype(np.float64)[i]
+    return [a.transpose(0, 2, 1, 3).reshape(B * L, h * 64) for a in ((e @ v) * r, (np.abs(e) @ np.abs(v)) * np.abs(r))]
+
+
+@pytest.mark.parametrize("algo,L", [("simt", 100), ("auto", 37), ("auto", 100), ("auto", 333), ("auto", 128), ("auto", 256), ("resident", 256)])
+@pytest.mark.parametrize("n", [64, 256])
+@pytest.mark.parametrize("scale,unit", [(0.1, 512), (0.1, 4096), (0.3, 1), (0.125, 1)])
+def test_attention_scales(nm, ctx, algo, L, n, scale, unit):
+    """Scales that are no power of two, scores up to 4e8: the largest score of a row stays inside the table.  (A score's
+    neighbours then lie far below the table and its first segment is extrapolated; the kernels do so alike.)"""
+    B, h = 2, 2
+    tabs = load_tables_both(ctx, n, ranges(L))
+    rng = np.random.default_rng(L + n)
+    qkv = rng.integers(-2, 3, (B * L, 3 * 64 * h)).astype(np.float32)
+    qkv[:, :2 * 64 * h] *= unit
+    out = torch.full((B * L, 64 * h), float("nan"), dtype=torch.bfloat16, device="cuda")
+    ctx.attention_pwl(torch.from_numpy(qkv).cuda().bfloat16(), out, B, L, h, 64, scale=scale,
+                      algo={"simt": nm.ALGO_SIMT, "auto": nm.ALGO_AUTO, "resident": nm.ALGO_ATTN_RESIDENT}[algo])
+    ctx.check_device_status()
+    ref, mag = scaled_scores(qkv, B, L, h, scale, tabs, two_roundings=L % 128 != 0)
+    # a rounding to bf16, 8 significant bits, is at most 2^-8 of the value: the output's, and at multiples of 128 the
+    # probabilities' as well; fp32 sums of L terms and of the row sum add 1e-5 of the terms' magnitudes
+    got = to_np(out)
+    assert np.all(np.isfinite(got))
+    err, bound = np.abs(got - ref), 2.0 ** -8 * np.abs(ref) + (2.0 ** -8 if L % 128 == 0 else 0.0) * mag + 1e-5 * mag
+    assert np.all(err <= bound), (err / bound).max()
+
+
 def test_attention_full_size_sampled(nm, ctx):
     """B=32, L=512, 12 heads of 64: the launch the benchmark times; three sampled batch entries
     are checked in full against the oracle."""

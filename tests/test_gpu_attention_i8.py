@@ -54,6 +54,22 @@ def test_int8_attention_bit_exact(nm, ctx, B, L, h, qk):
     assert torch.equal(ob.cpu(), want), "bf16 output = the fp32 value rounded once"
 
 
+@pytest.mark.parametrize("scale", [0.3, 30.0, 3000.0, 3e6])
+@pytest.mark.parametrize("n", [64, 127])
+def test_int8_attention_large_scales(nm, ctx, scale, n):
+    """fma(acc, sc, -(m * sc)) lies above 0 by up to half an ulp of m * sc, many segments for large scales."""
+    B, L, h, d = 2, 128, 2, 64
+    tabs = load_tables_both(ctx, n, {"exp": (-8.0, 0.0), "recip": (L / 16.0, float(L))})
+    codes, _, _ = _codes(B, L, h, d, n, 1.0)
+    out = torch.full((B * L, h * d), float("nan"), dtype=torch.float32, device="cuda")
+    pc = torch.full((B, h, L, L), -7, dtype=torch.int8, device="cuda")
+    ctx.attention_pwl_i8(torch.from_numpy(codes).cuda(), out, B, L, h, d, 0.7, 0.7, 0.04, scale=scale, p_dump=pc)
+    ctx.check_device_status()
+    r = oracle.attention_i8(codes, B, L, h, d, 0.7, 0.7, 0.04, tabs["exp"], tabs["recip"], scale=scale, want_dumps=True)
+    assert np.array_equal(pc.cpu().numpy(), r["p"])
+    assert np.array_equal(out.cpu().numpy().view(np.uint32), r["out"].view(np.uint32))
+
+
 def test_int8_attention_full_size_sampled(nm, ctx):
     """The config-3 launch shape (B 32, L 512, 12 heads): three batch entries checked in full, bit for bit."""
     B, L, h, d = 32, 512, 12, 64
