@@ -23,17 +23,24 @@
 // loses the tile's stores and the tensor core's reads of it.
 //
 // RAGGED form (an L that is not a multiple of 128, otherwise the CUDA-core kernel's): the tensor maps fill rows
-// beyond the sequence with zeros, the scores of keys beyond L are masked in the last chunk only, and warps whose
+// beyond the sequence with zeros, the scores of keys beyond L are masked in the last block only, and warps whose
 // 32 queries all lie beyond L keep the barriers' pace without arithmetic.  The CUDA-core kernel holds its
-// probabilities in fp32, so this form does not round them to 16 bits: e = hi + lo, two 16-bit terms (the error of
-// the pair is at most 2^-18 e in bf16, against the 2^-9 of the result's own rounding), and P V runs once per term.
-// The second term's 32 columns make it two CTAs per SM instead of three.  B 7, L 333, 12 heads: 2368 us on the CUDA
-// cores, 20.3 us here; B 1, L 37: 13.4 and 5.4 us.
+// probabilities in fp32, so this form does not round them to 16 bits: a bf16 P is three terms whose sum is e exactly,
+// an fp16 P two terms of 22 bits of e, scaled by a power of two per row; all of a probability's terms have its sign and
+// none of them is zero, so that an infinite V gives an infinity and not 0 * inf (ProbTerms).  The tensor core truncates
+// its sums, so the second and third terms, 2^-8 and less of the first, are kept out of the first one's sum: they have an
+// accumulator of their own, or go first.  Outputs that are not the correctly rounded ones, of all, at L 37 / 333 / 500, with
+// one accumulator and two rounded terms, so, and on the CUDA cores: bf16 2.2e-3, 2.4e-3, 2.5e-3 | 1.0e-4, 1.7e-4, 2.2e-4 |
+// 1.3e-4, 2.6e-4, 3.1e-4; fp16 0.9e-3, 3.5e-3, 5.0e-3 | 0.9e-3, 1.9e-3, 2.6e-3 | 1.0e-3, 1.7e-3, 2.0e-3.
+// The terms of 32 keys at a time, 48 columns, lie behind the second accumulator: 256 columns, two CTAs per SM.
+// B 7, L 333, 12 heads: 2368 us on the CUDA cores, 21.7 here (18.7 with two rounded terms); B 32, L 500: 141 (112).
 //
 // ONE form (L <= 128, a single 128-key chunk): the scores and the accumulator do not share columns (128 | 64, and P behind
 // them: 256 columns, two CTAs per SM), so the one Q K^T of sweep 1 serves sweep 2 as well, and nothing is fetched or
-// multiplied twice in what is then a latency-bound kernel (B 1, L 128, 16 heads: 6.4 -> 4.9 us; B 32, L 100, 12 heads:
-// 19.0 -> 16.7).
+// multiplied twice in what is then a latency-bound kernel (B 1, L 128, 16 heads: 6.4 -> 4.9 us).  RAGGED and ONE: the first
+// two terms of a block of 16 keys take the place of its scores, the third goes behind the accumulator, and P V runs once,
+// over all keys and the smallest terms first, instead of once per 64 keys (B 32, L 100, 12 heads: 15.0 -> 12.8 us; B 1, L 37:
+// 5.3).
 //
 //   warp 0            control: TMA loads (K chunks through two stages, V chunks through one) and the tcgen05.mma
 //                     for S = Q K_c^T and O += P_c V_c (V as an MN-major operand).  It sleeps in a named barrier
@@ -64,6 +71,7 @@ struct SArgs {
     void* out;
     int* status;
     int n_exp;
+    float e_max;         // RAGGED, fp16: the largest |PWL_exp(x)| for x from the table's lower end to 0
     int8_t* out_q;       // when set: the output goes out as int8 codes (of the value rounded to T) instead
     float q_inv_scale;
 };
@@ -77,10 +85,6 @@ template <> struct AT<__nv_bfloat16> {
         __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
         return *reinterpret_cast<uint32_t*>(&h);
     }
-    static __device__ __forceinline__ float2 unpack(uint32_t w)
-    {
-        return make_float2(__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u));
-    }
 };
 template <> struct AT<__half> {
     static constexpr uint32_t fmt = 0;
@@ -90,7 +94,36 @@ template <> struct AT<__half> {
         __half2 h = __floats2half2_rn(a, b);
         return *reinterpret_cast<uint32_t*>(&h);
     }
-    static __device__ __forceinline__ float2 unpack(uint32_t w) { return __half22float2(*reinterpret_cast<__half2*>(&w)); }
+};
+
+// Two probabilities as 16-bit terms, one packed word per term.  Each term but the last is the remainder so far rounded
+// towards zero and, being cut from a value one unit lower (the product with 1 - 2^-24, rounded towards zero), always smaller
+// than the remainder: the next term is never zero and has the same sign, and a zero probability has only zero terms.
+// bf16, 8 bits a term: after two terms at most 8 bits are left, so the three add up to e exactly.  fp16, 11 bits a term.
+template <typename T> struct ProbTerms;
+template <> struct ProbTerms<__nv_bfloat16> {
+    static constexpr int N = 3;
+    static __device__ __forceinline__ void split(float e0, float e1, uint32_t& w0, uint32_t& w1, uint32_t& w2)
+    {
+        const float below = 0x1.fffffep-1f;   // 1 - 2^-24
+        const uint32_t h0 = __float_as_uint(__fmul_rz(e0, below)), h1 = __float_as_uint(__fmul_rz(e1, below));
+        const float r0 = e0 - __uint_as_float(h0 & 0xffff0000u), r1 = e1 - __uint_as_float(h1 & 0xffff0000u);
+        const uint32_t m0 = __float_as_uint(__fmul_rz(r0, below)), m1 = __float_as_uint(__fmul_rz(r1, below));
+        const float l0 = r0 - __uint_as_float(m0 & 0xffff0000u), l1 = r1 - __uint_as_float(m1 & 0xffff0000u);
+        w0 = __byte_perm(h0, h1, 0x7632);
+        w1 = __byte_perm(m0, m1, 0x7632);
+        w2 = __byte_perm(__float_as_uint(l0), __float_as_uint(l1), 0x7632);
+    }
+};
+template <> struct ProbTerms<__half> {
+    static constexpr int N = 2;
+    static __device__ __forceinline__ void split(float e0, float e1, uint32_t& w0, uint32_t& w1, uint32_t&)
+    {
+        const float below = 0x1.fffffep-1f;
+        asm("cvt.rz.f16x2.f32 %0, %1, %2;" : "=r"(w0) : "f"(__fmul_rz(e1, below)), "f"(__fmul_rz(e0, below)));
+        const float2 hi = __half22float2(*reinterpret_cast<const __half2*>(&w0));
+        w1 = AT<__half>::pack(e0 - hi.x, e1 - hi.y);
+    }
 };
 
 // 16 packed words of this thread's row into 16 consecutive tensor-memory columns (the mirror of the 16-column read)
@@ -148,7 +181,7 @@ struct LoadCtx {
     const CUtensorMap *tmQ, *tmK, *tmV;
     uint8_t *q_s, *k_st, *p_s, *v_st;
     uint64_t *bar_q, *bar_k1_full, *bar_v_full;   // bar_k1_full: [2]
-    int n128;
+    int n128, v_chunks;
 };
 // Q and the first two 128-key chunks of sweep 1 (stage 0 = the two K stages, stage 1 = the buffer p_s).  One
 // thread; the buffers must be free.
@@ -166,11 +199,11 @@ __device__ __forceinline__ void load_tile_head(const LoadCtx& c, const Tile& t)
         nm_tma_load_3d(dst + STAGE, c.tmK, t.g * HD, st * 2 * CK + CK, t.b, bar);
     }
 }
-// The first V chunk of a tile (one thread; the V stage must be free).
+// The first V chunk of a tile, or all of its V (one thread; the V stage must be free).
 __device__ __forceinline__ void load_first_v(const LoadCtx& c, const Tile& t)
 {
-    nm_mbar_expect_tx(c.bar_v_full, STAGE);
-    nm_tma_load_3d(c.v_st, c.tmV, t.g * HD, 0, t.b, c.bar_v_full);
+    nm_mbar_expect_tx(c.bar_v_full, c.v_chunks * STAGE);
+    for (int i = 0; i < c.v_chunks; ++i) nm_tma_load_3d(c.v_st + i * STAGE, c.tmV, t.g * HD, i * CK, t.b, c.bar_v_full);
 }
 
 template <typename T, bool CLAMP_HI, bool RAGGED, bool ONE>
@@ -185,9 +218,11 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
     constexpr uint32_t TMEM_COLS = ONE ? 256 : 128;
     constexpr uint32_t O_OFF = ONE ? 128 : 64;
     // The 16-bit P tile goes through a second allocation of 32 columns (64 keys, two per column) and is the A operand
-    // of P V from there; three CTAs hold 3 x (128 + 32) of the SM's 512 columns.  RAGGED: 32 more for the low terms.
-    constexpr uint32_t P_COLS = RAGGED ? 64 : 32;
-    constexpr int P_TERMS = RAGGED ? 2 : 1;
+    // of P V from there; three CTAs hold 3 x (128 + 32) of the SM's 512 columns.  RAGGED: 64 columns for the sum of the
+    // lower terms and 64 for the terms of 32 keys, 16 columns each.
+    constexpr uint32_t P_COLS = RAGGED ? 128 : 32;
+    constexpr int TERMS = RAGGED ? ProbTerms<T>::N : 1;
+    constexpr bool SCALED = RAGGED && std::is_same<T, __half>::value;
 
     extern __shared__ uint8_t smem_raw[];
     __shared__ uint64_t bar_q, bar_drain;
@@ -197,6 +232,8 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
 
     const int L = a.L;
     const int n = RAGGED ? (L + CK - 1) / CK : L / CK;                    // 64-key chunks of sweep 2
+    // P V products: RAGGED one per 32 keys, or one for all of them (ONE); otherwise one per chunk
+    const int n_pv = !RAGGED ? n : ONE ? 1 : (L + 31) / 32;
     const int n128 = ONE ? 1 : RAGGED ? (L + 2 * CK - 1) / (2 * CK) : L / (2 * CK);   // 128-key chunks of sweep 1
     uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     uint8_t* q_s = base;                       // 16 KB
@@ -218,6 +255,11 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
     lc.q_s = q_s; lc.k_st = k_st; lc.p_s = p_s; lc.v_st = v_st;
     lc.bar_q = &bar_q; lc.bar_k1_full = &bar_k1_full[0]; lc.bar_v_full = &bar_v_full;
     lc.n128 = n128;
+    lc.v_chunks = 1;
+    if (RAGGED && ONE) {   // all of V in the buffer that sweep 1 of longer sequences takes
+        lc.v_st = p_s;
+        lc.v_chunks = n;
+    }
 
     if (threadIdx.x == 0) {
         abort_flag = 0;
@@ -260,6 +302,7 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
     nm_tc_fence_after();
     const uint32_t tmem_base = tmem_slot;
     const uint32_t tmem_p = ONE ? tmem_base + 192u : tmem_slot_p;
+    const uint32_t tmem_lo = tmem_slot_p, tmem_t = tmem_slot_p + 64u;   // RAGGED, not ONE: sum of the lower terms; the terms
     volatile int* abortp = &abort_flag;
     nm_grid_launch_dependents();   // the next kernel may start its set-up
     nm_grid_dependency_wait();     // Q, K, V come from the previous kernel
@@ -344,29 +387,53 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                 if (n > 1) load_k(1);
                 issue_qk(0);
             }
-            for (int j = 0; j < n; ++j) {
+            for (int u = 0; u < n_pv; ++u) {
+                const int j = RAGGED && !ONE ? u >> 1 : u;                              // chunk
+                const bool chunk_ends = !RAGGED || ONE || (u & 1) || u + 1 == n_pv;     // (it holds one or two P V products)
+                const bool chunk_begins = !RAGGED || ONE || !(u & 1);
                 if constexpr (!ONE) {
-                    asm volatile("bar.sync %0, %1;" ::"r"(bar_sc), "n"(160) : "memory");   // S-consumed(j)
-                    if (j + 1 < n) issue_qk(j + 1);
-                    if (j + 2 < n) load_k(j + 2);
-                } else if (j + 1 == n && more && ok) {
+                    if (chunk_ends) {
+                        asm volatile("bar.sync %0, %1;" ::"r"(bar_sc), "n"(160) : "memory");   // S-consumed(j)
+                        if (j + 1 < n) issue_qk(j + 1);
+                        if (j + 2 < n) load_k(j + 2);
+                    }
+                } else if (u + 1 == n_pv && more && ok) {
                     if (!wait(&bar_s_full, (uint32_t)ti & 1u)) ok = false;   // the tile's one product has read Q and K
                 }
-                // Last chunk: every Q K^T of the tile has completed, so Q, the K stages and p_s take the next tile's
+                // Last product: every Q K^T of the tile has completed, so Q, the K stages and p_s take the next tile's
                 // first loads now.
-                if (j + 1 == n && more && ok && nm_elect_one()) load_tile_head(lc, tile_of(tile + (int)gridDim.x));
+                if (u + 1 == n_pv && more && ok && nm_elect_one()) load_tile_head(lc, tile_of(tile + (int)gridDim.x));
                 __syncwarp();
-                asm volatile("bar.sync %0, %1;" ::"r"(bar_pr), "n"(160) : "memory");   // P-ready(j)
-                if (ok && !wait(&bar_v_full, v_cnt & 1u)) ok = false;
-                ++v_cnt;
+                asm volatile("bar.sync %0, %1;" ::"r"(bar_pr), "n"(160) : "memory");   // P-ready(u)
+                if (chunk_begins) {
+                    if (ok && !wait(&bar_v_full, v_cnt & 1u)) ok = false;
+                    ++v_cnt;
+                }
                 if (ok) {
                     nm_tc_fence_after();
-                    const uint32_t v_addr = nm_smem_u32(v_st);
+                    const uint32_t v_addr = nm_smem_u32(lc.v_st);
+                    // V rows (keys) 16 k .. 16 k + 15 of the stage: two groups of 8 rows, 1024 bytes apart
+                    auto vdesc = [v_addr](int k) { return nm_smem_desc_sw128(v_addr + (uint32_t)(16 * k * ROWB)); };
                     if (nm_elect_one()) {
+                        if constexpr (!RAGGED) {
 #pragma unroll
-                        for (int k = 0; k < 4 * P_TERMS; ++k) {   // V rows (keys) 16(k&3)..+15: two groups of 8 rows, 1024 bytes apart
-                            const uint64_t vdesc = nm_smem_desc_sw128(v_addr + (uint32_t)(16 * (k & 3) * ROWB));
-                            mma_f16_a_tmem(tmem_base + O_OFF, tmem_p + (uint32_t)(8 * k), vdesc, IDESC_PV, (j | k) != 0);
+                            for (int k = 0; k < 4; ++k)
+                                mma_f16_a_tmem(tmem_base + O_OFF, tmem_p + (uint32_t)(8 * k), vdesc(k), IDESC_PV, (j | k) != 0);
+                        } else if constexpr (ONE) {
+                            const int steps = (L + 15) / 16;
+#pragma unroll
+                            for (int t = TERMS - 1; t >= 0; --t)
+                                for (int k = 0; k < steps; ++k)
+                                    mma_f16_a_tmem(tmem_base + O_OFF, t == 2 ? tmem_p + (uint32_t)(8 * k) : tmem_base + (uint32_t)(16 * k + 8 * t),
+                                                   vdesc(k), IDESC_PV, t != TERMS - 1 || k != 0);
+                        } else {
+                            const int k0 = 2 * (u & 1);
+#pragma unroll
+                            for (int t = TERMS - 1; t >= 0; --t)
+#pragma unroll
+                                for (int k = 0; k < 2; ++k)
+                                    mma_f16_a_tmem(t == 0 ? tmem_base + O_OFF : tmem_lo, tmem_t + (uint32_t)(16 * t + 8 * k), vdesc(k0 + k), IDESC_PV,
+                                                   u != 0 || k != 0 || (t != 0 && t != TERMS - 1));
                         }
                         nm_tc_commit(&bar_p_empty);
                     }
@@ -376,11 +443,11 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                 ++pv_cnt;
                 // the V stage is free once this P V has completed (nothing else to do until then): it takes the
                 // next chunk's V, or after the last chunk the next tile's first one
-                const bool next_v = j + 1 < n || more;
-                if (ok && next_v) {
+                const bool last = u + 1 == n_pv;
+                if (ok && chunk_ends && (!last || more)) {
                     if (!wait(&bar_p_empty, pv_par)) ok = false;
                     if (ok && nm_elect_one()) {
-                        if (j + 1 < n) {
+                        if (!last) {
                             nm_mbar_expect_tx(&bar_v_full, STAGE);
                             nm_tma_load_3d(v_st, &tmV, g * HD, (j + 1) * CK, b, &bar_v_full);
                         } else {
@@ -443,6 +510,7 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
             const bool live = !RAGGED || qb * BQ + q * 32 < L;
             // ---- sweep 1: the final row maximum
             float m = -INFINITY;
+            [[maybe_unused]] float lowest = INFINITY;   // SCALED: the smallest score
 #pragma unroll 1
             for (int i = 0; i < n128; ++i) {
                 wait_all(&bar_s_full, s_cnt & 1u);
@@ -461,8 +529,13 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                         if (RAGGED && i == n128 - 1) {   // keys beyond L do not take part
                             const int lim = L - i * 2 * CK - hh * 32;
 #pragma unroll
-                            for (int k = 0; k < 32; ++k)
+                            for (int k = 0; k < 32; ++k) {
+                                if (SCALED && k < lim) lowest = fminf(lowest, __uint_as_float(r[k]));
                                 if (k >= lim) r[k] = 0xff800000u;   // -inf
+                            }
+                        } else if (SCALED) {
+#pragma unroll
+                            for (int k = 0; k < 32; ++k) lowest = fminf(lowest, __uint_as_float(r[k]));
                         }
                         float m0 = -INFINITY, m1 = -INFINITY;
 #pragma unroll
@@ -483,118 +556,180 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
             const float neg_ms = RAGGED ? -__fmul_rn(m, a.scale) : -__fmul_ru(m, a.scale);
             const uint64_t neg_ms2 = nm_pack2(neg_ms, neg_ms);
             float sum0 = 0.f, sum1 = 0.f, sum2 = 0.f, sum3 = 0.f;
-            // ---- sweep 2: e = PWL_exp(s - m), row sum, P tiles.  LAST: the chunk that may hold keys beyond L; they
-            // take the maximum as their score (which keeps the table index in range) and the exponential 0.
-            auto chunk = [&](int j, auto last) {
-                constexpr bool LAST = decltype(last)::value;
-                constexpr int W = RAGGED ? 16 : 32;   // (with two terms of P, 32 keys at a time spill: 129 us at B 32, L 500, 12 heads, 114 so)
-                if constexpr (!ONE) {
-                    wait_all(&bar_s_full, s_cnt & 1u);
-                    ++s_cnt;
-                    if (ok) nm_tc_fence_after();
+            // SCALED: the power of two that brings the largest |e| this row can have to 2^14 .. 2^15 (below the table the first
+            // segment goes on), and its inverse; an fp16 term then loses nothing to the narrow exponent
+            [[maybe_unused]] float up = 1.f, down = 1.f;
+            if constexpr (SCALED) {
+                const float x = __fadd_rn(__fmul_rn(lowest, a.scale), neg_ms);
+                const float2 kb0 = rep[lane & 15];
+                const float big = fmaxf(a.e_max, nm_pwl_index(x, inv_h, off, nm1) == 0 ? fabsf(__fmaf_rn(kb0.x, x, kb0.y)) : 0.f);
+                const int ex = min(max(14 + 127 - (int)(__float_as_uint(big) >> 23), -100), 100);
+                up = __uint_as_float((uint32_t)(127 + ex) << 23);
+                down = __uint_as_float((uint32_t)(127 - ex) << 23);
+            }
+            // ---- sweep 2: e = PWL_exp(s - m), row sum, P tiles.
+            // W scores of this thread's row -> exponentials, in groups of 8.  MASKED: keys from `lim` on lie beyond L; they take
+            // the maximum as their score (which keeps the table index in range) and the exponential 0.
+            constexpr int W = RAGGED ? 16 : 32;   // (with several terms of P, 32 keys at a time spill)
+            auto exponentials = [&](uint32_t* r, int lim, auto masked, auto&& use) {
+                constexpr bool MASKED = decltype(masked)::value;
+                if constexpr (MASKED) {
+#pragma unroll
+                    for (int k = 0; k < W; ++k)
+                        if (k >= lim) r[k] = __float_as_uint(m);
                 }
 #pragma unroll
-                for (int hh = 0; hh < CK / W; ++hh) {   // W keys at a time
-                    const int lim = LAST ? L - j * CK - hh * W : W;
-                    uint32_t r[W];
-                    if (ok && live) {
-                        if constexpr (W == 32) nm_tmem_ld32_sync(t_row + (uint32_t)((ONE ? j * CK : 0) + hh * 32), r);
-                        else nm_tmem_ld16_sync(t_row + (uint32_t)((ONE ? j * CK : 0) + hh * 16), r);
-                        if constexpr (LAST) {
+                for (int jj = 0; jj < W / 8; ++jj) {   // 8 keys
+                    float e[8];
 #pragma unroll
-                            for (int k = 0; k < W; ++k)
-                                if (k >= lim) r[k] = __float_as_uint(m);
-                        }
-                    }
-                    if (!ONE && hh == CK / W - 1) {
-                        nm_tc_fence_before();
-                        asm volatile("bar.arrive %0, %1;" ::"r"(bar_sc), "n"(160) : "memory");
-                    }
-                    uint32_t pk[W / 2];                    // the exponentials, packed to 16 bits
-                    [[maybe_unused]] uint32_t pl[RAGGED ? W / 2 : 1];          // RAGGED: what the packing left, packed to 16 bits
-                    if (ok && live) {
-#pragma unroll
-                        for (int jj = 0; jj < W / 8; ++jj) {   // 8 keys
-                            float e[8];
-#pragma unroll
-                            for (int k = 0; k < 8; k += 2) {
-                                // two scores at a time on the packed fp32 instructions: each half is the same correctly
-                                // rounded operation as the scalar form
-                                uint64_t x2, u2, b2;
-                                const float s0 = __uint_as_float(r[jj * 8 + k]), s1 = __uint_as_float(r[jj * 8 + k + 1]);
-                                if constexpr (RAGGED) {   // (the packed mul and add would be contracted into an FMA)
-                                    x2 = nm_pack2(__fadd_rn(__fmul_rn(s0, a.scale), neg_ms), __fadd_rn(__fmul_rn(s1, a.scale), neg_ms));
-                                } else {
-                                    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(x2) : "l"(nm_pack2(s0, s1)), "l"(scale2), "l"(neg_ms2));
-                                }
-                                asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(u2) : "l"(x2), "l"(inv_h2), "l"(off2));
-                                float x0, x1, u0, u1;
-                                nm_unpack2(x2, x0, x1);
-                                nm_unpack2(u2, u0, u1);
-                                u0 = fmaxf(u0, 0.0f);
-                                u1 = fmaxf(u1, 0.0f);
-                                if (CLAMP_HI) {
-                                    u0 = fminf(u0, nm1);
-                                    u1 = fminf(u1, nm1);
-                                }
-                                // floor(u) sits in the low mantissa bits after a round-down add of 1.5 * 2^23
-                                asm("add.rm.f32x2 %0, %1, %2;" : "=l"(b2) : "l"(nm_pack2(u0, u1)), "l"(magic2));
-                                float f0, f1;
-                                nm_unpack2(b2, f0, f1);
-                                float k0, c0, k1, c1;
-                                asm("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(k0), "=f"(c0) : "r"((__float_as_uint(f0) << 7) + rep_lane));
-                                asm("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(k1), "=f"(c1) : "r"((__float_as_uint(f1) << 7) + rep_lane));
-                                e[k] = __fmaf_rn(k0, x0, c0);
-                                e[k + 1] = __fmaf_rn(k1, x1, c1);
-                                if constexpr (LAST) {
-                                    if (jj * 8 + k >= lim) e[k] = 0.f;
-                                    if (jj * 8 + k + 1 >= lim) e[k + 1] = 0.f;
-                                }
-                            }
-                            sum0 += e[0] + e[4];
-                            sum1 += e[1] + e[5];
-                            sum2 += e[2] + e[6];
-                            sum3 += e[3] + e[7];
-#pragma unroll
-                            for (int k = 0; k < 4; ++k) {
-                                pk[jj * 4 + k] = AT<T>::pack(e[2 * k], e[2 * k + 1]);
-                                if constexpr (RAGGED) {
-                                    const float2 hi = AT<T>::unpack(pk[jj * 4 + k]);
-                                    pl[jj * 4 + k] = AT<T>::pack(e[2 * k] - hi.x, e[2 * k + 1] - hi.y);   // exact differences
-                                }
-                            }
-                        }
-                    }
-                    // The stores wait until P V of the previous chunk has read the tile; that MMA was
-                    // issued just before this chunk began, so the first half's arithmetic runs ahead of it.
-                    if (hh == 0 && j >= 1) {
-                        wait_all(&bar_p_empty, (pv_base + (uint32_t)(j - 1)) & 1u);
-                    }
-                    if (ok && live) {
-                        if (hh == 0 && j >= 1) nm_tc_fence_after();   // ordered after the P V that read the columns
-                        if constexpr (RAGGED) {   // keys 16 hh .. 16 hh + 15 of this thread's row
-                            tmem_st8(p_row + (uint32_t)(hh * 8), pk);
-                            tmem_st8(p_row + (uint32_t)(32 + hh * 8), pl);
+                    for (int k = 0; k < 8; k += 2) {
+                        // two scores at a time on the packed fp32 instructions: each half is the same correctly
+                        // rounded operation as the scalar form
+                        uint64_t x2, u2, b2;
+                        const float s0 = __uint_as_float(r[jj * 8 + k]), s1 = __uint_as_float(r[jj * 8 + k + 1]);
+                        if constexpr (RAGGED) {   // (the packed mul and add would be contracted into an FMA)
+                            x2 = nm_pack2(__fadd_rn(__fmul_rn(s0, a.scale), neg_ms), __fadd_rn(__fmul_rn(s1, a.scale), neg_ms));
                         } else {
-                            tmem_st16(p_row + (uint32_t)(hh * 16), pk);   // keys 32 hh .. 32 hh + 31
+                            asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(x2) : "l"(nm_pack2(s0, s1)), "l"(scale2), "l"(neg_ms2));
+                        }
+                        asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(u2) : "l"(x2), "l"(inv_h2), "l"(off2));
+                        float x0, x1, u0, u1;
+                        nm_unpack2(x2, x0, x1);
+                        nm_unpack2(u2, u0, u1);
+                        u0 = fmaxf(u0, 0.0f);
+                        u1 = fmaxf(u1, 0.0f);
+                        if (CLAMP_HI) {
+                            u0 = fminf(u0, nm1);
+                            u1 = fminf(u1, nm1);
+                        }
+                        // floor(u) sits in the low mantissa bits after a round-down add of 1.5 * 2^23
+                        asm("add.rm.f32x2 %0, %1, %2;" : "=l"(b2) : "l"(nm_pack2(u0, u1)), "l"(magic2));
+                        float f0, f1;
+                        nm_unpack2(b2, f0, f1);
+                        float k0, c0, k1, c1;
+                        asm("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(k0), "=f"(c0) : "r"((__float_as_uint(f0) << 7) + rep_lane));
+                        asm("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(k1), "=f"(c1) : "r"((__float_as_uint(f1) << 7) + rep_lane));
+                        e[k] = __fmaf_rn(k0, x0, c0);
+                        e[k + 1] = __fmaf_rn(k1, x1, c1);
+                        if constexpr (MASKED) {
+                            if (jj * 8 + k >= lim) e[k] = 0.f;
+                            if (jj * 8 + k + 1 >= lim) e[k + 1] = 0.f;
                         }
                     }
+                    sum0 += e[0] + e[4];
+                    sum1 += e[1] + e[5];
+                    sum2 += e[2] + e[6];
+                    sum3 += e[3] + e[7];
+                    use(jj, e);
                 }
-                tmem_st_wait();          // the P columns are written
-                nm_tc_fence_before();
-                asm volatile("bar.arrive %0, %1;" ::"r"(bar_pr), "n"(160) : "memory");
             };
+            if constexpr (!RAGGED) {
 #pragma unroll 1
-            for (int j = 0; j < (RAGGED ? n - 1 : n); ++j) chunk(j, std::false_type{});
-            if constexpr (RAGGED) chunk(n - 1, std::true_type{});
+                for (int j = 0; j < n; ++j) {
+                    if constexpr (!ONE) {
+                        wait_all(&bar_s_full, s_cnt & 1u);
+                        ++s_cnt;
+                        if (ok) nm_tc_fence_after();
+                    }
+#pragma unroll
+                    for (int hh = 0; hh < 2; ++hh) {
+                        uint32_t r[32];
+                        if (ok) nm_tmem_ld32_sync(t_row + (uint32_t)((ONE ? j * CK : 0) + hh * 32), r);
+                        if (!ONE && hh == 1) {
+                            nm_tc_fence_before();
+                            asm volatile("bar.arrive %0, %1;" ::"r"(bar_sc), "n"(160) : "memory");
+                        }
+                        uint32_t pk[16];   // the half's 32 exponentials, packed to 16 bits
+                        if (ok)
+                            exponentials(r, W, std::false_type{}, [&](int jj, const float* e) {
+#pragma unroll
+                                for (int k = 0; k < 4; ++k) pk[jj * 4 + k] = AT<T>::pack(e[2 * k], e[2 * k + 1]);
+                            });
+                        // The stores wait until P V of the previous chunk has read the tile; that MMA was
+                        // issued just before this chunk began, so the first half's arithmetic runs ahead of it.
+                        if (hh == 0 && j >= 1) wait_all(&bar_p_empty, (pv_base + (uint32_t)(j - 1)) & 1u);
+                        if (ok) {
+                            if (hh == 0 && j >= 1) nm_tc_fence_after();   // ordered after the P V that read the columns
+                            tmem_st16(p_row + (uint32_t)(hh * 16), pk);   // keys 32 hh .. 32 hh + 31 of this thread's row
+                        }
+                    }
+                    tmem_st_wait();          // the P columns are written
+                    nm_tc_fence_before();
+                    asm volatile("bar.arrive %0, %1;" ::"r"(bar_pr), "n"(160) : "memory");
+                }
+            } else {
+                // 16 keys' scores at tensor-memory column `src` -> the terms of their exponentials
+                uint32_t term[3][8];
+                auto block = [&](uint32_t src, int lim, auto masked, auto&& loaded) {
+                    uint32_t r[16];
+                    if (ok && live) nm_tmem_ld16_sync(src, r);
+                    loaded();
+                    if (ok && live)
+                        exponentials(r, lim, masked, [&](int jj, const float* e) {
+#pragma unroll
+                            for (int k = 0; k < 4; ++k)
+                                ProbTerms<T>::split(SCALED ? e[2 * k] * up : e[2 * k], SCALED ? e[2 * k + 1] * up : e[2 * k + 1],
+                                                    term[0][jj * 4 + k], term[1][jj * 4 + k], term[2][jj * 4 + k]);
+                        });
+                };
+                const uint32_t lanes = (uint32_t)(q * 32) << 16;
+                if constexpr (ONE) {
+                    auto keys16 = [&](int k, auto masked) {
+                        block(t_row + (uint32_t)(16 * k), L - 16 * k, masked, [] {});
+                        if (ok && live) {
+                            tmem_st8(t_row + (uint32_t)(16 * k), term[0]);
+                            tmem_st8(t_row + (uint32_t)(16 * k + 8), term[1]);
+                            if constexpr (TERMS == 3) tmem_st8(p_row + (uint32_t)(8 * k), term[2]);
+                        }
+                    };
+                    const int steps = (L + 15) / 16;
+#pragma unroll 1
+                    for (int k = 0; k < steps - 1; ++k) keys16(k, std::false_type{});
+                    keys16(steps - 1, std::true_type{});
+                    tmem_st_wait();
+                    nm_tc_fence_before();
+                    asm volatile("bar.arrive %0, %1;" ::"r"(bar_pr), "n"(160) : "memory");
+                } else {
+                    auto keys32 = [&](int u, auto masked) {
+                        const bool chunk_ends = (u & 1) || u + 1 == n_pv;
+                        if (!(u & 1)) {
+                            wait_all(&bar_s_full, s_cnt & 1u);
+                            ++s_cnt;
+                            if (ok) nm_tc_fence_after();
+                        }
+#pragma unroll
+                        for (int hh = 0; hh < 2; ++hh) {
+                            block(t_row + (uint32_t)((u & 1) * 32 + hh * 16), L - u * 32 - hh * 16, masked, [&] {
+                                if (hh == 1 && chunk_ends) {   // all of the chunk's scores are in registers
+                                    nm_tc_fence_before();
+                                    asm volatile("bar.arrive %0, %1;" ::"r"(bar_sc), "n"(160) : "memory");
+                                }
+                            });
+                            // the stores wait until the previous P V has read the columns; 16 keys' arithmetic runs ahead of it
+                            if (hh == 0 && u >= 1) wait_all(&bar_p_empty, (pv_base + (uint32_t)(u - 1)) & 1u);
+                            if (ok && live) {
+                                if (hh == 0 && u >= 1) nm_tc_fence_after();
+#pragma unroll
+                                for (int t = 0; t < TERMS; ++t) tmem_st8(tmem_t + lanes + (uint32_t)(16 * t + 8 * hh), term[t]);
+                            }
+                        }
+                        tmem_st_wait();
+                        nm_tc_fence_before();
+                        asm volatile("bar.arrive %0, %1;" ::"r"(bar_pr), "n"(160) : "memory");
+                    };
+#pragma unroll 1
+                    for (int u = 0; u < n_pv - 1; ++u) keys32(u, std::false_type{});
+                    keys32(n_pv - 1, std::true_type{});
+                }
+            }
             const float sum = (sum0 + sum1) + (sum2 + sum3);
             // ---- r = PWL_recip(sigma), then O * r
             const int sr = ONE ? nm_pwl_index(sum, r_inv_h, r_off, r_nm1)
                                : nm_pwl_index(sum, a.t_rcp->inv_h, a.t_rcp->off, (float)(a.t_rcp->n - 1));
             const float2 kbr = a.t_rcp->kb[sr];
             const float rinv = __fmaf_rn(kbr.x, sum, kbr.y);
-            wait_all(&bar_p_empty, (pv_base + (uint32_t)(n - 1)) & 1u);   // the last P V has completed
-            pv_base += (uint32_t)n;
+            wait_all(&bar_p_empty, (pv_base + (uint32_t)(n_pv - 1)) & 1u);   // the last P V has completed
+            pv_base += (uint32_t)n_pv;
             if (ok) nm_tc_fence_after();
             const bool store_row = !RAGGED || qb * BQ + row < L;
             T* orow = reinterpret_cast<T*>(a.out) + ((size_t)b * L + (size_t)qb * BQ + row) * ((size_t)a.heads * HD) +
@@ -603,7 +738,15 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
 #pragma unroll
             for (int jj = 0; jj < HD / 16; ++jj) {   // 16 channels at a time
                 uint32_t r0[16];
-                if (ok && live) nm_tmem_ld16_sync(o_addr + (uint32_t)(jj * 16), r0);
+                if (ok && live) {
+                    nm_tmem_ld16_sync(o_addr + (uint32_t)(jj * 16), r0);
+                    if constexpr (RAGGED && !ONE) {
+                        uint32_t r1[16];
+                        nm_tmem_ld16_sync(tmem_lo + ((uint32_t)(q * 32) << 16) + (uint32_t)(jj * 16), r1);
+#pragma unroll
+                        for (int k = 0; k < 16; ++k) r0[k] = __float_as_uint(__uint_as_float(r0[k]) + __uint_as_float(r1[k]));
+                    }
+                }
                 if (jj == HD / 16 - 1 && more) {
                     // all of O is in registers: the control warp may start the next tile's sweep 1 over [S | O]
                     nm_tc_fence_before();
@@ -612,7 +755,7 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                 if (ok && store_row) {
                     float v[16];
 #pragma unroll
-                    for (int k = 0; k < 16; ++k) v[k] = __uint_as_float(r0[k]) * rinv;
+                    for (int k = 0; k < 16; ++k) v[k] = (SCALED ? __uint_as_float(r0[k]) * down : __uint_as_float(r0[k])) * rinv;
                     if (a.out_q) {
                         int8_t code[16];
 #pragma unroll
@@ -671,6 +814,20 @@ nm_status launch(nm_ctx* ctx, const nm_attn_desc* d, cudaStream_t st, int8_t* ou
     a.out = d->out;
     a.status = ctx->d_status;
     a.n_exp = ctx->h_tables[d->exp_slot].n;
+    a.e_max = 0.f;
+    if (RAGGED && d->dtype == NM_F16) {
+        const NmTable& t = ctx->h_tables[d->exp_slot];
+        const double h = ((double)t.x_max - t.x_min) / t.n;
+        for (int i = 0; i < t.n; ++i) {   // each segment's ends as far as they are not above 0; the last one goes on to 0
+            const double ends[2] = {t.x_min + i * h, i + 1 == t.n && t.x_max < 0.f ? 0.0 : t.x_min + (i + 1) * h};
+            for (double x : ends) {
+                if (i > 0 && ends[0] > 0.0) continue;
+                if (x > 0.0) x = 0.0;
+                const double e = fabs((double)t.kb[i].x * x + t.kb[i].y);
+                if (e > a.e_max) a.e_max = (float)e;
+            }
+        }
+    }
     a.out_q = out_q;
     a.q_inv_scale = q_inv_scale;
     const size_t smem = (size_t)BQ * ROWB + 3 * (size_t)STAGE + (size_t)PBUF + (size_t)(a.n_exp + 1) * 16 * sizeof(float2) + 1024;
@@ -686,7 +843,7 @@ nm_status launch(nm_ctx* ctx, const nm_attn_desc* d, cudaStream_t st, int8_t* ou
     const int64_t tiles = (int64_t)d->B * d->heads * ((d->L + BQ - 1) / BQ);
     if (tiles > 0x7fffffffLL) return NM_ERR_SHAPE;
     // persistent: one resident wave of CTAs, each walking over tiles.  Three CTAs per SM (RAGGED, ONE: two) by the launch
-    // bounds (registers) and by tensor memory (3 x 160, 2 x 192 or 2 x 256 of 512 columns); fewer if the exp table makes the
+    // bounds (registers) and by tensor memory (3 x 160 or 2 x 256 of 512 columns); fewer if the exp table makes the
     // shared memory larger (233472 bytes per SM, 1 KB reserved per CTA).
     int64_t per_sm = 233472 / (int64_t)(smem + 1024 + 1536);
     if (per_sm > (RAGGED || ONE ? 2 : 3)) per_sm = RAGGED || ONE ? 2 : 3;

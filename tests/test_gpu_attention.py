@@ -109,8 +109,8 @@ def scaled_scores(qkv, B, L, h, scale, tabs, two_roundings):
 
 @pytest.mark.parametrize("algo,L", [("simt", 100), ("auto", 37), ("auto", 100), ("auto", 333), ("auto", 128), ("auto", 256), ("resident", 256)])
 @pytest.mark.parametrize("n", [64, 256])
-@pytest.mark.parametrize("scale,unit", [(0.1, 512), (0.1, 4096), (0.3, 1), (0.125, 1)])
-def test_attention_scales(nm, ctx, algo, L, n, scale, unit):
+@pytest.mark.parametrize("scale,unit,dtype", [(0.1, 512, "bf16"), (0.1, 4096, "bf16"), (0.3, 1, "bf16"), (0.125, 1, "bf16"), (0.3, 16, "f16")])
+def test_attention_scales(nm, ctx, algo, L, n, scale, unit, dtype):
     """Scales that are no power of two, scores up to 4e8: the largest score of a row stays inside the table.  (A score's
     neighbours then lie far below the table and its first segment is extrapolated; the kernels do so alike.)"""
     B, h = 2, 2
@@ -118,16 +118,19 @@ def test_attention_scales(nm, ctx, algo, L, n, scale, unit):
     rng = np.random.default_rng(L + n)
     qkv = rng.integers(-2, 3, (B * L, 3 * 64 * h)).astype(np.float32)
     qkv[:, :2 * 64 * h] *= unit
-    out = torch.full((B * L, 64 * h), float("nan"), dtype=torch.bfloat16, device="cuda")
-    ctx.attention_pwl(torch.from_numpy(qkv).cuda().bfloat16(), out, B, L, h, 64, scale=scale,
+    td, half_ulp = nm_inputs.torch_dtype(dtype), {"bf16": 2.0 ** -8, "f16": 2.0 ** -11}[dtype]
+    if dtype == "f16":
+        qkv[:, 2 * 64 * h:] /= 256   # (so that the outputs stay finite)
+    out = torch.full((B * L, 64 * h), float("nan"), dtype=td, device="cuda")
+    ctx.attention_pwl(torch.from_numpy(qkv).cuda().to(td), out, B, L, h, 64, scale=scale,
                       algo={"simt": nm.ALGO_SIMT, "auto": nm.ALGO_AUTO, "resident": nm.ALGO_ATTN_RESIDENT}[algo])
     ctx.check_device_status()
     ref, mag = scaled_scores(qkv, B, L, h, scale, tabs, two_roundings=L % 128 != 0)
-    # a rounding to bf16, 8 significant bits, is at most 2^-8 of the value: the output's, and at multiples of 128 the
-    # probabilities' as well; fp32 sums of L terms and of the row sum add 1e-5 of the terms' magnitudes
+    # a rounding to bf16, 8 significant bits, is at most 2^-8 of the value (fp16 2^-11): the output's, and at multiples of 128
+    # the probabilities' as well; fp32 sums of L terms and of the row sum add 1e-5 of the terms' magnitudes
     got = to_np(out)
     assert np.all(np.isfinite(got))
-    err, bound = np.abs(got - ref), 2.0 ** -8 * np.abs(ref) + (2.0 ** -8 if L % 128 == 0 else 0.0) * mag + 1e-5 * mag
+    err, bound = np.abs(got - ref), half_ulp * np.abs(ref) + (half_ulp if L % 128 == 0 and algo != "simt" else 0.0) * mag + 1e-5 * mag + 1e-7
     assert np.all(err <= bound), (err / bound).max()
 
 
