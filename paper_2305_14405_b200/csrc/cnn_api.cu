@@ -15,7 +15,7 @@ enum ConvPath {
     CONV_ROWTAP,    // Cin <= 8, kw <= 8 (an RGB first layer): implicit GEMM over a zero-padded 8-channel copy of the
                     // input, one K-block per filter row: 8 taps x 8 channels = 64 contiguous elements
     CONV_PAIRTAP,   // the same with stride 2 and Cin <= 4: image rows in pairs, a K-block is two filter rows of 8 taps x 4
-                    // channels (128 images of 224 x 224 x 3, 7 x 7: 279 us with one row per K-block, 179 so, copies included)
+                    // channels (128 images of 224 x 224 x 3, 7 x 7: 279 us with one row per K-block, 178 so, copies included)
     CONV_GATHER     // anything else: explicit gather (im2col) into the workspace, then the GEMM
 };
 
@@ -25,6 +25,7 @@ struct ConvGeom {
     ConvPath path;
     bool pad_w;       // CONV_GATHER: weights need their rows padded to Kpad
     int Hp, Wp;       // CONV_ROWTAP, CONV_PAIRTAP: extent of the padded input copy
+    int pair_rows;    // CONV_PAIRTAP: rows of it that are pairs
     size_t a_bytes, w_bytes;
 };
 
@@ -48,9 +49,12 @@ bool conv_geom(const nm_conv_desc* d, ConvGeom* g)
         g->path = CONV_IMPLICIT;
     } else if (d->Cin <= 4 && d->kw <= 8 && d->stride == 2 && d->algo != 1) {
         g->path = CONV_PAIRTAP;
-        // output row oy reads pair rows oy .. oy + pairs - 1, output pixel ox pixels 2 ox .. 2 ox + 7
+        // Output row oy reads pair rows oy .. oy + kh / 2 - 1, output pixel ox pixels 2 ox .. 2 ox + 7.  The last row of an odd
+        // kh is not read as half of a pair, whose other half lies below the window (0 * inf is NaN): it has a row of the copy to
+        // itself, with zeros beside it, behind the pair rows.
+        g->pair_rows = d->kh / 2 ? g->Ho - 1 + d->kh / 2 : 0;
+        g->Hp = g->pair_rows + (d->kh % 2 ? g->Ho : 0);
         const int pairs = (d->kh + 1) / 2;
-        g->Hp = g->Ho - 1 + pairs;
         g->Wp = (g->Wo - 1) * 2 + 8;
         g->a_bytes = align256((size_t)d->N * g->Hp * g->Wp * 8 * 2);
         g->w_bytes = align256((size_t)d->Cout * pairs * 64 * 2);
@@ -143,8 +147,8 @@ nm_status nm_conv2d_dispatch(nm_ctx* ctx, const nm_conv_desc* d, void* workspace
             void* xp = workspace;
             void* wp = (uint8_t*)workspace + g.a_bytes;
             const int pairs = (d->kh + 1) / 2;
-            const nm_status s = nm_launch_pad_pairs(ctx, d->x, xp, d->w, wp, d->dtype, d->N, d->H, d->W, d->Cin, d->pad, g.Hp, g.Wp,
-                                                    d->Cout, d->kh, d->kw, st);
+            const nm_status s = nm_launch_pad_pairs(ctx, d->x, xp, d->w, wp, d->dtype, d->N, d->H, d->W, d->Cin, d->pad, g.pair_rows,
+                                                    g.Hp, g.Wp, d->Cout, d->kh, d->kw, st);
             if (s != NM_OK) return s;
             c.a_base = xp;
             c.a_dim[0] = 64; c.a_dim[1] = (uint64_t)g.Wo; c.a_dim[2] = (uint64_t)g.Hp; c.a_dim[3] = (uint64_t)d->N;
@@ -153,6 +157,7 @@ nm_status nm_conv2d_dispatch(nm_ctx* ctx, const nm_conv_desc* d, void* workspace
             c.a_stride[2] = (uint64_t)g.Hp * g.Wp * 8 * 2;
             c.sw = c.sh = 1; c.pw = c.ph = 0;
             c.taps_y = pairs; c.taps_x = 1; c.cblocks = 1;
+            c.last_row_jump = d->kh % 2 ? g.pair_rows - d->kh / 2 : 0;
             c.w = wp; c.ldw = (int64_t)pairs * 64; c.Ktot = (int64_t)pairs * 64;
         } else {
             // the input with its border and five zero channels written out once (xp), the weights likewise (wp);

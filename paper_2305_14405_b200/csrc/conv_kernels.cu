@@ -138,12 +138,12 @@ __global__ void pad_weight_kernel(const T* __restrict__ w, T* __restrict__ wp, i
 }
 
 // The same for a stride-2 layer of at most four channels, two image rows to a row of the copy: x [N,H,W,Cin] ->
-// xp [N,Hp,Wp,2,4], pixel px of pair row r holding rows 2r - pad and 2r + 1 - pad of column px - pad.  Half the bytes of the
-// 8-channel copy, and a K-block of the convolution is two filter rows of 8 taps x 4 channels instead of one.  One thread
-// per 16-byte pixel pair.
+// xp [N,Hp,Wp,2,4], pixel px of pair row r holding rows 2r - pad and 2r + 1 - pad of column px - pad, and a K-block of the
+// convolution is two filter rows of 8 taps x 4 channels instead of one.  Behind the pair_rows pairs, where kh is odd: row r
+// holds row 2 (r - pair_rows) + kh - 1 - pad, an output row's last, and zeros.  One thread per 16-byte pixel pair.
 template <typename T>
 __global__ void __launch_bounds__(256) pad_input_pairs_kernel(const T* __restrict__ x, T* __restrict__ xp, int Nb, int H, int W,
-                                                              int Cin, int pad, int Hp, int Wp)
+                                                              int Cin, int pad, int kh, int pair_rows, int Hp, int Wp)
 {
     const int px = (int)(blockIdx.x * 256 + threadIdx.x);
     if (px >= Wp) return;
@@ -154,10 +154,12 @@ __global__ void __launch_bounds__(256) pad_input_pairs_kernel(const T* __restric
 #pragma unroll
             for (int c = 0; c < 8; ++c) v[c] = NmType<T>::from_f(0.f);
             if (ix >= 0 && ix < W) {
+                const bool single = r >= pair_rows;
+                const int iy0 = (single ? 2 * (r - pair_rows) + kh - 1 : 2 * r) - pad;
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
-                    const int iy = 2 * r + h - pad;
-                    if (iy < 0 || iy >= H) continue;
+                    const int iy = iy0 + h;
+                    if (iy < 0 || iy >= H || (h && single)) continue;
                     const T* src = x + (((int64_t)n * H + iy) * W + ix) * Cin;
 #pragma unroll
                     for (int c = 0; c < 4; ++c)
@@ -375,14 +377,14 @@ nm_status nm_launch_pad_weight(nm_ctx* ctx, const void* w, void* wp, nm_dtype dt
 }
 
 nm_status nm_launch_pad_pairs(nm_ctx* ctx, const void* x, void* xp, const void* w, void* wp, nm_dtype dt, int Nb, int H, int W,
-                              int Cin, int pad, int Hp, int Wp, int Cout, int kh, int kw, cudaStream_t st)
+                              int Cin, int pad, int pair_rows, int Hp, int Wp, int Cout, int kh, int kw, cudaStream_t st)
 {
     const dim3 grid((unsigned)((Wp + 255) / 256), (unsigned)(Hp < 65535 ? Hp : 65535), (unsigned)(Nb < 65535 ? Nb : 65535));
     const int64_t wtotal = (int64_t)Cout * ((kh + 1) / 2) * 64;
     {
         NmLaunchScope scope(ctx, NM_KERNEL_IM2COL, ((double)Nb * H * W * Cin + (double)Nb * Hp * Wp * 8) * nm_dtype_size(dt), st);
-        if (dt == NM_F16) pad_input_pairs_kernel<__half><<<grid, 256, 0, st>>>((const __half*)x, (__half*)xp, Nb, H, W, Cin, pad, Hp, Wp);
-        else pad_input_pairs_kernel<__nv_bfloat16><<<grid, 256, 0, st>>>((const __nv_bfloat16*)x, (__nv_bfloat16*)xp, Nb, H, W, Cin, pad, Hp, Wp);
+        if (dt == NM_F16) pad_input_pairs_kernel<__half><<<grid, 256, 0, st>>>((const __half*)x, (__half*)xp, Nb, H, W, Cin, pad, kh, pair_rows, Hp, Wp);
+        else pad_input_pairs_kernel<__nv_bfloat16><<<grid, 256, 0, st>>>((const __nv_bfloat16*)x, (__nv_bfloat16*)xp, Nb, H, W, Cin, pad, kh, pair_rows, Hp, Wp);
     }
     {
         NmLaunchScope scope(ctx, NM_KERNEL_IM2COL, (double)wtotal * 2.0 * nm_dtype_size(dt), st);

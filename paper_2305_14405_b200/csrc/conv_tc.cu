@@ -49,6 +49,7 @@ int64_t fill_args(nm_ctx* ctx, const NmConvTc* c, NmChain chain, TcArgs* a)
     cv.tiles_y = ceil_div(c->Ho, cv.TH);
     cv.sw = c->sw; cv.sh = c->sh; cv.pw = c->pw; cv.ph = c->ph;
     cv.kw_eff = c->taps_x; cv.cblocks = c->cblocks;
+    cv.ky_last = c->taps_y - 1; cv.ky_jump = c->last_row_jump;
     cv.Ho = c->Ho; cv.Nimg = c->N;
     cv.dw = c->depthwise;
     a->M = (int64_t)c->N * c->Ho * c->Wo; a->N = c->Cout; a->K = c->Ktot;

@@ -350,7 +350,7 @@ linear_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                 if constexpr (CONV) {
                     c_c = cb * BK_ELEMS;
                     c_w = pt.ox0 * a.cv.sw - a.cv.pw + kx;
-                    c_h = pt.oy0 * a.cv.sh - a.cv.ph + ky;
+                    c_h = pt.oy0 * a.cv.sh - a.cv.ph + ky + (ky == a.cv.ky_last ? a.cv.ky_jump : 0);
                     if (a.cv.dw) {   // pooling: channel block = column tile, one constant matrix for every tap and tile
                         c_c = nt * BK_ELEMS;
                         w_k = 0;

@@ -64,6 +64,7 @@ struct ConvDev {
     int sw, sh, pw, ph;     // tap (ky, kx) of output pixel (oy, ox) reads input (oy*sh - ph + ky, ox*sw - pw + kx)
     int kw_eff, cblocks;    // K-block kb = (ky*kw_eff + kx)*cblocks + cb; 64 channels per block
     int Ho, Nimg;           // output rows per image, images
+    int ky_last, ky_jump;   // the last filter row's input lies ky_jump rows further down (first layer, see conv_geom)
     int dw;                 // nonzero: "depthwise" form for pooling as a GEMM: column tile nt (64 channels) reads channel
                             // block nt of the activation at every tap and multiplies by ONE constant 64 x 64 matrix
 };
@@ -352,7 +353,7 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                         if constexpr (CONV) {
                             c_c = cb * BK_ELEMS;
                             c_w = pt.ox0 * a.cv.sw - a.cv.pw + kx;
-                            c_h = pt.oy0 * a.cv.sh - a.cv.ph + ky;
+                            c_h = pt.oy0 * a.cv.sh - a.cv.ph + ky + (ky == a.cv.ky_last ? a.cv.ky_jump : 0);
                             if (a.cv.dw) {   // pooling: channel block = column tile, one constant matrix for every tap and tile
                                 c_c = (tile % a.num_n_tiles) * BK_ELEMS;
                                 w_k = 0;

@@ -710,7 +710,8 @@ nm_status nm_launch_attention_i8(nm_ctx* ctx, const nm_attn_i8_desc* d, cudaStre
 // Implicit-GEMM convolution on the tensor-core kernel.  The A operand is described as a 4-D view
 // {inner, x, y, image} of the activation (dims in elements, strides in bytes); K-block
 // kb = (ky*taps_x + kx)*cblocks + cb reads the 64 inner elements cb*64.. at x = ox*sw - pw + kx,
-// y = oy*sh - ph + ky for every output pixel (oy, ox) of the tile; W is [Cout, Ktot] with row pitch ldw.
+// y = oy*sh - ph + ky for every output pixel (oy, ox) of the tile (for the last ky last_row_jump further down); W is
+// [Cout, Ktot] with row pitch ldw.
 struct NmConvTc {
     nm_dtype dtype;
     const void* a_base;
@@ -718,6 +719,7 @@ struct NmConvTc {
     uint64_t a_stride[3];
     int sw, sh, pw, ph;
     int taps_y, taps_x, cblocks;
+    int last_row_jump;
     const void* w;
     int64_t ldw, Ktot;
     int N, Ho, Wo, Cout;
@@ -736,9 +738,10 @@ nm_status nm_launch_pad_input(nm_ctx* ctx, const void* x, void* xp, nm_dtype dt,
                               int Hp, int Wp, cudaStream_t st);
 nm_status nm_launch_pad_weight(nm_ctx* ctx, const void* w, void* wp, nm_dtype dt, int Cout, int kh, int kw, int Cin,
                                cudaStream_t st);
-// the same for a stride-2 layer of at most 4 channels, rows in pairs: xp [N,Hp,Wp,2,4], wp [Cout,(kh+1)/2,8,2,4]
+// the same for a stride-2 layer of at most 4 channels, rows in pairs: xp [N,Hp,Wp,2,4] of pair_rows pairs and, behind them, an
+// odd kh's last filter row with zeros beside it, wp [Cout,(kh+1)/2,8,2,4]
 nm_status nm_launch_pad_pairs(nm_ctx* ctx, const void* x, void* xp, const void* w, void* wp, nm_dtype dt, int Nb, int H, int W,
-                              int Cin, int pad, int Hp, int Wp, int Cout, int kh, int kw, cudaStream_t st);
+                              int Cin, int pad, int pair_rows, int Hp, int Wp, int Cout, int kh, int kw, cudaStream_t st);
 nm_status nm_launch_im2col(nm_ctx* ctx, const void* x, void* A, nm_dtype dt, int Nb, int H, int W, int Cin, int kh,
                            int kw, int stride, int pad, int Ho, int Wo, int Kpad, cudaStream_t st);
 nm_status nm_launch_pad_rows(nm_ctx* ctx, const void* w, void* wp, nm_dtype dt, int rows, int K, int Kpad,

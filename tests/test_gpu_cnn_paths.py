@@ -50,6 +50,25 @@ def test_first_layer_row_pairs(nm, ctx, dtype, N, H, W, Cin, Cout, kh, kw, pad):
     conv_both(nm, ctx, x, w, b, 2, pad)
 
 
+@pytest.mark.parametrize("N,H,W,Cin,Cout,kh,kw,pad", [(2, 32, 24, 3, 64, 7, 7, 3), (1, 33, 20, 3, 16, 3, 3, 1), (2, 31, 17, 4, 8, 5, 8, 2),
+                                                      (1, 20, 20, 3, 8, 1, 1, 0), (1, 30, 30, 3, 24, 4, 7, 1), (70, 32, 32, 3, 64, 7, 7, 3)])
+def test_first_layer_reads_no_row_outside_the_window(nm, ctx, N, H, W, Cin, Cout, kh, kw, pad):
+    """Rows of NaN and infinities reach the outputs whose window holds them and no others."""
+    x, w, b, _ = operands(N, H, W, Cin, Cout, kh, kw, torch.float16, H)
+    Ho, Wo = (H + 2 * pad - kh) // 2 + 1, (W + 2 * pad - kw) // 2 + 1
+    for rows in ([H // 2], [H // 2 + 1], [0, H - 1], [3]):
+        xr = x.clone()
+        xr[:, rows] = float("nan")
+        xr[0, rows] = float("inf")
+        out = torch.zeros((N, Ho, Wo, Cout), device="cuda").half()
+        d = ctx.conv_desc(xr, w, out, 2, pad, bias=b, slot=nm.SLOT_NONE)
+        ctx.conv2d_pwl(d, torch.empty(max(256, ctx.conv2d_workspace_bytes(d)), dtype=torch.uint8, device="cuda"))
+        ctx.check_device_status()
+        holds = [any(2 * oy - pad <= r < 2 * oy - pad + kh for r in rows) for oy in range(Ho)]
+        finite = torch.isfinite(out).all(3).all(2).all(0).tolist()
+        assert [not f for f in finite] == holds, (rows, finite, holds)
+
+
 @pytest.mark.parametrize("dtype", [torch.float16, torch.bfloat16])
 @pytest.mark.parametrize("N,H,W,Cin,Cout,res", [(30, 56, 56, 64, 64, False), (85, 28, 28, 128, 128, False), (150, 24, 20, 64, 40, True),
                                                 (75, 33, 31, 128, 72, True), (41, 50, 40, 192, 128, False), (199, 32, 18, 64, 64, True)])
