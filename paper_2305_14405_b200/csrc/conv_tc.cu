@@ -146,6 +146,7 @@ nm_status launch_split(nm_ctx* ctx, const NmConvTc* c, int S, NmChain chain, cud
     const int64_t patches = fill_args(ctx, c, chain, &s.t);
     s.t.num_n_tiles = ceil_div(c->Cout, BN);
     const int64_t tiles = patches * s.t.num_n_tiles;
+    if (tiles > 0x7fffffffLL / S) return NM_ERR_SHAPE;
     s.S = S;
     s.t.num_tiles = (int)tiles;
     s.residual = c->residual; s.ldr = c->Cout;
@@ -196,7 +197,8 @@ nm_status launch_sel(nm_ctx* ctx, const NmConvTc* c, NmChain chain, cudaStream_t
             const nm_status e = c->Cout <= 64 ? launch_halo<T, 64>(ctx, c, chain, st) : launch_halo<T, 128>(ctx, c, chain, st);
             if (e != NM_ERR_UNSUPPORTED) return e;
         }
-        t = choose_tile((int64_t)c->N * c->Ho * c->Wo, patches, c->Cout, (int64_t)c->taps_y * c->taps_x * c->cblocks, true, c->slot != NM_SLOT_NONE,
+        t = choose_tile((int64_t)c->N * c->Ho * c->Wo, patches, c->Cout, (int64_t)c->taps_y * c->taps_x * c->cblocks, true,
+                        EpiNeeds{c->slot == NM_SLOT_NONE ? 0 : ctx->h_tables[c->slot].n, c->residual != nullptr, c->bias != nullptr},
                         c->depthwise != 0, true, chain, ctx->sm_count);
     } else {
         t.S = 0;

@@ -510,21 +510,23 @@ inline int split_stages(int BN, int S, int64_t ctas, int sms, bool back_to_back)
     return BN == 64 ? (split_alone(S, ctas, sms) ? 5 : 3) : (split_alone(S, ctas, sms) ? 6 : 4);
 }
 
-inline TileChoice choose_tile(int64_t rows, int64_t m_tiles, int64_t N, int64_t k_blocks, bool narrow_tiles, bool has_table, bool only64,
+inline TileChoice choose_tile(int64_t rows, int64_t m_tiles, int64_t N, int64_t k_blocks, bool narrow_tiles, const EpiNeeds& epi, bool only64,
                               bool whole_chunks, NmChain chain, int sms)
 {
+    const bool has_table = epi.n_seg > 0;
     struct P { int BN; bool two; double base, kb, round; };
     static const P apart[6] = {{256, true, 5.56, 0.420, 4.4}, {256, false, 4.72, 0.461, 4.8}, {128, true, 4.07, 0.233, 1.8},
                                {128, false, 2.94, 0.315, 1.95}, {64, true, 3.19, 0.251, 1.15}, {64, false, 3.00, 0.218, 1.25}};
     static const P joined[6] = {{256, true, 4.9, 0.386, 3.6}, {256, false, 5.4, 0.43, 3.6}, {128, true, 4.5, 0.26, 1.8},
                                 {128, false, 3.9, 0.322, 1.8}, {64, true, 3.9, 0.26, 0.9}, {64, false, 3.5, 0.30, 0.9}};
     const bool in_cnn = chain.back_to_back;
-    TileChoice best = {0, 0, false};
+    TileChoice best = {1, 64, false};   // the split kernel takes anything
     double best_t = 1e30;
     for (int i = 0; i < 6; ++i) {
         const P& p = in_cnn ? joined[i] : apart[i];
         if (!whole_chunks || (!narrow_tiles && p.BN != 256) || (only64 && p.BN != 64) || (p.two && m_tiles < 2)) continue;
         if (narrow_tiles && p.BN > 64 && N <= p.BN / 2) continue;   // half the tile would be padding
+        if (ring_stages(p.BN, p.two, epi) < 2) continue;            // no room beside a large table
         const int64_t tiles = (p.two ? (m_tiles + 1) / 2 : m_tiles) * ((N + p.BN - 1) / p.BN), slots = p.two ? sms / 2 : sms;
         const int64_t rounds = (tiles + slots - 1) / slots;
         const double share = tiles < slots ? (double)tiles / slots : 1.0;

@@ -63,6 +63,7 @@ nm_status launch_split(nm_ctx* ctx, const nm_linear_desc* d, int S, NmChain chai
     const int64_t k_blocks = (d->K + bk - 1) / bk, n_tiles = (d->N + BN - 1) / BN, tiles = (d->M + BM - 1) / BM * n_tiles;
     SplitArgs s;
     memset(&s, 0, sizeof(s));
+    if (tiles > 0x7fffffffLL / S) return NM_ERR_SHAPE;
     s.S = S;
     fill_args(ctx, d, chain, &s.t);
     s.t.num_n_tiles = (int)n_tiles;
@@ -84,9 +85,10 @@ nm_status launch_sel(nm_ctx* ctx, const nm_linear_desc* d, NmChain chain, cudaSt
     constexpr bool NARROW = !TcIn<InT>::is_int;   // tiles of 64 and 128 columns are built for the 16-bit types
     const int bk = ROW_BYTES / (int)sizeof(InT);
     const int64_t m_tiles = (d->M + BM - 1) / BM, k_blocks = (d->K + bk - 1) / bk;
+    const int n_seg = d->slot == NM_SLOT_NONE ? 0 : ctx->h_tables[d->slot].n;
     TileChoice c;
-    if (d->algo == 0) c = choose_tile(d->M, m_tiles, d->N, k_blocks, NARROW, d->slot != NM_SLOT_NONE, false, d->N * sizeof(OutT) % 16 == 0, chain,
-                                      ctx->sm_count);
+    if (d->algo == 0) c = choose_tile(d->M, m_tiles, d->N, k_blocks, NARROW, EpiNeeds{n_seg, d->residual != nullptr, d->bias != nullptr || TcIn<InT>::is_int}, false,
+                                      d->N * sizeof(OutT) % 16 == 0, chain, ctx->sm_count);
     else {
         // a forced kernel: by width alone; algo 3 asks for one CTA per tile, otherwise CTA pairs from one 256-row tile on
         c.S = 0;

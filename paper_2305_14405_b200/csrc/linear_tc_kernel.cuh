@@ -763,21 +763,34 @@ inline nm_status make_tmap(nm_ctx* ctx, CUtensorMap* m, const void* base, nm_dty
     return r == CUDA_SUCCESS ? NM_OK : NM_ERR_CUDA;
 }
 
+// What an epilogue keeps in shared memory beside the operand ring: a replicated table of n_seg segments, the staged output
+// and residual, the column vectors (bias, scales).
+struct EpiNeeds {
+    int n_seg;
+    bool res, vec;
+    size_t bytes() const
+    {
+        return (size_t)n_seg * 32 * sizeof(float2) + (size_t)NUM_EPI_WARPS * STAGE_BUF * (res ? 2 : 1) +
+               (vec ? (size_t)NUM_EPI_WARPS * 256 * sizeof(float) : 0);
+    }
+};
+constexpr int stage_bytes(int BN, bool two) { return A_BYTES + (two ? BN / 2 : BN) * ROW_BYTES; }
+// Ring stages of the persistent kernel that fit beside the epilogue (with 256 segments, a residual and a bias one of the one-CTA
+// 256-column tile, where two are needed, and two of the pair's).
+inline int ring_stages(int BN, bool two, const EpiNeeds& e)
+{
+    const int stages = (int)((227 * 1024 - 1024 /*alignment slack*/ - 1024 /*static*/ - e.bytes()) / stage_bytes(BN, two));
+    return stages > MAX_STAGES ? MAX_STAGES : stages;
+}
+
 // Shared-memory bytes and stage count of one launch; false if the kernel cannot run with this table size.
 template <typename InT, bool TWO, int BN>
 inline bool plan_smem(TcArgs* a, bool has_vec, size_t* smem_out)
 {
-    constexpr int B_ROWS = TWO ? BN / 2 : BN;
-    constexpr int STAGE_BYTES = A_BYTES + B_ROWS * ROW_BYTES;
-    const size_t table_bytes = (size_t)a->n_seg * 32 * sizeof(float2);
-    const size_t vec_bytes = has_vec ? (size_t)NUM_EPI_WARPS * 256 * sizeof(float) : 0;
-    const size_t staging = (size_t)NUM_EPI_WARPS * STAGE_BUF * (a->has_res ? 2 : 1) + vec_bytes;
-    const size_t budget = 227 * 1024 - 1024 /*alignment slack*/ - 1024 /*static*/ - table_bytes - staging;
-    int stages = (int)(budget / STAGE_BYTES);
-    if (stages > MAX_STAGES) stages = MAX_STAGES;
-    if (stages < 2) return false;
-    a->stages = stages;
-    *smem_out = (size_t)stages * STAGE_BYTES + staging + table_bytes + 1024;
+    const EpiNeeds e = {a->n_seg, a->has_res != 0, has_vec};
+    a->stages = ring_stages(BN, TWO, e);
+    if (a->stages < 2) return false;
+    *smem_out = (size_t)a->stages * stage_bytes(BN, TWO) + e.bytes() + 1024;
     return true;
 }
 

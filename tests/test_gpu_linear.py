@@ -143,3 +143,36 @@ def test_linear_argument_errors(nm, ctx):
     assert ei.value.code == 3
     e = torch.zeros(0, 64, dtype=torch.bfloat16, device="cuda")
     ctx.linear_pwl(e, A, torch.zeros(0, 64, dtype=torch.bfloat16, device="cuda"))   # empty: no-op
+
+
+@pytest.mark.parametrize("dtype,M,N,K", [("bf16", 8192, 1024, 256), ("f16", 4096, 2048, 256), ("bf16", 300, 512, 128), ("bf16", 100, 4096, 512)])
+def test_large_table_with_residual_and_bias(nm, ctx, dtype, M, N, K):
+    """256 segments, a residual and a bias leave room for one operand stage of the widest one-CTA tile: another is taken."""
+    tabs = load_tables_both(ctx, 256, RANGES)
+    td = nm_inputs.torch_dtype(dtype)
+    A, W = nm_inputs.matrix((M, K), 1, dtype, 1.0), nm_inputs.matrix((N, K), 2, dtype, 0.05)
+    rng = np.random.default_rng(3)
+    bias = (0.1 * rng.standard_normal(N)).astype(np.float32)
+    res = nm_inputs.round_to(rng.standard_normal((M, N)).astype(np.float32), dtype)
+    out = torch.full((M, N), float("nan"), dtype=td, device="cuda")
+    ctx.linear_pwl(torch.from_numpy(A).cuda().to(td), torch.from_numpy(W).cuda().to(td), out, bias=torch.from_numpy(bias).cuda(),
+                   residual=torch.from_numpy(res).cuda().to(td), slot=nm.SLOT_GELU)
+    ctx.check_device_status()
+    assert_close_bf16(to_np(out), oracle.linear(A, W, bias, res, tabs["gelu"]), "linear, 256 segments")
+
+
+@pytest.mark.parametrize("M,N,K", [(512, 4096, 128), (2048, 2048, 128), (200, 1024, 256)])
+def test_int8_large_table_with_residual_and_bias(nm, ctx, M, N, K):
+    tabs = load_tables_both(ctx, 256, RANGES)
+    Aq, Wq = nm_inputs.int8_matrix((M, K), 21), nm_inputs.int8_matrix((N, K), 22)
+    rng = np.random.default_rng(23)
+    ws = (rng.uniform(0.5, 1.5, N) * 0.08 / 127).astype(np.float32)
+    bias = (0.1 * rng.standard_normal(N)).astype(np.float32)
+    res = rng.standard_normal((M, N)).astype(np.float32)
+    out = torch.full((M, N), float("nan"), device="cuda")
+    ctx.linear_pwl(torch.from_numpy(Aq).cuda(), torch.from_numpy(Wq).cuda(), out, bias=torch.from_numpy(bias).cuda(),
+                   residual=torch.from_numpy(res).cuda(), slot=nm.SLOT_GELU, a_scale=float(np.float32(4.0 / 127)),
+                   w_scale=torch.from_numpy(ws).cuda())
+    ctx.check_device_status()
+    r = oracle.linear_i8(Aq, Wq, np.float32(4.0 / 127), ws, bias, res, tabs["gelu"])
+    assert np.array_equal(out.cpu().numpy().view(np.uint32), r["y"].view(np.uint32))
