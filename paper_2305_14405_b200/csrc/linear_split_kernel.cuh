@@ -223,7 +223,7 @@ struct Finisher {
                 }
                 if constexpr (INT) {
                     if (a.acc_dump)
-                        *reinterpret_cast<int4*>(a.acc_dump + grow * a.N + col) =
+                        *reinterpret_cast<int4*>(a.acc_dump + grow * a.ldd + col) =
                             make_int4((int)acc[u][0], (int)acc[u][1], (int)acc[u][2], (int)acc[u][3]);
                 }
                 float4 rv = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -238,7 +238,7 @@ struct Finisher {
                         x[i] = __fmaf_rn(t.x, x[i], t.y);
                     }
                 }
-                if (a.idx_dump) *reinterpret_cast<int4*>(a.idx_dump + grow * a.N + col) = make_int4(seg[0], seg[1], seg[2], seg[3]);
+                if (a.idx_dump) *reinterpret_cast<int4*>(a.idx_dump + grow * a.ldd + col) = make_int4(seg[0], seg[1], seg[2], seg[3]);
                 if (s.residual && !a.res_first) { x[0] += rv.x; x[1] += rv.y; x[2] += rv.z; x[3] += rv.w; }
                 Quad<OutT>::store(reinterpret_cast<OutT*>(s.out) + grow * s.ldo + col, make_float4(x[0], x[1], x[2], x[3]), a.inv_out_scale);
             }
@@ -494,6 +494,7 @@ struct TileChoice {
     int S;      // CTAs per cluster of the split kernel; 0: the persistent kernel
     int BN;
     bool two;   // persistent kernel: CTA pairs
+    double us;  // by the model
 };
 
 // A cluster's CTAs share a GPC, so not every SM is in one: the CTAs, in clusters of S, that certainly find an SM each.
@@ -520,8 +521,7 @@ inline TileChoice choose_tile(int64_t rows, int64_t m_tiles, int64_t N, int64_t 
     static const P joined[6] = {{256, true, 4.9, 0.386, 3.6}, {256, false, 5.4, 0.43, 3.6}, {128, true, 4.5, 0.26, 1.8},
                                 {128, false, 3.9, 0.322, 1.8}, {64, true, 3.9, 0.26, 0.9}, {64, false, 3.5, 0.30, 0.9}};
     const bool in_cnn = chain.back_to_back;
-    TileChoice best = {1, 64, false};   // the split kernel takes anything
-    double best_t = 1e30;
+    TileChoice best = {1, 64, false, 1e30};   // the split kernel takes anything
     for (int i = 0; i < 6; ++i) {
         const P& p = in_cnn ? joined[i] : apart[i];
         if (!whole_chunks || (!narrow_tiles && p.BN != 256) || (only64 && p.BN != 64) || (p.two && m_tiles < 2)) continue;
@@ -535,7 +535,7 @@ inline TileChoice choose_tile(int64_t rows, int64_t m_tiles, int64_t N, int64_t 
         if ((in_cnn || rounds > 2) && loop < p.round) loop = p.round;
         const double t = p.base + (double)rounds * loop + (in_cnn ? 0.0 : (chain.weights_ready ? 0.4 : 0.0) + 0.32 * share * p.BN / 64) +
                          (has_table ? (in_cnn ? 1.8 : 1.5) * p.BN / 256 : 0.0);
-        if (t < best_t * (in_cnn ? 0.97 : 1.0)) { best_t = t; best = {0, p.BN, p.two}; }
+        if (t < best.us * (in_cnn ? 0.97 : 1.0)) best = {0, p.BN, p.two, t};
     }
     const double tile_rows = (rows < BM ? (double)rows : (double)BM) / BM;
     for (int BN = 64; BN >= (only64 ? 64 : 32); BN /= 2) {
@@ -548,7 +548,7 @@ inline TileChoice choose_tile(int64_t rows, int64_t m_tiles, int64_t N, int64_t 
                              (BN == 64 ? 0.235 : 0.179) * (beyond > 0 ? beyond : 0) * (share > 1 ? share : 1) +
                              (S == 1 ? 0.0 : S == 2 ? 0.21 : S == 4 ? 0.26 : 0.56) +
                              (0.35 * (share < 1 ? share : 1) + 0.85 * (share > 1 ? share - 1 : 0)) * BN / 32 + (has_table ? 0.42 * BN / 64 : 0.0);
-            if (t < best_t * (in_cnn || best.S ? 0.97 : 1.0)) { best_t = t; best = {S, BN, false}; }
+            if (t < best.us * (in_cnn || best.S ? 0.97 : 1.0)) best = {S, BN, false, t};
         }
     }
     return best;

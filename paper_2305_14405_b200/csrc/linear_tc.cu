@@ -6,7 +6,7 @@ using namespace nm_tc;
 
 namespace {
 
-void fill_args(nm_ctx* ctx, const nm_linear_desc* d, NmChain chain, TcArgs* a)
+void fill_args(nm_ctx* ctx, const nm_linear_desc* d, int64_t ldd, NmChain chain, TcArgs* a)
 {
     memset(a, 0, sizeof(*a));
     a->M = d->M; a->N = d->N; a->K = d->K;
@@ -16,19 +16,19 @@ void fill_args(nm_ctx* ctx, const nm_linear_desc* d, NmChain chain, TcArgs* a)
     a->tab = d->slot == NM_SLOT_NONE ? nullptr : ctx->d_tables + d->slot;
     a->n_seg = d->slot == NM_SLOT_NONE ? 0 : ctx->h_tables[d->slot].n;
     a->a_scale = d->a_scale; a->w_scale = d->w_scale; a->inv_out_scale = d->inv_out_scale;
-    a->acc_dump = d->acc_dump; a->idx_dump = d->idx_dump;
+    a->acc_dump = d->acc_dump; a->idx_dump = d->idx_dump; a->ldd = ldd;
     a->status = ctx->d_status;
     a->weights_ready = chain.weights_ready;
     a->late_trigger = chain.late_trigger;
 }
 
 template <typename InT, typename OutT, bool TWO, int BN>
-nm_status launch(nm_ctx* ctx, const nm_linear_desc* d, NmChain chain, cudaStream_t st)
+nm_status launch(nm_ctx* ctx, const nm_linear_desc* d, int64_t ldd, NmChain chain, cudaStream_t st)
 {
     constexpr int B_ROWS = TWO ? BN / 2 : BN;
     constexpr int TILE_M = TWO ? 2 * BM : BM;
     TcArgs a;
-    fill_args(ctx, d, chain, &a);
+    fill_args(ctx, d, ldd, chain, &a);
     const int bk = ROW_BYTES / (int)sizeof(InT);
     const int64_t m_tiles = (d->M + TILE_M - 1) / TILE_M;
     a.num_n_tiles = (int)((d->N + BN - 1) / BN);
@@ -57,7 +57,7 @@ nm_status launch(nm_ctx* ctx, const nm_linear_desc* d, NmChain chain, cudaStream
 }
 
 template <typename InT, typename OutT, int BN>
-nm_status launch_split(nm_ctx* ctx, const nm_linear_desc* d, int S, NmChain chain, cudaStream_t st)
+nm_status launch_split(nm_ctx* ctx, const nm_linear_desc* d, int64_t ldd, int S, NmChain chain, cudaStream_t st)
 {
     const int bk = ROW_BYTES / (int)sizeof(InT);
     const int64_t k_blocks = (d->K + bk - 1) / bk, n_tiles = (d->N + BN - 1) / BN, tiles = (d->M + BM - 1) / BM * n_tiles;
@@ -65,7 +65,7 @@ nm_status launch_split(nm_ctx* ctx, const nm_linear_desc* d, int S, NmChain chai
     memset(&s, 0, sizeof(s));
     if (tiles > 0x7fffffffLL / S) return NM_ERR_SHAPE;
     s.S = S;
-    fill_args(ctx, d, chain, &s.t);
+    fill_args(ctx, d, ldd, chain, &s.t);
     s.t.num_n_tiles = (int)n_tiles;
     s.t.num_tiles = (int)tiles;
     s.t.num_k_blocks = (int)k_blocks;
@@ -79,28 +79,56 @@ nm_status launch_split(nm_ctx* ctx, const nm_linear_desc* d, int S, NmChain chai
     return launch_split_kernel<InT, OutT, BN, false>(ctx, tmA, tmW, s, chain.back_to_back, 2.0 * (double)d->M * (double)d->N * (double)d->K, st);
 }
 
+// Kernel and tile for d: the cheapest by the model, or (algo 2, 3) a forced one: the persistent kernel with a tile by the width
+// alone; algo 3 asks for one CTA per tile, otherwise CTA pairs from one 256-row tile on.
+template <typename InT, typename OutT>
+TileChoice choose(nm_ctx* ctx, const nm_linear_desc* d, NmChain chain)
+{
+    constexpr bool NARROW = !TcIn<InT>::is_int;   // tiles of 64 and 128 columns are built for the 16-bit types
+    const bool whole_chunks = d->N * sizeof(OutT) % 16 == 0;
+    if (d->algo != 0 && whole_chunks)
+        return {0, NARROW && d->N <= 64 ? 64 : (NARROW && d->N <= 128 ? 128 : 256), d->algo != 3 && d->M >= 256, 0.0};
+    const int bk = ROW_BYTES / (int)sizeof(InT);
+    const EpiNeeds epi = {d->slot == NM_SLOT_NONE ? 0 : ctx->h_tables[d->slot].n, d->residual != nullptr, d->bias != nullptr || TcIn<InT>::is_int};
+    return choose_tile(d->M, (d->M + BM - 1) / BM, d->N, (d->K + bk - 1) / bk, NARROW, epi, false, whole_chunks, chain, ctx->sm_count);
+}
+
+// ldd: row pitch of the dumps
+template <typename InT, typename OutT>
+nm_status launch_choice(nm_ctx* ctx, const nm_linear_desc* d, const TileChoice& c, int64_t ldd, NmChain chain, cudaStream_t st)
+{
+    if (c.S) return c.BN == 32 ? launch_split<InT, OutT, 32>(ctx, d, ldd, c.S, chain, st) : launch_split<InT, OutT, 64>(ctx, d, ldd, c.S, chain, st);
+    if constexpr (!TcIn<InT>::is_int) {
+        if (c.BN == 64) return c.two ? launch<InT, OutT, true, 64>(ctx, d, ldd, chain, st) : launch<InT, OutT, false, 64>(ctx, d, ldd, chain, st);
+        if (c.BN == 128) return c.two ? launch<InT, OutT, true, 128>(ctx, d, ldd, chain, st) : launch<InT, OutT, false, 128>(ctx, d, ldd, chain, st);
+    }
+    return c.two ? launch<InT, OutT, true, 256>(ctx, d, ldd, chain, st) : launch<InT, OutT, false, 256>(ctx, d, ldd, chain, st);
+}
+
 template <typename InT, typename OutT>
 nm_status launch_sel(nm_ctx* ctx, const nm_linear_desc* d, NmChain chain, cudaStream_t st)
 {
-    constexpr bool NARROW = !TcIn<InT>::is_int;   // tiles of 64 and 128 columns are built for the 16-bit types
-    const int bk = ROW_BYTES / (int)sizeof(InT);
-    const int64_t m_tiles = (d->M + BM - 1) / BM, k_blocks = (d->K + bk - 1) / bk;
-    const int n_seg = d->slot == NM_SLOT_NONE ? 0 : ctx->h_tables[d->slot].n;
-    TileChoice c;
-    if (d->algo == 0) c = choose_tile(d->M, m_tiles, d->N, k_blocks, NARROW, EpiNeeds{n_seg, d->residual != nullptr, d->bias != nullptr || TcIn<InT>::is_int}, false,
-                                      d->N * sizeof(OutT) % 16 == 0, chain, ctx->sm_count);
-    else {
-        // a forced kernel: by width alone; algo 3 asks for one CTA per tile, otherwise CTA pairs from one 256-row tile on
-        c.S = 0;
-        c.BN = NARROW && d->N <= 64 ? 64 : (NARROW && d->N <= 128 ? 128 : 256);
-        c.two = d->algo != 3 && d->M >= 256;
-    }
-    if (c.S) return c.BN == 32 ? launch_split<InT, OutT, 32>(ctx, d, c.S, chain, st) : launch_split<InT, OutT, 64>(ctx, d, c.S, chain, st);
-    if constexpr (NARROW) {
-        if (c.BN == 64) return c.two ? launch<InT, OutT, true, 64>(ctx, d, chain, st) : launch<InT, OutT, false, 64>(ctx, d, chain, st);
-        if (c.BN == 128) return c.two ? launch<InT, OutT, true, 128>(ctx, d, chain, st) : launch<InT, OutT, false, 128>(ctx, d, chain, st);
-    }
-    return c.two ? launch<InT, OutT, true, 256>(ctx, d, chain, st) : launch<InT, OutT, false, 256>(ctx, d, chain, st);
+    constexpr int64_t CHUNK = 16 / sizeof(OutT);
+    const TileChoice c = choose<InT, OutT>(ctx, d, chain);
+    const int64_t main_n = d->N / CHUNK * CHUNK;
+    if (main_n == d->N || main_n < 8) return launch_choice<InT, OutT>(ctx, d, c, d->N, chain, st);
+    // A row that is no multiple of 16 bytes: all of it by the split kernel, or the last 4 to 12 columns by the split kernel and the
+    // others by themselves, whichever the model finds cheaper (16384 x 1004 x 1024: 61 us and 36).
+    nm_linear_desc m = *d, r = *d;
+    m.N = main_n;
+    r.N = d->N - main_n;
+    r.W = (const uint8_t*)d->W + main_n * d->ldw * sizeof(InT);
+    r.out = (uint8_t*)d->out + main_n * sizeof(OutT);
+    if (d->residual) r.residual = (const uint8_t*)d->residual + main_n * sizeof(OutT);
+    if (d->bias) r.bias = d->bias + main_n;
+    if (d->w_scale) r.w_scale = d->w_scale + main_n;
+    if (d->acc_dump) r.acc_dump = d->acc_dump + main_n;
+    if (d->idx_dump) r.idx_dump = d->idx_dump + main_n;
+    const TileChoice cm = choose<InT, OutT>(ctx, &m, chain), cr = choose<InT, OutT>(ctx, &r, chain);
+    if (d->algo == 0 && c.us <= cm.us + cr.us) return launch_choice<InT, OutT>(ctx, d, c, d->N, chain, st);
+    const nm_status e = launch_choice<InT, OutT>(ctx, &m, cm, d->N, chain, st);
+    if (e != NM_OK) return e;
+    return launch_choice<InT, OutT>(ctx, &r, cr, d->N, chain, st);
 }
 
 }  // namespace

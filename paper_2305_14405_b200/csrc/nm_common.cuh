@@ -303,8 +303,8 @@ __device__ __forceinline__ void nm_tma_prefetch_2d(const CUtensorMap* tmap, int 
     asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global [%0, {%1, %2}];" ::"l"(tmap), "r"(c0), "r"(c1) : "memory");
 }
 
-// TMA: 2-D tiled store shared -> global as one bulk group; parts of the box beyond the
-// tensor's extents are not written.  c0 (innermost) must be a multiple of 16 bytes.
+// TMA: 2-D tiled store shared -> global as one bulk group; parts of the box beyond the tensor's extents are not written,
+// except that a row is written in whole 16-byte chunks.  c0 (innermost) must be a multiple of 16 bytes.
 __device__ __forceinline__ void nm_tma_store_2d(const CUtensorMap* tmap, const void* smem_src, int c0, int c1)
 {
     asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%2, %3}], [%1];" ::"l"(tmap),

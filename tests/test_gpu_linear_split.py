@@ -34,7 +34,7 @@ SHAPES = [(1, 8, 8), (1, 768, 768), (31, 64, 72), (33, 68, 128), (37, 2304, 768)
 @pytest.mark.parametrize("dtype", ["bf16", "f16"])
 @pytest.mark.parametrize("M,N,K", SHAPES)
 @pytest.mark.parametrize("epi", ["plain", "gelu_bias", "bias_res", "relu_res_first"])
-def test_16_bit(nm, ctx, dtype, M, N, K, epi):
+def test_16_bit(nm, ctx, dtype, M, N, K, epi, algo=0):
     tabs = load_tables_both(ctx, 64, RANGES)
     td = nm_inputs.torch_dtype(dtype)
     A, W = nm_inputs.matrix((M, K), M + K, dtype, 1.0), nm_inputs.matrix((N, K), N, dtype, 0.05)
@@ -45,7 +45,7 @@ def test_16_bit(nm, ctx, dtype, M, N, K, epi):
     first = epi == "relu_res_first"
     pad = 8 if (M + N) % 2 else 0
     out = torch.full((M, N + 8 - N % 8 + pad), float("nan"), dtype=td, device="cuda")
-    ctx.linear_pwl(strided(A, td, pad + 8 - K % 8), strided(W, td, 8 - K % 8), out[:, :N], slot=slot, res_first=first,
+    ctx.linear_pwl(strided(A, td, pad + 8 - K % 8), strided(W, td, 8 - K % 8), out[:, :N], slot=slot, res_first=first, algo=algo,
                    bias=None if bias is None else torch.from_numpy(bias).cuda(),
                    residual=None if res is None else strided(res, td, 8 - N % 8 + pad))
     ctx.check_device_status()
@@ -66,9 +66,22 @@ def test_16_bit(nm, ctx, dtype, M, N, K, epi):
     assert np.all(np.abs(got - ref) <= half_ulp * 1.01 * np.abs(ref) + 1e-5 * max(rms, 1.0)), np.abs(got - ref).max()
 
 
+@pytest.mark.parametrize("algo", [0, 2, 3])
+@pytest.mark.parametrize("M,N,K", [(40, 8, 64), (130, 12, 72), (300, 60, 64), (300, 68, 128), (513, 132, 136), (700, 260, 64), (9000, 1004, 64)])
+def test_rows_that_are_no_multiple_of_16_bytes(nm, ctx, M, N, K, algo):
+    """Nothing is written beyond a row (the border holds NaN), by no kernel."""
+    test_16_bit(nm, ctx, "bf16", M, N, K, "bias_res", algo)
+
+
+@pytest.mark.parametrize("algo", [0, 2, 3])
+@pytest.mark.parametrize("M,N,K,out", [(300, 68, 128, "i8"), (140, 332, 144, "bf16"), (600, 268, 64, "i8"), (600, 1020, 64, "bf16")])
+def test_int8_rows_that_are_no_multiple_of_16_bytes(nm, ctx, M, N, K, out, algo):
+    test_int8_bit_exact(nm, ctx, M, N, K, out, algo)
+
+
 @pytest.mark.parametrize("M,N,K,out", [(1, 8, 16, "f32"), (33, 68, 128, "i8"), (128, 1024, 1024, "bf16"), (128, 4096, 1024, "i8"),
                                        (128, 1024, 4096, "f32"), (200, 328, 144, "bf16")])
-def test_int8_bit_exact(nm, ctx, M, N, K, out):
+def test_int8_bit_exact(nm, ctx, M, N, K, out, algo=0):
     tabs = load_tables_both(ctx, 64, RANGES)
     Aq, Wq = nm_inputs.int8_matrix((M, K), 21), nm_inputs.int8_matrix((N, K), 22)
     rng = np.random.default_rng(23)
@@ -78,13 +91,14 @@ def test_int8_bit_exact(nm, ctx, M, N, K, out):
     out_scale = np.float32(0.02)
     td = {"bf16": torch.bfloat16, "i8": torch.int8, "f32": torch.float32}[out]
     ldo = (N + 15) // 16 * 16
-    o = torch.zeros((M, ldo), dtype=td, device="cuda")
+    o = torch.full((M, ldo), 99, dtype=td, device="cuda")
     acc = torch.full((M, N), -1, dtype=torch.int32, device="cuda")
     idx = torch.full((M, N), -7, dtype=torch.int32, device="cuda")
     ctx.linear_pwl(torch.from_numpy(Aq).cuda(), torch.from_numpy(Wq).cuda(), o[:, :N], bias=torch.from_numpy(bias).cuda(),
                    slot=nm.SLOT_GELU, a_scale=float(a_scale), w_scale=torch.from_numpy(ws).cuda(),
-                   inv_out_scale=float(np.float32(1.0) / out_scale), acc_dump=acc, idx_dump=idx)
+                   inv_out_scale=float(np.float32(1.0) / out_scale), acc_dump=acc, idx_dump=idx, algo=algo)
     ctx.check_device_status()
+    assert (o[:, N:] == 99).all()
     r = oracle.linear_i8(Aq, Wq, a_scale, ws, bias, None, tabs["gelu"], out_scale=out_scale)
     assert np.array_equal(acc.cpu().numpy(), r["acc"])
     assert np.array_equal(idx.cpu().numpy(), r["idx"])
