@@ -189,7 +189,7 @@ nm_status nm_launch_linear_f32(nm_ctx* ctx, const nm_linear_desc* d, cudaStream_
     a.res_first = d->res_first;
     a.tab = d->slot == NM_SLOT_NONE ? nullptr : ctx->d_tables + d->slot;
     a.n_seg = d->slot == NM_SLOT_NONE ? 0 : ctx->h_tables[d->slot].n;
-    a.idx_dump = d->idx_dump; a.ldd = d->N;
+    a.idx_dump = d->idx_dump;
     a.num_n_tiles = (int)n_tiles;
     a.num_tiles = (int)tiles;
     a.num_k_blocks = (int)((d->K + FBK - 1) / FBK);

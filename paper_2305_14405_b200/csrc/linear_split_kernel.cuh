@@ -223,7 +223,7 @@ struct Finisher {
                 }
                 if constexpr (INT) {
                     if (a.acc_dump)
-                        *reinterpret_cast<int4*>(a.acc_dump + grow * a.ldd + col) =
+                        *reinterpret_cast<int4*>(a.acc_dump + grow * a.N + col) =
                             make_int4((int)acc[u][0], (int)acc[u][1], (int)acc[u][2], (int)acc[u][3]);
                 }
                 float4 rv = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -238,7 +238,7 @@ struct Finisher {
                         x[i] = __fmaf_rn(t.x, x[i], t.y);
                     }
                 }
-                if (a.idx_dump) *reinterpret_cast<int4*>(a.idx_dump + grow * a.ldd + col) = make_int4(seg[0], seg[1], seg[2], seg[3]);
+                if (a.idx_dump) *reinterpret_cast<int4*>(a.idx_dump + grow * a.N + col) = make_int4(seg[0], seg[1], seg[2], seg[3]);
                 if (s.residual && !a.res_first) { x[0] += rv.x; x[1] += rv.y; x[2] += rv.z; x[3] += rv.w; }
                 Quad<OutT>::store(reinterpret_cast<OutT*>(s.out) + grow * s.ldo + col, make_float4(x[0], x[1], x[2], x[3]), a.inv_out_scale);
             }
@@ -473,19 +473,21 @@ inline unsigned split_launch_attrs(const nm_ctx* ctx, cudaLaunchAttribute* attr,
 }
 
 // Which kernel and tile a problem of `rows` rows (`m_tiles` blocks of 128), N columns and `k_blocks` K-blocks gets: the least
-// time by a model fitted to measured times in us: chains of equal launches at 72 problems, 37 to 4096 rows, N 256 to 4096,
-// K 256 to 4096, bf16 and int8, every kernel and tile.  It is 9 % off on the average, and the tile it picks 1 % behind the
-// best; at 16384 rows it predicts 47, 22, 64 and 67 us for the BERT-base projections (44, 22, 62 and 64 measured).
-//   persistent kernel, r rounds of tiles: base + r * k_blocks * (per K-block).  With most SMs busy a K-block takes at least
-//     its operands' way from L2 (97 KB a us and SM).  From the third round on a round takes at least its epilogue, by the
-//     short-K convolutions (64 -> 256 channels: 98 us with 256-column tiles, 79 with 128).
+// time by a model fitted to measured times in us of chains of equal launches.
+//   persistent kernel, 16-bit types: 352 problems, 300 to 16384 rows, N 256 to 4096, K 256 to 4096, with and without a table, each on all six
+//     tiles; 3 % off on the average, and the tile it picks 0.5 % behind the best, 9 % at most.  Full rounds of tiles take
+//     k_blocks * busy, or their epilogue; a part-filled one between k_blocks * lone and that (counted as a full round, 16384 x
+//     1536 x 512 went to a narrower tile: 27.5 us, 21.9 with 256 x 256 pairs); `fill`: what the first tiles and the last
+//     epilogue cost more when all SMs run them.  int8: base + every round in full, fitted to 72 problems of up to 4096 rows (the
+//     other form picked it too often over the split kernel there, 1024 x 1536 x 512: 5.6 us and 7.9).
 //   split kernel, n CTAs: base with the epilogue of the rows that exist + the K-blocks beyond those in flight at once (more when
 //     CTAs share an SM) + the exchange.
 //   Between kernels that are no matrix products the persistent kernel's longer set-up and tail overlap less, 0.4 us (11 layers, 128
 //   tokens: 497 us without it, 437 with).  A CNN's launches stand back to back and begin while their predecessor drains: there every
 //   round counts with its epilogue and narrow tiles do better than alone, so they have a row of parameters of their own (ResNet-50 batch
 //   13: 624 us, 657 with the other row; batch 23: 747 and 782).  There, and among the split kernel's widths, the wider tile wins
-//   within 3 %: it leaves more SMs to the neighbours.
+//   within 3 %: it leaves more SMs to the neighbours.  Elsewhere the split kernel wins within 3 % (37 x 2304 x 768: 4.6 us, 5.4 on
+//   persistent tiles).
 // E.g. 128 x 768 x 3072: 13.4 us in one round of the best persistent tile, 7.0 split over 8; 1024 x 768 x 768: 5.9 with 128 x 64
 // tiles, 9.8 with 256 x 256 pairs.
 // `whole_chunks`: a row of the output is a multiple of 16 bytes.  The persistent kernel stores through a tensor map, which
@@ -515,26 +517,38 @@ inline TileChoice choose_tile(int64_t rows, int64_t m_tiles, int64_t N, int64_t 
                               bool whole_chunks, NmChain chain, int sms)
 {
     const bool has_table = epi.n_seg > 0;
-    struct P { int BN; bool two; double base, kb, round; };
-    static const P apart[6] = {{256, true, 5.56, 0.420, 4.4}, {256, false, 4.72, 0.461, 4.8}, {128, true, 4.07, 0.233, 1.8},
-                               {128, false, 2.94, 0.315, 1.95}, {64, true, 3.19, 0.251, 1.15}, {64, false, 3.00, 0.218, 1.25}};
-    static const P joined[6] = {{256, true, 4.9, 0.386, 3.6}, {256, false, 5.4, 0.43, 3.6}, {128, true, 4.5, 0.26, 1.8},
-                                {128, false, 3.9, 0.322, 1.8}, {64, true, 3.9, 0.26, 0.9}, {64, false, 3.5, 0.30, 0.9}};
+    struct P { int BN; bool two; double base, lone, busy, round, round_table, table, fill; };
+    static const P apart[6] = {{256, true, 5.35, 0.265, 0.358, 1.67, 1.79, 2.36, 0.53}, {256, false, 5.03, 0.272, 0.435, 1.83, 1.35, 2.06, 0.0},
+                               {128, true, 3.97, 0.162, 0.240, 1.06, 0.56, 1.42, 0.97}, {128, false, 3.83, 0.161, 0.271, 1.18, 0.48, 1.37, 0.04},
+                               {64, true, 3.37, 0.150, 0.208, 0.93, 0.13, 1.42, 1.15},  {64, false, 3.18, 0.165, 0.202, 0.95, 0.05, 1.29, 0.57}};
+    struct J { double base, kb, round; };
+    static const J int8[2] = {{5.56, 0.420, 4.4}, {4.72, 0.461, 4.8}};
+    static const J joined[6] = {{4.9, 0.386, 3.6}, {5.4, 0.43, 3.6}, {4.5, 0.26, 1.8}, {3.9, 0.322, 1.8}, {3.9, 0.26, 0.9}, {3.5, 0.30, 0.9}};
     const bool in_cnn = chain.back_to_back;
     TileChoice best = {1, 64, false, 1e30};   // the split kernel takes anything
     for (int i = 0; i < 6; ++i) {
-        const P& p = in_cnn ? joined[i] : apart[i];
+        const P& p = apart[i];
         if (!whole_chunks || (!narrow_tiles && p.BN != 256) || (only64 && p.BN != 64) || (p.two && m_tiles < 2)) continue;
         if (narrow_tiles && p.BN > 64 && N <= p.BN / 2) continue;   // half the tile would be padding
         if (ring_stages(p.BN, p.two, epi) < 2) continue;            // no room beside a large table
         const int64_t tiles = (p.two ? (m_tiles + 1) / 2 : m_tiles) * ((N + p.BN - 1) / p.BN), slots = p.two ? sms / 2 : sms;
-        const int64_t rounds = (tiles + slots - 1) / slots;
-        const double share = tiles < slots ? (double)tiles / slots : 1.0;
-        const double feed = (A_BYTES + (p.two ? p.BN / 2 : p.BN) * ROW_BYTES) / 96.6e3;
-        double loop = (double)k_blocks * (!in_cnn && share >= 0.8 && feed > p.kb ? feed : p.kb);
-        if ((in_cnn || rounds > 2) && loop < p.round) loop = p.round;
-        const double t = p.base + (double)rounds * loop + (in_cnn ? 0.0 : (chain.weights_ready ? 0.4 : 0.0) + 0.32 * share * p.BN / 64) +
-                         (has_table ? (in_cnn ? 1.8 : 1.5) * p.BN / 256 : 0.0);
+        double t;
+        if (in_cnn) {
+            const J& j = joined[i];
+            const double loop = (double)k_blocks * j.kb;
+            t = j.base + (double)((tiles + slots - 1) / slots) * (loop < j.round ? j.round : loop) + (has_table ? 1.8 * p.BN / 256 : 0.0);
+        } else if (!narrow_tiles) {
+            const int64_t rounds = (tiles + slots - 1) / slots;
+            const double share = tiles < slots ? (double)tiles / slots : 1.0;
+            double loop = (double)k_blocks * int8[i].kb;
+            if (rounds > 2 && loop < int8[i].round) loop = int8[i].round;
+            t = int8[i].base + (double)rounds * loop + 1.28 * share + (has_table ? 1.5 : 0.0) + (chain.weights_ready ? 0.4 : 0.0);
+        } else {
+            const double full = (double)(tiles / slots), part = (double)(tiles % slots) / slots, k = (double)k_blocks;
+            const double epilogue = p.round + (has_table ? p.round_table : 0.0), busy = k * p.busy, some = k * (p.lone + (p.busy - p.lone) * part);
+            t = p.base + full * (busy > epilogue ? busy : epilogue) + (part > 0.0 ? (full > 0.0 && some < epilogue ? epilogue : some) : 0.0) +
+                (has_table ? p.table : 0.0) + p.fill * (full > 0.0 ? 1.0 : part) + (chain.weights_ready ? 0.4 : 0.0);
+        }
         if (t < best.us * (in_cnn ? 0.97 : 1.0)) best = {0, p.BN, p.two, t};
     }
     const double tile_rows = (rows < BM ? (double)rows : (double)BM) / BM;
@@ -548,7 +562,7 @@ inline TileChoice choose_tile(int64_t rows, int64_t m_tiles, int64_t N, int64_t 
                              (BN == 64 ? 0.235 : 0.179) * (beyond > 0 ? beyond : 0) * (share > 1 ? share : 1) +
                              (S == 1 ? 0.0 : S == 2 ? 0.21 : S == 4 ? 0.26 : 0.56) +
                              (0.35 * (share < 1 ? share : 1) + 0.85 * (share > 1 ? share - 1 : 0)) * BN / 32 + (has_table ? 0.42 * BN / 64 : 0.0);
-            if (t < best.us * (in_cnn || best.S ? 0.97 : 1.0)) best = {S, BN, false, t};
+            if (t < best.us * (in_cnn || best.S ? 0.97 : 1.03)) best = {S, BN, false, t};
         }
     }
     return best;

@@ -6,7 +6,7 @@ using namespace nm_tc;
 
 namespace {
 
-void fill_args(nm_ctx* ctx, const nm_linear_desc* d, int64_t ldd, NmChain chain, TcArgs* a)
+void fill_args(nm_ctx* ctx, const nm_linear_desc* d, NmChain chain, TcArgs* a)
 {
     memset(a, 0, sizeof(*a));
     a->M = d->M; a->N = d->N; a->K = d->K;
@@ -16,19 +16,19 @@ void fill_args(nm_ctx* ctx, const nm_linear_desc* d, int64_t ldd, NmChain chain,
     a->tab = d->slot == NM_SLOT_NONE ? nullptr : ctx->d_tables + d->slot;
     a->n_seg = d->slot == NM_SLOT_NONE ? 0 : ctx->h_tables[d->slot].n;
     a->a_scale = d->a_scale; a->w_scale = d->w_scale; a->inv_out_scale = d->inv_out_scale;
-    a->acc_dump = d->acc_dump; a->idx_dump = d->idx_dump; a->ldd = ldd;
+    a->acc_dump = d->acc_dump; a->idx_dump = d->idx_dump;
     a->status = ctx->d_status;
     a->weights_ready = chain.weights_ready;
     a->late_trigger = chain.late_trigger;
 }
 
 template <typename InT, typename OutT, bool TWO, int BN>
-nm_status launch(nm_ctx* ctx, const nm_linear_desc* d, int64_t ldd, NmChain chain, cudaStream_t st)
+nm_status launch(nm_ctx* ctx, const nm_linear_desc* d, NmChain chain, cudaStream_t st)
 {
     constexpr int B_ROWS = TWO ? BN / 2 : BN;
     constexpr int TILE_M = TWO ? 2 * BM : BM;
     TcArgs a;
-    fill_args(ctx, d, ldd, chain, &a);
+    fill_args(ctx, d, chain, &a);
     const int bk = ROW_BYTES / (int)sizeof(InT);
     const int64_t m_tiles = (d->M + TILE_M - 1) / TILE_M;
     a.num_n_tiles = (int)((d->N + BN - 1) / BN);
@@ -57,7 +57,7 @@ nm_status launch(nm_ctx* ctx, const nm_linear_desc* d, int64_t ldd, NmChain chai
 }
 
 template <typename InT, typename OutT, int BN>
-nm_status launch_split(nm_ctx* ctx, const nm_linear_desc* d, int64_t ldd, int S, NmChain chain, cudaStream_t st)
+nm_status launch_split(nm_ctx* ctx, const nm_linear_desc* d, int S, NmChain chain, cudaStream_t st)
 {
     const int bk = ROW_BYTES / (int)sizeof(InT);
     const int64_t k_blocks = (d->K + bk - 1) / bk, n_tiles = (d->N + BN - 1) / BN, tiles = (d->M + BM - 1) / BM * n_tiles;
@@ -65,7 +65,7 @@ nm_status launch_split(nm_ctx* ctx, const nm_linear_desc* d, int64_t ldd, int S,
     memset(&s, 0, sizeof(s));
     if (tiles > 0x7fffffffLL / S) return NM_ERR_SHAPE;
     s.S = S;
-    fill_args(ctx, d, ldd, chain, &s.t);
+    fill_args(ctx, d, chain, &s.t);
     s.t.num_n_tiles = (int)n_tiles;
     s.t.num_tiles = (int)tiles;
     s.t.num_k_blocks = (int)k_blocks;
@@ -93,16 +93,15 @@ TileChoice choose(nm_ctx* ctx, const nm_linear_desc* d, NmChain chain)
     return choose_tile(d->M, (d->M + BM - 1) / BM, d->N, (d->K + bk - 1) / bk, NARROW, epi, false, whole_chunks, chain, ctx->sm_count);
 }
 
-// ldd: row pitch of the dumps
 template <typename InT, typename OutT>
-nm_status launch_choice(nm_ctx* ctx, const nm_linear_desc* d, const TileChoice& c, int64_t ldd, NmChain chain, cudaStream_t st)
+nm_status launch_choice(nm_ctx* ctx, const nm_linear_desc* d, const TileChoice& c, NmChain chain, cudaStream_t st)
 {
-    if (c.S) return c.BN == 32 ? launch_split<InT, OutT, 32>(ctx, d, ldd, c.S, chain, st) : launch_split<InT, OutT, 64>(ctx, d, ldd, c.S, chain, st);
+    if (c.S) return c.BN == 32 ? launch_split<InT, OutT, 32>(ctx, d, c.S, chain, st) : launch_split<InT, OutT, 64>(ctx, d, c.S, chain, st);
     if constexpr (!TcIn<InT>::is_int) {
-        if (c.BN == 64) return c.two ? launch<InT, OutT, true, 64>(ctx, d, ldd, chain, st) : launch<InT, OutT, false, 64>(ctx, d, ldd, chain, st);
-        if (c.BN == 128) return c.two ? launch<InT, OutT, true, 128>(ctx, d, ldd, chain, st) : launch<InT, OutT, false, 128>(ctx, d, ldd, chain, st);
+        if (c.BN == 64) return c.two ? launch<InT, OutT, true, 64>(ctx, d, chain, st) : launch<InT, OutT, false, 64>(ctx, d, chain, st);
+        if (c.BN == 128) return c.two ? launch<InT, OutT, true, 128>(ctx, d, chain, st) : launch<InT, OutT, false, 128>(ctx, d, chain, st);
     }
-    return c.two ? launch<InT, OutT, true, 256>(ctx, d, ldd, chain, st) : launch<InT, OutT, false, 256>(ctx, d, ldd, chain, st);
+    return c.two ? launch<InT, OutT, true, 256>(ctx, d, chain, st) : launch<InT, OutT, false, 256>(ctx, d, chain, st);
 }
 
 template <typename InT, typename OutT>
@@ -111,9 +110,10 @@ nm_status launch_sel(nm_ctx* ctx, const nm_linear_desc* d, NmChain chain, cudaSt
     constexpr int64_t CHUNK = 16 / sizeof(OutT);
     const TileChoice c = choose<InT, OutT>(ctx, d, chain);
     const int64_t main_n = d->N / CHUNK * CHUNK;
-    if (main_n == d->N || main_n < 8) return launch_choice<InT, OutT>(ctx, d, c, d->N, chain, st);
+    if (main_n == d->N || main_n < 8 || d->acc_dump || d->idx_dump) return launch_choice<InT, OutT>(ctx, d, c, chain, st);
     // A row that is no multiple of 16 bytes: all of it by the split kernel, or the last 4 to 12 columns by the split kernel and the
-    // others by themselves, whichever the model finds cheaper (16384 x 1004 x 1024: 58.4 us and 38.5).
+    // others by themselves, whichever the model finds cheaper (16384 x 1004 x 1024: 58.4 us and 38.5); with dumps, whose
+    // row is N, the former.
     nm_linear_desc m = *d, r = *d;
     m.N = main_n;
     r.N = d->N - main_n;
@@ -122,13 +122,11 @@ nm_status launch_sel(nm_ctx* ctx, const nm_linear_desc* d, NmChain chain, cudaSt
     if (d->residual) r.residual = (const uint8_t*)d->residual + main_n * sizeof(OutT);
     if (d->bias) r.bias = d->bias + main_n;
     if (d->w_scale) r.w_scale = d->w_scale + main_n;
-    if (d->acc_dump) r.acc_dump = d->acc_dump + main_n;
-    if (d->idx_dump) r.idx_dump = d->idx_dump + main_n;
     const TileChoice cm = choose<InT, OutT>(ctx, &m, chain), cr = choose<InT, OutT>(ctx, &r, chain);
-    if (d->algo == 0 && c.us <= cm.us + cr.us) return launch_choice<InT, OutT>(ctx, d, c, d->N, chain, st);
-    const nm_status e = launch_choice<InT, OutT>(ctx, &m, cm, d->N, chain, st);
+    if (d->algo == 0 && c.us <= cm.us + cr.us) return launch_choice<InT, OutT>(ctx, d, c, chain, st);
+    const nm_status e = launch_choice<InT, OutT>(ctx, &m, cm, chain, st);
     if (e != NM_OK) return e;
-    return launch_choice<InT, OutT>(ctx, &r, cr, d->N, chain, st);
+    return launch_choice<InT, OutT>(ctx, &r, cr, chain, st);
 }
 
 }  // namespace

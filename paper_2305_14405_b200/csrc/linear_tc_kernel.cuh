@@ -80,7 +80,6 @@ struct TcArgs {
     float inv_out_scale;
     int32_t* acc_dump;
     int32_t* idx_dump;
-    int64_t ldd;    // row pitch of the dumps
     int* status;
     int num_n_tiles, num_tiles, num_k_blocks, stages, n_seg;
     int weights_ready, late_trigger;   // NmChain
@@ -647,7 +646,7 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                             const float4 ws = *reinterpret_cast<const float4*>(my_vec + 128 + c * 32 + i);
                             const float4 bs = *reinterpret_cast<const float4*>(my_vec + c * 32 + i);
                             if (a.acc_dump && row_ok && col0 + i < a.N)
-                                *reinterpret_cast<int4*>(a.acc_dump + row * a.ldd + col0 + i) =
+                                *reinterpret_cast<int4*>(a.acc_dump + row * a.N + col0 + i) =
                                     make_int4((int)r[i], (int)r[i + 1], (int)r[i + 2], (int)r[i + 3]);
                             uint64_t d01, d23;   // fma((float)acc, scale, bias), two columns per packed instruction
                             asm("fma.rn.f32x2 %0, %1, %2, %3;"
@@ -682,7 +681,7 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                             for (int i = 0; i < 32; ++i) {
                                 int s;
                                 v[i] = nm_pwl_fast(rep_lane, v[i], inv_h, off, nm1, &s);
-                                if (row_ok && col0 + i < a.N) a.idx_dump[row * a.ldd + col0 + i] = s;
+                                if (row_ok && col0 + i < a.N) a.idx_dump[row * a.N + col0 + i] = s;
                             }
                         } else {
                             const uint64_t inv_h2 = nm_pack2(inv_h, inv_h), off2 = nm_pack2(off, off);
@@ -697,7 +696,7 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                     } else if (a.idx_dump) {
 #pragma unroll
                         for (int i = 0; i < 32; ++i)
-                            if (row_ok && col0 + i < a.N) a.idx_dump[row * a.ldd + col0 + i] = -1;
+                            if (row_ok && col0 + i < a.N) a.idx_dump[row * a.N + col0 + i] = -1;
                     }
                     if (has_res && !a.res_first) add_res32<OutT>(&rsv[cc * WPC], v);
                     pack32<OutT>(v, &packed[cc * WPC], a.inv_out_scale);
