@@ -439,7 +439,7 @@ linear_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         }
     }
     __syncthreads();
-    if (S > 1 && ok && !nm_mbar_wait(&bar_part, 0, abortp, a.status)) ok = false;
+    if (S > 1 && ok && !nm_mbar_wait_cluster(&bar_part, 0, abortp, a.status)) ok = false;   // (other CTAs wrote the rows)
 
     if (ok) fin.run(part, s_tab);
 
