@@ -62,6 +62,7 @@ int64_t fill_args(nm_ctx* ctx, const NmConvTc* c, NmChain chain, TcArgs* a)
     a->weights_ready = chain.weights_ready && !c->depthwise;
     a->late_trigger = chain.late_trigger;
     a->num_k_blocks = c->taps_y * c->taps_x * c->cblocks;
+    a->accs = 1;
     return (int64_t)cv.tiles_x * cv.tiles_y * ceil_div(c->N, cv.NB);
 }
 
@@ -199,7 +200,7 @@ nm_status launch_sel(nm_ctx* ctx, const NmConvTc* c, NmChain chain, cudaStream_t
         }
         t = choose_tile((int64_t)c->N * c->Ho * c->Wo, patches, c->Cout, (int64_t)c->taps_y * c->taps_x * c->cblocks, true,
                         EpiNeeds{c->slot == NM_SLOT_NONE ? 0 : ctx->h_tables[c->slot].n, c->residual != nullptr, c->bias != nullptr},
-                        c->depthwise != 0, true, chain, ctx->sm_count);
+                        c->depthwise != 0, true, false, chain, ctx->sm_count);
     } else {
         t.S = 0;
         t.BN = c->Cout <= 64 || c->depthwise ? 64 : (c->Cout <= 128 ? 128 : 256);

@@ -290,8 +290,9 @@ linear_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         // what the others will send: their columns of each of this CTA's rows
         if (S > 1) nm_mbar_expect_tx(&bar_part, (uint32_t)((rows - rank + S - 1) / S) * (uint32_t)(S - 1) * BN * 4u);
     }
+    const uint32_t tmem_cols = INT ? BN : a.accs <= 1 ? BN : a.accs <= 2 ? 2 * BN : a.accs <= 4 ? 4 * BN : 8 * BN;
     if (warp == 1) {
-        nm_tmem_alloc(&tmem_slot, BN);
+        nm_tmem_alloc(&tmem_slot, tmem_cols);
         nm_tmem_relinquish();
     }
     if (a.tab) {
@@ -383,6 +384,9 @@ linear_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
             int stage = 0;
             uint32_t phase = 0;
             bool ready = false;
+            [[maybe_unused]] uint32_t acc = tmem;
+            [[maybe_unused]] int left = a.acc_steps;   // steps that the accumulator still takes (0: no limit)
+            [[maybe_unused]] uint32_t accum = 0;
             for (int kb = kb0; kb < kb1; ++kb) {
                 if (!ready && !vote(nm_mbar_wait(&bar_full[stage], phase, abortp, a.status))) { ok = false; break; }
                 if constexpr (ONE_LANE) {   // look at the next stage while this one's MMAs are issued
@@ -395,9 +399,17 @@ linear_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                 if (ONE_LANE || nm_elect_one()) {
 #pragma unroll
                     for (int k = 0; k < 4; ++k) {  // 4 x 32 bytes of K per 128-byte row
-                        const uint32_t accum = (kb != kb0 || k != 0) ? 1u : 0u;
-                        if constexpr (INT) nm_mma_i8(tmem, adesc + 2 * k, bdesc + 2 * k, IDESC, accum);
-                        else nm_mma_f16(tmem, adesc + 2 * k, bdesc + 2 * k, IDESC, accum);
+                        if constexpr (INT) {
+                            nm_mma_i8(tmem, adesc + 2 * k, bdesc + 2 * k, IDESC, (kb != kb0 || k != 0) ? 1u : 0u);
+                        } else {
+                            nm_mma_f16(acc, adesc + 2 * k, bdesc + 2 * k, IDESC, accum);
+                            accum = 1u;
+                            if (--left == 0) {
+                                acc += BN;
+                                left = a.acc_steps;
+                                accum = 0u;
+                            }
+                        }
                     }
                     nm_tc_commit(&bar_empty[stage]);
                 }
@@ -421,11 +433,20 @@ linear_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         uint32_t* mine = part + (((rank * BM + row) >> (31 - __clz(S))) * PITCH + c0);   // the row's place, in the owner
         const uint32_t t_addr = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)c0;
         const uint32_t dst = nm_mapa(nm_smem_u32(mine), (uint32_t)owner), bar = nm_mapa(nm_smem_u32(&bar_part), (uint32_t)owner);
+        const int used = a.acc_steps ? (4 * (kb1 - kb0) + a.acc_steps - 1) / a.acc_steps : 1;   // this CTA's accumulators
         if (ok && q * 32 < rows) {
 #pragma unroll
             for (int c = 0; c < BN / 2; c += 16) {
                 uint32_t r[16];
                 nm_tmem_ld16_sync(t_addr + (uint32_t)c, r);
+                if constexpr (!INT) {
+                    for (int i = 1; i < used; ++i) {
+                        uint32_t o[16];
+                        nm_tmem_ld16_sync(t_addr + (uint32_t)(i * BN + c), o);
+#pragma unroll
+                        for (int j = 0; j < 16; ++j) r[j] = __float_as_uint(__uint_as_float(r[j]) + __uint_as_float(o[j]));
+                    }
+                }
                 if (row >= rows) continue;
                 if (owner == rank) {
 #pragma unroll
@@ -449,7 +470,7 @@ linear_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     if (warp == 1) {
         __syncwarp();
         nm_tc_fence_after();
-        nm_tmem_dealloc(tmem, BN);
+        nm_tmem_dealloc(tmem, tmem_cols);
     }
     // Every row sent to this CTA has arrived before it gets here, unless something timed out: then it stays until the others,
     // who may still be sending, have got as far or are gone.
@@ -497,7 +518,19 @@ struct TileChoice {
     int BN;
     bool two;   // persistent kernel: CTA pairs
     double us;  // by the model
+    int steps;  // MMA steps per accumulator (TcArgs::acc_steps), 0: all
 };
+
+// How many MMA steps of 16 K-elements an accumulator may take if the sum is to be no further from the exact one than a chain of
+// fp32 FMAs.  The tensor core truncates the sum at every step: measured against float64, a chain of n steps is off by 1.55e-8 n of
+// the sum's rms, a chain of K FMAs by 7.4e-9 sqrt(K) = 3.0e-8 sqrt(steps) (bf16, K 16 to 4096: 2.1e-8, 6.6e-8, 2.4e-7, 7.3e-7, 3.3e-6,
+// 4.4e-6 for one accumulator at K 16, 64, 256, 768, 3072, 4096; FMAs 1.9e-8, 5.1e-8, 1.1e-7, 2.1e-7, 5.2e-7, 6.0e-7).
+inline int steps_like_fma(int64_t k_blocks)
+{
+    const int n = (int)(1.5 * sqrt(4.0 * (double)k_blocks) - 1.0);
+    return n < 1 ? 1 : n;
+}
+constexpr int SPLIT_ACC_COLS = 256;   // tensor-memory columns of a CTA: two of them share an SM
 
 // A cluster's CTAs share a GPC, so not every SM is in one: the CTAs, in clusters of S, that certainly find an SM each.
 inline bool split_alone(int S, int64_t ctas, int sms) { return ctas <= (S == 8 ? sms * 3 / 4 : sms * 7 / 8); }
@@ -514,7 +547,7 @@ inline int split_stages(int BN, int S, int64_t ctas, int sms, bool back_to_back)
 }
 
 inline TileChoice choose_tile(int64_t rows, int64_t m_tiles, int64_t N, int64_t k_blocks, bool narrow_tiles, const EpiNeeds& epi, bool only64,
-                              bool whole_chunks, NmChain chain, int sms)
+                              bool whole_chunks, bool like_fma, NmChain chain, int sms)
 {
     const bool has_table = epi.n_seg > 0;
     struct P { int BN; bool two; double base, lone, busy, round, round_table, table, fill; };
@@ -525,13 +558,16 @@ inline TileChoice choose_tile(int64_t rows, int64_t m_tiles, int64_t N, int64_t 
     static const J int8[2] = {{5.56, 0.420, 4.4}, {4.72, 0.461, 4.8}};
     static const J joined[6] = {{4.9, 0.386, 3.6}, {5.4, 0.43, 3.6}, {4.5, 0.26, 1.8}, {3.9, 0.322, 1.8}, {3.9, 0.26, 0.9}, {3.5, 0.30, 0.9}};
     const bool in_cnn = chain.back_to_back;
-    TileChoice best = {1, 64, false, 1e30};   // the split kernel takes anything
+    TileChoice best = {1, 64, false, 1e30, 0};   // the split kernel takes anything
     for (int i = 0; i < 6; ++i) {
         const P& p = apart[i];
         if (!whole_chunks || (!narrow_tiles && p.BN != 256) || (only64 && p.BN != 64) || (p.two && m_tiles < 2)) continue;
         if (narrow_tiles && p.BN > 64 && N <= p.BN / 2) continue;   // half the tile would be padding
         if (ring_stages(p.BN, p.two, epi) < 2) continue;            // no room beside a large table
         const int64_t tiles = (p.two ? (m_tiles + 1) / 2 : m_tiles) * ((N + p.BN - 1) / p.BN), slots = p.two ? sms / 2 : sms;
+        // (like_fma: the 64-column tiles have room for up to four accumulators in each of their two buffers)
+        const int steps = like_fma ? steps_like_fma(k_blocks) : 0;
+        if (like_fma && (p.BN != 64 || 4 * k_blocks > 4 * steps)) continue;
         double t;
         if (in_cnn) {
             const J& j = joined[i];
@@ -549,20 +585,30 @@ inline TileChoice choose_tile(int64_t rows, int64_t m_tiles, int64_t N, int64_t 
             t = p.base + full * (busy > epilogue ? busy : epilogue) + (part > 0.0 ? (full > 0.0 && some < epilogue ? epilogue : some) : 0.0) +
                 (has_table ? p.table : 0.0) + p.fill * (full > 0.0 ? 1.0 : part) + (chain.weights_ready ? 0.4 : 0.0);
         }
-        if (t < best.us * (in_cnn ? 0.97 : 1.0)) best = {0, p.BN, p.two, t};
+        if (t < best.us * (in_cnn ? 0.97 : 1.0)) best = {0, p.BN, p.two, t, steps};
     }
     const double tile_rows = (rows < BM ? (double)rows : (double)BM) / BM;
     for (int BN = 64; BN >= (only64 ? 64 : 32); BN /= 2) {
         const int64_t tiles = m_tiles * ((N + BN - 1) / BN);
         for (int S = 1; S <= 8 && S <= k_blocks; S *= 2) {
             const int64_t n = tiles * S;
-            if (n > 2 * sms && (whole_chunks || S > 1 || n > 0x7fffffffLL)) break;
+            if (n > 0x7fffffffLL || (n > 2 * sms && (like_fma ? best.us < 1e30 : whole_chunks || S > 1))) break;
+            int steps = 0;
+            if (like_fma) {
+                const int64_t mine = 4 * ((k_blocks + S - 1) / S), most = SPLIT_ACC_COLS / BN;
+                steps = steps_like_fma(k_blocks);
+                if (mine > steps * most) {
+                    // (more than 150 000 K-elements: nothing does, and the last form takes longer chains)
+                    if (BN > 32 || best.us < 1e30 || (S < 8 && 2 * S <= k_blocks)) continue;
+                    steps = (int)((mine + most - 1) / most);
+                }
+            }
             const double per = (double)((k_blocks + S - 1) / S), share = (double)n / sms, beyond = per - split_stages(BN, S, n, sms, in_cnn);
             const double t = 4.29 + 0.73 * tile_rows * BN / 64 + 0.038 * per +
                              (BN == 64 ? 0.235 : 0.179) * (beyond > 0 ? beyond : 0) * (share > 1 ? share : 1) +
                              (S == 1 ? 0.0 : S == 2 ? 0.21 : S == 4 ? 0.26 : 0.56) +
                              (0.35 * (share < 1 ? share : 1) + 0.85 * (share > 1 ? share - 1 : 0)) * BN / 32 + (has_table ? 0.42 * BN / 64 : 0.0);
-            if (t < best.us * (in_cnn || best.S ? 0.97 : 1.03)) best = {S, BN, false, t};
+            if (t < best.us * (in_cnn || best.S ? 0.97 : 1.03)) best = {S, BN, false, t, steps};
         }
     }
     return best;
@@ -577,6 +623,7 @@ inline nm_status launch_split_kernel(nm_ctx* ctx, const CUtensorMap& tmA, const 
     constexpr int MIN_STAGES = (PART_BYTES + STAGE_BYTES - 1) / STAGE_BYTES;
     static_assert(MIN_STAGES <= 3, "partial tile");
     const int per = (s.t.num_k_blocks + s.S - 1) / s.S, most = split_stages(BN, s.S, (int64_t)s.t.num_tiles * s.S, ctx->sm_count, back_to_back);
+    s.t.accs = s.t.acc_steps ? (4 * per + s.t.acc_steps - 1) / s.t.acc_steps : 1;
     s.t.stages = per < MIN_STAGES ? MIN_STAGES : (per > most ? most : per);
     const size_t smem = (size_t)s.t.stages * STAGE_BYTES + (s.S > 1 ? PART_BYTES : 0) + 1024;
     auto kern = s.S == 1   ? linear_split_kernel<InT, OutT, BN, CONV, 1>

@@ -23,7 +23,7 @@ void fill_args(nm_ctx* ctx, const nm_linear_desc* d, NmChain chain, TcArgs* a)
 }
 
 template <typename InT, typename OutT, bool TWO, int BN>
-nm_status launch(nm_ctx* ctx, const nm_linear_desc* d, NmChain chain, cudaStream_t st)
+nm_status launch(nm_ctx* ctx, const nm_linear_desc* d, int steps, NmChain chain, cudaStream_t st)
 {
     constexpr int B_ROWS = TWO ? BN / 2 : BN;
     constexpr int TILE_M = TWO ? 2 * BM : BM;
@@ -35,6 +35,8 @@ nm_status launch(nm_ctx* ctx, const nm_linear_desc* d, NmChain chain, cudaStream
     if (m_tiles * a.num_n_tiles > 0x7fffffffLL) return NM_ERR_SHAPE;
     a.num_tiles = (int)(m_tiles * a.num_n_tiles);
     a.num_k_blocks = (int)((d->K + bk - 1) / bk);
+    a.acc_steps = steps;
+    a.accs = steps ? (4 * a.num_k_blocks + steps - 1) / steps : 1;
     // Weights of 2 MB and less stay in L2 from pass to pass unless the stack is very deep, and asking for them then costs up to 1.5 %
     // (7 layers, 432 tokens, H 512: 356 against 361 us; ResNet-50 batch 7: 964 and 977); larger ones do not: 12 layers, 7 x 333
     // tokens, 170 MB of weights: 1008 -> 998 us, int8 24 layers, 128 tokens, 300 MB: 870 -> 859.
@@ -57,8 +59,9 @@ nm_status launch(nm_ctx* ctx, const nm_linear_desc* d, NmChain chain, cudaStream
 }
 
 template <typename InT, typename OutT, int BN>
-nm_status launch_split(nm_ctx* ctx, const nm_linear_desc* d, int S, NmChain chain, cudaStream_t st)
+nm_status launch_split(nm_ctx* ctx, const nm_linear_desc* d, const TileChoice& c, NmChain chain, cudaStream_t st)
 {
+    const int S = c.S;
     const int bk = ROW_BYTES / (int)sizeof(InT);
     const int64_t k_blocks = (d->K + bk - 1) / bk, n_tiles = (d->N + BN - 1) / BN, tiles = (d->M + BM - 1) / BM * n_tiles;
     SplitArgs s;
@@ -66,6 +69,7 @@ nm_status launch_split(nm_ctx* ctx, const nm_linear_desc* d, int S, NmChain chai
     if (tiles > 0x7fffffffLL / S) return NM_ERR_SHAPE;
     s.S = S;
     fill_args(ctx, d, chain, &s.t);
+    s.t.acc_steps = c.steps;
     s.t.num_n_tiles = (int)n_tiles;
     s.t.num_tiles = (int)tiles;
     s.t.num_k_blocks = (int)k_blocks;
@@ -79,38 +83,40 @@ nm_status launch_split(nm_ctx* ctx, const nm_linear_desc* d, int S, NmChain chai
     return launch_split_kernel<InT, OutT, BN, false>(ctx, tmA, tmW, s, chain.back_to_back, 2.0 * (double)d->M * (double)d->N * (double)d->K, st);
 }
 
-// Kernel and tile for d: the cheapest by the model, or (algo 2, 3) a forced one: the persistent kernel with a tile by the width
+// Kernel and tile for d: the cheapest by the model (like_fma: with accumulators as good as a chain of fp32 FMAs), or (algo 2, 3) a forced one: the persistent kernel with a tile by the width
 // alone; algo 3 asks for one CTA per tile, otherwise CTA pairs from one 256-row tile on.
 template <typename InT, typename OutT>
-TileChoice choose(nm_ctx* ctx, const nm_linear_desc* d, NmChain chain)
+TileChoice choose(nm_ctx* ctx, const nm_linear_desc* d, bool like_fma, NmChain chain)
 {
     constexpr bool NARROW = !TcIn<InT>::is_int;   // tiles of 64 and 128 columns are built for the 16-bit types
     const bool whole_chunks = d->N * sizeof(OutT) % 16 == 0;
     if (d->algo != 0 && whole_chunks)
-        return {0, NARROW && d->N <= 64 ? 64 : (NARROW && d->N <= 128 ? 128 : 256), d->algo != 3 && d->M >= 256, 0.0};
+        return {0, NARROW && d->N <= 64 ? 64 : (NARROW && d->N <= 128 ? 128 : 256), d->algo != 3 && d->M >= 256, 0.0, 0};
     const int bk = ROW_BYTES / (int)sizeof(InT);
     const EpiNeeds epi = {d->slot == NM_SLOT_NONE ? 0 : ctx->h_tables[d->slot].n, d->residual != nullptr, d->bias != nullptr || TcIn<InT>::is_int};
-    return choose_tile(d->M, (d->M + BM - 1) / BM, d->N, (d->K + bk - 1) / bk, NARROW, epi, false, whole_chunks, chain, ctx->sm_count);
+    return choose_tile(d->M, (d->M + BM - 1) / BM, d->N, (d->K + bk - 1) / bk, NARROW, epi, false, whole_chunks, like_fma, chain, ctx->sm_count);
 }
 
 template <typename InT, typename OutT>
 nm_status launch_choice(nm_ctx* ctx, const nm_linear_desc* d, const TileChoice& c, NmChain chain, cudaStream_t st)
 {
-    if (c.S) return c.BN == 32 ? launch_split<InT, OutT, 32>(ctx, d, c.S, chain, st) : launch_split<InT, OutT, 64>(ctx, d, c.S, chain, st);
+    if (c.S) return c.BN == 32 ? launch_split<InT, OutT, 32>(ctx, d, c, chain, st) : launch_split<InT, OutT, 64>(ctx, d, c, chain, st);
     if constexpr (!TcIn<InT>::is_int) {
-        if (c.BN == 64) return c.two ? launch<InT, OutT, true, 64>(ctx, d, chain, st) : launch<InT, OutT, false, 64>(ctx, d, chain, st);
-        if (c.BN == 128) return c.two ? launch<InT, OutT, true, 128>(ctx, d, chain, st) : launch<InT, OutT, false, 128>(ctx, d, chain, st);
+        if (c.BN == 64) return c.two ? launch<InT, OutT, true, 64>(ctx, d, c.steps, chain, st) : launch<InT, OutT, false, 64>(ctx, d, c.steps, chain, st);
+        if (c.BN == 128) return c.two ? launch<InT, OutT, true, 128>(ctx, d, c.steps, chain, st) : launch<InT, OutT, false, 128>(ctx, d, c.steps, chain, st);
     }
-    return c.two ? launch<InT, OutT, true, 256>(ctx, d, chain, st) : launch<InT, OutT, false, 256>(ctx, d, chain, st);
+    return c.two ? launch<InT, OutT, true, 256>(ctx, d, c.steps, chain, st) : launch<InT, OutT, false, 256>(ctx, d, c.steps, chain, st);
 }
 
 template <typename InT, typename OutT>
 nm_status launch_sel(nm_ctx* ctx, const nm_linear_desc* d, NmChain chain, cudaStream_t st)
 {
     constexpr int64_t CHUNK = 16 / sizeof(OutT);
-    const TileChoice c = choose<InT, OutT>(ctx, d, chain);
+    // Few rows or columns had the CUDA cores' fp32 FMA chains before the split kernel took them: no sum of theirs gets worse.
+    const bool like_fma = !TcIn<InT>::is_int && d->algo == 0 && (d->M < 64 || d->N < 64);
+    const TileChoice c = choose<InT, OutT>(ctx, d, like_fma, chain);
     const int64_t main_n = d->N / CHUNK * CHUNK;
-    if (main_n == d->N || main_n < 8 || d->acc_dump || d->idx_dump) return launch_choice<InT, OutT>(ctx, d, c, chain, st);
+    if (like_fma || main_n == d->N || main_n < 8 || d->acc_dump || d->idx_dump) return launch_choice<InT, OutT>(ctx, d, c, chain, st);
     // A row that is no multiple of 16 bytes: all of it by the split kernel, or the last 4 to 12 columns by the split kernel and the
     // others by themselves, whichever the model finds cheaper (16384 x 1004 x 1024: 58.4 us and 38.5); with dumps, whose
     // row is N, the former.
@@ -122,7 +128,7 @@ nm_status launch_sel(nm_ctx* ctx, const nm_linear_desc* d, NmChain chain, cudaSt
     if (d->residual) r.residual = (const uint8_t*)d->residual + main_n * sizeof(OutT);
     if (d->bias) r.bias = d->bias + main_n;
     if (d->w_scale) r.w_scale = d->w_scale + main_n;
-    const TileChoice cm = choose<InT, OutT>(ctx, &m, chain), cr = choose<InT, OutT>(ctx, &r, chain);
+    const TileChoice cm = choose<InT, OutT>(ctx, &m, false, chain), cr = choose<InT, OutT>(ctx, &r, false, chain);
     if (d->algo == 0 && c.us <= cm.us + cr.us) return launch_choice<InT, OutT>(ctx, d, c, chain, st);
     const nm_status e = launch_choice<InT, OutT>(ctx, &m, cm, chain, st);
     if (e != NM_OK) return e;

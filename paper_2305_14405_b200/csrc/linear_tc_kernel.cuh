@@ -87,6 +87,8 @@ struct TcArgs {
     int w_stages;                      // HALO: weight tiles in shared memory; w_resident: all of them, loaded once
     int w_resident;
     ConvDev cv;
+    int acc_steps;   // MMA steps (16 K-elements) per accumulator, 0: one accumulator takes them all; otherwise there are
+    int accs;        // `accs` of them, BN columns each and side by side, and the epilogue adds them up in fp32
 };
 
 template <typename InT> struct TcIn;
@@ -218,6 +220,10 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     // one's MMAs, 281 and less (128 images, 28 x 28, 128 -> 128, 3 x 3: 45.6 -> 39.2 us).  With 256 columns the tensor core
     // covers it, and all lanes, whose stage numbers and descriptors stay in uniform registers, are 1 % faster.
     constexpr bool ONE_LANE = BN < 256;
+    // Several accumulators per tile (TcArgs::acc_steps): matrices of few columns.
+    constexpr bool MULTI = BN == 64 && !CONV && !TcIn<InT>::is_int;
+    const uint32_t buf_cols = MULTI ? BN * (uint32_t)a.accs : BN;
+    const uint32_t tmem_cols = !MULTI || a.accs <= 1 ? TMEM_COLS : a.accs <= 2 ? 2 * TMEM_COLS : 4 * TMEM_COLS;
     auto vote = [](bool done) { return ONE_LANE ? done : __all_sync(0xffffffffu, done) != 0; };
 
     extern __shared__ uint8_t smem_raw[];
@@ -275,10 +281,10 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     }
     if (warp == 1) {
         if constexpr (TWO) {
-            nm_tmem_alloc2(&tmem_slot, TMEM_COLS);
+            nm_tmem_alloc2(&tmem_slot, tmem_cols);
             nm_tmem_relinquish2();
         } else {
-            nm_tmem_alloc(&tmem_slot, TMEM_COLS);
+            nm_tmem_alloc(&tmem_slot, tmem_cols);
             nm_tmem_relinquish();
         }
     }
@@ -408,7 +414,9 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                 // tcgen05 operations, ordered by tcgen05.fence (a cluster-scope acquire costs ~400 cycles per tile)
                 if (!vote(nm_mbar_wait(&bar_acc_empty[buf], acc_phase ^ 1u, abortp, a.status))) { ok = false; break; }
                 nm_tc_fence_after();
-                const uint32_t d_tmem = tmem_base + (uint32_t)(buf * BN);
+                uint32_t d_tmem = tmem_base + (uint32_t)buf * buf_cols;
+                [[maybe_unused]] int left = a.acc_steps;
+                [[maybe_unused]] uint32_t multi_accum = 0;
                 if constexpr (HALO) {
                     const bool wait_w = !a.w_resident || tile == tile_first;
                     for (int cb = 0; ok && cb < a.cv.cblocks; ++cb) {
@@ -445,13 +453,21 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                     if (ONE_LANE || nm_elect_one()) {
 #pragma unroll
                         for (int k = 0; k < 4; ++k) {  // 4 x 32 bytes of K per 128-byte row
-                            const uint32_t accum = (kb | k) != 0 ? 1u : 0u;
+                            const uint32_t accum = MULTI ? multi_accum : (kb | k) != 0 ? 1u : 0u;
                             if constexpr (TWO) {
                                 if constexpr (TcIn<InT>::is_int) nm_mma_i8_2cta(d_tmem, adesc + 2 * k, bdesc + 2 * k, IDESC, accum);
                                 else nm_mma_f16_2cta(d_tmem, adesc + 2 * k, bdesc + 2 * k, IDESC, accum);
                             } else {
                                 if constexpr (TcIn<InT>::is_int) nm_mma_i8(d_tmem, adesc + 2 * k, bdesc + 2 * k, IDESC, accum);
                                 else nm_mma_f16(d_tmem, adesc + 2 * k, bdesc + 2 * k, IDESC, accum);
+                            }
+                            if constexpr (MULTI) {
+                                multi_accum = 1u;
+                                if (--left == 0) {
+                                    d_tmem += BN;
+                                    left = a.acc_steps;
+                                    multi_accum = 0u;
+                                }
                             }
                         }
                         // smem stage reusable (in both CTAs of a pair) once these MMAs retire
@@ -572,7 +588,7 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             bool store_rows;   // do this warp's 32 rows exist at all?
             if constexpr (CONV) store_rows = pt.oy0 + sub_h < a.cv.Ho && pt.img0 + sub_n < a.cv.Nimg;
             else store_rows = (int64_t)m0 + q * 32 < a.M;
-            const uint32_t t_addr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * BN + col_off);
+            const uint32_t t_addr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)buf * buf_cols + (uint32_t)col_off;
             uint32_t r[32];
 #pragma unroll
             for (int g = 0; g < NG; ++g) {
@@ -624,6 +640,14 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                     // arithmetic measured no faster (the quarter's other warp covers the latency), and registers
                     // with a load in flight are not safe from compiler-made copies until the wait.
                     nm_tmem_ld32_sync(t_addr + (uint32_t)(c * 32), r);
+                    if constexpr (MULTI) {
+                        for (int i = 1; i < a.accs; ++i) {
+                            uint32_t o[32];
+                            nm_tmem_ld32_sync(t_addr + (uint32_t)(i * BN + c * 32), o);
+#pragma unroll
+                            for (int j = 0; j < 32; ++j) r[j] = __float_as_uint(__uint_as_float(r[j]) + __uint_as_float(o[j]));
+                        }
+                    }
                     if (c + 1 == NCH) {
                         // this warp's share of the accumulator is in registers: hand the buffer back
                         nm_tc_fence_before();
@@ -731,8 +755,8 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     if (warp == 1) {
         __syncwarp();
         nm_tc_fence_after();
-        if constexpr (TWO) nm_tmem_dealloc2(tmem_base, TMEM_COLS);
-        else nm_tmem_dealloc(tmem_base, TMEM_COLS);
+        if constexpr (TWO) nm_tmem_dealloc2(tmem_base, tmem_cols);
+        else nm_tmem_dealloc(tmem_base, tmem_cols);
     }
 }
 

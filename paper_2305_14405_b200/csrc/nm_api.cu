@@ -334,6 +334,8 @@ nm_status nm_linear_dispatch(nm_ctx* ctx, const nm_linear_desc* d, cudaStream_t 
     if (d->algo == 2 || d->algo == 3) return tc ? nm_launch_linear_tc(ctx, d, st, chain) : NM_ERR_UNSUPPORTED;
     // (narrow matrices of more rows than the CUDA-core kernel's grid takes have always been refused)
     if (d->N < 64 && (d->M + 63) / 64 > 65535) return NM_ERR_SHAPE;
+    // (few rows or columns: one MMA step's truncated sum is further from the exact one than 16 FMAs, see steps_like_fma)
+    if (d->in_dtype != NM_I8 && (d->M < 64 || d->N < 64) && d->K <= 16) return nm_launch_linear_simt(ctx, d, st);
     return tc ? nm_launch_linear_tc(ctx, d, st, chain) : nm_launch_linear_simt(ctx, d, st);
 }
 
