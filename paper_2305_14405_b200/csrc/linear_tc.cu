@@ -90,7 +90,7 @@ TileChoice choose(nm_ctx* ctx, const nm_linear_desc* d, bool like_fma, NmChain c
 {
     constexpr bool NARROW = !TcIn<InT>::is_int;   // tiles of 64 and 128 columns are built for the 16-bit types
     const bool whole_chunks = d->N * sizeof(OutT) % 16 == 0;
-    if (d->algo != 0 && whole_chunks)
+    if (nm_algo_forced(d->algo) && whole_chunks)
         return {0, NARROW && d->N <= 64 ? 64 : (NARROW && d->N <= 128 ? 128 : 256), d->algo != 3 && d->M >= 256, 0.0, 0};
     const int bk = ROW_BYTES / (int)sizeof(InT);
     const EpiNeeds epi = {d->slot == NM_SLOT_NONE ? 0 : ctx->h_tables[d->slot].n, d->residual != nullptr, d->bias != nullptr || TcIn<InT>::is_int};
@@ -113,7 +113,7 @@ nm_status launch_sel(nm_ctx* ctx, const nm_linear_desc* d, NmChain chain, cudaSt
 {
     constexpr int64_t CHUNK = 16 / sizeof(OutT);
     // Few rows or columns had the CUDA cores' fp32 FMA chains before the split kernel took them: no sum of theirs gets worse.
-    const bool like_fma = !TcIn<InT>::is_int && d->algo == 0 && (d->M < 64 || d->N < 64);
+    const bool like_fma = !TcIn<InT>::is_int && !nm_algo_forced(d->algo) && (d->M < 64 || d->N < 64);
     const TileChoice c = choose<InT, OutT>(ctx, d, like_fma, chain);
     const int64_t main_n = d->N / CHUNK * CHUNK;
     if (like_fma || main_n == d->N || main_n < 8 || d->acc_dump || d->idx_dump) return launch_choice<InT, OutT>(ctx, d, c, chain, st);
@@ -129,7 +129,7 @@ nm_status launch_sel(nm_ctx* ctx, const nm_linear_desc* d, NmChain chain, cudaSt
     if (d->bias) r.bias = d->bias + main_n;
     if (d->w_scale) r.w_scale = d->w_scale + main_n;
     const TileChoice cm = choose<InT, OutT>(ctx, &m, false, chain), cr = choose<InT, OutT>(ctx, &r, false, chain);
-    if (d->algo == 0 && c.us <= cm.us + cr.us) return launch_choice<InT, OutT>(ctx, d, c, chain, st);
+    if (!nm_algo_forced(d->algo) && c.us <= cm.us + cr.us) return launch_choice<InT, OutT>(ctx, d, c, chain, st);
     const nm_status e = launch_choice<InT, OutT>(ctx, &m, cm, chain, st);
     if (e != NM_OK) return e;
     return launch_choice<InT, OutT>(ctx, &r, cr, chain, st);
