@@ -94,7 +94,8 @@ __global__ void __launch_bounds__(256, MINB) layernorm_kernel(const NmTable* __r
 {
     // A warp walks over rows with a grid-wide stride; the raw 16-byte vectors of its NEXT row are
     // already in flight while the current row is reduced and written, so every SM keeps several
-    // rows per warp outstanding instead of one short-lived row.
+    // rows per warp outstanding instead of one short-lived row.  (Rows of more than 16 vectors per lane are 16 KB and leave
+    // no registers for a second one.)
     constexpr int N = VecOf<T>::N;
     const int lane = threadIdx.x & 31;
     const int64_t warp0 = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -102,7 +103,7 @@ __global__ void __launch_bounds__(256, MINB) layernorm_kernel(const NmTable* __r
     const int nvec = H / N;  // H is a multiple of N
     const float inv_h = tab->inv_h, off = tab->off, nm1 = (float)(tab->n - 1);
     nm_grid_launch_dependents();   // the next kernel may start its set-up
-    constexpr bool GB_REGS = MODE != LN_SMEM, ONE_ROW = MODE == LN_ONE_ROW;
+    constexpr bool GB_REGS = MODE != LN_SMEM, ONE_ROW = MODE == LN_ONE_ROW, NEXT_ROW = !ONE_ROW && ITERS <= 16;
     constexpr int Q = N / 4;           // 16-byte groups of gamma (and of beta) per vector
     extern __shared__ float4 s_gb[];   // LN_SMEM: gamma, then beta: [ITERS][Q][32]
     __shared__ float2 s_tab[MODE != LN_REGS ? NM_MAX_SEGMENTS : 1];
@@ -130,13 +131,16 @@ __global__ void __launch_bounds__(256, MINB) layernorm_kernel(const NmTable* __r
         __syncthreads();
     }
     nm_grid_dependency_wait();     // x comes from the previous kernel
-    uint4 nxt[ITERS];
-    if (warp0 < rows) {
+    uint4 nxt[NEXT_ROW || ONE_ROW ? ITERS : 1];
+    [[maybe_unused]] auto load_row = [&](int64_t row) {
 #pragma unroll
         for (int it = 0; it < ITERS; ++it) {
             const int v = it * 32 + lane;
-            if (v < nvec) nxt[it] = *reinterpret_cast<const uint4*>(x + warp0 * H + v * N);
+            if (v < nvec) nxt[it] = *reinterpret_cast<const uint4*>(x + row * H + v * N);
         }
+    };
+    if constexpr (NEXT_ROW || ONE_ROW) {
+        if (warp0 < rows) load_row(warp0);
     }
     if (!ONE_ROW || !early) fetch_gb();
     if constexpr (MODE == LN_SMEM) {
@@ -150,25 +154,28 @@ __global__ void __launch_bounds__(256, MINB) layernorm_kernel(const NmTable* __r
     for (int64_t row = warp0; row < rows; row += nwarps) {
         float f[ITERS][N];
         float sum = 0.f;
+        if constexpr (!NEXT_ROW && !ONE_ROW) {
+#pragma unroll
+            for (int it = 0; it < ITERS; ++it) {
+                const int v = it * 32 + lane;
+                if (v < nvec) load16<T>(x + row * H + v * N, f[it]);
+            }
+        }
 #pragma unroll
         for (int it = 0; it < ITERS; ++it) {
             const int v = it * 32 + lane;
             if (v < nvec) {
-                const T* e = reinterpret_cast<const T*>(&nxt[it]);
+                if constexpr (NEXT_ROW || ONE_ROW) {
+                    const T* e = reinterpret_cast<const T*>(&nxt[it]);
 #pragma unroll
-                for (int i = 0; i < N; ++i) {
-                    f[it][i] = NmType<T>::to_f(e[i]);
-                    sum += f[it][i];
+                    for (int i = 0; i < N; ++i) f[it][i] = NmType<T>::to_f(e[i]);
                 }
+#pragma unroll
+                for (int i = 0; i < N; ++i) sum += f[it][i];
             }
         }
-        const int64_t nrow = row + nwarps;
-        if (!ONE_ROW && nrow < rows) {
-#pragma unroll
-            for (int it = 0; it < ITERS; ++it) {
-                const int v = it * 32 + lane;
-                if (v < nvec) nxt[it] = *reinterpret_cast<const uint4*>(x + nrow * H + v * N);
-            }
+        if constexpr (NEXT_ROW) {
+            if (row + nwarps < rows) load_row(row + nwarps);
         }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
@@ -295,7 +302,7 @@ nm_status launch_ln(nm_ctx* ctx, const NmTable* tab, const NmTable* tab2, const 
     // launch in a chain, 2.8 so; 37 x 768: 3.2 and 2.3).
     const bool one_row = rows <= (int64_t)ctx->sm_count * (threads / 32) && iters * N <= 32;
     int64_t blocks = (rows + 7) / 8;
- NmLaunchScope scope(ctx, NM_KERNEL_LAYERNORM, 2.0 * (double)rows * H * sizeof(T), st);
+    NmLaunchScope scope(ctx, NM_KERNEL_LAYERNORM, 2.0 * (double)rows * H * sizeof(T), st);
     cudaLaunchConfig_t cfg;
     memset(&cfg, 0, sizeof(cfg));
     cfg.gridDim = dim3((unsigned)blocks);
@@ -310,18 +317,24 @@ nm_status launch_ln(nm_ctx* ctx, const NmTable* tab, const NmTable* tab2, const 
     T* yt = (T*)y;
 #define NM_LN_CASE(I, MODE, MINB)                                                                             \
     do {                                                                                                      \
-        const int64_t cap = (int64_t)ctx->sm_count * MINB;                                                    \
+        const int64_t cap = (int64_t)ctx->sm_count * MINB;                                                 \
         cfg.gridDim = dim3((unsigned)(blocks > cap ? cap : blocks));                                          \
         cfg.dynamicSmemBytes = MODE == LN_SMEM ? (size_t)I * 32 * N * 2 * sizeof(float) : 0;                  \
         cudaLaunchKernelEx(&cfg, layernorm_kernel<T, I, MODE, MINB>, tab, tab2, xt, gamma, beta, yt, rows, H,  \
                            eps, q, q_inv_scale, early ? 1 : 0);                                               \
     } while (0)
-    if constexpr (N == 4) {
-        if (one_row && iters <= 4) NM_LN_CASE(4, LN_ONE_ROW, 1);
-        else if (one_row) NM_LN_CASE(8, LN_ONE_ROW, 1);
+    const auto status = [] { return cudaGetLastError() == cudaSuccess ? NM_OK : NM_ERR_CUDA; };
+    if constexpr (N == 4) {   // fp32: twice the vectors per row
+        if (one_row && iters > 4) {
+            NM_LN_CASE(8, LN_ONE_ROW, 1);
+            return status();
+        }
+        if (iters > 16 && iters <= 32) {
+            NM_LN_CASE(32, LN_SMEM, 1);
+            return status();
+        }
     }
-    if (one_row && N == 4) {}
-    else if (one_row && iters <= 2) NM_LN_CASE(2, LN_ONE_ROW, 1);
+    if (one_row && iters <= 2) NM_LN_CASE(2, LN_ONE_ROW, 1);
     else if (one_row && iters <= 3) NM_LN_CASE(3, LN_ONE_ROW, 1);
     else if (one_row) NM_LN_CASE(4, LN_ONE_ROW, 1);
     else if (small && iters <= 1) NM_LN_CASE(1, LN_REGS, 2);
@@ -335,7 +348,7 @@ nm_status launch_ln(nm_ctx* ctx, const NmTable* tab, const NmTable* tab2, const 
     else if (iters <= 16) NM_LN_CASE(16, LN_SMEM, 1);
     else return NM_ERR_UNSUPPORTED;
 #undef NM_LN_CASE
-    return cudaGetLastError() == cudaSuccess ? NM_OK : NM_ERR_CUDA;
+    return status();
 }
 
 }  // namespace

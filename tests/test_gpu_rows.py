@@ -90,6 +90,53 @@ def test_layernorm_parity(nm, ctx, dtype, rows, H):
         assert_close_bf16(to_np(yd), ref, "layernorm " + dtype)
 
 
+# 1 to 3 vectors per lane with gamma and beta in registers (tensors up to 48 MB, more rows than one per warp) and in shared
+# memory (larger ones, and every row wider than that), up to the widest row
+FORMS = [("bf16", 3001, 136), ("bf16", 2400, 504), ("bf16", 1500, 768), ("f16", 3001, 256), ("f32", 2000, 128), ("f32", 1201, 200), ("f32", 1300, 384),
+         ("bf16", 94003, 256), ("bf16", 47001, 512), ("f16", 31300, 768), ("bf16", 31300, 768), ("f32", 94003, 128), ("f32", 47001, 256), ("f32", 31251, 384),
+         ("bf16", 1301, 1024), ("bf16", 1301, 1536), ("f16", 40, 2048), ("bf16", 1300, 3000), ("f32", 1300, 512), ("f32", 1201, 768), ("f32", 30, 1024), ("f32", 1300, 1000),
+         ("f32", 1300, 1504), ("f32", 70, 2048), ("f32", 1, 2056), ("f32", 1400, 2560), ("f32", 1300, 4096)]
+
+
+@pytest.mark.parametrize("dtype,rows,H", FORMS)
+@pytest.mark.parametrize("two_tables", [False, True])
+def test_layernorm_forms(nm, ctx, dtype, rows, H, two_tables):
+    td = nm_inputs.torch_dtype(dtype)
+    gen = torch.Generator(device="cuda").manual_seed(H)
+    z = (torch.randn((rows, H), generator=gen, device="cuda") * (0.6 + 1.2 * torch.rand((rows, 1), generator=gen, device="cuda")) + 0.3).to(td)
+    g, b = 1 + 0.1 * torch.randn(H, generator=gen, device="cuda"), 0.1 * torch.randn(H, generator=gen, device="cuda")
+    y = torch.full((rows + 1, H), float("nan"), device="cuda").to(td)
+    some = [r for r in range(rows) if r < 40 or r >= rows - 40 or r % 997 == 0]
+    zs, gs, bs = to_np(z[some]), to_np(g), to_np(b)
+    if two_tables:
+        tabs = []
+        for slot, func, (lo, hi) in ((nm.SLOT_USER0, nm.FUNC_SQRT, (0.0625, 9.0)), (nm.SLOT_USER0 + 1, nm.FUNC_RECIP, (0.2, 3.2))):
+            ctx.load_function_table(slot, func, 64, lo, hi)
+            tabs.append(oracle.Table.secant(func, 64, lo, hi))
+        ctx.layernorm_pwl_sqrt_recip(z, g, b, y[:rows], nm.SLOT_USER0, nm.SLOT_USER0 + 1, eps=1e-5)
+        ref = oracle.layernorm_sqrt_recip(zs, gs, bs, 1e-5, *tabs)
+    else:
+        tabs = load_tables_both(ctx, 64, {"rsqrt": RANGES["rsqrt"]})
+        ctx.layernorm_pwl(z, g, b, y[:rows], eps=1e-5)
+        ref = oracle.layernorm(zs, gs, bs, 1e-5, tabs["rsqrt"])
+    ctx.check_device_status()
+    assert torch.isnan(y[rows].float()).all() and not torch.isnan(y[:rows].float()).any()
+    if dtype == "f32":
+        assert_close_f32(to_np(y[some]), ref, "layernorm f32")
+    else:
+        assert_close_bf16(to_np(y[some]), ref, "layernorm " + dtype)
+
+
+@pytest.mark.parametrize("dtype,H", [("f32", 4104), ("bf16", 4104)])
+def test_layernorm_refuses_wider_rows(nm, ctx, dtype, H):
+    load_tables_both(ctx, 64, {"rsqrt": RANGES["rsqrt"]})
+    z = torch.zeros((4, H), device="cuda").to(nm_inputs.torch_dtype(dtype))
+    g = torch.ones(H, device="cuda")
+    with pytest.raises(nm.NmError) as ei:
+        ctx.layernorm_pwl(z, g, g, torch.empty_like(z))
+    assert ei.value.code == 5
+
+
 @pytest.mark.parametrize("dtype,rows,H,n", [("f32", 96, 256, 64), ("bf16", 1024, 768, 64), ("bf16", 333, 1024, 16),
                                             ("f16", 100, 768, 256), ("bf16", 5, 8, 64)])
 def test_layernorm_sqrt_recip_parity(nm, ctx, dtype, rows, H, n):
