@@ -23,15 +23,25 @@ __device__ __forceinline__ void load16(const T* p, float* f)
     for (int i = 0; i < N; ++i) f[i] = NmType<T>::to_f(e[i]);
 }
 
+__device__ __forceinline__ uint32_t pack_pair(float a, float b, __nv_bfloat16)
+{
+    const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
+    return *reinterpret_cast<const uint32_t*>(&h);
+}
+__device__ __forceinline__ uint32_t pack_pair(float a, float b, __half)
+{
+    const __half2 h = __floats2half2_rn(a, b);
+    return *reinterpret_cast<const uint32_t*>(&h);
+}
+// (Two values per conversion: one at a time, bf16 rows spilled and ran at 5.66 TB/s instead of 6.06, 2^19 x 768.)
 template <typename T>
 __device__ __forceinline__ void store16(T* p, const float* f)
 {
-    constexpr int N = VecOf<T>::N;
-    uint4 raw;
-    T* e = reinterpret_cast<T*>(&raw);
-#pragma unroll
-    for (int i = 0; i < N; ++i) e[i] = NmType<T>::from_f(f[i]);
-    *reinterpret_cast<uint4*>(p) = raw;
+    if constexpr (sizeof(T) == 4)
+        *reinterpret_cast<float4*>(p) = make_float4(f[0], f[1], f[2], f[3]);
+    else
+        *reinterpret_cast<uint4*>(p) = make_uint4(pack_pair(f[0], f[1], T()), pack_pair(f[2], f[3], T()), pack_pair(f[4], f[5], T()),
+                                                  pack_pair(f[6], f[7], T()));
 }
 
 // ---- y = k[s]*x + b[s] element-wise (Section 3.2: S, then Y = X.K + B) ----------
@@ -293,10 +303,12 @@ nm_status launch_ln(nm_ctx* ctx, const NmTable* tab, const NmTable* tab2, const 
     const int nvec = H / N;
     const int iters = (nvec + 31) / 32;
     const int threads = 256;
+    // fp32 rows beyond the L2, bound by memory alone, come in three waves of blocks, which even out what the SMs get of it
+    // (2^18 x 768: 269 us in one wave, 257 so; 2^16 x 2048: 185 and 175; 16-bit rows are 1 % slower that way).
     // Tensors that fit the L2 (the encoder's: 16384 x 768 is 25 MB) are latency-bound: gamma and beta in registers, one resident
-    // wave of 2 blocks per SM, 12.8 us for that shape as with 4 blocks and shared memory, and 3.2 against 3.8 for 2331 rows,
-    // which pay for filling it.  Tensors far beyond the L2 want more warps per SM: 284 us at 2^19 x 768 (5.68 TB/s; 291 with
-    // per-row fetches), 182 at 2^18 x 1024 (196); 8192 x 1024: 9.7 (12.4).
+    // wave of 2 blocks per SM (9.1 us for that shape back to back, 3.2 for 2331 rows; shared memory would have to be filled
+    // first).  Tensors far beyond the L2 want more warps per SM: 265 us at 2^19 x 768 (6.07 TB/s; 291 with per-row fetches), 173
+    // at 2^18 x 1024 (196), and so do rows too wide for the registers: 8192 x 1024 7.9 (11.0).
     const bool small = (double)rows * H * sizeof(T) <= 48e6 && iters <= 3;
     // At most one row per warp of one block per SM: bound by latency alone (128 x 1024 bf16 with int8 codes: 4.6 us per
     // launch in a chain, 2.8 so; 37 x 768: 3.2 and 2.3).
@@ -317,7 +329,7 @@ nm_status launch_ln(nm_ctx* ctx, const NmTable* tab, const NmTable* tab2, const 
     T* yt = (T*)y;
 #define NM_LN_CASE(I, MODE, MINB)                                                                             \
     do {                                                                                                      \
-        const int64_t cap = (int64_t)ctx->sm_count * MINB;                                                 \
+        const int64_t cap = (int64_t)ctx->sm_count * MINB * (MODE == LN_SMEM && N == 4 && I <= 16 ? 3 : 1);   \
         cfg.gridDim = dim3((unsigned)(blocks > cap ? cap : blocks));                                          \
         cfg.dynamicSmemBytes = MODE == LN_SMEM ? (size_t)I * 32 * N * 2 * sizeof(float) : 0;                  \
         cudaLaunchKernelEx(&cfg, layernorm_kernel<T, I, MODE, MINB>, tab, tab2, xt, gamma, beta, yt, rows, H,  \
@@ -344,6 +356,7 @@ nm_status launch_ln(nm_ctx* ctx, const NmTable* tab, const NmTable* tab2, const 
     else if (iters <= 2) NM_LN_CASE(2, LN_SMEM, 4);
     else if (iters <= 3) NM_LN_CASE(3, LN_SMEM, 4);
     else if (iters <= 4) NM_LN_CASE(4, LN_SMEM, 3);
+    else if (iters <= 6) NM_LN_CASE(6, LN_SMEM, 2);
     else if (iters <= 8) NM_LN_CASE(8, LN_SMEM, 2);
     else if (iters <= 16) NM_LN_CASE(16, LN_SMEM, 1);
     else return NM_ERR_UNSUPPORTED;
