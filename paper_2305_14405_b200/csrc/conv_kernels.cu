@@ -7,6 +7,8 @@
 // CUDA-core kernels around it: the zero-padded copies that let a few-channel first layer run as an
 // implicit GEMM, the explicit gather (im2col) kept for channel counts the implicit form does not
 // take, and the pools.
+#include <type_traits>
+
 #include "nm_common.cuh"
 
 namespace {
@@ -252,38 +254,50 @@ __device__ __forceinline__ __nv_bfloat162 max2(__nv_bfloat162 a, __nv_bfloat162 
 // The plain window maximum: bound by reading x once, so a thread's arithmetic is kept to packed 16-bit maxima and
 // 32-bit indexes (the maximum of 16-bit values needs no fp32).  One thread per output pixel and 8 channels; a block's
 // threads run along channels, then pixels of one output row, and share the window's columns through L1.
-// 128 x 112 x 112 x 64, 3 x 3 / 2: 105 us with fp32 maxima and 64-bit index divisions, 55 us so.
-template <typename T>
+// 128 x 112 x 112 x 64, 3 x 3 / 2: 106 us with fp32 maxima and 64-bit index divisions, 48 us so.
+// SHORT: rows of at most half a block's work; a block takes as many as it has threads for, of all images' rows one after another
+// (65536 x 2 x 2 x 8, 2 x 2: 49.8 us with a row per block, 2.8 so).
+template <typename T, bool SHORT>
 __global__ void __launch_bounds__(256) maxpool_plain_kernel(const T* __restrict__ x, T* __restrict__ y, int Nb, int H, int W,
                                                             int C, int ks, int stride, int pad, int Ho, int Wo)
 {
     using V2 = typename Vec2<T>::type;
     const uint32_t c8n = (uint32_t)C >> 3;
-    const uint32_t i = blockIdx.x * 256u + threadIdx.x;
-    if (i >= (uint32_t)Wo * c8n) return;
-    const int ox = (int)(i / c8n), c8 = (int)(i - (uint32_t)ox * c8n);
+    const uint64_t row_work = (uint64_t)Wo * c8n;
+    const uint32_t r = SHORT ? threadIdx.x / (uint32_t)row_work : 0u, rows_per_block = SHORT ? 256u / (uint32_t)row_work : 1u;
+    const uint64_t i = (uint64_t)blockIdx.x * 256u + threadIdx.x - r * (uint32_t)row_work;
+    if (r >= rows_per_block || i >= row_work) return;
+    const int ox = row_work >> 32 ? (int)(i / c8n) : (int)((uint32_t)i / c8n), c8 = (int)(i - (uint64_t)ox * c8n);
     const int x0 = max(ox * stride - pad, 0), x1 = min(ox * stride - pad + ks, W);
     const V2 lowest = Vec2<T>::make(-INFINITY, -INFINITY);
-    for (int n = blockIdx.z; n < Nb; n += gridDim.z) {
-        for (int oy = blockIdx.y; oy < Ho; oy += gridDim.y) {
-            const int y0 = max(oy * stride - pad, 0), y1 = min(oy * stride - pad + ks, H);
-            V2 best[4] = {lowest, lowest, lowest, lowest};
-            for (int iy = y0; iy < y1; ++iy) {
-                const T* row = x + ((int64_t)n * H + iy) * W * C + c8 * 8;
+    auto pixel = [&](int n, int oy) {
+        const int y0 = max(oy * stride - pad, 0), y1 = min(oy * stride - pad + ks, H);
+        V2 best[4] = {lowest, lowest, lowest, lowest};
+        for (int iy = y0; iy < y1; ++iy) {
+            const T* row = x + ((int64_t)n * H + iy) * W * C + c8 * 8;
 #pragma unroll 3
-                for (int ix = x0; ix < x1; ++ix) {
-                    const uint4 raw = __ldg(reinterpret_cast<const uint4*>(row + (int64_t)ix * C));
-                    const V2* h = reinterpret_cast<const V2*>(&raw);
+            for (int ix = x0; ix < x1; ++ix) {
+                const uint4 raw = __ldg(reinterpret_cast<const uint4*>(row + (int64_t)ix * C));
+                const V2* h = reinterpret_cast<const V2*>(&raw);
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) best[j] = max2(best[j], h[j]);
-                }
+                for (int j = 0; j < 4; ++j) best[j] = max2(best[j], h[j]);
             }
-            uint4 out;
-            V2* o = reinterpret_cast<V2*>(&out);
-#pragma unroll
-            for (int j = 0; j < 4; ++j) o[j] = best[j];
-            *reinterpret_cast<uint4*>(y + (((int64_t)n * Ho + oy) * Wo + ox) * C + c8 * 8) = out;
         }
+        uint4 out;
+        V2* o = reinterpret_cast<V2*>(&out);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) o[j] = best[j];
+        *reinterpret_cast<uint4*>(y + (((int64_t)n * Ho + oy) * Wo + ox) * C + c8 * 8) = out;
+    };
+    if constexpr (SHORT) {
+        const int64_t rows = (int64_t)Nb * Ho;
+        for (int64_t row = (int64_t)blockIdx.y * rows_per_block + r; row < rows; row += (int64_t)gridDim.y * rows_per_block) {
+            const int n = rows >> 32 ? (int)(row / Ho) : (int)((uint32_t)row / (uint32_t)Ho);
+            pixel(n, (int)(row - (int64_t)n * Ho));
+        }
+    } else {
+        for (int n = blockIdx.z; n < Nb; n += gridDim.z)
+            for (int oy = blockIdx.y; oy < Ho; oy += gridDim.y) pixel(n, oy);
     }
 }
 
@@ -411,9 +425,17 @@ nm_status nm_launch_maxpool(nm_ctx* ctx, const void* x, void* y, nm_dtype dt, in
     const int64_t total = (int64_t)Nb * Ho * Wo * (C / 8);
     NmLaunchScope scope(ctx, NM_KERNEL_POOL, ((double)Nb * H * W * C + (double)Nb * Ho * Wo * C) * nm_dtype_size(dt), st);
     if (!relu) {
-        const dim3 grid((unsigned)(((int64_t)Wo * (C / 8) + 255) / 256), (unsigned)(Ho < 65535 ? Ho : 65535), (unsigned)(Nb < 65535 ? Nb : 65535));
-        if (dt == NM_F16) maxpool_plain_kernel<__half><<<grid, 256, 0, st>>>((const __half*)x, (__half*)y, Nb, H, W, C, ks, stride, pad, Ho, Wo);
-        else maxpool_plain_kernel<__nv_bfloat16><<<grid, 256, 0, st>>>((const __nv_bfloat16*)x, (__nv_bfloat16*)y, Nb, H, W, C, ks, stride, pad, Ho, Wo);
+        const int64_t row_work = (int64_t)Wo * (C / 8), per_block = row_work <= 128 ? 256 / row_work : 1;
+        const int64_t blocks = ((int64_t)Nb * Ho + per_block - 1) / per_block;
+        const dim3 grid = per_block > 1 ? dim3(1, (unsigned)(blocks < 65535 ? blocks : 65535))
+                                        : dim3((unsigned)((row_work + 255) / 256), (unsigned)(Ho < 65535 ? Ho : 65535), (unsigned)(Nb < 65535 ? Nb : 65535));
+        auto go = [&](auto t, auto form) {
+            using T = decltype(t);
+            maxpool_plain_kernel<T, decltype(form)::value><<<grid, 256, 0, st>>>((const T*)x, (T*)y, Nb, H, W, C, ks, stride, pad, Ho, Wo);
+        };
+        auto typed = [&](auto form) { dt == NM_F16 ? go(__half(), form) : go(__nv_bfloat16(), form); };
+        if (per_block > 1) typed(std::true_type());
+        else typed(std::false_type());
         return cudaGetLastError() == cudaSuccess ? NM_OK : NM_ERR_CUDA;
     }
     if (dt == NM_F16)

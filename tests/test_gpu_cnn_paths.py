@@ -81,11 +81,12 @@ def test_halo(nm, ctx, dtype, N, H, W, Cin, Cout, res):
 
 @pytest.mark.parametrize("dtype", [torch.float16, torch.bfloat16])
 @pytest.mark.parametrize("N,H,W,C,ks,stride,pad", [(2, 112, 112, 64, 3, 2, 1), (1, 7, 5, 8, 3, 2, 1), (3, 9, 13, 24, 2, 2, 0), (1, 8, 8, 136, 5, 1, 4),
-                                                   (2, 6, 6, 16, 1, 1, 0), (1, 3, 300, 8, 3, 3, 2)])
+                                                   (2, 6, 6, 16, 1, 1, 0), (1, 3, 300, 8, 3, 3, 2), (65539, 2, 2, 8, 2, 2, 0), (70001, 1, 1, 24, 1, 1, 0),
+                                                   (333, 5, 4, 40, 3, 1, 1), (20, 7, 7, 1024, 7, 1, 0), (2, 70000, 2, 8, 1, 1, 0)])
 def test_maxpool_is_exact(ctx, dtype, N, H, W, C, ks, stride, pad):
     g = torch.Generator(device="cuda").manual_seed(C)
     x = torch.randn((N, H, W, C), generator=g, device="cuda").to(dtype)
-    x[0, 0, 0, 0], x[0, -1, -1, 1], x[0, 1, 1, 2] = float("inf"), float("-inf"), torch.finfo(dtype).min
+    x[0, 0, 0, 0], x[0, -1, -1, 1], x[0, min(1, H - 1), min(1, W - 1), 2] = float("inf"), float("-inf"), torch.finfo(dtype).min
     Ho, Wo = (H + 2 * pad - ks) // stride + 1, (W + 2 * pad - ks) // stride + 1
     y = torch.full((N, Ho, Wo, C), float("nan"), device="cuda").to(dtype)
     ctx.maxpool2d(x, y, ks, stride, pad)
