@@ -206,17 +206,21 @@ nm_status nm_launch_linear_f32(nm_ctx* ctx, const nm_linear_desc* d, cudaStream_
     cfg.stream = st;
     cudaLaunchAttribute attr[2];
     cfg.attrs = attr;
-    int* resident = ctx->f32_resident;   // clusters of 1..8 CTAs the device holds, asked for once per context
-    if (resident[0] == 0) {
+    // clusters of 1..8 CTAs the device holds, asked for once per context (or by several threads, which find the same; the first
+    // word is set when the others are, and orders them for a thread that did not ask)
+    int* resident = ctx->f32_resident;
+    if (__atomic_load_n(&resident[0], __ATOMIC_ACQUIRE) == 0) {
         for (int S = 1; S <= 8; ++S) {
+            int n = 0;
             cfg.numAttrs = split_launch_attrs(ctx, attr, S);
             cfg.gridDim = dim3((unsigned)(S * ctx->sm_count));
-            if (cudaOccupancyMaxActiveClusters(&resident[S], linear_f32_kernel, &cfg) != cudaSuccess) {
+            if (cudaOccupancyMaxActiveClusters(&n, linear_f32_kernel, &cfg) != cudaSuccess) {
                 (void)cudaGetLastError();
-                resident[S] = S == 1 ? ctx->sm_count : 0;
+                n = S == 1 ? ctx->sm_count : 0;
             }
+            __atomic_store_n(&resident[S], n, __ATOMIC_RELAXED);
         }
-        resident[0] = 1;
+        __atomic_store_n(&resident[0], 1, __ATOMIC_RELEASE);
     }
     s.S = choose_f32_split(tiles, a.num_k_blocks, resident);
     cfg.numAttrs = split_launch_attrs(ctx, attr, s.S);

@@ -86,3 +86,23 @@ def test_the_plain_kernels_can_be_forced(nm, ctx):
         ctx.attention_pwl(qkv, att[algo], 1, 128, 1, 64, algo=algo)
     ctx.check_device_status()
     assert not torch.equal(*lin) and not torch.equal(*att)
+
+
+def test_first_calls_from_several_threads(nm):
+    """The first fp32 products of a context, on a stream per thread."""
+    import threading
+    ctx = nm.Context(0)
+    try:
+        A, W = [torch.from_numpy(nm_inputs.matrix(s, 3, "f32", 1.0)).cuda() for s in ((100, 768), (768, 768))]
+        outs = [torch.zeros(100, 768, device="cuda") for _ in range(8)]
+        streams = [torch.cuda.Stream() for _ in outs]
+        torch.cuda.synchronize()
+        threads = [threading.Thread(target=lambda o=o, s=s: ctx.linear_pwl(A, W, o, stream=s)) for o, s in zip(outs, streams)]
+        for t in threads:
+            t.start()
+        for t in threads:
+            t.join()
+        torch.cuda.synchronize()
+        assert all(torch.equal(o, outs[0]) for o in outs) and outs[0].abs().sum() > 0
+    finally:
+        ctx.close()
