@@ -135,9 +135,16 @@ nm_status nm_pwl_apply(nm_ctx* ctx, int slot, const void* x, void* y, int64_t co
  *   acc_dump / idx_dump: device int32[M*N] (row-major, ld N) or NULL: the raw
  *   accumulators and the segment numbers, for bit-exact checks.
  * All pointers 16-byte aligned, lda/ldw/ldo/ldr multiples of 16 bytes.
- * algo: 0 = pick; 1 = force the plain SIMT kernel; 2 = force the tcgen05 kernel
- * (NM_ERR_UNSUPPORTED if the shape or dtype has none); 3 = tcgen05 with one CTA per
- * tile even where the two-CTA (cta_group::2) tile would be chosen. */
+ * algo: 0 = pick; 1 = force the plain SIMT kernel; 2 = force the persistent tcgen05
+ * kernel (NM_ERR_UNSUPPORTED if the shape or dtype has none); 3 = the same with one CTA per
+ * tile even where the two-CTA (cta_group::2) tile would be chosen; NM_ALGO_SPLIT(ctas, columns) =
+ * force the tcgen05 kernel that splits K over a cluster of 1, 2, 4 or 8 CTAs, tiles of 32 or 64
+ * columns (NM_ERR_UNSUPPORTED likewise, and if K has fewer 128-byte blocks than CTAs).  With 2 and 3 the last
+ * 4 to 12 columns of rows that are no multiple of 16 bytes go to that kernel too.
+ * Picked for fp32: a tiled CUDA-core kernel where N is a multiple of 4, else the plain one.  Picked for 16-bit types:
+ * a tcgen05 kernel where K is a multiple of 8 and N of 4 and at least 8; sums with M < 64 or N < 64 are no less
+ * accurate than a chain of fp32 FMAs. */
+#define NM_ALGO_SPLIT(ctas, columns) (0x1000 | (ctas) | ((columns) << 4))
 typedef struct {
     int64_t M, N, K;
     nm_dtype in_dtype;
@@ -175,9 +182,11 @@ nm_status nm_linear_pwl(nm_ctx* ctx, const nm_linear_desc* desc, void* stream);
  * [B*L, 3*heads*d] projection.  out: device [B*L, heads*d], leading dimension
  * heads*d.  dtype F32, BF16 or F16 (fp32 arithmetic inside).  scale must be positive and finite
  * (NM_ERR_INVALID_ARG otherwise).
- * algo: 0 = pick; 1 = CUDA-core kernel; 2 = tensor-core kernel that streams K and V and computes
- * Q K^T twice (d = 64, L a multiple of 128); 3 = tensor-core kernel that keeps the whole score block
- * in tensor memory (d = 64, L in {128, 256, 384, 512}). */
+ * algo: 0 = pick; 1 = the plain CUDA-core kernel; 2 = tensor-core kernel that streams K and V (d = 64, L a multiple
+ * of 128); 3 = tensor-core kernel that keeps the whole score block in tensor memory (d = 64, L in {128, 256, 384, 512}).
+ * Picked for d = 64: fp32 a tiled CUDA-core kernel as long as 32 rows of scores fit shared memory (L up to 1408);
+ * 16-bit types the streaming kernel at any L.  At multiples of 128 it rounds the probabilities e_j to the storage type
+ * before the second product; at other lengths they keep 24 bits (fp16: 22), and all sums are fp32 everywhere. */
 typedef struct {
     int32_t B, L, heads, d;
     nm_dtype dtype;

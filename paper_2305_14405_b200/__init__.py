@@ -20,6 +20,13 @@ F32, BF16, F16, I8 = 0, 1, 2, 3
 SLOT_NONE, SLOT_GELU, SLOT_EXP, SLOT_RECIP, SLOT_RSQRT, SLOT_RELU, SLOT_USER0 = -1, 0, 1, 2, 3, 4, 5
 FUNC_GELU, FUNC_EXP, FUNC_RECIP, FUNC_RSQRT, FUNC_RELU, FUNC_SQRT, FUNC_IDENTITY = range(7)
 ALGO_AUTO, ALGO_SIMT, ALGO_TC, ALGO_TC_1CTA = 0, 1, 2, 3
+
+
+def algo_split(ctas, columns):
+    """NM_ALGO_SPLIT: forces the linear operator's or convolution's split-K kernel."""
+    return 0x1000 | ctas | columns << 4
+
+
 ALGO_ATTN_RESIDENT = 3   # attention only: the kernel that keeps the score block in tensor memory
 STATIC_WS_BYTES = 32 << 20
 

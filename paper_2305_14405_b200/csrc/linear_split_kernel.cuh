@@ -546,6 +546,13 @@ inline int split_stages(int BN, int S, int64_t ctas, int sms, bool back_to_back)
     return BN == 64 ? (split_alone(S, ctas, sms) ? 5 : 3) : (split_alone(S, ctas, sms) ? 6 : 4);
 }
 
+// The form NM_ALGO_SPLIT asks for; S = -1 if K has too few K-blocks for it.
+inline TileChoice forced_split(int32_t algo, int64_t k_blocks)
+{
+    const int S = algo & 15;
+    return {S <= k_blocks ? S : -1, (algo & 0xff0) >> 4, false, 0.0, 0};
+}
+
 inline TileChoice choose_tile(int64_t rows, int64_t m_tiles, int64_t N, int64_t k_blocks, bool narrow_tiles, const EpiNeeds& epi, bool only64,
                               bool whole_chunks, bool like_fma, NmChain chain, int sms)
 {

@@ -83,16 +83,17 @@ nm_status launch_split(nm_ctx* ctx, const nm_linear_desc* d, const TileChoice& c
     return launch_split_kernel<InT, OutT, BN, false>(ctx, tmA, tmW, s, chain.back_to_back, 2.0 * (double)d->M * (double)d->N * (double)d->K, st);
 }
 
-// Kernel and tile for d: the cheapest by the model (like_fma: with accumulators as good as a chain of fp32 FMAs), or (algo 2, 3) a forced one: the persistent kernel with a tile by the width
+// Kernel and tile for d: the cheapest by the model (like_fma: with accumulators as good as a chain of fp32 FMAs), or a forced one, with algo 2 and 3 the persistent kernel with a tile by the width
 // alone; algo 3 asks for one CTA per tile, otherwise CTA pairs from one 256-row tile on.
 template <typename InT, typename OutT>
 TileChoice choose(nm_ctx* ctx, const nm_linear_desc* d, bool like_fma, NmChain chain)
 {
     constexpr bool NARROW = !TcIn<InT>::is_int;   // tiles of 64 and 128 columns are built for the 16-bit types
     const bool whole_chunks = d->N * sizeof(OutT) % 16 == 0;
+    const int bk = ROW_BYTES / (int)sizeof(InT);
+    if (nm_algo_is_split(d->algo)) return forced_split(d->algo, (d->K + bk - 1) / bk);
     if (nm_algo_forced(d->algo) && whole_chunks)
         return {0, NARROW && d->N <= 64 ? 64 : (NARROW && d->N <= 128 ? 128 : 256), d->algo != 3 && d->M >= 256, 0.0, 0};
-    const int bk = ROW_BYTES / (int)sizeof(InT);
     const EpiNeeds epi = {d->slot == NM_SLOT_NONE ? 0 : ctx->h_tables[d->slot].n, d->residual != nullptr, d->bias != nullptr || TcIn<InT>::is_int};
     return choose_tile(d->M, (d->M + BM - 1) / BM, d->N, (d->K + bk - 1) / bk, NARROW, epi, false, whole_chunks, like_fma, chain, ctx->sm_count);
 }
@@ -116,7 +117,8 @@ nm_status launch_sel(nm_ctx* ctx, const nm_linear_desc* d, NmChain chain, cudaSt
     const bool like_fma = !TcIn<InT>::is_int && !nm_algo_forced(d->algo) && (d->M < 64 || d->N < 64);
     const TileChoice c = choose<InT, OutT>(ctx, d, like_fma, chain);
     const int64_t main_n = d->N / CHUNK * CHUNK;
-    if (like_fma || main_n == d->N || main_n < 8 || d->acc_dump || d->idx_dump) return launch_choice<InT, OutT>(ctx, d, c, chain, st);
+    if (c.S < 0) return NM_ERR_UNSUPPORTED;
+    if (like_fma || nm_algo_is_split(d->algo) || main_n == d->N || main_n < 8 || d->acc_dump || d->idx_dump) return launch_choice<InT, OutT>(ctx, d, c, chain, st);
     // A row that is no multiple of 16 bytes: all of it by the split kernel, or the last 4 to 12 columns by the split kernel and the
     // others by themselves, whichever the model finds cheaper (16384 x 1004 x 1024: 58.4 us and 38.5); with dumps, whose
     // row is N, the former.

@@ -331,7 +331,7 @@ nm_status nm_linear_dispatch(nm_ctx* ctx, const nm_linear_desc* d, cudaStream_t 
     if (!nm_algo_forced(d->algo) && nm_linear_f32_supported(d)) return nm_launch_linear_f32(ctx, d, st);
     if (d->algo == 1) return nm_launch_linear_simt(ctx, d, st);
     const bool tc = nm_linear_tc_supported(d);
-    if (d->algo == 2 || d->algo == 3) return tc ? nm_launch_linear_tc(ctx, d, st, chain) : NM_ERR_UNSUPPORTED;
+    if (d->algo == 2 || d->algo == 3 || nm_algo_is_split(d->algo)) return tc ? nm_launch_linear_tc(ctx, d, st, chain) : NM_ERR_UNSUPPORTED;
     // (narrow matrices of more rows than the CUDA-core kernel's grid takes have always been refused)
     if (d->N < 64 && (d->M + 63) / 64 > 65535) return NM_ERR_SHAPE;
     // (few rows or columns: one MMA step's truncated sum is further from the exact one than 16 FMAs, see steps_like_fma)
@@ -371,7 +371,7 @@ static nm_status attention_dispatch(nm_ctx* ctx, const nm_attn_desc* d, void* st
     // equals the maximum of the scaled scores only for a positive scale
     if (!(d->scale > 0.0f) || !isfinite(d->scale)) return NM_ERR_INVALID_ARG;
     cudaStream_t st = (cudaStream_t)stream;
-    if (!nm_algo_forced(d->algo) && nm_attention_f32_supported(d)) {
+    if ((d->algo < 1 || d->algo > 3) && nm_attention_f32_supported(d)) {
         const nm_status s = nm_launch_attention_f32(ctx, d, st);
         if (s != NM_ERR_UNSUPPORTED) return s;
     }

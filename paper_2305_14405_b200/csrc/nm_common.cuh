@@ -679,8 +679,13 @@ nm_status nm_launch_layernorm(nm_ctx* ctx, const void* x, const float* gamma, co
 nm_status nm_launch_wait_selftest(nm_ctx* ctx, long long limit_cycles, cudaStream_t st);
 nm_status nm_launch_quantize(nm_ctx* ctx, const void* x, nm_dtype dtype, int64_t count, float inv_scale,
                              int8_t* q, cudaStream_t st);
-// algo 1, 2 and 3 of a descriptor force a kernel, anything else leaves the choice to the library
-static inline bool nm_algo_forced(int32_t algo) { return algo >= 1 && algo <= 3; }
+// algo 1, 2, 3 and NM_ALGO_SPLIT of a descriptor force a kernel, anything else leaves the choice to the library
+static inline bool nm_algo_is_split(int32_t algo)
+{
+    const int S = algo & 15, BN = (algo & 0xff0) >> 4;
+    return (algo & ~0xfff) == 0x1000 && (S == 1 || S == 2 || S == 4 || S == 8) && (BN == 32 || BN == 64);
+}
+static inline bool nm_algo_forced(int32_t algo) { return (algo >= 1 && algo <= 3) || nm_algo_is_split(algo); }
 nm_status nm_launch_linear_simt(nm_ctx* ctx, const nm_linear_desc* d, cudaStream_t st);
 nm_status nm_launch_linear_f32(nm_ctx* ctx, const nm_linear_desc* d, cudaStream_t st);
 bool nm_linear_f32_supported(const nm_linear_desc* d);   // fp32, N a multiple of 4; linear_simt takes the rest

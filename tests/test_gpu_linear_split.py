@@ -66,6 +66,41 @@ def test_16_bit(nm, ctx, dtype, M, N, K, epi, algo=0):
     assert np.all(np.abs(got - ref) <= half_ulp * 1.01 * np.abs(ref) + 1e-5 * max(rms, 1.0)), np.abs(got - ref).max()
 
 
+@pytest.mark.parametrize("dtype", ["bf16", "f16"])
+@pytest.mark.parametrize("S", [1, 2, 4, 8])
+@pytest.mark.parametrize("BN", [32, 64])
+@pytest.mark.parametrize("M,N,K,epi", [(1, 36, 520, "bias_res"), (37, 100, 1032, "gelu_bias"), (127, 64, 512, "plain"), (130, 196, 904, "relu_res_first")])
+def test_every_form_16_bit(nm, ctx, dtype, S, BN, M, N, K, epi):
+    """Every cluster size and width of the kernel: fewer rows than CTAs, a row less than a tile and two more, columns and K ragged."""
+    test_16_bit(nm, ctx, dtype, M, N, K, epi, nm.algo_split(S, BN))
+
+
+@pytest.mark.parametrize("out", ["bf16", "i8", "f32"])
+@pytest.mark.parametrize("S", [1, 2, 4, 8])
+@pytest.mark.parametrize("BN", [32, 64])
+@pytest.mark.parametrize("M,N,K", [(1, 36, 1040), (37, 100, 2000), (127, 64, 1024), (130, 196, 1808)])
+def test_every_form_int8(nm, ctx, out, S, BN, M, N, K):
+    test_int8_bit_exact(nm, ctx, M, N, K, out, nm.algo_split(S, BN))
+
+
+@pytest.mark.parametrize("S", [1, 2, 4, 8])
+@pytest.mark.parametrize("BN", [32, 64])
+@pytest.mark.parametrize("N,H,Cin,Cout,k,stride,pad,res", [(1, 13, 64, 72, 3, 1, 1, True), (3, 9, 64, 200, 3, 2, 1, False), (2, 7, 512, 40, 1, 2, 0, True)])
+def test_every_form_convolution(nm, ctx, S, BN, N, H, Cin, Cout, k, stride, pad, res):
+    test_convolution(nm, ctx, N, H, Cin, Cout, k, stride, pad, res, nm.algo_split(S, BN))
+
+
+def test_forced_forms_are_refused_where_they_do_not_fit(nm, ctx):
+    A, W = [torch.zeros(s, dtype=torch.bfloat16, device="cuda") for s in ((8, 256), (64, 256))]   # four K-blocks
+    out = torch.zeros(8, 64, dtype=torch.bfloat16, device="cuda")
+    with pytest.raises(nm.NmError) as ei:
+        ctx.linear_pwl(A, W, out, algo=nm.algo_split(8, 64))
+    assert ei.value.code == 5
+    with pytest.raises(nm.NmError) as ei:
+        ctx.linear_pwl(A.float(), W.float(), out.float(), algo=nm.algo_split(1, 64))
+    assert ei.value.code == 5
+
+
 @pytest.mark.parametrize("algo", [0, 2, 3])
 @pytest.mark.parametrize("M,N,K", [(40, 8, 64), (130, 12, 72), (300, 60, 64), (300, 68, 128), (513, 132, 136), (700, 260, 64), (9000, 1004, 64)])
 def test_rows_that_are_no_multiple_of_16_bytes(nm, ctx, M, N, K, algo):
@@ -114,7 +149,7 @@ def test_int8_bit_exact(nm, ctx, M, N, K, out, algo=0):
 @pytest.mark.parametrize("N,H,Cin,Cout,k,stride,pad,res", [(1, 14, 256, 256, 3, 1, 1, False), (1, 7, 512, 512, 3, 1, 1, False),
                                                            (2, 7, 512, 72, 1, 2, 0, False), (1, 56, 64, 64, 3, 1, 1, True),
                                                            (3, 9, 64, 200, 3, 2, 1, True)])
-def test_convolution(nm, ctx, N, H, Cin, Cout, k, stride, pad, res):
+def test_convolution(nm, ctx, N, H, Cin, Cout, k, stride, pad, res, forced=0):
     """The split kernel's implicit GEMM against the explicit gather on the CUDA cores."""
     ctx.load_function_table(nm.SLOT_RELU, nm.FUNC_RELU, 2, -8.0, 8.0)
     g = torch.Generator(device="cuda").manual_seed(H + Cin)
@@ -124,7 +159,7 @@ def test_convolution(nm, ctx, N, H, Cin, Cout, k, stride, pad, res):
     Ho = (H + 2 * pad - k) // stride + 1
     r = torch.randn((N, Ho, Ho, Cout), generator=g, device="cuda").half() if res else None
     outs = []
-    for algo in (nm.ALGO_AUTO, nm.ALGO_SIMT):
+    for algo in (forced, nm.ALGO_SIMT):
         out = torch.full((N, Ho, Ho, Cout), float("nan"), device="cuda").half()
         d = ctx.conv_desc(x, w, out, stride, pad, bias=b, residual=r, slot=nm.SLOT_RELU, res_first=res, algo=algo)
         ctx.conv2d_pwl(d, torch.empty(max(256, ctx.conv2d_workspace_bytes(d)), dtype=torch.uint8, device="cuda"))
