@@ -200,7 +200,7 @@ nm_status launch_sel(nm_ctx* ctx, const NmConvTc* c, NmChain chain, cudaStream_t
         }
         t = choose_tile((int64_t)c->N * c->Ho * c->Wo, patches, c->Cout, (int64_t)c->taps_y * c->taps_x * c->cblocks, true,
                         EpiNeeds{c->slot == NM_SLOT_NONE ? 0 : ctx->h_tables[c->slot].n, c->residual != nullptr, c->bias != nullptr},
-                        c->depthwise != 0, true, false, chain, ctx->sm_count);
+                        c->depthwise != 0, true, 0, chain, ctx->sm_count);
     } else if (nm_algo_is_split(c->algo)) {
         t = forced_split(c->algo, (int64_t)c->taps_y * c->taps_x * c->cblocks);
         if (t.S < 0) return NM_ERR_UNSUPPORTED;

@@ -290,7 +290,8 @@ linear_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         // what the others will send: their columns of each of this CTA's rows
         if (S > 1) nm_mbar_expect_tx(&bar_part, (uint32_t)((rows - rank + S - 1) / S) * (uint32_t)(S - 1) * BN * 4u);
     }
-    const uint32_t tmem_cols = INT ? BN : a.accs <= 1 ? BN : a.accs <= 2 ? 2 * BN : a.accs <= 4 ? 4 * BN : 8 * BN;
+    constexpr bool MULTI = !INT && !CONV;   // several accumulators (TcArgs::acc_steps)
+    const uint32_t tmem_cols = !MULTI ? BN : a.accs <= 1 ? BN : a.accs <= 2 ? 2 * BN : a.accs <= 4 ? 4 * BN : 8 * BN;
     if (warp == 1) {
         nm_tmem_alloc(&tmem_slot, tmem_cols);
         nm_tmem_relinquish();
@@ -386,7 +387,7 @@ linear_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
             bool ready = false;
             [[maybe_unused]] uint32_t acc = tmem;
             [[maybe_unused]] int left = a.acc_steps;   // steps that the accumulator still takes (0: no limit)
-            [[maybe_unused]] uint32_t accum = 0;
+            [[maybe_unused]] uint32_t accum_on = 0;
             for (int kb = kb0; kb < kb1; ++kb) {
                 if (!ready && !vote(nm_mbar_wait(&bar_full[stage], phase, abortp, a.status))) { ok = false; break; }
                 if constexpr (ONE_LANE) {   // look at the next stage while this one's MMAs are issued
@@ -399,15 +400,15 @@ linear_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                 if (ONE_LANE || nm_elect_one()) {
 #pragma unroll
                     for (int k = 0; k < 4; ++k) {  // 4 x 32 bytes of K per 128-byte row
-                        if constexpr (INT) {
-                            nm_mma_i8(tmem, adesc + 2 * k, bdesc + 2 * k, IDESC, (kb != kb0 || k != 0) ? 1u : 0u);
-                        } else {
-                            nm_mma_f16(acc, adesc + 2 * k, bdesc + 2 * k, IDESC, accum);
-                            accum = 1u;
+                        const uint32_t accum = MULTI ? accum_on : (kb != kb0 || k != 0) ? 1u : 0u;
+                        if constexpr (INT) nm_mma_i8(tmem, adesc + 2 * k, bdesc + 2 * k, IDESC, accum);
+                        else nm_mma_f16(MULTI ? acc : tmem, adesc + 2 * k, bdesc + 2 * k, IDESC, accum);
+                        if constexpr (MULTI) {
+                            accum_on = 1u;
                             if (--left == 0) {
                                 acc += BN;
                                 left = a.acc_steps;
-                                accum = 0u;
+                                accum_on = 0u;
                             }
                         }
                     }
@@ -433,13 +434,13 @@ linear_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         uint32_t* mine = part + (((rank * BM + row) >> (31 - __clz(S))) * PITCH + c0);   // the row's place, in the owner
         const uint32_t t_addr = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)c0;
         const uint32_t dst = nm_mapa(nm_smem_u32(mine), (uint32_t)owner), bar = nm_mapa(nm_smem_u32(&bar_part), (uint32_t)owner);
-        const int used = a.acc_steps ? (4 * (kb1 - kb0) + a.acc_steps - 1) / a.acc_steps : 1;   // this CTA's accumulators
+        const int used = MULTI && a.accs > 1 ? (4 * (kb1 - kb0) + a.acc_steps - 1) / a.acc_steps : 1;   // this CTA's accumulators
         if (ok && q * 32 < rows) {
 #pragma unroll
             for (int c = 0; c < BN / 2; c += 16) {
                 uint32_t r[16];
                 nm_tmem_ld16_sync(t_addr + (uint32_t)c, r);
-                if constexpr (!INT) {
+                if constexpr (MULTI) {
                     for (int i = 1; i < used; ++i) {
                         uint32_t o[16];
                         nm_tmem_ld16_sync(t_addr + (uint32_t)(i * BN + c), o);
@@ -459,8 +460,11 @@ linear_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
             }
         }
     }
+    // The rows of other CTAs: one thread acquires them, at cluster scope, and hands them on through the block's barrier (256
+    // threads that each acquire at cluster scope cost 0.13 us a launch: int8 24 layers, 128 tokens 878 -> 890 us).
+    if (S > 1 && ok && threadIdx.x == 0) (void)nm_mbar_wait_cluster(&bar_part, 0, abortp, a.status);
     __syncthreads();
-    if (S > 1 && ok && !nm_mbar_wait_cluster(&bar_part, 0, abortp, a.status)) ok = false;   // (other CTAs wrote the rows)
+    ok = ok && !abort_flag;
 
     if (ok) fin.run(part, s_tab);
 
@@ -504,13 +508,16 @@ inline unsigned split_launch_attrs(const nm_ctx* ctx, cudaLaunchAttribute* attr,
 //   split kernel, n CTAs: base with the epilogue of the rows that exist + the K-blocks beyond those in flight at once (more when
 //     CTAs share an SM) + the exchange.
 //   Between kernels that are no matrix products the persistent kernel's longer set-up and tail overlap less, 0.4 us (11 layers, 128
-//   tokens: 497 us without it, 437 with).  A CNN's launches stand back to back and begin while their predecessor drains: there every
+//   tokens: 497 us without it, 437 with), and by how much depends on the tile: fitted to encoders of 300 to 12800 rows with each of
+//   their four products on each tile, the picked one is 0.27 us behind the best there, 0.64 without.  A CNN's launches stand back to back and begin while their predecessor drains: there every
 //   round counts with its epilogue and narrow tiles do better than alone, so they have a row of parameters of their own (ResNet-50 batch
 //   13: 624 us, 657 with the other row; batch 23: 747 and 782).  There, and among the split kernel's widths, the wider tile wins
 //   within 3 %: it leaves more SMs to the neighbours.  Elsewhere the split kernel wins within 3 % (37 x 2304 x 768: 4.6 us, 5.4 on
 //   persistent tiles).
 // E.g. 128 x 768 x 3072: 13.4 us in one round of the best persistent tile, 7.0 split over 8; 1024 x 768 x 768: 5.9 with 128 x 64
 // tiles, 9.8 with 256 x 256 pairs.
+// `fma_steps`: 0, or the K-steps of 16 of a sum that is to be as good as a chain of FMAs (steps_like_fma; each further
+// accumulator costs 0.3 us, 0.9 between other kernels, which wait for its tensor memory).
 // `whole_chunks`: a row of the output is a multiple of 16 bytes.  The persistent kernel stores through a tensor map, which
 // writes whole 16-byte chunks and would reach beyond a row that is not; the split kernel stores four columns at a time.
 struct TileChoice {
@@ -525,9 +532,9 @@ struct TileChoice {
 // fp32 FMAs.  The tensor core truncates the sum at every step: measured against float64, a chain of n steps is off by 1.55e-8 n of
 // the sum's rms, a chain of K FMAs by 7.4e-9 sqrt(K) = 3.0e-8 sqrt(steps) (bf16, K 16 to 4096: 2.1e-8, 6.6e-8, 2.4e-7, 7.3e-7, 3.3e-6,
 // 4.4e-6 for one accumulator at K 16, 64, 256, 768, 3072, 4096; FMAs 1.9e-8, 5.1e-8, 1.1e-7, 2.1e-7, 5.2e-7, 6.0e-7).
-inline int steps_like_fma(int64_t k_blocks)
+inline int steps_like_fma(int64_t k_steps)
 {
-    const int n = (int)(1.5 * sqrt(4.0 * (double)k_blocks) - 1.0);
+    const int n = (int)((k_steps < 32 ? 1.4 : 1.75) * sqrt((double)k_steps) - 0.1);
     return n < 1 ? 1 : n;
 }
 constexpr int SPLIT_ACC_COLS = 256;   // tensor-memory columns of a CTA: two of them share an SM
@@ -554,7 +561,7 @@ inline TileChoice forced_split(int32_t algo, int64_t k_blocks)
 }
 
 inline TileChoice choose_tile(int64_t rows, int64_t m_tiles, int64_t N, int64_t k_blocks, bool narrow_tiles, const EpiNeeds& epi, bool only64,
-                              bool whole_chunks, bool like_fma, NmChain chain, int sms)
+                              bool whole_chunks, int64_t fma_steps, NmChain chain, int sms)
 {
     const bool has_table = epi.n_seg > 0;
     struct P { int BN; bool two; double base, lone, busy, round, round_table, table, fill; };
@@ -572,9 +579,9 @@ inline TileChoice choose_tile(int64_t rows, int64_t m_tiles, int64_t N, int64_t 
         if (narrow_tiles && p.BN > 64 && N <= p.BN / 2) continue;   // half the tile would be padding
         if (ring_stages(p.BN, p.two, epi) < 2) continue;            // no room beside a large table
         const int64_t tiles = (p.two ? (m_tiles + 1) / 2 : m_tiles) * ((N + p.BN - 1) / p.BN), slots = p.two ? sms / 2 : sms;
-        // (like_fma: the 64-column tiles have room for up to four accumulators in each of their two buffers)
-        const int steps = like_fma ? steps_like_fma(k_blocks) : 0;
-        if (like_fma && (p.BN != 64 || 4 * k_blocks > 4 * steps)) continue;
+        // (the 64-column tiles have room for up to four accumulators in each of their two buffers)
+        const int steps = fma_steps ? steps_like_fma(fma_steps) : 0;
+        if (fma_steps && (p.BN != 64 || 4 * k_blocks > 4 * steps)) continue;
         double t;
         if (in_cnn) {
             const J& j = joined[i];
@@ -590,7 +597,9 @@ inline TileChoice choose_tile(int64_t rows, int64_t m_tiles, int64_t N, int64_t 
             const double full = (double)(tiles / slots), part = (double)(tiles % slots) / slots, k = (double)k_blocks;
             const double epilogue = p.round + (has_table ? p.round_table : 0.0), busy = k * p.busy, some = k * (p.lone + (p.busy - p.lone) * part);
             t = p.base + full * (busy > epilogue ? busy : epilogue) + (part > 0.0 ? (full > 0.0 && some < epilogue ? epilogue : some) : 0.0) +
-                (has_table ? p.table : 0.0) + p.fill * (full > 0.0 ? 1.0 : part) + (chain.weights_ready ? 0.4 : 0.0);
+                (has_table ? p.table : 0.0) + p.fill * (full > 0.0 ? 1.0 : part);
+            if (chain.weights_ready)
+                t += 0.8 + (p.BN == 256 ? (has_table ? 1.5 : 0.5) : p.BN == 64 ? (has_table ? -0.8 : -0.4) : has_table || (epi.res && !p.two) ? 0.4 : -0.4);
         }
         if (t < best.us * (in_cnn ? 0.97 : 1.0)) best = {0, p.BN, p.two, t, steps};
     }
@@ -599,11 +608,11 @@ inline TileChoice choose_tile(int64_t rows, int64_t m_tiles, int64_t N, int64_t 
         const int64_t tiles = m_tiles * ((N + BN - 1) / BN);
         for (int S = 1; S <= 8 && S <= k_blocks; S *= 2) {
             const int64_t n = tiles * S;
-            if (n > 0x7fffffffLL || (n > 2 * sms && (like_fma ? best.us < 1e30 : whole_chunks || S > 1))) break;
+            if (n > 0x7fffffffLL || (n > 2 * sms && (fma_steps ? best.us < 1e30 : whole_chunks || S > 1))) break;
             int steps = 0;
-            if (like_fma) {
+            if (fma_steps) {
                 const int64_t mine = 4 * ((k_blocks + S - 1) / S), most = SPLIT_ACC_COLS / BN;
-                steps = steps_like_fma(k_blocks);
+                steps = steps_like_fma(fma_steps);
                 if (mine > steps * most) {
                     // (more than 150 000 K-elements: nothing does, and the last form takes longer chains)
                     if (BN > 32 || best.us < 1e30 || (S < 8 && 2 * S <= k_blocks)) continue;
@@ -614,7 +623,8 @@ inline TileChoice choose_tile(int64_t rows, int64_t m_tiles, int64_t N, int64_t 
             const double t = 4.29 + 0.73 * tile_rows * BN / 64 + 0.038 * per +
                              (BN == 64 ? 0.235 : 0.179) * (beyond > 0 ? beyond : 0) * (share > 1 ? share : 1) +
                              (S == 1 ? 0.0 : S == 2 ? 0.21 : S == 4 ? 0.26 : 0.56) +
-                             (0.35 * (share < 1 ? share : 1) + 0.85 * (share > 1 ? share - 1 : 0)) * BN / 32 + (has_table ? 0.42 * BN / 64 : 0.0);
+                             (0.35 * (share < 1 ? share : 1) + 0.85 * (share > 1 ? share - 1 : 0)) * BN / 32 + (has_table ? 0.42 * BN / 64 : 0.0) +
+                             (steps ? (chain.weights_ready ? 0.9 : 0.3) * (double)(int)((4.0 * per - 1.0) / steps) : 0.0);
             if (t < best.us * (in_cnn || best.S ? 0.97 : 1.03)) best = {S, BN, false, t, steps};
         }
     }

@@ -95,7 +95,8 @@ TileChoice choose(nm_ctx* ctx, const nm_linear_desc* d, bool like_fma, NmChain c
     if (nm_algo_forced(d->algo) && whole_chunks)
         return {0, NARROW && d->N <= 64 ? 64 : (NARROW && d->N <= 128 ? 128 : 256), d->algo != 3 && d->M >= 256, 0.0, 0};
     const EpiNeeds epi = {d->slot == NM_SLOT_NONE ? 0 : ctx->h_tables[d->slot].n, d->residual != nullptr, d->bias != nullptr || TcIn<InT>::is_int};
-    return choose_tile(d->M, (d->M + BM - 1) / BM, d->N, (d->K + bk - 1) / bk, NARROW, epi, false, whole_chunks, like_fma, chain, ctx->sm_count);
+    return choose_tile(d->M, (d->M + BM - 1) / BM, d->N, (d->K + bk - 1) / bk, NARROW, epi, false, whole_chunks, like_fma ? (d->K + 15) / 16 : 0, chain,
+                       ctx->sm_count);
 }
 
 template <typename InT, typename OutT>
