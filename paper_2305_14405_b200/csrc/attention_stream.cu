@@ -126,38 +126,6 @@ template <> struct ProbTerms<__half> {
     }
 };
 
-// 16 packed words of this thread's row into 16 consecutive tensor-memory columns (the mirror of the 16-column read)
-__device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t* r)
-{
-    asm volatile(
-        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], "
-        "{%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};" ::"r"(taddr),
-        "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]),
-        "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
-        : "memory");
-}
-__device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t* r)
-{
-    asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"r"(taddr), "r"(r[0]), "r"(r[1]),
-                 "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7])
-                 : "memory");
-}
-__device__ __forceinline__ void tmem_st_wait()
-{
-    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-}
-// D (+)= A B with the A operand in tensor memory: row m of A in lane m, elements 2c and 2c + 1 of the row in the
-// low and high half of column c (16 elements = 8 columns per instruction)
-__device__ __forceinline__ void mma_f16_a_tmem(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc, uint32_t idesc,
-                                               uint32_t accumulate)
-{
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
-        ::"r"(d_tmem), "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accumulate)
-        : "memory");
-}
-
 __device__ __forceinline__ float max3f(float a, float b, float c)
 {
     float d;
@@ -418,13 +386,13 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                         if constexpr (!RAGGED) {
 #pragma unroll
                             for (int k = 0; k < 4; ++k)
-                                mma_f16_a_tmem(tmem_base + O_OFF, tmem_p + (uint32_t)(8 * k), vdesc(k), IDESC_PV, (j | k) != 0);
+                                nm_mma_f16_a_tmem(tmem_base + O_OFF, tmem_p + (uint32_t)(8 * k), vdesc(k), IDESC_PV, (j | k) != 0);
                         } else if constexpr (ONE) {
                             const int steps = (L + 15) / 16;
 #pragma unroll
                             for (int t = TERMS - 1; t >= 0; --t)
                                 for (int k = 0; k < steps; ++k)
-                                    mma_f16_a_tmem(tmem_base + O_OFF, t == 2 ? tmem_p + (uint32_t)(8 * k) : tmem_base + (uint32_t)(16 * k + 8 * t),
+                                    nm_mma_f16_a_tmem(tmem_base + O_OFF, t == 2 ? tmem_p + (uint32_t)(8 * k) : tmem_base + (uint32_t)(16 * k + 8 * t),
                                                    vdesc(k), IDESC_PV, t != TERMS - 1 || k != 0);
                         } else {
                             const int k0 = 2 * (u & 1);
@@ -432,7 +400,7 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                             for (int t = TERMS - 1; t >= 0; --t)
 #pragma unroll
                                 for (int k = 0; k < 2; ++k)
-                                    mma_f16_a_tmem(t == 0 ? tmem_base + O_OFF : tmem_lo, tmem_t + (uint32_t)(16 * t + 8 * k), vdesc(k0 + k), IDESC_PV,
+                                    nm_mma_f16_a_tmem(t == 0 ? tmem_base + O_OFF : tmem_lo, tmem_t + (uint32_t)(16 * t + 8 * k), vdesc(k0 + k), IDESC_PV,
                                                    u != 0 || k != 0 || (t != 0 && t != TERMS - 1));
                         }
                         nm_tc_commit(&bar_p_empty);
@@ -650,10 +618,10 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                         if (hh == 0 && j >= 1) wait_all(&bar_p_empty, (pv_base + (uint32_t)(j - 1)) & 1u);
                         if (ok) {
                             if (hh == 0 && j >= 1) nm_tc_fence_after();   // ordered after the P V that read the columns
-                            tmem_st16(p_row + (uint32_t)(hh * 16), pk);   // keys 32 hh .. 32 hh + 31 of this thread's row
+                            nm_tmem_st16(p_row + (uint32_t)(hh * 16), pk);   // keys 32 hh .. 32 hh + 31 of this thread's row
                         }
                     }
-                    tmem_st_wait();          // the P columns are written
+                    nm_tmem_st_wait();          // the P columns are written
                     nm_tc_fence_before();
                     asm volatile("bar.arrive %0, %1;" ::"r"(bar_pr), "n"(160) : "memory");
                 }
@@ -677,16 +645,16 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                     auto keys16 = [&](int k, auto masked) {
                         block(t_row + (uint32_t)(16 * k), L - 16 * k, masked, [] {});
                         if (ok && live) {
-                            tmem_st8(t_row + (uint32_t)(16 * k), term[0]);
-                            tmem_st8(t_row + (uint32_t)(16 * k + 8), term[1]);
-                            if constexpr (TERMS == 3) tmem_st8(p_row + (uint32_t)(8 * k), term[2]);
+                            nm_tmem_st8(t_row + (uint32_t)(16 * k), term[0]);
+                            nm_tmem_st8(t_row + (uint32_t)(16 * k + 8), term[1]);
+                            if constexpr (TERMS == 3) nm_tmem_st8(p_row + (uint32_t)(8 * k), term[2]);
                         }
                     };
                     const int steps = (L + 15) / 16;
 #pragma unroll 1
                     for (int k = 0; k < steps - 1; ++k) keys16(k, std::false_type{});
                     keys16(steps - 1, std::true_type{});
-                    tmem_st_wait();
+                    nm_tmem_st_wait();
                     nm_tc_fence_before();
                     asm volatile("bar.arrive %0, %1;" ::"r"(bar_pr), "n"(160) : "memory");
                 } else {
@@ -710,10 +678,10 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                             if (ok && live) {
                                 if (hh == 0 && u >= 1) nm_tc_fence_after();
 #pragma unroll
-                                for (int t = 0; t < TERMS; ++t) tmem_st8(tmem_t + lanes + (uint32_t)(16 * t + 8 * hh), term[t]);
+                                for (int t = 0; t < TERMS; ++t) nm_tmem_st8(tmem_t + lanes + (uint32_t)(16 * t + 8 * hh), term[t]);
                             }
                         }
-                        tmem_st_wait();
+                        nm_tmem_st_wait();
                         nm_tc_fence_before();
                         asm volatile("bar.arrive %0, %1;" ::"r"(bar_pr), "n"(160) : "memory");
                     };

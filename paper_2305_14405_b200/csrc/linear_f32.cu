@@ -1,173 +1,357 @@
-// fp32 linear operator with PWL epilogue on the CUDA cores (the fp32 tolerance rules out tf32, and three-way bf16
-// splits lose bits in the tensor cores' accumulation).
+// fp32 linear operator with PWL epilogue on the tensor cores: every fp32 operand is the sum of three bf16 terms
+// (f32_terms.cuh: the terms, their six products, and why an accumulator of the first product takes four steps only, one K-block;
+// the sum warps add it to their fp32 registers while the other one fills).
 //
-// Bound by the register file behind the FMA pipe: an 8 x 8 outer product with three distinct operands per instruction
-// runs at 49 TFLOP/s as scalar FFMA and at 63 with the packed form (registers only, no loads), so the packed form it is,
-// and it runs along K, where both operands lie as they are needed: a thread's accumulator is a PAIR of partial sums
-// (even and odd k, added at the end), fma.rn.f32x2 takes two adjacent k of a row of A and of W, and nothing is transposed
-// or duplicated.  One CTA per SM (two smaller ones are not placed evenly) computes a 128 x 64 tile with two groups of 128
-// threads, 8 x 8 elements per thread; a group takes every other K-block of 32 with a cp.async ring and a named barrier of
-// its own, so that the groups drift apart and one's barrier and first fragments hide behind the other's arithmetic
-// (against one ring for both: 98 -> 89 us at 1024 x 2304 x 768).  Fragments are double-buffered in registers.  Problems of
-// few tiles split K over a thread-block cluster.  1024 x 2304 x 768: 41 TFLOP/s; the 64 x 64-tile kernel before: 16.
+// A CTA takes a 128 x BN tile (BN = 128 or 64): eight warps fetch the fp32 operands, split them and write the terms into a ring
+// of K-major, 128-byte-swizzled operand tiles; one warp issues the products; eight warps add the accumulators up.  Problems of few tiles
+// split K over a thread-block cluster, whose partial tiles are added through distributed shared memory.
+// A result that is not finite (an infinite or NaN operand, one of 2^112 or more, sums beyond the fp32 range) is
+// computed again as a chain of FMAs, so that infinities come out as they do there and not as the difference of two.
+//
+// Bound by the shared-memory port with 128 columns: per K-block of 64 k the terms' stores take 768 cycles, the products' operand reads
+// 1536, the fp32 fetch 1390 beside them; 2700 were measured.  The fetch loop must not spill (beside 200 KB of shared memory the L1 is
+// too small to hold a spilled register: 5000 cycles), hence the two chunks at a time, the one walking pointer and the tail apart.
+// Relative errors against float64 here and with packed FMAs on the CUDA cores, which this kernel replaced: 1024 x 768 x 768
+// 9.0e-8 and 2.5e-7, x 3072 1.2e-7 and 2.5e-7, 128 x 768 x 256 8.1e-8 and 9.7e-8.  Times: 1024 x 2304 x 768 24.5 us and 84.3,
+// 1024 x 768 x 3072 42.3 and 132.0, 40 x 768 x 3072 14.2 and 24.0, 128 x 768 x 256 7.3 and 7.6.
+#include "f32_terms.cuh"
 #include "linear_split_kernel.cuh"
 
 using namespace nm_tc;
 
 namespace {
 
-constexpr int FBM = BM;       // 128 rows, as Finisher expects
-constexpr int FBN = 64;
-constexpr int FG = 2;             // thread groups
-constexpr int FBK = 32;
-constexpr int FPITCH = FBK + 4;   // words per operand row: 8 rows of a warp's loads fall on distinct banks
-constexpr int FSTAGES = 3;
-constexpr int F_THREADS = 128 * FG;
-constexpr int FSTAGE_WORDS = (FBM + FBN) * FPITCH;
-constexpr int PART_WORDS = FBM * part_pitch(FBN);
+constexpr int FBK = 64;           // K-elements of a stage: 128 bytes of bf16 per row and term
+constexpr int F_PROD = 256;       // threads that fetch and split: warps 0 to 7; warp 8 issues the products
+constexpr int F_SUM_WARPS = 8;    // warps 9 to 16
+constexpr int F_THREADS = F_PROD + 32 + 32 * F_SUM_WARPS;
+constexpr int FIN_THREADS = 512;  // of them run the final sum
 
-__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, int bytes)
-{
-    // bytes < 16: the rest of the 16 are zero-filled and not read
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
-}
+template <int BN> struct F32Tile {
+    static constexpr int B_BYTES = BN * ROW_BYTES;
+    static constexpr int STAGE_BYTES = 3 * (A_BYTES + B_BYTES);
+    static constexpr int STAGES = BN == 128 ? 2 : 3;
+    static constexpr int SMEM = STAGES * STAGE_BYTES + 1024;
+    static constexpr int CHUNKS = (BM + BN) / 16;      // 16-byte chunks of fp32 per thread and stage
+    static constexpr int AHEAD = BN == 128 ? 8 : 12;   // of them in flight, in registers
+    static constexpr int GROUP = BN == 128 ? 2 : 1;    // split together
+    static_assert(BM * part_pitch(BN) * 4 <= STAGES * STAGE_BYTES, "the partial tile takes the ring's place");
+};
 
+template <int BN>
 __global__ void __launch_bounds__(F_THREADS, 1)
 linear_f32_kernel(const float* __restrict__ A, const float* __restrict__ W, int64_t lda, int64_t ldw, const SplitArgs s)
 {
+    using T = F32Tile<BN>;
     const TcArgs& a = s.t;
-    extern __shared__ __align__(16) float fsm[];
+    constexpr int PITCH = part_pitch(BN);
+    constexpr uint32_t IDESC = nm_idesc(1, 1, 0, 0, BM, BN);
+    constexpr uint32_t TMEM_COLS = 4 * BN;   // two accumulators of h h', one of the 2^-16 and one of the 2^-32 products
+
+    extern __shared__ uint8_t smem_raw[];
+    __shared__ uint64_t bar_full[T::STAGES], bar_empty[T::STAGES], bar_acc_full[2], bar_acc_empty[2], bar_end;
+    __shared__ uint32_t tmem_slot;
+    __shared__ int abort_flag;
     __shared__ float2 s_tab[NM_MAX_SEGMENTS];
+
+    uint8_t* ring = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+    float* part = reinterpret_cast<float*>(ring);
     const int S = s.S;
     const int rank = S > 1 ? (int)nm_cluster_ctarank() : 0;
     const int tile = (int)blockIdx.x / S;
     const int mt = tile / a.num_n_tiles, nt = tile % a.num_n_tiles;
     const int kb0 = (int)((int64_t)rank * a.num_k_blocks / S), kb1 = (int)((int64_t)(rank + 1) * a.num_k_blocks / S);
-    const int tid = threadIdx.x;
-    const int64_t m0 = (int64_t)mt * FBM, n0 = (int64_t)nt * FBN;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int64_t m0 = (int64_t)mt * BM, n0 = (int64_t)nt * BN;
+    const int rows = (int)min((int64_t)BM, a.M - m0), cols = (int)min((int64_t)BN, a.N - n0);
+
+    if (tid == 0) {
+        abort_flag = 0;
+        for (int i = 0; i < T::STAGES; ++i) {
+            nm_mbar_init(&bar_full[i], F_PROD / 32);
+            nm_mbar_init(&bar_empty[i], 1);
+        }
+        for (int i = 0; i < 2; ++i) {
+            nm_mbar_init(&bar_acc_full[i], 1);
+            nm_mbar_init(&bar_acc_empty[i], F_SUM_WARPS);
+        }
+        nm_mbar_init(&bar_end, 1);
+        nm_fence_barrier_init();
+    }
+    if (warp == F_PROD / 32) {
+        nm_tmem_alloc(&tmem_slot, TMEM_COLS);
+        nm_tmem_relinquish();
+    }
     if (a.tab) {
         for (int i = tid; i < a.n_seg; i += F_THREADS) s_tab[i] = a.tab->kb[i];
     }
-    nm_grid_launch_dependents();
-    nm_grid_dependency_wait();
-
-    // 192 operand rows of 8 chunks per stage, 12 chunks per thread of a group: rows gt/8 + 16 i (i < 8: A, else W)
-    const int grp = tid >> 7, gt = tid & 127;
-    float* ring = fsm + grp * FSTAGES * FSTAGE_WORDS;
-    const int c4 = (gt & 7) * 4;
-    const float* srcA = A + (m0 + (gt >> 3)) * lda + c4;
-    const float* srcW = W + (n0 + (gt >> 3)) * ldw + c4;
-    const int rowsA = (int)min((int64_t)FBM, a.M - m0) - (gt >> 3), rowsW = (int)min((int64_t)FBN, a.N - n0) - (gt >> 3);
-    const uint32_t dst = nm_smem_u32(ring) + (uint32_t)((gt >> 3) * FPITCH + c4) * 4u;
-    auto load = [&](int kb, int stage) {
-        const int64_t left = a.K - ((int64_t)kb * FBK + c4);   // valid elements from this chunk's first k on
-        const int bytes = left >= 4 ? 16 : (left > 0 ? (int)left * 4 : 0);
-        const uint32_t d = dst + (uint32_t)(stage * FSTAGE_WORDS) * 4u;
-        const float* pa = srcA + (int64_t)kb * FBK;
-        const float* pw = srcW + (int64_t)kb * FBK;
-#pragma unroll
-        for (int i = 0; i < FBM / 16; ++i) {
-            const int n = 16 * i < rowsA ? bytes : 0;
-            cp_async16(d + (uint32_t)(16 * i * FPITCH) * 4u, n ? (const void*)(pa + 16 * i * lda) : (const void*)A, n);
-        }
-#pragma unroll
-        for (int i = 0; i < FBN / 16; ++i) {
-            const int n = 16 * i < rowsW ? bytes : 0;
-            cp_async16(d + (uint32_t)((FBM + 16 * i) * FPITCH) * 4u, n ? (const void*)(pw + 16 * i * ldw) : (const void*)A, n);
-        }
-    };
-    const int ty = (gt >> 5) * 4 + ((gt & 31) >> 3), tx = gt & 7;   // rows ty + 16 i, columns tx + 8 j
-    uint64_t acc[8][8];   // sums over the even and the odd k
-#pragma unroll
-    for (int i = 0; i < 8; ++i)
-#pragma unroll
-        for (int j = 0; j < 8; ++j) acc[i][j] = 0ull;
-
-#pragma unroll
-    for (int i = 0; i < FSTAGES - 1; ++i) {
-        if (kb0 + grp + FG * i < kb1) load(kb0 + grp + FG * i, i);
-        asm volatile("cp.async.commit_group;" ::: "memory");
-    }
-    int stage = 0;
-    for (int kb = kb0 + grp; kb < kb1; kb += FG) {
-        asm volatile("cp.async.wait_group %0;" ::"n"(FSTAGES - 2) : "memory");
-        // this K-block has landed for the whole group, and all of it has left the stage loaded next
-        asm volatile("bar.sync %0, %1;" ::"r"(1 + grp), "n"(128) : "memory");
-        if (kb + FG * (FSTAGES - 1) < kb1) load(kb + FG * (FSTAGES - 1), stage == 0 ? FSTAGES - 1 : stage - 1);
-        asm volatile("cp.async.commit_group;" ::: "memory");
-        const float* sa = ring + stage * FSTAGE_WORDS + ty * FPITCH;
-        const float* sb = ring + stage * FSTAGE_WORDS + (FBM + tx) * FPITCH;
-        uint64_t ra[2][8], rb[2][8];
-        auto frag = [&](int b, int k2) {
-#pragma unroll
-            for (int i = 0; i < 8; ++i) ra[b][i] = *reinterpret_cast<const uint64_t*>(sa + 16 * i * FPITCH + k2);
-#pragma unroll
-            for (int j = 0; j < 8; ++j) rb[b][j] = *reinterpret_cast<const uint64_t*>(sb + 8 * j * FPITCH + k2);
-        };
-        frag(0, 0);
-#pragma unroll
-        for (int k2 = 0; k2 < FBK; k2 += 2) {
-            const int b = (k2 >> 1) & 1;
-            if (k2 + 2 < FBK) frag(b ^ 1, k2 + 2);
-#pragma unroll
-            for (int j = 0; j < 8; ++j)
-#pragma unroll
-                for (int i = 0; i < 8; ++i) asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc[i][j]) : "l"(ra[b][i]), "l"(rb[b][j]));
-        }
-        stage = stage + 1 == FSTAGES ? 0 : stage + 1;
-    }
-    asm volatile("cp.async.wait_group 0;" ::: "memory");
-    __syncthreads();   // everyone is done with the rings: the groups' tiles take their place
-    constexpr int PITCH = part_pitch(FBN);
-    float* part = fsm;
-    {
-        float* mine = part + grp * PART_WORDS;
-#pragma unroll
-        for (int i = 0; i < 8; ++i)
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                float lo, hi;
-                nm_unpack2(acc[i][j], lo, hi);
-                mine[(ty + 16 * i) * PITCH + tx + 8 * j] = lo + hi;
-            }
-    }
+    nm_tc_fence_before();
     __syncthreads();
+    nm_tc_fence_after();
+    const uint32_t tmem = tmem_slot;
+    volatile int* abortp = &abort_flag;
+    if (!a.late_trigger) nm_grid_launch_dependents();
+    // weights that were complete before the previous kernel started are fetched before the wait for it
+    if (!a.weights_ready || warp >= F_PROD / 32) nm_grid_dependency_wait();
+    if (a.late_trigger) nm_grid_launch_dependents();
+    bool ok = true;
+
+    if (warp < F_PROD / 32) {
+        // ------------------------------------------------ operands
+        // This thread's: chunk tid % 16 (four k) of rows tid / 16 + 16 i, first of W, then of A.  Rows that do not exist are
+        // not read: what their registers hold goes into rows and columns of the product that are not stored.
+        const int c4 = (tid & 15) * 4, r0 = tid >> 4;
+        uint32_t exists = 0;   // bit i: row i of this thread does
 #pragma unroll
-    for (int i = 0; i < FBM * FBN / 4 / F_THREADS; ++i) {   // the groups' sum
-        const int u = tid + i * F_THREADS;
-        float* p = part + (u / (FBN / 4)) * PITCH + (u % (FBN / 4)) * 4;
-        float4 v = *reinterpret_cast<const float4*>(p);
-#pragma unroll
-        for (int g = 1; g < FG; ++g) {
-            const float4 o = *reinterpret_cast<const float4*>(p + g * PART_WORDS);
-            v.x += o.x; v.y += o.y; v.z += o.z; v.w += o.w;
+        for (int i = 0; i < T::CHUNKS; ++i) {
+            if (i < BN / 16 ? 16 * i + r0 < cols : 16 * i - BN + r0 < rows) exists |= 1u << i;
         }
-        *reinterpret_cast<float4*>(p) = v;
+        const int64_t stepA = 16 * lda, stepW = 16 * ldw;
+        const float* pA = A + (m0 + r0) * lda + c4 + (int64_t)kb0 * FBK;   // row 0 in the K-block that is fetched next
+        const float* pW = W + (n0 + r0) * ldw + c4 + (int64_t)kb0 * FBK;
+        const int full = min(kb1, (int)(a.K / FBK));   // K-blocks that are all there end here
+        // (one pointer walks along the rows: an address per row would be kept in registers)
+        const float* pf = pW;
+        uint32_t mask = kb0 < full ? exists : 0u;
+        float4 reg[T::AHEAD];
+        auto fetch = [&](int i) {
+            if (i == 0) pf = pW;
+            if (i == BN / 16) pf = pA;
+            float4& v = reg[i % T::AHEAD];
+            asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %5, 0;\n\t"
+                         "@p ld.global.cg.v4.f32 {%0, %1, %2, %3}, [%4];\n\t}"
+                         : "+f"(v.x), "+f"(v.y), "+f"(v.z), "+f"(v.w)
+                         : "l"(pf), "r"(mask & (1u << i)));
+            pf += i < BN / 16 ? stepW : stepA;
+        };
+        // row r of a term's tile at byte 128 r, its 16-byte chunk j at j ^ (r % 8); this thread's rows all have r % 8 = r0 % 8
+        const uint32_t dst0 = nm_smem_u32(ring) + (uint32_t)(r0 * ROW_BYTES + (((c4 >> 3) ^ (r0 & 7)) << 4) + ((c4 & 4) << 1));
+        auto put = [&](uint32_t d, uint32_t term, const uint2& h, const uint2& m, const uint2& l) {
+            asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(d), "r"(h.x), "r"(h.y) : "memory");
+            asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(d + term), "r"(m.x), "r"(m.y) : "memory");
+            asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(d + 2 * term), "r"(l.x), "r"(l.y) : "memory");
+        };
+#pragma unroll
+        for (int i = 0; i < T::AHEAD; ++i) {
+            if (i == BN / 16 && a.weights_ready) nm_grid_dependency_wait();
+            reg[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+            fetch(i);
+        }
+        if (T::AHEAD == BN / 16 && a.weights_ready) nm_grid_dependency_wait();
+        // where a thread's row i goes in a stage: the terms of A lie before those of W
+        auto place = [](int i) { return (uint32_t)(i < BN / 16 ? 3 * A_BYTES + i * 16 * ROW_BYTES : (i - BN / 16) * 16 * ROW_BYTES); };
+        int stage = 0;
+        uint32_t phase = 0;
+        for (int kb = kb0; kb < kb1; ++kb) {
+            if (!nm_mbar_wait(&bar_empty[stage], phase ^ 1u, abortp, a.status)) { ok = false; break; }
+            const uint32_t dst = dst0 + (uint32_t)(stage * T::STAGE_BYTES);
+            if (kb < full) {
+#pragma unroll
+                for (int i = 0; i < T::CHUNKS; i += T::GROUP) {
+                    uint2 h[T::GROUP], m[T::GROUP], l[T::GROUP];
+#pragma unroll
+                    for (int j = 0; j < T::GROUP; ++j) nm_f32_terms4(reg[(i + j) % T::AHEAD], h[j], m[j], l[j]);
+#pragma unroll
+                    for (int j = 0; j < T::GROUP; ++j) {
+                        const int n = (i + j + T::AHEAD) % T::CHUNKS;
+                        if (n == 0) {
+                            pA += FBK;
+                            pW += FBK;
+                            mask = kb + 1 < full ? exists : 0u;
+                        }
+                        fetch(n);
+                    }
+#pragma unroll
+                    for (int j = 0; j < T::GROUP; ++j) put(dst + place(i + j), i < BN / 16 ? T::B_BYTES : A_BYTES, h[j], m[j], l[j]);
+                }
+            } else {
+                // K ends in this one: zeros beyond it, and the last one to three k of a row, whose end may be the memory's, singly
+                const int left = (int)a.K - (kb * FBK + c4);
+#pragma unroll 4
+                for (int i = 0; i < T::CHUNKS; ++i) {
+                    const float* p = (i < BN / 16 ? W + (n0 + r0 + 16 * i) * ldw : A + (m0 + r0 + 16 * i - BN) * lda) + (int64_t)kb * FBK + c4;
+                    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+                    if (exists & (1u << i)) {
+                        if (left >= 4) v = __ldcg(reinterpret_cast<const float4*>(p));
+                        else {
+                            if (left > 0) v.x = __ldcg(p);
+                            if (left > 1) v.y = __ldcg(p + 1);
+                            if (left > 2) v.z = __ldcg(p + 2);
+                        }
+                    }
+                    uint2 h, m, l;
+                    nm_f32_terms4(v, h, m, l);
+                    put(dst + place(i), i < BN / 16 ? T::B_BYTES : A_BYTES, h, m, l);
+                }
+            }
+            nm_fence_proxy_async();
+            __syncwarp();
+            if (lane == 0) nm_mbar_arrive(&bar_full[stage]);
+            if (++stage == T::STAGES) { stage = 0; phase ^= 1u; }
+        }
+    } else if (warp == F_PROD / 32) {
+        // ------------------------------------------------ products, those of an accumulator together
+        int stage = 0;
+        uint32_t phase = 0, acc_phase = 0;
+        for (int kb = kb0; kb < kb1; ++kb) {
+            if (!__all_sync(0xffffffffu, nm_mbar_wait(&bar_full[stage], phase, abortp, a.status))) { ok = false; break; }
+            const uint32_t sa = nm_smem_u32(ring + (size_t)stage * T::STAGE_BYTES), sb = sa + 3 * A_BYTES;
+            const uint64_t ah = nm_smem_desc_sw128(sa), bh = nm_smem_desc_sw128(sb);
+            constexpr uint64_t AT = A_BYTES >> 4, BT = T::B_BYTES >> 4;   // from term to term
+            const int buf = (kb - kb0) & 1;
+            if (!__all_sync(0xffffffffu, nm_mbar_wait(&bar_acc_empty[buf], acc_phase ^ 1u, abortp, a.status))) { ok = false; break; }
+            nm_tc_fence_after();
+            if (nm_elect_one()) {
+#pragma unroll
+                for (int k = 0; k < 4; ++k) nm_mma_f16(tmem + (uint32_t)(buf * BN), ah + 2 * k, bh + 2 * k, IDESC, k != 0);   // 32 bytes of K per row
+                nm_tc_commit(&bar_acc_full[buf]);
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    nm_mma_f16(tmem + 2 * BN, ah + 2 * k, bh + BT + 2 * k, IDESC, kb != kb0 || k != 0);
+                    nm_mma_f16(tmem + 2 * BN, ah + AT + 2 * k, bh + 2 * k, IDESC, 1u);
+                }
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    nm_mma_f16(tmem + 3 * BN, ah + AT + 2 * k, bh + BT + 2 * k, IDESC, kb != kb0 || k != 0);
+                    nm_mma_f16(tmem + 3 * BN, ah + 2 * k, bh + 2 * BT + 2 * k, IDESC, 1u);
+                    nm_mma_f16(tmem + 3 * BN, ah + 2 * AT + 2 * k, bh + 2 * k, IDESC, 1u);
+                }
+                nm_tc_commit(&bar_empty[stage]);
+            }
+            __syncwarp();
+            if (++stage == T::STAGES) { stage = 0; phase ^= 1u; }
+            acc_phase ^= (uint32_t)buf;
+        }
+        if (nm_elect_one()) nm_tc_commit(&bar_end);   // (after a timeout it still counts what was issued)
+        __syncwarp();
+    } else {
+        // ------------------------------------------------ sums: 32 rows and half of the columns per warp
+        const int c0 = ((warp - F_PROD / 32 - 1) >> 2) * (BN / 2), q = warp & 3, row = q * 32 + lane;
+        const uint32_t t_addr = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)c0;
+        uint64_t acc[BN / 4];   // pairs of columns
+#pragma unroll
+        for (int i = 0; i < BN / 4; ++i) acc[i] = 0ull;
+        uint32_t phase = 0;
+        for (int kb = kb0; kb < kb1; ++kb) {
+            const int buf = (kb - kb0) & 1;
+            if (!__all_sync(0xffffffffu, nm_mbar_wait(&bar_acc_full[buf], phase, abortp, a.status))) { ok = false; break; }
+            nm_tc_fence_after();
+#pragma unroll
+            for (int c = 0; c < BN / 2; c += 16) {
+                uint32_t r[16];
+                nm_tmem_ld16_sync(t_addr + (uint32_t)(buf * BN + c), r);
+#pragma unroll
+                for (int i = 0; i < 16; i += 2)
+                    asm("add.rn.f32x2 %0, %0, %1;" : "+l"(acc[(c + i) / 2]) : "l"(nm_pack2(__uint_as_float(r[i]), __uint_as_float(r[i + 1]))));
+            }
+            nm_tc_fence_before();
+            __syncwarp();
+            if (lane == 0) nm_mbar_arrive(&bar_acc_empty[buf]);
+            phase ^= (uint32_t)buf;
+        }
+        // every product is done, and has read the ring, whose place the partial tile takes
+        if (!nm_mbar_wait(&bar_end, 0, abortp, a.status)) ok = false;
+        __syncwarp();
+        nm_tc_fence_after();
+        bool odd = false;   // a sum that is not finite
+        float* mine = part + row * PITCH + c0;
+        if (__all_sync(0xffffffffu, ok && !*abortp)) {
+#pragma unroll
+            for (int c = 0; c < BN / 2; c += 4) {
+                float v[4];
+                nm_unpack2(acc[c / 2], v[0], v[1]);
+                nm_unpack2(acc[c / 2 + 1], v[2], v[3]);
+                *reinterpret_cast<float4*>(mine + c) = make_float4(v[0], v[1], v[2], v[3]);
+            }
+#pragma unroll 1
+            for (int c = 0; c < BN / 2; c += 16) {
+                uint32_t mid[16], low[16];
+                nm_tmem_ld16_sync(t_addr + (uint32_t)(2 * BN + c), mid);
+                nm_tmem_ld16_sync(t_addr + (uint32_t)(3 * BN + c), low);
+#pragma unroll
+                for (int i = 0; i < 16; i += 4) {
+                    float4* p = reinterpret_cast<float4*>(mine + c + i);
+                    float4 v = *p;
+                    auto add = [&](float& x, int j) {
+                        x = nm_f32_sum(x, mid[j], low[j]);
+                        odd |= !(fabsf(x) <= 3.402823466e38f);
+                    };
+                    add(v.x, i);
+                    add(v.y, i + 1);
+                    add(v.z, i + 2);
+                    add(v.w, i + 3);
+                    *p = v;
+                }
+            }
+            if (odd && row < rows) {
+                const int64_t k0 = (int64_t)kb0 * FBK, k1 = min((int64_t)kb1 * FBK, a.K);
+                for (int j = 0; j < BN / 2 && c0 + j < cols; ++j) {
+                    if (fabsf(mine[j]) <= 3.402823466e38f) continue;
+                    const float *pa = A + (m0 + row) * lda, *pw = W + (n0 + c0 + j) * ldw;
+                    float v = 0.f;
+                    for (int64_t k = k0; k < k1; ++k) v = __fmaf_rn(__ldcg(pa + k), __ldcg(pw + k), v);
+                    mine[j] = v;
+                }
+            }
+        }
+        nm_tc_fence_before();
     }
-    const int rows = (int)(a.M - m0 < FBM ? a.M - m0 : FBM);
-    Finisher<false, float, FBN, false, F_THREADS, false> fin(s, rank, mt, nt, rows, Patch{0, 0, 0});
+    Finisher<false, float, BN, false, FIN_THREADS, false> fin(s, rank, mt, nt, rows, Patch{0, 0, 0});
     fin.prefetch_vectors();
     fin.load_res(0);
     if (S > 1) nm_cluster_sync();
     else __syncthreads();
-    fin.run(reinterpret_cast<const uint32_t*>(part), s_tab);
+    if (tid < FIN_THREADS && !*abortp) fin.run(reinterpret_cast<const uint32_t*>(part), s_tab);
     if (S > 1) nm_cluster_sync();   // a peer may still be reading this CTA's partial tile
+    if (warp == F_PROD / 32) {
+        nm_tc_fence_after();
+        nm_tmem_dealloc(tmem, TMEM_COLS);
+    }
 }
 
-// CTAs per cluster: the least time by measured figures, in us: 1.65 per K-block of 32, 4.9 per round of CTAs for the
-// launch, the ring's fill and the epilogue, 0.7 + 0.25 S for the exchange.  A round is what the GPU holds of clusters of S,
-// which is less than its SMs for most S.
-int choose_f32_split(int64_t tiles, int k_blocks, const int* resident)
+struct F32Choice {
+    int BN, S;
+};
+
+// Columns per tile and CTAs per cluster: the least time by a model of 18 problems of 16 to 1024 rows, N 256 to 3072, K 256 to 3072, each
+// with nine forms (6 % off on the average; the form it picks is 0.7 % behind the best, 3 % at most), in us: the launch, the first
+// operands and the epilogue, the K-blocks of 64, more when all SMs fetch, the exchange of a split, and what a further round of CTAs costs
+// beside its K-blocks.  A round is what the GPU holds of clusters of S, which is less than its SMs for most S (1024 x 768 x 768
+// with 128 columns: 22.6, 16.6 and, in two rounds, 30.2 us for S = 1, 2, 3).
+F32Choice choose_f32(int64_t M, int64_t N, int k_blocks, const int* resident)
 {
-    int best = 1;
+    struct P { int BN; double base, kb, busy, split, per_cta, round; };
+    static const P forms[2] = {{128, 5.56, 1.34, 0.22, 0.1, 0.46, 8.0}, {64, 3.93, 1.12, 0.0, 1.19, 0.14, 7.1}};
+    F32Choice best = {64, 1};
     double best_t = 1e30;
-    for (int S = 1; S <= 8 && S <= k_blocks; ++S) {
-        if (resident[S] < 1) continue;
-        const double rounds = (double)((tiles + resident[S] - 1) / resident[S]);
-        const double t = rounds * (1.65 * ((k_blocks + S - 1) / S) + 4.9 + (S > 1 ? 0.7 + 0.25 * S : 0.0));
-        if (t < best_t * 0.98) { best_t = t; best = S; }
+    for (const P& p : forms) {
+        const int64_t tiles = ((M + BM - 1) / BM) * ((N + p.BN - 1) / p.BN);
+        for (int S = 1; S <= 8 && S <= k_blocks; ++S) {
+            if (resident[S] < 1) continue;
+            const double rounds = (double)((tiles + resident[S] - 1) / resident[S]);
+            const double share = tiles < resident[S] ? (double)tiles / resident[S] : 1.0;
+            const double t = p.base + rounds * (p.kb + p.busy * share) * ((k_blocks + S - 1) / S) + (S > 1 ? p.split + p.per_cta * S : 0.0) + p.round * (rounds - 1.0);
+            if (t < best_t * 0.98) { best_t = t; best = {p.BN, S}; }
+        }
     }
     return best;
+}
+
+template <int BN>
+nm_status launch_f32(nm_ctx* ctx, const nm_linear_desc* d, SplitArgs& s, cudaLaunchConfig_t& cfg, cudaLaunchAttribute* attr, cudaStream_t st)
+{
+    const int64_t n_tiles = (d->N + BN - 1) / BN, tiles = (d->M + BM - 1) / BM * n_tiles;
+    s.t.num_n_tiles = (int)n_tiles;
+    s.t.num_tiles = (int)tiles;
+    if (cudaFuncSetAttribute(linear_f32_kernel<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, F32Tile<BN>::SMEM) != cudaSuccess)
+        return NM_ERR_CUDA;
+    cfg.dynamicSmemBytes = F32Tile<BN>::SMEM;
+    cfg.numAttrs = split_launch_attrs(ctx, attr, s.S);
+    cfg.gridDim = dim3((unsigned)(tiles * s.S));
+    NmLaunchScope scope(ctx, NM_KERNEL_LINEAR_TC, 2.0 * (double)d->M * (double)d->N * (double)d->K, st);
+    if (cudaLaunchKernelEx(&cfg, linear_f32_kernel<BN>, (const float*)d->A, (const float*)d->W, d->lda, d->ldw, s) != cudaSuccess)
+        return NM_ERR_CUDA;
+    return cudaGetLastError() == cudaSuccess ? NM_OK : NM_ERR_CUDA;
 }
 
 }  // namespace
@@ -177,10 +361,9 @@ bool nm_linear_f32_supported(const nm_linear_desc* d)
     return d->in_dtype == NM_F32 && d->N % 4 == 0 && d->K <= 0x7fffffffLL;
 }
 
-nm_status nm_launch_linear_f32(nm_ctx* ctx, const nm_linear_desc* d, cudaStream_t st)
+nm_status nm_launch_linear_f32(nm_ctx* ctx, const nm_linear_desc* d, cudaStream_t st, NmChain chain)
 {
-    const int64_t m_tiles = (d->M + FBM - 1) / FBM, n_tiles = (d->N + FBN - 1) / FBN, tiles = m_tiles * n_tiles;
-    if ((d->M + 63) / 64 > 65535 || tiles > 0x7fffffffLL / 8) return NM_ERR_SHAPE;
+    if ((d->M + 63) / 64 > 65535 || (d->M + BM - 1) / BM * ((d->N + 63) / 64) > 0x7fffffffLL / 8) return NM_ERR_SHAPE;
     SplitArgs s;
     memset(&s, 0, sizeof(s));
     TcArgs& a = s.t;
@@ -190,31 +373,30 @@ nm_status nm_launch_linear_f32(nm_ctx* ctx, const nm_linear_desc* d, cudaStream_
     a.tab = d->slot == NM_SLOT_NONE ? nullptr : ctx->d_tables + d->slot;
     a.n_seg = d->slot == NM_SLOT_NONE ? 0 : ctx->h_tables[d->slot].n;
     a.idx_dump = d->idx_dump;
-    a.num_n_tiles = (int)n_tiles;
-    a.num_tiles = (int)tiles;
+    a.status = ctx->d_status;
+    a.weights_ready = chain.weights_ready;
+    a.late_trigger = chain.late_trigger;
     a.num_k_blocks = (int)((d->K + FBK - 1) / FBK);
     s.residual = d->residual; s.ldr = d->ldr;
     s.out = d->out; s.ldo = d->ldo;
-    constexpr size_t smem = (size_t)FG * FSTAGES * FSTAGE_WORDS * 4;
-    static_assert(PART_WORDS <= FSTAGES * FSTAGE_WORDS, "partial tiles");
-    if (cudaFuncSetAttribute(linear_f32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-        return NM_ERR_CUDA;
     cudaLaunchConfig_t cfg;
     memset(&cfg, 0, sizeof(cfg));
     cfg.blockDim = dim3(F_THREADS);
-    cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cudaLaunchAttribute attr[2];
     cfg.attrs = attr;
-    // clusters of 1..8 CTAs the device holds, asked for once per context (or by several threads, which find the same; the first
-    // word is set when the others are, and orders them for a thread that did not ask)
+    // clusters of 1..8 CTAs the device holds (one CTA of either width per SM), asked for once per context (or by several threads,
+    // which find the same; the first word is set when the others are, and orders them for a thread that did not ask)
     int* resident = ctx->f32_resident;
     if (__atomic_load_n(&resident[0], __ATOMIC_ACQUIRE) == 0) {
+        cfg.dynamicSmemBytes = F32Tile<64>::SMEM;
+        if (cudaFuncSetAttribute(linear_f32_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, F32Tile<64>::SMEM) != cudaSuccess)
+            return NM_ERR_CUDA;
         for (int S = 1; S <= 8; ++S) {
             int n = 0;
             cfg.numAttrs = split_launch_attrs(ctx, attr, S);
             cfg.gridDim = dim3((unsigned)(S * ctx->sm_count));
-            if (cudaOccupancyMaxActiveClusters(&n, linear_f32_kernel, &cfg) != cudaSuccess) {
+            if (cudaOccupancyMaxActiveClusters(&n, linear_f32_kernel<64>, &cfg) != cudaSuccess) {
                 (void)cudaGetLastError();
                 n = S == 1 ? ctx->sm_count : 0;
             }
@@ -222,11 +404,7 @@ nm_status nm_launch_linear_f32(nm_ctx* ctx, const nm_linear_desc* d, cudaStream_
         }
         __atomic_store_n(&resident[0], 1, __ATOMIC_RELEASE);
     }
-    s.S = choose_f32_split(tiles, a.num_k_blocks, resident);
-    cfg.numAttrs = split_launch_attrs(ctx, attr, s.S);
-    cfg.gridDim = dim3((unsigned)(tiles * s.S));
-    NmLaunchScope scope(ctx, NM_KERNEL_LINEAR_SIMT, 2.0 * (double)d->M * (double)d->N * (double)d->K, st);
-    if (cudaLaunchKernelEx(&cfg, linear_f32_kernel, (const float*)d->A, (const float*)d->W, d->lda, d->ldw, s) != cudaSuccess)
-        return NM_ERR_CUDA;
-    return cudaGetLastError() == cudaSuccess ? NM_OK : NM_ERR_CUDA;
+    const F32Choice c = choose_f32(d->M, d->N, a.num_k_blocks, resident);
+    s.S = c.S;
+    return c.BN == 128 ? launch_f32<128>(ctx, d, s, cfg, attr, st) : launch_f32<64>(ctx, d, s, cfg, attr, st);
 }

@@ -328,7 +328,7 @@ nm_status nm_linear_dispatch(nm_ctx* ctx, const nm_linear_desc* d, cudaStream_t 
         if (d->out_dtype != d->in_dtype) return NM_ERR_UNSUPPORTED;
         if (d->acc_dump) return NM_ERR_UNSUPPORTED;
     }
-    if (!nm_algo_forced(d->algo) && nm_linear_f32_supported(d)) return nm_launch_linear_f32(ctx, d, st);
+    if (!nm_algo_forced(d->algo) && nm_linear_f32_supported(d)) return nm_launch_linear_f32(ctx, d, st, chain);
     if (d->algo == 1) return nm_launch_linear_simt(ctx, d, st);
     const bool tc = nm_linear_tc_supported(d);
     if (d->algo == 2 || d->algo == 3 || nm_algo_is_split(d->algo)) return tc ? nm_launch_linear_tc(ctx, d, st, chain) : NM_ERR_UNSUPPORTED;
@@ -610,7 +610,7 @@ static nm_status encoder_layer_impl(nm_ctx* ctx, const nm_encoder_weights* w, co
     s = linear(a_in, H, w->Wo, H, w->bo, x, NM_SLOT_NONE, z, act, w->a_attn, w->s_wo, 0.f);
     if (s != NM_OK) return s;
     s = layernorm_checked(ctx, z, w->g1, w->be1, x1, T, H, c->eps, c->rsqrt_slot, act, stream, i8 ? q8 : nullptr,
-                          i8 ? 1.0f / w->a_x1 : 0.f, act != NM_F32);
+                          i8 ? 1.0f / w->a_x1 : 0.f, true);
     if (s != NM_OK) return s;
 
     // g = PWLgelu(x1 W1^T + b1)   (int8 path: requantised in the epilogue with the scale of g)
@@ -624,7 +624,7 @@ static nm_status encoder_layer_impl(nm_ctx* ctx, const nm_encoder_weights* w, co
     if (s != NM_OK) return s;
     const bool next_codes = i8 && next_a_x > 0.f;
     return layernorm_checked(ctx, z, w->g2, w->be2, y, T, H, c->eps, c->rsqrt_slot, act, stream, next_codes ? q8 : nullptr,
-                             next_codes ? 1.0f / next_a_x : 0.f, act != NM_F32);
+                             next_codes ? 1.0f / next_a_x : 0.f, true);
 }
 
 nm_status nm_encoder_stack(nm_ctx* ctx, const nm_encoder_weights* layers, int32_t n_layers, const nm_encoder_cfg* c,

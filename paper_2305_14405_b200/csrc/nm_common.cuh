@@ -648,6 +648,38 @@ __device__ __forceinline__ void nm_tmem_ld16_sync(uint32_t taddr, uint32_t* r)
         : "memory");
 }
 
+// 16 packed words of this thread's row into 16 consecutive tensor-memory columns (the mirror of the 16-column read)
+__device__ __forceinline__ void nm_tmem_st16(uint32_t taddr, const uint32_t* r)
+{
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], "
+        "{%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};" ::"r"(taddr),
+        "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]),
+        "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
+        : "memory");
+}
+__device__ __forceinline__ void nm_tmem_st8(uint32_t taddr, const uint32_t* r)
+{
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"r"(taddr), "r"(r[0]), "r"(r[1]),
+                 "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7])
+                 : "memory");
+}
+__device__ __forceinline__ void nm_tmem_st_wait()
+{
+    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+}
+// D (+)= A B with the A operand in tensor memory: row m of A in lane m, elements 2c and 2c + 1 of the row in the
+// low and high half of column c (16 elements = 8 columns per instruction)
+__device__ __forceinline__ void nm_mma_f16_a_tmem(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc, uint32_t idesc,
+                                               uint32_t accumulate)
+{
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
+        ::"r"(d_tmem), "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accumulate)
+        : "memory");
+}
+
 // ---------------------------------------------------------------- host --------
 
 #define NM_CUDA_TRY(expr)                         \
@@ -687,8 +719,6 @@ static inline bool nm_algo_is_split(int32_t algo)
 }
 static inline bool nm_algo_forced(int32_t algo) { return (algo >= 1 && algo <= 3) || nm_algo_is_split(algo); }
 nm_status nm_launch_linear_simt(nm_ctx* ctx, const nm_linear_desc* d, cudaStream_t st);
-nm_status nm_launch_linear_f32(nm_ctx* ctx, const nm_linear_desc* d, cudaStream_t st);
-bool nm_linear_f32_supported(const nm_linear_desc* d);   // fp32, N a multiple of 4; linear_simt takes the rest
 // What a caller that enqueues a whole chain of kernels knows about a launch's neighbours in the stream.
 //   weights_ready: everything the call was given (weights, biases, scales) was complete before the previous kernel
 //     started, so the kernel may fetch it before its grid-dependency wait; only the activation comes from that kernel.
@@ -698,6 +728,8 @@ bool nm_linear_f32_supported(const nm_linear_desc* d);   // fp32, N a multiple o
 struct NmChain {
     bool weights_ready = false, late_trigger = false, back_to_back = false;
 };
+nm_status nm_launch_linear_f32(nm_ctx* ctx, const nm_linear_desc* d, cudaStream_t st, NmChain chain);
+bool nm_linear_f32_supported(const nm_linear_desc* d);   // fp32, N a multiple of 4; linear_simt takes the rest
 nm_status nm_launch_linear_tc(nm_ctx* ctx, const nm_linear_desc* d, cudaStream_t st, NmChain chain = NmChain());
 nm_status nm_linear_dispatch(nm_ctx* ctx, const nm_linear_desc* d, cudaStream_t st, NmChain chain);
 nm_status nm_conv2d_dispatch(nm_ctx* ctx, const nm_conv_desc* d, void* workspace, size_t ws_bytes, cudaStream_t st, NmChain chain);

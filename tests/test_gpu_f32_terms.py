@@ -1,0 +1,57 @@
+"""GPU parity, fp32 products as bf16 terms on the tensor cores: precision, the ends of the exponent range, infinities and NaN."""
+import pytest
+import torch
+
+import nm_inputs
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ctx(nm):
+    c = nm.Context(0)
+    yield c
+    c.close()
+
+
+def linear(ctx, A, W, algo=0):
+    out = torch.full((A.shape[0], W.shape[0]), float("nan"), device="cuda")
+    ctx.linear_pwl(A, W, out, algo=algo)
+    ctx.check_device_status()
+    return out
+
+
+# one CTA, both tile widths, splits, remainders of rows, columns and K
+@pytest.mark.parametrize("M,N,K", [(5, 8, 40), (128, 64, 64), (129, 196, 132), (300, 512, 2048), (1000, 1600, 768), (128, 768, 3072), (2000, 2304, 260)])
+def test_linear_precision(ctx, M, N, K):
+    """Four truncated steps of a sum, 4 * 1.55e-8, a chain of K / 64 rounded additions, 7.4e-9 sqrt(K / 64), and the rounding of the
+    result, 2.5e-8, all relative to the sums' rms.  They are added up, since the truncations all go towards zero."""
+    A, W = [torch.from_numpy(nm_inputs.matrix(s, K, "f32", d)).cuda() for s, d in (((M, K), 1.0), ((N, K), 0.02))]
+    ref = A.double() @ W.double().t()
+    err = ((linear(ctx, A, W).double() - ref).norm() / ref.norm()).item()
+    assert err < 4 * 1.55e-8 + 7.4e-9 * (K / 64) ** 0.5 + 2.5e-8
+
+
+@pytest.mark.parametrize("a_exp,w_exp", [(0, 0), (-110, 0), (0, -110), (-110, 100), (40, 40), (100, -100)])
+def test_linear_exponents(ctx, a_exp, w_exp):
+    """The terms' scaling keeps the range of fp32: the same result times a power of two."""
+    A, W = [torch.from_numpy(nm_inputs.matrix(s, 7, "f32", 1.0)).cuda() for s in ((70, 200), (68, 200))]
+    A, W = A.sign() * (A.abs() + 0.1), W.sign() * (W.abs() + 0.1)
+    base = linear(ctx, A, W)
+    got = linear(ctx, torch.ldexp(A, torch.tensor(a_exp)), torch.ldexp(W, torch.tensor(w_exp)))
+    assert torch.equal(got, torch.ldexp(base, torch.tensor(a_exp + w_exp)))
+
+
+@pytest.mark.parametrize("M,N,K", [(37, 60, 100), (200, 132, 320)])
+def test_linear_not_finite(nm, ctx, M, N, K):
+    A, W = [torch.from_numpy(nm_inputs.matrix(s, 9, "f32", 1.0)).cuda() for s in ((M, K), (N, K))]
+    big = torch.finfo(torch.float32).max
+    for i, v in enumerate([float("inf"), -float("inf"), float("nan"), big, -big]):
+        A[3 * i, (7 * i + 1) % K] = v
+        W[2 * i + 1, (11 * i + 5) % K] = v
+    W[20, :] = 0
+    W[20, 1] = 0.25   # exact in bf16: its lower terms are zero
+    got, ref = linear(ctx, A, W), linear(ctx, A, W, nm.ALGO_SIMT)
+    assert torch.equal(got.isnan(), ref.isnan()) and torch.equal(got.isinf(), ref.isinf())
+    assert torch.equal(got[got.isinf()], ref[got.isinf()]) and ref.isinf().any() and ref.isnan().any()
+    f = ref.isfinite()
+    assert ((got - ref)[f].abs() <= 1e-5 * ref[f].abs().clamp(min=K ** 0.5)).all()
