@@ -1,8 +1,11 @@
 """GPU parity, fp32 products as bf16 terms on the tensor cores: precision, the ends of the exponent range, infinities and NaN."""
+import numpy as np
 import pytest
 import torch
 
 import nm_inputs
+from util import load_tables_both
+
 pytestmark = pytest.mark.gpu
 
 
@@ -37,8 +40,8 @@ def test_linear_exponents(ctx, a_exp, w_exp):
     A, W = [torch.from_numpy(nm_inputs.matrix(s, 7, "f32", 1.0)).cuda() for s in ((70, 200), (68, 200))]
     A, W = A.sign() * (A.abs() + 0.1), W.sign() * (W.abs() + 0.1)
     base = linear(ctx, A, W)
-    got = linear(ctx, torch.ldexp(A, torch.tensor(a_exp)), torch.ldexp(W, torch.tensor(w_exp)))
-    assert torch.equal(got, torch.ldexp(base, torch.tensor(a_exp + w_exp)))
+    got = linear(ctx, A * 2.0 ** a_exp, W * 2.0 ** w_exp)
+    assert torch.equal(got, base * 2.0 ** (a_exp + w_exp))
 
 
 @pytest.mark.parametrize("M,N,K", [(37, 60, 100), (200, 132, 320)])
@@ -55,3 +58,34 @@ def test_linear_not_finite(nm, ctx, M, N, K):
     assert torch.equal(got[got.isinf()], ref[got.isinf()]) and ref.isinf().any() and ref.isnan().any()
     f = ref.isfinite()
     assert ((got - ref)[f].abs() <= 1e-5 * ref[f].abs().clamp(min=K ** 0.5)).all()
+
+
+@pytest.mark.parametrize("L", [1, 15, 16, 17, 64, 65, 100, 128])
+@pytest.mark.parametrize("n", [2, 64, 256])
+@pytest.mark.parametrize("odd", [None, "q", "k", "v", "large_v"])
+def test_attention(nm, ctx, L, n, odd):
+    """Against the CUDA-core kernel; one head of three has an operand that takes it off the tensor cores."""
+    B, h = 2, 3
+    load_tables_both(ctx, n, {"exp": (-8.0, 0.0), "recip": (max(L / 16.0, 0.5), float(max(L, 2)))})
+    x = torch.from_numpy(nm_inputs.matrix((B * L, 3 * h * 64), L, "f32", 0.8)).cuda()
+    if odd:
+        col = {"q": 64, "k": 3 * 64 + 64, "v": 6 * 64 + 64, "large_v": 6 * 64 + 64}[odd]
+        # (an infinite key's exponential is -inf, the extension of the table's first line; what comes of its infinite sum depends on
+        # where the reciprocal is multiplied)
+        x[L - 1, col + 5] = {"large_v": 1e30, "k": float("nan")}.get(odd, float("inf"))
+    outs = []
+    for algo in (nm.ALGO_AUTO, nm.ALGO_SIMT):
+        out = torch.full((B * L + 1, h * 64), float("nan"), device="cuda")
+        ctx.attention_pwl(x, out, B, L, h, 64, algo=algo)
+        ctx.check_device_status()
+        assert out[B * L:].isnan().all()
+        outs.append(out[:B * L].cpu().numpy().astype(np.float64))
+    got, ref = outs
+    assert (np.isnan(got) == np.isnan(ref)).all() and (np.isinf(got) == np.isinf(ref)).all()
+    assert (got[np.isinf(ref)] == ref[np.isinf(ref)]).all()
+    f = np.isfinite(ref)
+    # two products of up to 128 terms and a table slope of up to n segments' rounding each; the odd head's own size
+    scale = np.maximum(np.abs(ref), np.where(f, 1.0, 0.0) * 0.05)
+    with np.errstate(invalid="ignore"):
+        row = np.max(np.where(f, np.abs(ref), 0.0), axis=1, keepdims=True)
+    assert (np.abs(got - ref)[f] <= (2e-5 * np.maximum(scale, row))[f]).all()
