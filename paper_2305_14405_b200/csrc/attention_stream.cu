@@ -37,15 +37,17 @@
 //
 // ONE form (L <= 128, a single 128-key chunk): the scores and the accumulator do not share columns (128 | 64, and P behind
 // them: 256 columns, two CTAs per SM), so the one Q K^T of sweep 1 serves sweep 2 as well, and nothing is fetched or
-// multiplied twice in what is then a latency-bound kernel (B 1, L 128, 16 heads: 6.4 -> 4.9 us).  RAGGED and ONE: the first
-// two terms of a block of 16 keys take the place of its scores, the third goes behind the accumulator, and P V runs once,
-// over all keys and the smallest terms first, instead of once per 64 keys (B 32, L 100, 12 heads: 15.0 -> 12.8 us; B 1, L 37:
-// 5.3).
+// multiplied twice in what is then a latency-bound kernel (B 1, L 128, 16 heads: 6.4 -> 4.9 us).  All of V is fetched at once and P V
+// runs once, over all keys.  Two softmax warps share 32 rows, half of the blocks of 16 keys each; the second one's sums go on from the
+// first one's, in the order that one warp would take (int8 24 layers, 128 tokens: 889 -> 849 us; with several chunks per tile, where
+// the shared-memory pipe is the bound, two warps per quarter lose: B 32, L 512, 12 heads 70.8 -> 80.1).  RAGGED and ONE: the first two
+// terms of a block of 16 keys take the place of its scores, the third goes behind the accumulator, and P V takes the smallest
+// terms first, instead of one product per 64 keys (B 32, L 100, 12 heads: 15.0 -> 12.8 us; B 1, L 37: 5.3).
 //
 //   warp 0            control: TMA loads (K chunks through two stages, V chunks through one) and the tcgen05.mma
 //                     for S = Q K_c^T and O += P_c V_c (V as an MN-major operand).  It sleeps in a named barrier
 //                     (bar.sync) that the softmax warps signal with bar.arrive, so hand-offs cost no polling.
-//   warps 1..4        softmax, one per tensor-memory lane quarter: tcgen05.ld, row maximum (sweep 1); PWL exp, row
+//   warps 1..4 (ONE: 1..8)  softmax, one (two) per tensor-memory lane quarter: tcgen05.ld, row maximum (sweep 1); PWL exp, row
 //                     sum, P tile (sweep 2); PWL reciprocal, scaling, store (optionally as int8 codes for the int8
 //                     encoder).
 #include <string.h>
@@ -174,8 +176,11 @@ __device__ __forceinline__ void load_first_v(const LoadCtx& c, const Tile& t)
     for (int i = 0; i < c.v_chunks; ++i) nm_tma_load_3d(c.v_st + i * STAGE, c.tmV, t.g * HD, i * CK, t.b, c.bar_v_full);
 }
 
+// Threads of a CTA: the control warp and one or (ONE) two softmax warps per lane quarter.
+template <bool ONE> constexpr int CTA_THREADS = ONE ? 288 : 160;
+
 template <typename T, bool CLAMP_HI, bool RAGGED, bool ONE>
-__global__ void __launch_bounds__(160, RAGGED || ONE ? 2 : 3)
+__global__ void __launch_bounds__(CTA_THREADS<ONE>, RAGGED || ONE ? 2 : 3)
 attention_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                         const __grid_constant__ CUtensorMap tmV, const SArgs a)
 {
@@ -191,17 +196,22 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
     constexpr uint32_t P_COLS = RAGGED ? 128 : 32;
     constexpr int TERMS = RAGGED ? ProbTerms<T>::N : 1;
     constexpr bool SCALED = RAGGED && std::is_same<T, __half>::value;
+    constexpr int NT = CTA_THREADS<ONE>;
+    constexpr int LD = ONE ? 16 : 32;   // scores read at a time
 
     extern __shared__ uint8_t smem_raw[];
     __shared__ uint64_t bar_q, bar_drain;
     __shared__ uint64_t bar_k_full[2], bar_k1_full[2], bar_v_full, bar_s_full, bar_p_empty;
     __shared__ uint32_t tmem_slot, tmem_slot_p;
     __shared__ int abort_flag;
+    // ONE: the two warps' row maxima (SCALED: and minima), and what they pass on to add a row up as one of them would
+    __shared__ float s_pair[ONE ? 2 : 1][2][BQ];
+    __shared__ float4 s_sum[ONE ? 9 : 1][ONE ? BQ : 1];
 
     const int L = a.L;
     const int n = RAGGED ? (L + CK - 1) / CK : L / CK;                    // 64-key chunks of sweep 2
-    // P V products: RAGGED one per 32 keys, or one for all of them (ONE); otherwise one per chunk
-    const int n_pv = !RAGGED ? n : ONE ? 1 : (L + 31) / 32;
+    // P V products: one for all keys (ONE), one per 32 keys (RAGGED), otherwise one per chunk
+    const int n_pv = ONE ? 1 : !RAGGED ? n : (L + 31) / 32;
     const int n128 = ONE ? 1 : RAGGED ? (L + 2 * CK - 1) / (2 * CK) : L / (2 * CK);   // 128-key chunks of sweep 1
     uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     uint8_t* q_s = base;                       // 16 KB
@@ -224,7 +234,7 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
     lc.bar_q = &bar_q; lc.bar_k1_full = &bar_k1_full[0]; lc.bar_v_full = &bar_v_full;
     lc.n128 = n128;
     lc.v_chunks = 1;
-    if (RAGGED && ONE) {   // all of V in the buffer that sweep 1 of longer sequences takes
+    if (ONE) {   // all of V in the buffer that sweep 1 of longer sequences takes
         lc.v_st = p_s;
         lc.v_chunks = n;
     }
@@ -263,7 +273,7 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
         // half a warp at a time, so 16 copies already make arbitrary lookups conflict-free.  One extra
         // entry (a copy of the last) lets input 0 of a table whose range ends at 0 go unclamped.
         const int ne = a.n_exp;
-        for (int i = threadIdx.x - 32; i < (ne + 1) * 16; i += 128) rep[i] = a.t_exp->kb[min(i >> 4, ne - 1)];
+        for (int i = threadIdx.x - 32; i < (ne + 1) * 16; i += NT - 32) rep[i] = a.t_exp->kb[min(i >> 4, ne - 1)];
     }
     nm_tc_fence_before();
     __syncthreads();
@@ -298,7 +308,7 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
             if (ok && !wait(&bar_q, q_cnt & 1u)) ok = false;
             ++q_cnt;
             // the previous tile's epilogue has read O out of tensor memory (sweep 1 writes over [S | O])
-            if (ti > 0) asm volatile("bar.sync %0, %1;" ::"r"(bar_oc), "n"(160) : "memory");
+            if (ti > 0) asm volatile("bar.sync %0, %1;" ::"r"(bar_oc), "n"(NT) : "memory");
             // ---- sweep 1: [S | O] = Q K^T for 128 keys at a time; K stage i & 1 (0: the two K stages
             // taken together, 1: the P tile)
             auto issue_qk1 = [&](int i) {
@@ -317,7 +327,7 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
             };
             if (n128 > 0) issue_qk1(0);
             for (int i = 0; !ONE && i < n128; ++i) {
-                asm volatile("bar.sync %0, %1;" ::"r"(bar_sc), "n"(160) : "memory");   // S-consumed: chunk i is in registers
+                asm volatile("bar.sync %0, %1;" ::"r"(bar_sc), "n"(NT) : "memory");   // S-consumed: chunk i is in registers
                 if (i + 1 < n128) issue_qk1(i + 1);
                 if (ok && i + 2 < n128 && nm_elect_one()) {   // its MMAs are complete: the stage takes the chunk after next
                     uint8_t* dst = (i & 1) ? p_s : k_st;
@@ -361,7 +371,7 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                 const bool chunk_begins = !RAGGED || ONE || !(u & 1);
                 if constexpr (!ONE) {
                     if (chunk_ends) {
-                        asm volatile("bar.sync %0, %1;" ::"r"(bar_sc), "n"(160) : "memory");   // S-consumed(j)
+                        asm volatile("bar.sync %0, %1;" ::"r"(bar_sc), "n"(NT) : "memory");   // S-consumed(j)
                         if (j + 1 < n) issue_qk(j + 1);
                         if (j + 2 < n) load_k(j + 2);
                     }
@@ -372,7 +382,7 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                 // first loads now.
                 if (u + 1 == n_pv && more && ok && nm_elect_one()) load_tile_head(lc, tile_of(tile + (int)gridDim.x));
                 __syncwarp();
-                asm volatile("bar.sync %0, %1;" ::"r"(bar_pr), "n"(160) : "memory");   // P-ready(u)
+                asm volatile("bar.sync %0, %1;" ::"r"(bar_pr), "n"(NT) : "memory");   // P-ready(u)
                 if (chunk_begins) {
                     if (ok && !wait(&bar_v_full, v_cnt & 1u)) ok = false;
                     ++v_cnt;
@@ -385,7 +395,7 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                     if (nm_elect_one()) {
                         if constexpr (!RAGGED) {
 #pragma unroll
-                            for (int k = 0; k < 4; ++k)
+                            for (int k = 0; k < (ONE ? 8 : 4); ++k)
                                 nm_mma_f16_a_tmem(tmem_base + O_OFF, tmem_p + (uint32_t)(8 * k), vdesc(k), IDESC_PV, (j | k) != 0);
                         } else if constexpr (ONE) {
                             const int steps = (L + 15) / 16;
@@ -440,7 +450,15 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
         // One row per thread.  A warp never blocks on the others: it signals the control warp with bar.arrive.
         const int q = warp & 3;
         const int row = q * 32 + lane;
+        const int part = ONE ? (warp - 1) >> 2 : 0;   // which of the two warps that share 32 rows, half of the blocks of 16 keys each
+        const int blocks = RAGGED ? (L + 15) / 16 : 8, first = part * ((blocks + 1) / 2), last = part ? blocks : (blocks + 1) / 2;   // ONE: its blocks
         const uint32_t bar_sc = 2, bar_pr = 3, bar_oc = 6;
+        // this row's value of the other warp, which takes the same steps
+        [[maybe_unused]] auto swap = [&](float (*buf)[BQ], float v) {
+            buf[part][row] = v;
+            asm volatile("bar.sync %0, 64;" ::"r"(8 + q) : "memory");
+            return buf[part ^ 1][row];
+        };
         const uint32_t t_row = tmem_base + ((uint32_t)(q * 32) << 16);
         const float inv_h = a.t_exp->inv_h, off = a.t_exp->off, nm1 = (float)(a.n_exp - 1);
         // this lane's copy of the replicated table, with the constant of the index trick folded in:
@@ -487,36 +505,40 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                     nm_tc_fence_after();
 #pragma unroll
                     for (int hh = 0; hh < 4; ++hh) {   // 128 keys: the scores span [S | O]
-                        uint32_t r[32];
-                        if (ONE && hh * 32 >= L) continue;   // no keys there
-                        nm_tmem_ld32_sync(t_row + (uint32_t)(hh * 32), r);
+                        uint32_t r[LD];
+                        const int key = ONE ? (first + hh) * 16 : hh * 32;
+                        if (ONE && first + hh >= last) continue;   // no keys there
+                        if constexpr (ONE) nm_tmem_ld16_sync(t_row + (uint32_t)key, r);
+                        else nm_tmem_ld32_sync(t_row + (uint32_t)key, r);
                         if (!ONE && hh == 3) {   // all of it is in registers: the control warp may overwrite S
                             nm_tc_fence_before();
-                            asm volatile("bar.arrive %0, %1;" ::"r"(bar_sc), "n"(160) : "memory");
+                            asm volatile("bar.arrive %0, %1;" ::"r"(bar_sc), "n"(NT) : "memory");
                         }
                         if (RAGGED && i == n128 - 1) {   // keys beyond L do not take part
-                            const int lim = L - i * 2 * CK - hh * 32;
+                            const int lim = L - i * 2 * CK - key;
 #pragma unroll
-                            for (int k = 0; k < 32; ++k) {
+                            for (int k = 0; k < LD; ++k) {
                                 if (SCALED && k < lim) lowest = fminf(lowest, __uint_as_float(r[k]));
                                 if (k >= lim) r[k] = 0xff800000u;   // -inf
                             }
                         } else if (SCALED) {
 #pragma unroll
-                            for (int k = 0; k < 32; ++k) lowest = fminf(lowest, __uint_as_float(r[k]));
+                            for (int k = 0; k < LD; ++k) lowest = fminf(lowest, __uint_as_float(r[k]));
                         }
                         float m0 = -INFINITY, m1 = -INFINITY;
 #pragma unroll
-                        for (int k = 0; k < 32; k += 4) {
+                        for (int k = 0; k < LD; k += 4) {
                             m0 = max3f(m0, __uint_as_float(r[k]), __uint_as_float(r[k + 1]));
                             m1 = max3f(m1, __uint_as_float(r[k + 2]), __uint_as_float(r[k + 3]));
                         }
                         m = max3f(m, m0, m1);
                     }
                 } else if (!ONE) {
-                    asm volatile("bar.arrive %0, %1;" ::"r"(bar_sc), "n"(160) : "memory");
+                    asm volatile("bar.arrive %0, %1;" ::"r"(bar_sc), "n"(NT) : "memory");
                 }
             }
+            if constexpr (ONE) m = fmaxf(m, swap(s_pair[0], m));
+            if constexpr (ONE && SCALED) lowest = fminf(lowest, swap(s_pair[1], lowest));
             // RAGGED: the scores are scaled and rounded before the maximum is subtracted, and the segment number is clamped on
             // both sides, as on the CUDA cores.  Otherwise one FMA does both, and its result must not lie above 0, which is what
             // bounds the segment number there: the product is rounded up.  Rounded to nearest, fma(m, scale, -m scale) lies up
@@ -524,6 +546,7 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
             const float neg_ms = RAGGED ? -__fmul_rn(m, a.scale) : -__fmul_ru(m, a.scale);
             const uint64_t neg_ms2 = nm_pack2(neg_ms, neg_ms);
             float sum0 = 0.f, sum1 = 0.f, sum2 = 0.f, sum3 = 0.f;
+            [[maybe_unused]] int groups = 0;   // ONE: groups of 8 keys that the second warp has put into s_sum
             // SCALED: the power of two that brings the largest |e| this row can have to 2^14 .. 2^15 (below the table the first
             // segment goes on), and its inverse; an fp16 term then loses nothing to the narrow exponent
             [[maybe_unused]] float up = 1.f, down = 1.f;
@@ -538,7 +561,7 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
             // ---- sweep 2: e = PWL_exp(s - m), row sum, P tiles.
             // W scores of this thread's row -> exponentials, in groups of 8.  MASKED: keys from `lim` on lie beyond L; they take
             // the maximum as their score (which keeps the table index in range) and the exponential 0.
-            constexpr int W = RAGGED ? 16 : 32;   // (with several terms of P, 32 keys at a time spill)
+            constexpr int W = RAGGED ? 16 : LD;   // (with several terms of P, 32 keys at a time spill)
             auto exponentials = [&](uint32_t* r, int lim, auto masked, auto&& use) {
                 constexpr bool MASKED = decltype(masked)::value;
                 if constexpr (MASKED) {
@@ -584,28 +607,46 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                             if (jj * 8 + k + 1 >= lim) e[k + 1] = 0.f;
                         }
                     }
-                    sum0 += e[0] + e[4];
-                    sum1 += e[1] + e[5];
-                    sum2 += e[2] + e[6];
-                    sum3 += e[3] + e[7];
+                    if (ONE && part == 1) {   // (to be added up behind the first warp's)
+                        s_sum[groups++][row] = make_float4(e[0] + e[4], e[1] + e[5], e[2] + e[6], e[3] + e[7]);
+                    } else {
+                        sum0 += e[0] + e[4];
+                        sum1 += e[1] + e[5];
+                        sum2 += e[2] + e[6];
+                        sum3 += e[3] + e[7];
+                    }
                     use(jj, e);
                 }
             };
-            if constexpr (!RAGGED) {
+            if constexpr (!RAGGED && ONE) {
+#pragma unroll 1
+                for (int k = first; k < last; ++k) {
+                    uint32_t r[16], pk[8];
+                    if (ok) {
+                        nm_tmem_ld16_sync(t_row + (uint32_t)(16 * k), r);
+                        exponentials(r, W, std::false_type{}, [&](int jj, const float* e) {
+#pragma unroll
+                            for (int i = 0; i < 4; ++i) pk[jj * 4 + i] = AT<T>::pack(e[2 * i], e[2 * i + 1]);
+                        });
+                        nm_tmem_st8(p_row + (uint32_t)(8 * k), pk);
+                    }
+                }
+                nm_tmem_st_wait();
+                nm_tc_fence_before();
+                asm volatile("bar.arrive %0, %1;" ::"r"(bar_pr), "n"(NT) : "memory");
+            } else if constexpr (!RAGGED) {
 #pragma unroll 1
                 for (int j = 0; j < n; ++j) {
-                    if constexpr (!ONE) {
-                        wait_all(&bar_s_full, s_cnt & 1u);
-                        ++s_cnt;
-                        if (ok) nm_tc_fence_after();
-                    }
+                    wait_all(&bar_s_full, s_cnt & 1u);
+                    ++s_cnt;
+                    if (ok) nm_tc_fence_after();
 #pragma unroll
                     for (int hh = 0; hh < 2; ++hh) {
                         uint32_t r[32];
-                        if (ok) nm_tmem_ld32_sync(t_row + (uint32_t)((ONE ? j * CK : 0) + hh * 32), r);
-                        if (!ONE && hh == 1) {
+                        if (ok) nm_tmem_ld32_sync(t_row + (uint32_t)(hh * 32), r);
+                        if (hh == 1) {
                             nm_tc_fence_before();
-                            asm volatile("bar.arrive %0, %1;" ::"r"(bar_sc), "n"(160) : "memory");
+                            asm volatile("bar.arrive %0, %1;" ::"r"(bar_sc), "n"(NT) : "memory");
                         }
                         uint32_t pk[16];   // the half's 32 exponentials, packed to 16 bits
                         if (ok)
@@ -623,7 +664,7 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                     }
                     nm_tmem_st_wait();          // the P columns are written
                     nm_tc_fence_before();
-                    asm volatile("bar.arrive %0, %1;" ::"r"(bar_pr), "n"(160) : "memory");
+                    asm volatile("bar.arrive %0, %1;" ::"r"(bar_pr), "n"(NT) : "memory");
                 }
             } else {
                 // 16 keys' scores at tensor-memory column `src` -> the terms of their exponentials
@@ -650,13 +691,12 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                             if constexpr (TERMS == 3) nm_tmem_st8(p_row + (uint32_t)(8 * k), term[2]);
                         }
                     };
-                    const int steps = (L + 15) / 16;
 #pragma unroll 1
-                    for (int k = 0; k < steps - 1; ++k) keys16(k, std::false_type{});
-                    keys16(steps - 1, std::true_type{});
+                    for (int k = first; k < (last < blocks ? last : blocks - 1); ++k) keys16(k, std::false_type{});
+                    if (first < last && last == blocks) keys16(blocks - 1, std::true_type{});
                     nm_tmem_st_wait();
                     nm_tc_fence_before();
-                    asm volatile("bar.arrive %0, %1;" ::"r"(bar_pr), "n"(160) : "memory");
+                    asm volatile("bar.arrive %0, %1;" ::"r"(bar_pr), "n"(NT) : "memory");
                 } else {
                     auto keys32 = [&](int u, auto masked) {
                         const bool chunk_ends = (u & 1) || u + 1 == n_pv;
@@ -670,7 +710,7 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                             block(t_row + (uint32_t)((u & 1) * 32 + hh * 16), L - u * 32 - hh * 16, masked, [&] {
                                 if (hh == 1 && chunk_ends) {   // all of the chunk's scores are in registers
                                     nm_tc_fence_before();
-                                    asm volatile("bar.arrive %0, %1;" ::"r"(bar_sc), "n"(160) : "memory");
+                                    asm volatile("bar.arrive %0, %1;" ::"r"(bar_sc), "n"(NT) : "memory");
                                 }
                             });
                             // the stores wait until the previous P V has read the columns; 16 keys' arithmetic runs ahead of it
@@ -683,14 +723,31 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                         }
                         nm_tmem_st_wait();
                         nm_tc_fence_before();
-                        asm volatile("bar.arrive %0, %1;" ::"r"(bar_pr), "n"(160) : "memory");
+                        asm volatile("bar.arrive %0, %1;" ::"r"(bar_pr), "n"(NT) : "memory");
                     };
 #pragma unroll 1
                     for (int u = 0; u < n_pv - 1; ++u) keys32(u, std::false_type{});
                     keys32(n_pv - 1, std::true_type{});
                 }
             }
-            const float sum = (sum0 + sum1) + (sum2 + sum3);
+            float sum = (sum0 + sum1) + (sum2 + sum3);
+            if constexpr (ONE) {
+                // Added up in the order that one warp would take, so that the last bit does not depend on the split (an int8
+                // network's codes do on that bit): the second warp goes on from the first one's four sums.
+                float* const total = &s_pair[0][0][row];   // (the maxima have been read: both warps are at the barrier below)
+                if (part == 0) s_sum[8][row] = make_float4(sum0, sum1, sum2, sum3);
+                asm volatile("bar.sync %0, 64;" ::"r"(8 + q) : "memory");
+                if (part == 1) {
+                    float4 c = s_sum[8][row];
+                    for (int i = 0; i < groups; ++i) {
+                        const float4 v = s_sum[i][row];
+                        c.x += v.x; c.y += v.y; c.z += v.z; c.w += v.w;
+                    }
+                    *total = sum = (c.x + c.y) + (c.z + c.w);
+                }
+                asm volatile("bar.sync %0, 64;" ::"r"(8 + q) : "memory");
+                sum = *total;
+            }
             // ---- r = PWL_recip(sigma), then O * r
             const int sr = ONE ? nm_pwl_index(sum, r_inv_h, r_off, r_nm1)
                                : nm_pwl_index(sum, a.t_rcp->inv_h, a.t_rcp->off, (float)(a.t_rcp->n - 1));
@@ -704,7 +761,8 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                       (size_t)g * HD;
             const uint32_t o_addr = t_row + O_OFF;
 #pragma unroll
-            for (int jj = 0; jj < HD / 16; ++jj) {   // 16 channels at a time
+            for (int j2 = 0; j2 < (ONE ? HD / 32 : HD / 16); ++j2) {   // 16 channels at a time
+                const int jj = ONE ? 2 * part + j2 : j2;
                 uint32_t r0[16];
                 if (ok && live) {
                     nm_tmem_ld16_sync(o_addr + (uint32_t)(jj * 16), r0);
@@ -715,10 +773,10 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                         for (int k = 0; k < 16; ++k) r0[k] = __float_as_uint(__uint_as_float(r0[k]) + __uint_as_float(r1[k]));
                     }
                 }
-                if (jj == HD / 16 - 1 && more) {
+                if (j2 == (ONE ? HD / 32 : HD / 16) - 1 && more) {
                     // all of O is in registers: the control warp may start the next tile's sweep 1 over [S | O]
                     nm_tc_fence_before();
-                    asm volatile("bar.arrive %0, %1;" ::"r"(bar_oc), "n"(160) : "memory");
+                    asm volatile("bar.arrive %0, %1;" ::"r"(bar_oc), "n"(NT) : "memory");
                 }
                 if (ok && store_row) {
                     float v[16];
@@ -813,7 +871,7 @@ nm_status launch(nm_ctx* ctx, const nm_attn_desc* d, cudaStream_t st, int8_t* ou
     // persistent: one resident wave of CTAs, each walking over tiles.  Three CTAs per SM (RAGGED, ONE: two) by the launch
     // bounds (registers) and by tensor memory (3 x 160 or 2 x 256 of 512 columns); fewer if the exp table makes the
     // shared memory larger (233472 bytes per SM, 1 KB reserved per CTA).
-    int64_t per_sm = 233472 / (int64_t)(smem + 1024 + 1536);
+    int64_t per_sm = 233472 / (int64_t)(smem + 1024 + (ONE ? 22 * 1024 : 1536));
     if (per_sm > (RAGGED || ONE ? 2 : 3)) per_sm = RAGGED || ONE ? 2 : 3;
     if (per_sm < 1) per_sm = 1;
     int64_t grid = (int64_t)ctx->sm_count * per_sm;
@@ -821,7 +879,7 @@ nm_status launch(nm_ctx* ctx, const nm_attn_desc* d, cudaStream_t st, int8_t* ou
     cudaLaunchConfig_t cfg;
     memset(&cfg, 0, sizeof(cfg));
     cfg.gridDim = dim3((unsigned)grid);
-    cfg.blockDim = dim3(160);
+    cfg.blockDim = dim3(CTA_THREADS<ONE>);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
