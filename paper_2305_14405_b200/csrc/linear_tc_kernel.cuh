@@ -8,7 +8,7 @@
 //   warp 0     TMA producer: 128 x 128-byte A tile and W tile per stage, 128-byte swizzle,
 //              multi-stage mbarrier ring
 //   warp 1     tcgen05.mma issuer (one lane); accumulators live in tensor memory, two
-//              buffers of BN columns so the epilogue of tile i overlaps the main loop
+//              or four buffers of BN columns so the epilogue of tile i overlaps the main loop
 //              of tile i+1
 //   warps 2-9  epilogue, two warps per tensor-memory lane quarter.  Per 32-column chunk:
 //              tcgen05.ld -> bias/scale -> segment index
@@ -21,7 +21,7 @@
 //
 // BN = 256, 128 or 64 columns per tile (the MMA's N): narrow layers get a narrow tile instead of
 //   multiplying zero-filled weight rows.  With BN = 64 the two warps of a lane quarter do not split
-//   the tile's columns but take alternate tiles (each warp always reads the same accumulator buffer).
+//   the tile's columns but take alternate tiles.
 // TWO = false: one CTA per 128 x BN tile (tcgen05 cta_group::1).
 // TWO = true:  a cluster of two CTAs per 256 x BN tile (cta_group::2): each CTA loads its
 //   own 128 rows of A and its own BN/2 rows of W, the leader CTA issues one MMA over both,
@@ -200,7 +200,6 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     static_assert(!HALO || (CONV && TWO), "the halo form is built for CTA pairs");
     constexpr int TILE_M = TWO ? 2 * BM : BM;
     constexpr int BK_ELEMS = ROW_BYTES / (int)sizeof(InT);
-    constexpr uint32_t TMEM_COLS = 2 * BN;
     constexpr uint32_t IDESC = nm_idesc(TcIn<InT>::c_fmt, TcIn<InT>::ab_fmt, 0, 0, TILE_M, BN);
     // epilogue geometry: the two warps of a lane quarter split the tile's columns (BN/2 each), or, for the
     // 64-column tile, take alternate tiles (64 columns each).  A chunk is 32 columns; a staging group is 128
@@ -223,14 +222,18 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     // Several accumulators per tile (TcArgs::acc_steps): matrices of few columns.
     constexpr bool MULTI = BN == 64 && !CONV && !TcIn<InT>::is_int;
     const uint32_t buf_cols = MULTI ? BN * (uint32_t)a.accs : BN;
-    const uint32_t tmem_cols = !MULTI || a.accs <= 1 ? TMEM_COLS : a.accs <= 2 ? 2 * TMEM_COLS : 4 * TMEM_COLS;
+    // Accumulator buffers: with two, a narrow tile waits for the hand-over to the epilogue and back (128 images, 56 x 56, 64 -> 256 with
+    // residual: 107 -> 102 us; ResNet-50 batch 128: 2299 -> 2285).
+    constexpr int MOST_BUFS = BN == 256 ? 2 : 4;
+    const int bufs = MULTI && a.accs > 1 ? 2 : MOST_BUFS, buf_shift = bufs == 4 ? 2 : 1;
+    const uint32_t tmem_cols = !MULTI || a.accs <= 1 ? MOST_BUFS * BN : a.accs <= 2 ? 4 * BN : 8 * BN;
     auto vote = [](bool done) { return ONE_LANE ? done : __all_sync(0xffffffffu, done) != 0; };
 
     extern __shared__ uint8_t smem_raw[];
     __shared__ uint64_t bar_full[MAX_STAGES];
     __shared__ uint64_t bar_empty[MAX_STAGES];
-    __shared__ uint64_t bar_acc_full[2];
-    __shared__ uint64_t bar_acc_empty[2];
+    __shared__ uint64_t bar_acc_full[MOST_BUFS];
+    __shared__ uint64_t bar_acc_empty[MOST_BUFS];
     __shared__ uint64_t bar_res[NUM_EPI_WARPS];
     __shared__ uint64_t bar_res_free[NUM_EPI_WARPS];
     __shared__ uint64_t bar_wfull[HALO ? MAX_W_STAGES : 1], bar_wempty[HALO ? MAX_W_STAGES : 1];
@@ -268,7 +271,7 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                 nm_mbar_init(&bar_wempty[i], 1);
             }
         }
-        for (int b = 0; b < 2; ++b) {
+        for (int b = 0; b < MOST_BUFS; ++b) {
             nm_mbar_init(&bar_acc_full[b], 1);
             nm_mbar_init(&bar_acc_empty[b], (ALT ? NUM_EPI_WARPS / 2 : NUM_EPI_WARPS) * (TWO ? 2 : 1));
         }
@@ -483,7 +486,7 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                     else nm_tc_commit(&bar_acc_full[buf]);
                 }
                 if constexpr (!ONE_LANE) __syncwarp();
-                buf ^= 1;
+                buf = (buf + 1) & (bufs - 1);
                 if (buf == 0) acc_phase ^= 1u;
             }
             if (!ok && (ONE_LANE || nm_elect_one())) {
@@ -564,10 +567,10 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             }
         };
         fetch_vec(my_first);
-        // the CTA's it-th tile uses accumulator buffer it & 1, in that buffer's (it >> 1)-th use
+        // the CTA's it-th tile uses accumulator buffer it % bufs, in that buffer's (it / bufs)-th use
         for (int tile = my_first, it = ALT ? wsel : 0; ok && tile < a.num_tiles; tile += my_step, it += EPI_STEP) {
-            const int buf = it & 1;
-            const uint32_t acc_phase = (uint32_t)((it >> 1) & 1);
+            const int buf = it & (bufs - 1);
+            const uint32_t acc_phase = (uint32_t)((it >> buf_shift) & 1);
             const int mt = tile / a.num_n_tiles;
             const int m0 = mt * TILE_M + (int)rank * BM;
             const int n0 = (tile % a.num_n_tiles) * BN + col_off;
