@@ -16,6 +16,7 @@ enum ConvPath {
                     // input, one K-block per filter row: 8 taps x 8 channels = 64 contiguous elements
     CONV_PAIRTAP,   // the same with stride 2 and Cin <= 4: image rows in pairs, a K-block is two filter rows of 8 taps x 4
                     // channels (128 images of 224 x 224 x 3, 7 x 7: 279 us with one row per K-block, 178 so, copies included)
+    CONV_STEM,      // the same where the kernel's form for it applies (linear_tc_kernel.cuh): 4 channels per pixel, no pairs
     CONV_GATHER     // anything else: explicit gather (im2col) into the workspace, then the GEMM
 };
 
@@ -47,6 +48,13 @@ bool conv_geom(const nm_conv_desc* d, ConvGeom* g)
         g->path = CONV_DIRECT;
     } else if (d->Cin % 64 == 0 && d->algo != 1) {
         g->path = CONV_IMPLICIT;
+    } else if (d->Cin <= 4 && d->kw <= 8 && d->kh <= 8 && d->stride == 2 && d->algo == 0 && d->Cout <= 128 && d->pad <= 64) {
+        // (wider outputs keep the row pairs: all weights have to stay in shared memory; so do forced kernels)
+        g->path = CONV_STEM;
+        g->Hp = d->H;
+        g->Wp = (d->W + d->pad + 1) & ~1;
+        g->a_bytes = align256((size_t)d->N * g->Hp * g->Wp * 4 * 2);
+        g->w_bytes = align256((size_t)d->Cout * ((d->kh + 1) / 2) * 64 * 2);
     } else if (d->Cin <= 4 && d->kw <= 8 && d->stride == 2 && d->algo != 1) {
         g->path = CONV_PAIRTAP;
         // Output row oy reads pair rows oy .. oy + kh / 2 - 1, output pixel ox pixels 2 ox .. 2 ox + 7.  The last row of an odd
@@ -127,7 +135,7 @@ nm_status nm_conv2d_dispatch(nm_ctx* ctx, const nm_conv_desc* d, void* workspace
         if (!workspace || ws_bytes < need) return NM_ERR_WORKSPACE;
         if (((uintptr_t)workspace & 255u) != 0) return NM_ERR_ALIGNMENT;
     }
-    if (g.path == CONV_IMPLICIT || g.path == CONV_ROWTAP || g.path == CONV_PAIRTAP) {
+    if (g.path == CONV_IMPLICIT || g.path == CONV_ROWTAP || g.path == CONV_PAIRTAP || g.path == CONV_STEM) {
         NmConvTc c;
         memset(&c, 0, sizeof(c));
         c.dtype = d->dtype;
@@ -143,6 +151,21 @@ nm_status nm_conv2d_dispatch(nm_ctx* ctx, const nm_conv_desc* d, void* workspace
             c.sw = c.sh = d->stride; c.pw = c.ph = d->pad;
             c.taps_y = d->kh; c.taps_x = d->kw; c.cblocks = d->Cin / 64;
             c.w = d->w; c.ldw = g.K; c.Ktot = g.K;
+        } else if (g.path == CONV_STEM) {
+            void* xp = workspace;
+            void* wp = (uint8_t*)workspace + g.a_bytes;
+            const int pairs = (d->kh + 1) / 2;
+            const nm_status s = nm_launch_pad_stem(ctx, d->x, xp, d->w, wp, d->dtype, d->N, d->H, d->W, d->Cin, d->pad, g.Wp, d->Cout, d->kh, d->kw, st);
+            if (s != NM_OK) return s;
+            c.a_base = xp;
+            c.a_dim[0] = (uint64_t)g.Wp * 4; c.a_dim[1] = (uint64_t)d->H; c.a_dim[2] = (uint64_t)d->N; c.a_dim[3] = 1;
+            c.a_stride[0] = (uint64_t)g.Wp * 8;
+            c.a_stride[1] = (uint64_t)d->H * g.Wp * 8;
+            c.a_stride[2] = (uint64_t)d->N * d->H * g.Wp * 8;
+            c.sw = c.sh = 2; c.pw = c.ph = d->pad;
+            c.taps_y = pairs; c.taps_x = 1; c.cblocks = 1;
+            c.stem_kh = d->kh;
+            c.w = wp; c.ldw = (int64_t)pairs * 64; c.Ktot = (int64_t)pairs * 64;
         } else if (g.path == CONV_PAIRTAP) {
             void* xp = workspace;
             void* wp = (uint8_t*)workspace + g.a_bytes;

@@ -9,14 +9,15 @@ using namespace nm_tc;
 namespace {
 
 nm_status make_tmap4(nm_ctx* ctx, CUtensorMap* m, const void* base, nm_dtype dt, const uint64_t dim[4],
-                     const uint64_t stride_bytes[3], const uint32_t box[4], const uint32_t estr[4])
+                     const uint64_t stride_bytes[3], const uint32_t box[4], const uint32_t estr[4],
+                     CUtensorMapSwizzle swizzle = CU_TENSOR_MAP_SWIZZLE_128B)
 {
     cuuint64_t gdim[4] = {dim[0], dim[1], dim[2], dim[3]};
     cuuint64_t gstr[3] = {stride_bytes[0], stride_bytes[1], stride_bytes[2]};
     cuuint32_t b[4] = {box[0], box[1], box[2], box[3]};
     cuuint32_t e[4] = {estr[0], estr[1], estr[2], estr[3]};
     CUresult r = ((EncodeTiledFn)ctx->encode_tiled)(m, tmap_type(dt), 4, const_cast<void*>(base), gdim, gstr, b, e,
-                                                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                                                    CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle,
                                                     CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                                                     CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return r == CUDA_SUCCESS ? NM_OK : NM_ERR_CUDA;
@@ -52,6 +53,7 @@ int64_t fill_args(nm_ctx* ctx, const NmConvTc* c, NmChain chain, TcArgs* a)
     cv.ky_last = c->taps_y - 1; cv.ky_jump = c->last_row_jump;
     cv.Ho = c->Ho; cv.Nimg = c->N;
     cv.dw = c->depthwise;
+    cv.stem_kh = c->stem_kh;
     a->M = (int64_t)c->N * c->Ho * c->Wo; a->N = c->Cout; a->K = c->Ktot;
     a->bias = c->bias;
     a->has_res = c->residual ? 1 : 0;
@@ -113,7 +115,8 @@ bool use_halo(const NmConvTc* c, int64_t free_patches, int sms)
     return t_halo < 0.9 * t_free;
 }
 
-template <typename T, int BN>
+// The forms that load a patch of 8 x 16 output pixels' input once: HALO3X3 and STEM.
+template <typename T, int BN, int FORM>
 nm_status launch_halo(nm_ctx* ctx, const NmConvTc* c, NmChain chain, cudaStream_t st)
 {
     TcArgs a;
@@ -127,16 +130,17 @@ nm_status launch_halo(nm_ctx* ctx, const NmConvTc* c, NmChain chain, cudaStream_
     if (patches / 2 > 0x7ffffffeLL) return NM_ERR_UNSUPPORTED;
     a.num_tiles = (int)((patches + 1) / 2);
     size_t smem = 0;
-    if (!plan_smem_halo<T, BN>(&a, c->bias != nullptr, &smem)) return NM_ERR_UNSUPPORTED;
+    if (!plan_smem_halo<T, BN, FORM>(&a, c->bias != nullptr, &smem)) return NM_ERR_UNSUPPORTED;
     CUtensorMap tmA, tmW, tmO, tmR;
-    const uint32_t abox[4] = {64u, HALO_W, HALO_H, 1u}, one[4] = {1u, 1u, 1u, 1u};
-    nm_status s = make_tmap4(ctx, &tmA, c->a_base, c->dtype, c->a_dim, c->a_stride, abox, one);
+    const uint32_t halo[4] = {64u, HALO_W, HALO_H, 1u}, stem[4] = {STEM_PITCH / 2, (uint32_t)(30 + c->stem_kh), 1u, 1u}, one[4] = {1u, 1u, 1u, 1u};
+    nm_status s = make_tmap4(ctx, &tmA, c->a_base, c->dtype, c->a_dim, c->a_stride, FORM == STEM ? stem : halo, one,
+                             FORM == STEM ? CU_TENSOR_MAP_SWIZZLE_NONE : CU_TENSOR_MAP_SWIZZLE_128B);
     if (s != NM_OK) return s;
     s = make_tmap(ctx, &tmW, c->w, c->dtype, c->Cout, c->Ktot, c->ldw, BN / 2);
     if (s != NM_OK) return s;
     s = make_tmaps_out(ctx, &tmO, &tmR, c, cv);
     if (s != NM_OK) return s;
-    return launch_kernel<T, T, true, BN, true, true>(ctx, tmA, tmW, tmO, tmR, a, smem, c->flops, st);
+    return launch_kernel<T, T, true, BN, true, FORM>(ctx, tmA, tmW, tmO, tmR, a, smem, c->flops, st);
 }
 
 template <typename T, int BN>
@@ -189,13 +193,14 @@ nm_status launch(nm_ctx* ctx, const NmConvTc* c, NmChain chain, cudaStream_t st)
 template <typename T>
 nm_status launch_sel(nm_ctx* ctx, const NmConvTc* c, NmChain chain, cudaStream_t st)
 {
+    if (c->stem_kh) return c->Cout <= 64 ? launch_halo<T, 64, STEM>(ctx, c, chain, st) : launch_halo<T, 128, STEM>(ctx, c, chain, st);
     TileChoice t;
     if (c->algo == 0) {
         int tw, th, nb;
         choose_patch(c->Wo, c->Ho, c->N, &tw, &th, &nb);
         const int64_t patches = (int64_t)ceil_div(c->Wo, tw) * ceil_div(c->Ho, th) * ceil_div(c->N, nb);
         if (use_halo(c, patches, ctx->sm_count)) {
-            const nm_status e = c->Cout <= 64 ? launch_halo<T, 64>(ctx, c, chain, st) : launch_halo<T, 128>(ctx, c, chain, st);
+            const nm_status e = c->Cout <= 64 ? launch_halo<T, 64, HALO3X3>(ctx, c, chain, st) : launch_halo<T, 128, HALO3X3>(ctx, c, chain, st);
             if (e != NM_ERR_UNSUPPORTED) return e;
         }
         t = choose_tile((int64_t)c->N * c->Ho * c->Wo, patches, c->Cout, (int64_t)c->taps_y * c->taps_x * c->cblocks, true,

@@ -38,6 +38,12 @@
 //   10 y + x of shared memory, eight output pixels of a patch row are one 8-row group of the operand, the groups lie 1280 bytes
 //   apart, and tap (ky, kx) is the same operand 10 ky + kx rows further on.  The swizzle follows the address, so an operand may
 //   start at any row.  The weights have a ring of their own, or stay in shared memory if all of them fit.
+// STEM: a first layer of stride 2, at most 4 channels and 8 x 8 taps, on a copy with 4 channels per pixel.  Pixel pairs of an image row
+// are 16 bytes, and output pixel x + 1 begins one pair after output pixel x: without a swizzle, 8 operand rows of 16 bytes are
+// 128 contiguous bytes of the image row itself, the next 16 bytes of K begin one pair further on and the next 8 rows (the patch is
+// 8 x 16) two image rows down.  So the 22 x (30 + kh) pixels of a patch are loaded once, 6.5 KB, instead of one 64-element row per
+// output pixel and pair of filter rows, 64 KB a tile (128 images of 224 x 224 x 3, 7 x 7, copies included: 179 -> 119 us; what
+// bounds it now is the epilogue of 64-column tiles: 120 of the 131 us before the issue below, 81 of 97 without the products).
 #pragma once
 #include <string.h>
 
@@ -56,6 +62,9 @@ constexpr int HALO_W = 10, HALO_H = 18;                    // input pixels of a 
 constexpr int HALO_LOAD = HALO_W * HALO_H * ROW_BYTES;     // bytes of one halo box
 constexpr int HALO_BYTES = (HALO_LOAD + 1023) / 1024 * 1024;
 constexpr int MAX_W_STAGES = 18;
+enum { NO_HALO = 0, HALO3X3 = 1, STEM = 2 };               // forms of the A operand's load
+constexpr int STEM_PITCH = (2 * 7 + 8) * 4 * 2;            // bytes of an image row of a patch
+constexpr int STEM_BYTES = ((2 * 15 + 8) * STEM_PITCH + 1023) / 1024 * 1024;
 
 // How a tile's 128 rows map onto the NHWC tensors of a convolution (CONV kernels only).
 struct ConvDev {
@@ -65,6 +74,7 @@ struct ConvDev {
     int kw_eff, cblocks;    // K-block kb = (ky*kw_eff + kx)*cblocks + cb; 64 channels per block
     int Ho, Nimg;           // output rows per image, images
     int ky_last, ky_jump;   // the last filter row's input lies ky_jump rows further down (first layer, see conv_geom)
+    int stem_kh;            // STEM: filter rows
     int dw;                 // nonzero: "depthwise" form for pooling as a GEMM: column tile nt (64 channels) reads channel
                             // block nt of the activation at every tap and multiplies by ONE constant 64 x 64 matrix
 };
@@ -188,7 +198,7 @@ __device__ __forceinline__ void res_tile_load(void* dst, const CUtensorMap* tmR,
     else nm_tma_load_2d(dst, tmR, col, row0, bar);
 }
 
-template <typename InT, typename OutT, bool TWO, int BN, bool CONV, bool HALO = false>
+template <typename InT, typename OutT, bool TWO, int BN, bool CONV, int HALO = NO_HALO>
 __global__ void __launch_bounds__(NUM_THREADS, 1)
 linear_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmW,
                  const __grid_constant__ CUtensorMap tmO, const __grid_constant__ CUtensorMap tmR, const TcArgs a)
@@ -196,7 +206,7 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     static_assert(BN == 64 || BN == 128 || BN == 256, "tile widths built");
     constexpr int B_ROWS = TWO ? BN / 2 : BN;
     constexpr int B_BYTES = B_ROWS * ROW_BYTES;
-    constexpr int STAGE_BYTES = HALO ? HALO_BYTES : A_BYTES + B_BYTES;
+    constexpr int STAGE_BYTES = HALO == STEM ? STEM_BYTES : HALO ? HALO_BYTES : A_BYTES + B_BYTES;
     static_assert(!HALO || (CONV && TWO), "the halo form is built for CTA pairs");
     constexpr int TILE_M = TWO ? 2 * BM : BM;
     constexpr int BK_ELEMS = ROW_BYTES / (int)sizeof(InT);
@@ -219,6 +229,9 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     // one's MMAs, 281 and less (128 images, 28 x 28, 128 -> 128, 3 x 3: 45.6 -> 39.2 us).  With 256 columns the tensor core
     // covers it, and all lanes, whose stage numbers and descriptors stay in uniform registers, are 1 % faster.
     constexpr bool ONE_LANE = BN < 256;
+    // STEM's issuer has all of a tile's products between two waits: there all lanes wait, and one elected lane issues them unrolled,
+    // 45 cycles each instead of 70 (128 images: 131 -> 97 us).
+    constexpr bool ONE_ISSUER = ONE_LANE && HALO != STEM;
     // Several accumulators per tile (TcArgs::acc_steps): matrices of few columns.
     constexpr bool MULTI = BN == 64 && !CONV && !TcIn<InT>::is_int;
     const uint32_t buf_cols = MULTI ? BN * (uint32_t)a.accs : BN;
@@ -228,6 +241,7 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     const int bufs = MULTI && a.accs > 1 ? 2 : MOST_BUFS, buf_shift = bufs == 4 ? 2 : 1;
     const uint32_t tmem_cols = !MULTI || a.accs <= 1 ? MOST_BUFS * BN : a.accs <= 2 ? 4 * BN : 8 * BN;
     auto vote = [](bool done) { return ONE_LANE ? done : __all_sync(0xffffffffu, done) != 0; };
+    auto issue_vote = [](bool done) { return ONE_ISSUER ? done : __all_sync(0xffffffffu, done) != 0; };
 
     extern __shared__ uint8_t smem_raw[];
     __shared__ uint64_t bar_full[MAX_STAGES];
@@ -328,10 +342,15 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                     for (int cb = 0; ok && cb < a.cv.cblocks; ++cb) {
                         if (!nm_mbar_wait(&bar_empty[stage], phase ^ 1u, abortp, a.status)) { ok = false; break; }
                         const uint32_t full = nm_mapa(nm_smem_u32(&bar_full[stage]), 0);
-                        if (rank == 0) nm_mbar_expect_tx(&bar_full[stage], 2 * HALO_LOAD);
-                        nm_tma_load_4d_2cta(tiles + (size_t)stage * STAGE_BYTES, &tmA, cb * BK_ELEMS, pt.ox0 - 1, pt.oy0 - 1, pt.img0, full);
+                        if constexpr (HALO == STEM) {
+                            if (rank == 0) nm_mbar_expect_tx(&bar_full[stage], (uint32_t)(2 * STEM_PITCH * (30 + a.cv.stem_kh)));
+                            nm_tma_load_4d_2cta(tiles + (size_t)stage * STAGE_BYTES, &tmA, pt.ox0 * 8, pt.oy0 * 2 - a.cv.ph, pt.img0, 0, full);
+                        } else {
+                            if (rank == 0) nm_mbar_expect_tx(&bar_full[stage], 2 * HALO_LOAD);
+                            nm_tma_load_4d_2cta(tiles + (size_t)stage * STAGE_BYTES, &tmA, cb * BK_ELEMS, pt.ox0 - 1, pt.oy0 - 1, pt.img0, full);
+                        }
                         if (++stage == stages) { stage = 0; phase ^= 1u; }
-                        for (int tap = 0; load_w && tap < 9; ++tap) {
+                        for (int tap = 0; load_w && tap < (HALO == STEM ? a.num_k_blocks : 9); ++tap) {
                             if (!nm_mbar_wait(&bar_wempty[ws], wphase ^ 1u, abortp, a.status)) { ok = false; break; }
                             const uint32_t full = nm_mapa(nm_smem_u32(&bar_wfull[ws]), 0);
                             if (rank == 0) nm_mbar_expect_tx(&bar_wfull[ws], 2 * B_BYTES);
@@ -403,7 +422,7 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         __syncwarp();
     } else if (warp == 1) {
         // ------------------------------------------------ MMA issuer (the leader CTA of a pair)
-        if (rank == 0 && (!ONE_LANE || nm_elect_one())) {
+        if (rank == 0 && (!ONE_ISSUER || nm_elect_one())) {
             int stage = 0;
             uint32_t phase = 0;
             int buf = 0;
@@ -415,7 +434,7 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             for (int tile = tile_first; ok && tile < a.num_tiles; tile += tile_step) {
                 // CTA-scope acquire also where the peer CTA's epilogue warps arrive: what the hand-back orders are
                 // tcgen05 operations, ordered by tcgen05.fence (a cluster-scope acquire costs ~400 cycles per tile)
-                if (!vote(nm_mbar_wait(&bar_acc_empty[buf], acc_phase ^ 1u, abortp, a.status))) { ok = false; break; }
+                if (!issue_vote(nm_mbar_wait(&bar_acc_empty[buf], acc_phase ^ 1u, abortp, a.status))) { ok = false; break; }
                 nm_tc_fence_after();
                 uint32_t d_tmem = tmem_base + (uint32_t)buf * buf_cols;
                 [[maybe_unused]] int left = a.acc_steps;
@@ -423,29 +442,55 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                 if constexpr (HALO) {
                     const bool wait_w = !a.w_resident || tile == tile_first;
                     for (int cb = 0; ok && cb < a.cv.cblocks; ++cb) {
-                        if (!ready && !nm_mbar_wait(&bar_full[stage], phase, abortp, a.status)) { ok = false; break; }
-                        const int nxt = stage + 1 == stages ? 0 : stage + 1;
-                        ready = nm_mbar_test_wait(&bar_full[nxt], nxt == 0 ? phase ^ 1u : phase);
+                        if (!ready && !issue_vote(nm_mbar_wait(&bar_full[stage], phase, abortp, a.status))) { ok = false; break; }
+                        if constexpr (ONE_ISSUER) {
+                            const int nxt = stage + 1 == stages ? 0 : stage + 1;
+                            ready = nm_mbar_test_wait(&bar_full[nxt], nxt == 0 ? phase ^ 1u : phase);
+                        }
                         const uint32_t sa = nm_smem_u32(tiles + (size_t)stage * STAGE_BYTES);
-                        for (int tap = 0; tap < 9; ++tap) {
-                            if (wait_w && !nm_mbar_wait(&bar_wfull[ws], wphase, abortp, a.status)) { ok = false; break; }
+                        if constexpr (HALO == STEM) {   // two filter rows of 32 elements per weight tile
+                            for (int i = 0; wait_w && ok && i < a.num_k_blocks; ++i)
+                                ok = issue_vote(nm_mbar_wait(&bar_wfull[i], 0, abortp, a.status));
+                            if (!ok) break;
                             nm_tc_fence_after();
-                            const int ky = tap / 3, kx = tap - 3 * ky;
-                            const uint64_t adesc = nm_smem_desc_sw128(sa + (uint32_t)((HALO_W * ky + kx) * ROW_BYTES), HALO_W * ROW_BYTES);
-                            const uint64_t bdesc = nm_smem_desc_sw128(nm_smem_u32(w_tiles + (size_t)ws * B_BYTES));
+                            const uint64_t bdesc = nm_smem_desc_sw128(nm_smem_u32(w_tiles));
+                            const uint64_t adesc = nm_smem_desc_plain(sa, 16, 2 * STEM_PITCH);
+                            if (nm_elect_one()) {
 #pragma unroll
-                            for (int k = 0; k < 4; ++k)
-                                nm_mma_f16_2cta(d_tmem, adesc + 2 * k, bdesc + 2 * k, IDESC, (cb | tap | k) != 0 ? 1u : 0u);
-                            if (!a.w_resident) nm_tc_commit2(&bar_wempty[ws], 3);
-                            if (tap == 8) nm_tc_commit2(&bar_empty[stage], 3);
-                            if (++ws == a.w_stages) { ws = 0; wphase ^= 1u; }
+                                for (int ky = 0; ky < 8; ++ky) {
+                                    if (ky >= a.cv.stem_kh) break;
+                                    const uint64_t ad = adesc + ky * (STEM_PITCH >> 4), bd = bdesc + (ky >> 1) * (B_BYTES >> 4) + 4 * (ky & 1);
+                                    nm_mma_f16_2cta(d_tmem, ad, bd, IDESC, ky != 0);
+                                    nm_mma_f16_2cta(d_tmem, ad + 2, bd + 2, IDESC, 1u);
+                                }
+                                nm_tc_commit2(&bar_empty[stage], 3);
+                            }
+                            __syncwarp();
+                        }
+                        else {
+                            for (int tap = 0; tap < 9; ++tap) {
+                                if (wait_w && !issue_vote(nm_mbar_wait(&bar_wfull[ws], wphase, abortp, a.status))) { ok = false; break; }
+                                nm_tc_fence_after();
+                                const int ky = tap / 3, kx = tap - 3 * ky;
+                                const uint64_t adesc = nm_smem_desc_sw128(sa + (uint32_t)((HALO_W * ky + kx) * ROW_BYTES), HALO_W * ROW_BYTES);
+                                const uint64_t bdesc = nm_smem_desc_sw128(nm_smem_u32(w_tiles + (size_t)ws * B_BYTES));
+                                if (ONE_ISSUER || nm_elect_one()) {
+#pragma unroll
+                                    for (int k = 0; k < 4; ++k)
+                                        nm_mma_f16_2cta(d_tmem, adesc + 2 * k, bdesc + 2 * k, IDESC, (cb | tap | k) != 0 ? 1u : 0u);
+                                    if (!a.w_resident) nm_tc_commit2(&bar_wempty[ws], 3);
+                                    if (tap == 8) nm_tc_commit2(&bar_empty[stage], 3);
+                                }
+                                if constexpr (!ONE_ISSUER) __syncwarp();
+                                if (++ws == a.w_stages) { ws = 0; wphase ^= 1u; }
+                            }
                         }
                         if (++stage == stages) { stage = 0; phase ^= 1u; }
                     }
                 }
                 for (int kb = 0; !HALO && kb < a.num_k_blocks; ++kb) {
-                    if (!ready && !vote(nm_mbar_wait(&bar_full[stage], phase, abortp, a.status))) { ok = false; break; }
-                    if constexpr (ONE_LANE) {
+                    if (!ready && !issue_vote(nm_mbar_wait(&bar_full[stage], phase, abortp, a.status))) { ok = false; break; }
+                    if constexpr (ONE_ISSUER) {
                         const int nxt = stage + 1 == stages ? 0 : stage + 1;
                         ready = nm_mbar_test_wait(&bar_full[nxt], nxt == 0 ? phase ^ 1u : phase);
                     }
@@ -453,7 +498,7 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                     const uint32_t sa = nm_smem_u32(tiles + (size_t)stage * STAGE_BYTES);
                     const uint64_t adesc = nm_smem_desc_sw128(sa);
                     const uint64_t bdesc = nm_smem_desc_sw128(sa + A_BYTES);
-                    if (ONE_LANE || nm_elect_one()) {
+                    if (ONE_ISSUER || nm_elect_one()) {
 #pragma unroll
                         for (int k = 0; k < 4; ++k) {  // 4 x 32 bytes of K per 128-byte row
                             const uint32_t accum = MULTI ? multi_accum : (kb | k) != 0 ? 1u : 0u;
@@ -477,19 +522,19 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                         if constexpr (TWO) nm_tc_commit2(&bar_empty[stage], 3);
                         else nm_tc_commit(&bar_empty[stage]);
                     }
-                    if constexpr (!ONE_LANE) __syncwarp();
+                    if constexpr (!ONE_ISSUER) __syncwarp();
                     if (++stage == stages) { stage = 0; phase ^= 1u; }
                 }
                 if (!ok) break;
-                if (ONE_LANE || nm_elect_one()) {
+                if (ONE_ISSUER || nm_elect_one()) {
                     if constexpr (TWO) nm_tc_commit2(&bar_acc_full[buf], 3);
                     else nm_tc_commit(&bar_acc_full[buf]);
                 }
-                if constexpr (!ONE_LANE) __syncwarp();
+                if constexpr (!ONE_ISSUER) __syncwarp();
                 buf = (buf + 1) & (bufs - 1);
                 if (buf == 0) acc_phase ^= 1u;
             }
-            if (!ok && (ONE_LANE || nm_elect_one())) {
+            if (!ok && (ONE_ISSUER || nm_elect_one())) {
                 if constexpr (TWO) nm_tc_commit2(&bar_drain, 1);
                 else nm_tc_commit(&bar_drain);
                 long long t0 = clock64();
@@ -823,32 +868,34 @@ inline bool plan_smem(TcArgs* a, bool has_vec, size_t* smem_out)
 }
 
 // The same for the halo form: all weight tiles if they leave room for two halo boxes and the columns are one tile, else a ring.
-template <typename T, int BN>
+template <typename T, int BN, int FORM>
 inline bool plan_smem_halo(TcArgs* a, bool has_vec, size_t* smem_out)
 {
-    constexpr int B_BYTES = BN / 2 * ROW_BYTES;
+    constexpr int B_BYTES = BN / 2 * ROW_BYTES, LOAD_BYTES = FORM == STEM ? STEM_BYTES : HALO_BYTES, MOST = FORM == STEM ? MAX_STAGES : 4;
     const size_t table_bytes = (size_t)a->n_seg * 32 * sizeof(float2);
     const size_t vec_bytes = has_vec ? (size_t)NUM_EPI_WARPS * 256 * sizeof(float) : 0;
     const size_t fixed = (size_t)NUM_EPI_WARPS * STAGE_BUF * (a->has_res ? 2 : 1) + vec_bytes + table_bytes + 2048;
     const long long room = 227 * 1024 - (long long)fixed;
     const int kb = a->num_k_blocks;
-    a->w_resident = a->num_n_tiles == 1 && kb <= MAX_W_STAGES && room >= (long long)kb * B_BYTES + 2 * HALO_BYTES;
+    a->w_resident = a->num_n_tiles == 1 && kb <= MAX_W_STAGES && room >= (long long)kb * B_BYTES + 2 * LOAD_BYTES;
     a->stages = 3;
     if (a->w_resident) {
         a->w_stages = kb;
-        a->stages = (int)((room - (long long)kb * B_BYTES) / HALO_BYTES);
-        if (a->stages > 4) a->stages = 4;
+        a->stages = (int)((room - (long long)kb * B_BYTES) / LOAD_BYTES);
+        if (a->stages > MOST) a->stages = MOST;
+    } else if (FORM == STEM) {
+        return false;
     } else {
-        a->w_stages = (int)((room - 3LL * HALO_BYTES) / B_BYTES);
+        a->w_stages = (int)((room - 3LL * LOAD_BYTES) / B_BYTES);
         if (a->w_stages > MAX_W_STAGES) a->w_stages = MAX_W_STAGES;
-        if (room < 3LL * HALO_BYTES + 4LL * B_BYTES) return false;
+        if (room < 3LL * LOAD_BYTES + 4LL * B_BYTES) return false;
     }
-    *smem_out = (size_t)a->stages * HALO_BYTES + (size_t)a->w_stages * B_BYTES + fixed - 1024;
+    *smem_out = (size_t)a->stages * LOAD_BYTES + (size_t)a->w_stages * B_BYTES + fixed - 1024;
     return true;
 }
 
 // Launches the persistent kernel over a.num_tiles tiles (one CTA, or one CTA pair, per resident slot).
-template <typename InT, typename OutT, bool TWO, int BN, bool CONV, bool HALO = false>
+template <typename InT, typename OutT, bool TWO, int BN, bool CONV, int HALO = NO_HALO>
 inline nm_status launch_kernel(nm_ctx* ctx, const CUtensorMap& tmA, const CUtensorMap& tmW, const CUtensorMap& tmO,
                                const CUtensorMap& tmR, const TcArgs& a, size_t smem, double work, cudaStream_t st)
 {

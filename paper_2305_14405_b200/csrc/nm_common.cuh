@@ -607,6 +607,13 @@ __device__ __forceinline__ uint64_t nm_smem_desc_sw128(uint32_t smem_addr, uint3
     return d;
 }
 
+// The same without a swizzle, K-major: 8 rows of 16 bytes are 128 contiguous bytes, the next 16 bytes of K of the same rows begin
+// `k_bytes` further on, the next 8 rows `group_bytes`.  Both may be any multiple of 16, so that operand rows may overlap in memory.
+__device__ __forceinline__ uint64_t nm_smem_desc_plain(uint32_t smem_addr, uint32_t k_bytes, uint32_t group_bytes)
+{
+    return (uint64_t)((smem_addr & 0x3FFFFu) >> 4) | (uint64_t)(k_bytes >> 4) << 16 | (uint64_t)(group_bytes >> 4) << 32 | (uint64_t)1 << 46;
+}
+
 // Instruction descriptor: D format (1 = f32, 2 = s32), A/B format (f16 kinds:
 // 0 = f16, 1 = bf16; i8 kind: 1 = signed), major-ness (0 = K-major), N>>3, M>>4.
 __host__ __device__ constexpr uint32_t nm_idesc(uint32_t c_fmt, uint32_t ab_fmt, uint32_t a_mn_major,
@@ -759,6 +766,7 @@ struct NmConvTc {
     int sw, sh, pw, ph;
     int taps_y, taps_x, cblocks;
     int last_row_jump;
+    int stem_kh;    // first layer (NM_STEM): filter rows; a_* describe the copy {4 W, H, N, 1}, ph and pw are the padding
     const void* w;
     int64_t ldw, Ktot;
     int N, Ho, Wo, Cout;
@@ -777,6 +785,9 @@ nm_status nm_launch_pad_input(nm_ctx* ctx, const void* x, void* xp, nm_dtype dt,
                               int Hp, int Wp, cudaStream_t st);
 nm_status nm_launch_pad_weight(nm_ctx* ctx, const void* w, void* wp, nm_dtype dt, int Cout, int kh, int kw, int Cin,
                                cudaStream_t st);
+// the same for the first layer's own form: xp [N,H,Wp,4] with `pad` zero pixels on the left and wp [Cout,(kh+1)/2,2,8,4]
+nm_status nm_launch_pad_stem(nm_ctx* ctx, const void* x, void* xp, const void* w, void* wp, nm_dtype dt, int Nb, int H, int W, int Cin,
+                             int pad, int Wp, int Cout, int kh, int kw, cudaStream_t st);
 // the same for a stride-2 layer of at most 4 channels, rows in pairs: xp [N,Hp,Wp,2,4] of pair_rows pairs and, behind them, an
 // odd kh's last filter row with zeros beside it, wp [Cout,(kh+1)/2,8,2,4]
 nm_status nm_launch_pad_pairs(nm_ctx* ctx, const void* x, void* xp, const void* w, void* wp, nm_dtype dt, int Nb, int H, int W,
