@@ -229,9 +229,10 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     // one's MMAs, 281 and less (128 images, 28 x 28, 128 -> 128, 3 x 3: 45.6 -> 39.2 us).  With 256 columns the tensor core
     // covers it, and all lanes, whose stage numbers and descriptors stay in uniform registers, are 1 % faster.
     constexpr bool ONE_LANE = BN < 256;
-    // STEM's issuer has all of a tile's products between two waits: there all lanes wait, and one elected lane issues them unrolled,
-    // 45 cycles each instead of 70 (128 images: 131 -> 97 us).
-    constexpr bool ONE_ISSUER = ONE_LANE && HALO != STEM;
+    // The halo forms' issuer has many products between two waits; with 64 columns, where all weights stay in shared memory, all lanes
+    // wait and one elected lane issues a patch's products unrolled, 45 cycles each instead of 70 (128 images: 56 x 56, 64 -> 64,
+    // 3 x 3: 50 -> 35 us, the first layer 131 -> 97; 28 x 28, 128 -> 128, with a wait per tap: 38 -> 43, so one lane there).
+    constexpr bool ONE_ISSUER = ONE_LANE && HALO != STEM && !(HALO && BN == 64);
     // Several accumulators per tile (TcArgs::acc_steps): matrices of few columns.
     constexpr bool MULTI = BN == 64 && !CONV && !TcIn<InT>::is_int;
     const uint32_t buf_cols = MULTI ? BN * (uint32_t)a.accs : BN;
@@ -467,7 +468,25 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                             }
                             __syncwarp();
                         }
-                        else {
+                        else if (!ONE_ISSUER && a.w_resident) {   // channel block cb's nine weight tiles lie behind one another
+                            for (int i = 0; wait_w && ok && i < 9; ++i)
+                                ok = issue_vote(nm_mbar_wait(&bar_wfull[9 * cb + i], 0, abortp, a.status));
+                            if (!ok) break;
+                            nm_tc_fence_after();
+                            const uint64_t adesc = nm_smem_desc_sw128(sa, HALO_W * ROW_BYTES);
+                            const uint64_t bdesc = nm_smem_desc_sw128(nm_smem_u32(w_tiles + (size_t)(9 * cb) * B_BYTES));
+                            if (nm_elect_one()) {
+#pragma unroll
+                                for (int tap = 0; tap < 9; ++tap) {
+#pragma unroll
+                                    for (int k = 0; k < 4; ++k)
+                                        nm_mma_f16_2cta(d_tmem, adesc + ((HALO_W * (tap / 3) + tap % 3) * ROW_BYTES >> 4) + 2 * k,
+                                                        bdesc + tap * (B_BYTES >> 4) + 2 * k, IDESC, (tap | k) != 0 || cb != 0);
+                                }
+                                nm_tc_commit2(&bar_empty[stage], 3);
+                            }
+                            __syncwarp();
+                        } else {
                             for (int tap = 0; tap < 9; ++tap) {
                                 if (wait_w && !issue_vote(nm_mbar_wait(&bar_wfull[ws], wphase, abortp, a.status))) { ok = false; break; }
                                 nm_tc_fence_after();
