@@ -796,8 +796,8 @@ def main():
         gemm_kind = "linear_tc" if prof["linear_tc"][0] else "linear_simt"
         n_l, ms_l, work_l = prof[gemm_kind]
         achieved = work_l / (ms_l * 1e-3) / 1e12 if ms_l > 0 else 0.0
-        # int8: the measured bf16 peak times the nominal 2:1 int8:bf16 ratio; fp32 runs on CUDA cores
-        scale = {"i8": 2.0, "f32": 0.5}.get(wl.dtype, 1.0)
+        # int8: the measured bf16 peak times the nominal 2:1 int8:bf16 ratio; an fp32 product is six bf16 products
+        scale = {"i8": 2.0, "f32": 1.0 / 6.0}.get(wl.dtype, 1.0)
         peak, which = pick_peak(peaks, prof_clocks, scale)
         roofline = {"bound": "tensor", "kernel": gemm_kind, "achieved": achieved, "peak": peak,
                     "unit": "TFLOP/s", "frac": achieved / peak, "traffic": None,

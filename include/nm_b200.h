@@ -141,8 +141,8 @@ nm_status nm_pwl_apply(nm_ctx* ctx, int slot, const void* x, void* y, int64_t co
  * force the tcgen05 kernel that splits K over a cluster of 1, 2, 4 or 8 CTAs, tiles of 32 or 64
  * columns (NM_ERR_UNSUPPORTED likewise, and if K has fewer 128-byte blocks than CTAs).  With 2 and 3 the last
  * 4 to 12 columns of rows that are no multiple of 16 bytes go to that kernel too.
- * Picked for fp32: a tiled CUDA-core kernel where N is a multiple of 4, else the plain one.  Picked for 16-bit types:
- * a tcgen05 kernel where K is a multiple of 8 and N of 4 and at least 8; sums with M < 64 or N < 64 are no less
+ * Picked for fp32: the tensor cores, on three bf16 terms per operand (sums no less accurate than chains of FMAs), where N is
+ * a multiple of 4, else the plain kernel.  Picked for 16-bit types: a tcgen05 kernel where K is a multiple of 8 and N of 4 and at least 8; sums with M < 64 or N < 64 are no less
  * accurate than a chain of fp32 FMAs. */
 #define NM_ALGO_SPLIT(ctas, columns) (0x1000 | (ctas) | ((columns) << 4))
 typedef struct {
@@ -184,7 +184,8 @@ nm_status nm_linear_pwl(nm_ctx* ctx, const nm_linear_desc* desc, void* stream);
  * (NM_ERR_INVALID_ARG otherwise).
  * algo: 0 = pick; 1 = the plain CUDA-core kernel; 2 = tensor-core kernel that streams K and V (d = 64, L a multiple
  * of 128); 3 = tensor-core kernel that keeps the whole score block in tensor memory (d = 64, L in {128, 256, 384, 512}).
- * Picked for d = 64: fp32 a tiled CUDA-core kernel as long as 32 rows of scores fit shared memory (L up to 1408);
+ * Picked for d = 64: fp32 the tensor cores up to L = 128 (three bf16 terms per operand), a tiled CUDA-core kernel as
+ * long as 32 rows of scores fit shared memory (L up to 1408);
  * 16-bit types the streaming kernel at any L.  At multiples of 128 it rounds the probabilities e_j to the storage type
  * before the second product; at other lengths they keep 24 bits (fp16: 22), and all sums are fp32 everywhere. */
 typedef struct {
