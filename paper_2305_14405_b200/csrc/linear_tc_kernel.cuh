@@ -40,9 +40,11 @@
 //   start at any row.  The weights have a ring of their own, or stay in shared memory if all of them fit.
 // STEM: a first layer of stride 2, at most 4 channels and 8 x 8 taps, on a copy with 4 channels per pixel.  Pixel pairs of an image row
 // are 16 bytes, and output pixel x + 1 begins one pair after output pixel x: without a swizzle, 8 operand rows of 16 bytes are
-// 128 contiguous bytes of the image row itself, the next 16 bytes of K begin one pair further on and the next 8 rows (the patch is
-// 8 x 16) two image rows down.  So the 22 x (30 + kh) pixels of a patch are loaded once, 6.5 KB, instead of one 64-element row per
-// output pixel and pair of filter rows, 64 KB a tile (128 images of 224 x 224 x 3, 7 x 7, copies included: 179 -> 119 us; what
+// 128 contiguous bytes of the image row itself, and the next 8 rows (the patch is 8 x 16) begin two image rows down.  The second
+// 16 bytes of a step of K are the same pixels one image row down, so that a step takes the 16 products that it takes in the row-pair
+// form (cnn_api.cu) and the truncated sums are the same, bit for bit; behind an odd last filter row they are zeros, a place of their own (0 * inf
+// is NaN).  So the 22 x (30 + kh) pixels of a patch are loaded once, 6.5 KB, instead of one 64-element row per output pixel and
+// pair of filter rows, 64 KB a tile (128 images of 224 x 224 x 3, 7 x 7, copies included: 179 -> 119 us; what
 // bounds it now is the epilogue of 64-column tiles: 120 of the 131 us before the issue below, 81 of 97 without the products).
 #pragma once
 #include <string.h>
@@ -258,7 +260,8 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
 
     const int stages = a.stages;
     uint8_t* tiles = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-    uint8_t* w_tiles = tiles + (size_t)stages * STAGE_BYTES;     // HALO: w_stages x B_BYTES
+    uint8_t* zeros = tiles + (size_t)stages * STAGE_BYTES;        // STEM: one stage more
+    uint8_t* w_tiles = zeros + (HALO == STEM ? STEM_BYTES : 0);   // HALO: w_stages x B_BYTES
     uint8_t* stage_out = w_tiles + (HALO ? (size_t)a.w_stages * B_BYTES : 0);   // 8 x 4 KB
     uint8_t* stage_res = stage_out + NUM_EPI_WARPS * STAGE_BUF;   // 8 x 4 KB when a residual is given
     float2* rep = reinterpret_cast<float2*>(stage_res + (a.has_res ? NUM_EPI_WARPS * STAGE_BUF : 0));
@@ -307,6 +310,10 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         }
     }
     if (a.tab) nm_table_replicate(rep, a.tab, a.n_seg, threadIdx.x, NUM_THREADS);
+    if constexpr (HALO == STEM) {
+        for (int i = threadIdx.x; i < STEM_BYTES / 16; i += NUM_THREADS) reinterpret_cast<uint4*>(zeros)[i] = make_uint4(0u, 0u, 0u, 0u);
+        nm_fence_proxy_async();
+    }
     nm_tc_fence_before();
     __syncthreads();
     if constexpr (TWO) nm_cluster_sync();  // both CTAs' barriers and tensor memory are ready
@@ -449,20 +456,23 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                             ready = nm_mbar_test_wait(&bar_full[nxt], nxt == 0 ? phase ^ 1u : phase);
                         }
                         const uint32_t sa = nm_smem_u32(tiles + (size_t)stage * STAGE_BYTES);
-                        if constexpr (HALO == STEM) {   // two filter rows of 32 elements per weight tile
+                        if constexpr (HALO == STEM) {   // two filter rows per weight tile, two taps of both per step
                             for (int i = 0; wait_w && ok && i < a.num_k_blocks; ++i)
                                 ok = issue_vote(nm_mbar_wait(&bar_wfull[i], 0, abortp, a.status));
                             if (!ok) break;
                             nm_tc_fence_after();
                             const uint64_t bdesc = nm_smem_desc_sw128(nm_smem_u32(w_tiles));
-                            const uint64_t adesc = nm_smem_desc_plain(sa, 16, 2 * STEM_PITCH);
+                            const uint64_t adesc = nm_smem_desc_plain(sa, STEM_PITCH, 2 * STEM_PITCH);
+                            const uint32_t last = sa + (uint32_t)((a.cv.stem_kh - 1) * STEM_PITCH);   // an odd one has zeros beside it
+                            const uint64_t odd_desc = nm_smem_desc_plain(last, nm_smem_u32(zeros) - last, 2 * STEM_PITCH);
                             if (nm_elect_one()) {
 #pragma unroll
-                                for (int ky = 0; ky < 8; ++ky) {
+                                for (int ky = 0; ky < 8; ky += 2) {
                                     if (ky >= a.cv.stem_kh) break;
-                                    const uint64_t ad = adesc + ky * (STEM_PITCH >> 4), bd = bdesc + (ky >> 1) * (B_BYTES >> 4) + 4 * (ky & 1);
-                                    nm_mma_f16_2cta(d_tmem, ad, bd, IDESC, ky != 0);
-                                    nm_mma_f16_2cta(d_tmem, ad + 2, bd + 2, IDESC, 1u);
+                                    const uint64_t ad = ky + 1 < a.cv.stem_kh ? adesc + ky * (STEM_PITCH >> 4) : odd_desc;
+                                    const uint64_t bd = bdesc + (ky >> 1) * (B_BYTES >> 4);
+#pragma unroll
+                                    for (int k = 0; k < 4; ++k) nm_mma_f16_2cta(d_tmem, ad + k, bd + 2 * k, IDESC, (ky | k) != 0);
                                 }
                                 nm_tc_commit2(&bar_empty[stage], 3);
                             }
@@ -894,7 +904,7 @@ inline bool plan_smem_halo(TcArgs* a, bool has_vec, size_t* smem_out)
     const size_t table_bytes = (size_t)a->n_seg * 32 * sizeof(float2);
     const size_t vec_bytes = has_vec ? (size_t)NUM_EPI_WARPS * 256 * sizeof(float) : 0;
     const size_t fixed = (size_t)NUM_EPI_WARPS * STAGE_BUF * (a->has_res ? 2 : 1) + vec_bytes + table_bytes + 2048;
-    const long long room = 227 * 1024 - (long long)fixed;
+    const long long room = 227 * 1024 - (long long)fixed - (FORM == STEM ? STEM_BYTES : 0);   // (STEM: the zeros)
     const int kb = a->num_k_blocks;
     a->w_resident = a->num_n_tiles == 1 && kb <= MAX_W_STAGES && room >= (long long)kb * B_BYTES + 2 * LOAD_BYTES;
     a->stages = 3;
@@ -909,7 +919,7 @@ inline bool plan_smem_halo(TcArgs* a, bool has_vec, size_t* smem_out)
         if (a->w_stages > MAX_W_STAGES) a->w_stages = MAX_W_STAGES;
         if (room < 3LL * LOAD_BYTES + 4LL * B_BYTES) return false;
     }
-    *smem_out = (size_t)a->stages * LOAD_BYTES + (size_t)a->w_stages * B_BYTES + fixed - 1024;
+    *smem_out = (size_t)(a->stages + (FORM == STEM ? 1 : 0)) * LOAD_BYTES + (size_t)a->w_stages * B_BYTES + fixed - 1024;
     return true;
 }
 

@@ -785,7 +785,7 @@ nm_status nm_launch_pad_input(nm_ctx* ctx, const void* x, void* xp, nm_dtype dt,
                               int Hp, int Wp, cudaStream_t st);
 nm_status nm_launch_pad_weight(nm_ctx* ctx, const void* w, void* wp, nm_dtype dt, int Cout, int kh, int kw, int Cin,
                                cudaStream_t st);
-// the same for the first layer's own form: xp [N,H,Wp,4] with `pad` zero pixels on the left and wp [Cout,(kh+1)/2,2,8,4]
+// the same for the first layer's own form: xp [N,H,Wp,4] with `pad` zero pixels on the left and wp [Cout,(kh+1)/2,4,2,2,4]
 nm_status nm_launch_pad_stem(nm_ctx* ctx, const void* x, void* xp, const void* w, void* wp, nm_dtype dt, int Nb, int H, int W, int Cin,
                              int pad, int Wp, int Cout, int kh, int kw, cudaStream_t st);
 // the same for a stride-2 layer of at most 4 channels, rows in pairs: xp [N,Hp,Wp,2,4] of pair_rows pairs and, behind them, an

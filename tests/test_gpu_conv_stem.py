@@ -19,3 +19,22 @@ def test_first_layer(nm, ctx, dtype, N, H, W, Cin, Cout, kh, kw, pad, res):  # n
     Ho, Wo = (H + 2 * pad - kh) // 2 + 1, (W + 2 * pad - kw) // 2 + 1
     r = torch.randn((N, Ho, Wo, Cout), generator=g, device="cuda").to(dtype) if res else None
     conv_both(nm, ctx, x, w, b, 2, pad, r)
+
+
+@pytest.mark.parametrize("dtype", [torch.float16, torch.bfloat16])
+@pytest.mark.parametrize("N,H,W,Cin,Cout,kh,kw,pad", [(40, 64, 66, 3, 64, 7, 7, 3), (16, 224, 224, 3, 64, 7, 7, 3), (9, 100, 70, 4, 128, 8, 8, 4),
+                                                      (24, 90, 64, 1, 16, 4, 2, 0), (70, 40, 48, 3, 72, 6, 5, 5), (33, 50, 50, 2, 40, 3, 3, 1)])
+@pytest.mark.parametrize("inf", [False, True])
+def test_the_forms_of_the_first_layer_agree_in_every_bit(nm, ctx, dtype, N, H, W, Cin, Cout, kh, kw, pad, inf):  # noqa: F811
+    """Both take the same 16 products per step of the sum, in the same order of steps."""
+    x, w, b, _ = operands(N, H, W, Cin, Cout, kh, kw, dtype, H + W)
+    if inf:
+        x[0, H // 2, W // 2, 0], x[0, H - 1, 0, Cin - 1] = float("inf"), float("-inf")
+    outs = []
+    for algo in (nm.ALGO_AUTO, nm.ALGO_TC):
+        out = torch.full((N, (H + 2 * pad - kh) // 2 + 1, (W + 2 * pad - kw) // 2 + 1, Cout), float("nan"), device="cuda").to(dtype)
+        d = ctx.conv_desc(x, w, out, 2, pad, bias=b, slot=nm.SLOT_RELU, algo=algo)
+        ctx.conv2d_pwl(d, torch.empty(ctx.conv2d_workspace_bytes(d), dtype=torch.uint8, device="cuda"))
+        ctx.check_device_status()
+        outs.append(out.nan_to_num(12345.0))
+    assert torch.equal(*outs)
