@@ -213,7 +213,8 @@ constexpr int LOADS = 128 / LOAD_ROWS;
 constexpr int TILE = 128 * 128;   // bytes of one term: 128 rows of 64 bf16
 constexpr int E_PITCH = 128 + 4;
 constexpr float TC_LIMIT = 0x1p48f;   // (a low term is up to 2^15 of its operand: 64 products stay finite)
-constexpr int TC_SMEM_MOST = 9 * TILE + 1024 + NM_MAX_SEGMENTS * 16 * (int)sizeof(float2);
+// room for the largest table: the segments are counted on the device, where a captured launch finds the table of its replay
+constexpr int TC_SMEM = 9 * TILE + 1024 + NM_MAX_SEGMENTS * 16 * (int)sizeof(float2);
 
 __global__ void __launch_bounds__(TC_THREADS, 1) attention_f32_tc_kernel(const F32AttnArgs a)
 {
@@ -490,8 +491,8 @@ nm_status nm_launch_attention_f32(nm_ctx* ctx, const nm_attn_desc* d, cudaStream
     const int64_t blocks = (int64_t)(tc ? 1 : a.q_blocks) * d->heads * d->B;
     if (blocks > 0x7fffffffLL) return NM_ERR_UNSUPPORTED;
     auto kern = tc ? attention_f32_tc_kernel : attention_f32_kernel;
-    const size_t smem = tc ? 9 * TILE + 1024 + (size_t)ctx->h_tables[d->exp_slot].n * 16 * sizeof(float2) : smem_bytes(d->L);
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, tc ? TC_SMEM_MOST : 226 * 1024) != cudaSuccess) return NM_ERR_CUDA;
+    const size_t smem = tc ? TC_SMEM : smem_bytes(d->L);
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, tc ? TC_SMEM : 226 * 1024) != cudaSuccess) return NM_ERR_CUDA;
     cudaLaunchConfig_t cfg;
     memset(&cfg, 0, sizeof(cfg));
     cfg.gridDim = dim3((unsigned)blocks);

@@ -89,3 +89,25 @@ def test_attention(nm, ctx, L, n, odd):
     with np.errstate(invalid="ignore"):
         row = np.max(np.where(f, np.abs(ref), 0.0), axis=1, keepdims=True)
     assert (np.abs(got - ref)[f] <= (2e-5 * np.maximum(scale, row))[f]).all()
+
+
+@pytest.mark.parametrize("L", [37, 128, 200])
+def test_attention_replay_takes_the_table_of_its_time(ctx, L):
+    """A launch captured with a small exp table and replayed with a large one."""
+    B, h = 2, 3
+    ranges = {"exp": (-8.0, 0.0), "recip": (L / 16.0, float(L))}
+    x = torch.from_numpy(nm_inputs.matrix((B * L, 3 * h * 64), L, "f32", 0.8)).cuda()
+    out, ref = torch.zeros(B * L, h * 64, device="cuda"), torch.zeros(B * L, h * 64, device="cuda")
+    load_tables_both(ctx, 16, ranges)
+    ctx.attention_pwl(x, out, B, L, h, 64)
+    graph, side = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+    side.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.graph(graph, stream=side):
+        ctx.attention_pwl(x, out, B, L, h, 64)
+    torch.cuda.synchronize()
+    load_tables_both(ctx, 256, ranges)
+    ctx.attention_pwl(x, ref, B, L, h, 64)
+    graph.replay()
+    torch.cuda.synchronize()
+    ctx.check_device_status()
+    assert torch.equal(out, ref)
