@@ -244,6 +244,9 @@ __global__ void __launch_bounds__(TC_THREADS, 1) attention_f32_tc_kernel(const F
     for (int i = tid; i < n_exp * 16; i += TC_THREADS) rep[i] = a.t_exp->kb[i >> 4];
     const float inv_h = a.t_exp->inv_h, off = a.t_exp->off, nm1 = (float)(n_exp - 1);
     const float r_inv_h = a.t_rcp->inv_h, r_off = a.t_rcp->off, r_nm1 = (float)(a.t_rcp->n - 1);
+    // The successor may start only when this CTA has its tensor memory: a successor that took columns first and then waited for this grid
+    // would wait for good.
+    __syncthreads();
     nm_grid_launch_dependents();
     nm_grid_dependency_wait();
 

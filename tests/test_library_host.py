@@ -163,3 +163,17 @@ def test_elastic_builder_against_numerical_means(lib, func, lo, hi, dLx):
     # with a large e_th no intercept moves
     _, _, b_off, _ = nm.pwl_table_build_elastic(func, lo, hi, dLx, 0.0, bias_correct=True, e_th=10.0)
     assert np.array_equal(np.asarray(b_off, np.float64), b0)
+
+
+def test_tensor_memory_is_allocated_before_the_next_kernel_may_start():
+    """A kernel that lets its successor start while its own allocation may still wait can lose the columns to it, and the
+    successor waits for the kernel: between the two there is a barrier of the block, in the source of every kernel."""
+    seen = 0
+    for name in sorted(os.listdir(os.path.join(os.path.dirname(nm.__file__), "csrc"))):
+        text = open(os.path.join(os.path.dirname(nm.__file__), "csrc", name)).read()
+        for m in re.finditer(r"nm_tmem_alloc2?\(&", text):
+            rest = text[m.end():]
+            trigger = rest.find("nm_grid_launch_dependents();")
+            assert trigger > 0 and "__syncthreads();" in rest[:trigger], (name, text[:m.start()].count("\n") + 1)
+            seen += 1
+    assert seen >= 8
