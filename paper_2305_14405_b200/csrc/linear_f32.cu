@@ -35,8 +35,86 @@ template <int BN> struct F32Tile {
     static constexpr int CHUNKS = (BM + BN) / 16;      // 16-byte chunks of fp32 per thread and stage
     static constexpr int AHEAD = BN == 128 ? 8 : 12;   // of them in flight, in registers
     static constexpr int GROUP = BN == 128 ? 2 : 1;    // split together
-    static_assert(BM * part_pitch(BN) * 4 <= STAGES * STAGE_BYTES, "the partial tile takes the ring's place");
+    static_assert((BM * part_pitch(BN) + F_SUM_WARPS * 2 * 64 * (16 + 4)) * 4 <= STAGES * STAGE_BYTES,
+                  "the partial tile and the slices of fma_chains take the ring's place");
 };
+
+// Sums that are not finite, among those of a warp's 32 rows and COLS columns at `sums`: chains of K FMAs instead.  16 rows and 32 columns
+// at a time, those without such a sum passed over; 4 x 4 chains per lane, the operands 16 k at a time through the warp's own CHAIN_WORDS of
+// shared memory, one buffer filling while the other is multiplied.  1024 x 768 x 3072, 48 us alone: one row of NaN or infinities 258 to 274 us,
+// nothing but NaN 521 (each such sum by its row's thread, from memory: 2240 and 28400); 37 x 768 x 3072, 16 us: 45 and 72.  The finite
+// product pays for the code with 0.5 us of 42.3 (8 x 4 chains, which need 40 more registers: with 1.3 us, and 360 and 369 us).
+constexpr int CHAIN_K = 16, CHAIN_PITCH = CHAIN_K + 4, CHAIN_BUF = 64 * CHAIN_PITCH, CHAIN_WORDS = 2 * CHAIN_BUF;
+
+template <int COLS>
+__device__ __forceinline__ void fma_chains(const float* A, const float* W, int64_t lda, int64_t ldw, int K, int rows, int cols, float* sums, int pitch, float* slice)
+{
+    const int lane = threadIdx.x & 31, ry = lane >> 3, cx = lane & 7;   // rows ry + 4 i, columns cx + 8 j
+    __syncwarp();
+#pragma unroll 1
+    for (int cr = 0; cr < COLS / 16; ++cr) {
+        const int c = (cr >> 1) * 32, r_lo = (cr & 1) * 16;
+        uint32_t odd = 0;   // bit 4 i + j
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int r = r_lo + ry + 4 * i, n = c + cx + 8 * j;
+                if (r < rows && n < cols && !(fabsf(sums[r * pitch + n]) <= 3.402823466e38f)) odd |= 1u << (4 * i + j);
+            }
+        if (!__any_sync(0xffffffffu, odd != 0)) continue;
+        float v[4][4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) v[i][j] = 0.f;
+        // row r of A at row r of a buffer, row c + r of W at 32 + r (for one that does not exist the first one again); zeros beyond K,
+        // which leave a chain as it is
+        auto fetch = [&](int k0) {
+            const int k = k0 + (lane & 3) * 4, left = min(K - k, 4), bytes = left > 0 ? 4 * left : 0;
+            const uint32_t dst = nm_smem_u32(slice + ((k0 / CHAIN_K) & 1) * CHAIN_BUF + (lane >> 2) * CHAIN_PITCH + (lane & 3) * 4);
+#pragma unroll 1
+            for (int i = 0; i < 8; ++i) {
+                const int r = (8 * i + (lane >> 2)) & 31;
+                const float* p = (i < 4 ? A + (r < rows ? r : 0) * lda : W + (c + r < cols ? c + r : c) * ldw) + (bytes ? k : 0);
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst + (uint32_t)(8 * i * CHAIN_PITCH * 4)), "l"(p), "r"(bytes) : "memory");
+            }
+            asm volatile("cp.async.commit_group;" ::: "memory");
+        };
+        __syncwarp();
+        fetch(0);
+#pragma unroll 1
+        for (int k0 = 0; k0 < K; k0 += CHAIN_K) {
+            if (k0 + CHAIN_K < K) {
+                fetch(k0 + CHAIN_K);
+                asm volatile("cp.async.wait_group 1;" ::: "memory");
+            } else {
+                asm volatile("cp.async.wait_group 0;" ::: "memory");
+            }
+            __syncwarp();
+            const float* buf = slice + ((k0 / CHAIN_K) & 1) * CHAIN_BUF;
+#pragma unroll 1
+            for (int kk = 0; kk < CHAIN_K; kk += 4) {
+                float4 w[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) w[j] = *reinterpret_cast<const float4*>(buf + (32 + cx + 8 * j) * CHAIN_PITCH + kk);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const float4 x = *reinterpret_cast<const float4*>(buf + (r_lo + ry + 4 * i) * CHAIN_PITCH + kk);
+#pragma unroll
+                    for (int j = 0; j < 4; ++j)
+                        v[i][j] = __fmaf_rn(x.w, w[j].w, __fmaf_rn(x.z, w[j].z, __fmaf_rn(x.y, w[j].y, __fmaf_rn(x.x, w[j].x, v[i][j]))));
+                }
+            }
+            __syncwarp();   // the buffer may be filled again
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                if (odd & (1u << (4 * i + j))) sums[(r_lo + ry + 4 * i) * pitch + c + cx + 8 * j] = v[i][j];
+    }
+}
 
 template <int BN>
 __global__ void __launch_bounds__(F_THREADS, 1)
@@ -283,15 +361,11 @@ linear_f32_kernel(const float* __restrict__ A, const float* __restrict__ W, int6
                     *p = v;
                 }
             }
-            if (odd && row < rows) {
-                const int64_t k0 = (int64_t)kb0 * FBK, k1 = min((int64_t)kb1 * FBK, a.K);
-                for (int j = 0; j < BN / 2 && c0 + j < cols; ++j) {
-                    if (fabsf(mine[j]) <= 3.402823466e38f) continue;
-                    const float *pa = A + (m0 + row) * lda, *pw = W + (n0 + c0 + j) * ldw;
-                    float v = 0.f;
-                    for (int64_t k = k0; k < k1; ++k) v = __fmaf_rn(__ldcg(pa + k), __ldcg(pw + k), v);
-                    mine[j] = v;
-                }
+            if (__builtin_expect(__any_sync(0xffffffffu, odd && row < rows), 0)) {
+                const int64_t k0 = (int64_t)kb0 * FBK;
+                float* slice = part + BM * PITCH + (warp - F_PROD / 32 - 1) * CHAIN_WORDS;
+                fma_chains<BN / 2>(A + (m0 + q * 32) * lda + k0, W + (n0 + c0) * ldw + k0, lda, ldw, (int)(min((int64_t)kb1 * FBK, a.K) - k0),
+                                   rows - q * 32, cols - c0, part + q * 32 * PITCH + c0, PITCH, slice);
             }
         }
         nm_tc_fence_before();

@@ -60,6 +60,48 @@ def test_linear_not_finite(nm, ctx, M, N, K):
     assert ((got - ref)[f].abs() <= 1e-5 * ref[f].abs().clamp(min=K ** 0.5)).all()
 
 
+# every sum of the tile by FMAs: remainders of rows, columns and K (of a row's last three k, too), one CTA and splits, both widths
+@pytest.mark.parametrize("M,N,K", [(1, 4, 7), (33, 36, 30), (128, 64, 64), (129, 100, 161), (200, 132, 320), (300, 512, 2048), (1000, 1600, 70)])
+def test_linear_of_large_operands(ctx, M, N, K):
+    """From 2^112 on a term of an operand is infinite, the product itself is not."""
+    A, W = [torch.from_numpy(nm_inputs.matrix(s, K, "f32", 1.0)).cuda() for s in ((M, K + -K % 4), (N, K + -K % 4))]
+    A[:, K:], W[:, K:] = float("nan"), float("inf")
+    A, W = (A * 2.0 ** 124)[:, :K], (W * 2.0 ** -100)[:, :K]
+    got, ref = linear(ctx, A, W), A.double() @ W.double().t()
+    # a chain of K rounded sums: 2^-24 of the running sum each, at most 2^-24 sqrt(K) of the rms here
+    assert ((got.double() - ref).norm() / ref.norm()).item() < 2.0 ** -24 * K ** 0.5 + 2.0 ** -24
+
+
+def time_of(call):
+    graph, side = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+    call()
+    side.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.graph(graph, stream=side):
+        call()
+        call()
+    times = []
+    for _ in range(5):
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        graph.replay()
+        b.record()
+        torch.cuda.synchronize()
+        times.append(a.elapsed_time(b))
+    return min(times)
+
+
+@pytest.mark.parametrize("M,N,K", [(1024, 768, 3072), (37, 768, 3072), (128, 768, 256)])
+def test_not_finite_linear_takes_no_longer_than_a_plain_product(ctx, M, N, K):
+    """2 to 6 times the finite product with one row, up to 11 with all; element by element it was 50 (one row) to 600 times."""
+    A, W = [torch.from_numpy(nm_inputs.matrix(s, 9, "f32", 1.0)).cuda() for s in ((M, K), (N, K))]
+    out = torch.empty(M, N, device="cuda")
+    finite = time_of(lambda: ctx.linear_pwl(A, W, out))
+    for rows, value in ((slice(5, 6), float("nan")), (slice(None), float("nan")), (slice(None), float("inf"))):
+        odd = A.clone()
+        odd[rows] = value
+        assert time_of(lambda: ctx.linear_pwl(odd, W, out)) < 16 * finite
+
+
 @pytest.mark.parametrize("L", [1, 15, 16, 17, 64, 65, 100, 128])
 @pytest.mark.parametrize("n", [2, 64, 256])
 @pytest.mark.parametrize("odd", [None, "q", "k", "v", "large_v"])
