@@ -211,10 +211,75 @@ constexpr int PART_KEYS = 128 / PARTS;
 constexpr int LOAD_ROWS = TC_THREADS / 16;   // rows that are fetched at a time
 constexpr int LOADS = 128 / LOAD_ROWS;
 constexpr int TILE = 128 * 128;   // bytes of one term: 128 rows of 64 bf16
-constexpr int E_PITCH = 128 + 4;
+constexpr int E_PITCH = 128 + 4, F_PITCH = HD + 4;   // words per row of scores, and of operands, for the CUDA cores' products
+static_assert((128 * E_PITCH + 2 * 128 * F_PITCH) * 4 <= 9 * TILE, "they take the place of the terms");
 constexpr float TC_LIMIT = 0x1p48f;   // (a low term is up to 2^15 of its operand: 64 products stay finite)
 // room for the largest table: the segments are counted on the device, where a captured launch finds the table of its replay
 constexpr int TC_SMEM = 9 * TILE + 1024 + NM_MAX_SEGMENTS * 16 * (int)sizeof(float2);
+
+// The products of a CTA as chains of FMAs, for operands that the terms do not take: the operands in shared memory behind the scores.
+// B 8, L 128, 12 heads with a NaN in every head: 58 us, 627 with each operand from memory.  Functions of their own: a launch runs the kernel's
+// code once or twice, from a cold instruction cache, and these should not lie in its way (inlined, finite B 8, L 37 8.0 -> 8.2 us).
+__device__ __forceinline__ void stage(const float* p, int64_t stride, int L, float* dst)
+{
+    const int c4 = ((int)threadIdx.x & 15) * 4;
+#pragma unroll 1
+    for (int r = (int)threadIdx.x >> 4; r < 128; r += LOAD_ROWS)
+        *reinterpret_cast<float4*>(dst + r * F_PITCH + c4) = r < L ? __ldcg(reinterpret_cast<const float4*>(p + r * stride + c4)) : make_float4(0.f, 0.f, 0.f, 0.f);
+}
+
+__device__ __noinline__ void scores_by_fma(const float* Q, const float* K, int64_t stride, int L, float* s_e)
+{
+    const int row = (int)threadIdx.x & 127, key0 = ((int)threadIdx.x >> 7) * PART_KEYS, lim = min(L - key0, PART_KEYS);
+    float *s_q = s_e + 128 * E_PITCH, *s_k = s_q + 128 * F_PITCH;
+    stage(Q, stride, L, s_q);
+    stage(K, stride, L, s_k);
+    __syncthreads();
+#pragma unroll 1
+    for (int j = 0; j < lim; j += 8) {
+        float s[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) s[i] = 0.f;
+#pragma unroll 1
+        for (int c = 0; c < HD; c += 4) {
+            const float4 x = *reinterpret_cast<const float4*>(s_q + row * F_PITCH + c);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const float4 y = *reinterpret_cast<const float4*>(s_k + (key0 + j + i) * F_PITCH + c);
+                s[i] = __fmaf_rn(x.w, y.w, __fmaf_rn(x.z, y.z, __fmaf_rn(x.y, y.y, __fmaf_rn(x.x, y.x, s[i]))));
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < 8; i += 4) *reinterpret_cast<float4*>(s_e + row * E_PITCH + key0 + j + i) = make_float4(s[i], s[i + 1], s[i + 2], s[i + 3]);
+    }
+}
+
+// 16 channels of a row: its exponentials, at s_e, times V, times rinv
+__device__ __noinline__ void output_by_fma(const float* V, int64_t stride, int L, float* s_e, float rinv, float* out)
+{
+    const int row = (int)threadIdx.x & 127, c0 = ((int)threadIdx.x >> 7) * 16;
+    float* s_v = s_e + 128 * E_PITCH;
+    stage(V, stride, L, s_v);
+    __syncthreads();
+    if (row >= L) return;
+    float x[16];
+#pragma unroll
+    for (int c = 0; c < 16; ++c) x[c] = 0.f;
+#pragma unroll 1
+    for (int j = 0; j < L; ++j) {
+        const float e = s_e[row * E_PITCH + j];
+#pragma unroll
+        for (int c = 0; c < 16; c += 4) {
+            const float4 y = *reinterpret_cast<const float4*>(s_v + j * F_PITCH + c0 + c);
+            x[c] = __fmaf_rn(e, y.x, x[c]);
+            x[c + 1] = __fmaf_rn(e, y.y, x[c + 1]);
+            x[c + 2] = __fmaf_rn(e, y.z, x[c + 2]);
+            x[c + 3] = __fmaf_rn(e, y.w, x[c + 3]);
+        }
+    }
+#pragma unroll
+    for (int c = 0; c < 16; c += 4) *reinterpret_cast<float4*>(out + c) = make_float4(x[c] * rinv, x[c + 1] * rinv, x[c + 2] * rinv, x[c + 3] * rinv);
+}
 
 __global__ void __launch_bounds__(TC_THREADS, 1) attention_f32_tc_kernel(const F32AttnArgs a)
 {
@@ -224,7 +289,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) attention_f32_tc_kernel(const F
     __shared__ int abort_flag;
     __shared__ float s_red[PARTS][128];
     uint8_t* tiles = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-    float* s_e = reinterpret_cast<float*>(tiles);   // 128 x E_PITCH in the place of Q and K, for the CUDA cores' products
+    float* s_e = reinterpret_cast<float*>(tiles);   // 128 x E_PITCH in the terms' place, for the CUDA cores' products; their operands behind it
     float2* rep = reinterpret_cast<float2*>(tiles + 9 * TILE);   // the exp table, 16-way replicated
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int g = (int)blockIdx.x % a.heads, b = (int)blockIdx.x / a.heads;
@@ -321,13 +386,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) attention_f32_tc_kernel(const F
     const uint32_t t_row = tmem + ((uint32_t)((warp & 3) * 32) << 16);
     bool ok = true;
     if (odd) {
-        if (row < L) {
-            for (int j = 0; j < lim; ++j) {
-                float s = 0.f;
-                for (int c = 0; c < HD; ++c) s = __fmaf_rn(__ldcg(Qp + (int64_t)row * a.stride_t + c), __ldcg(Kp + (int64_t)(key0 + j) * a.stride_t + c), s);
-                s_e[row * E_PITCH + key0 + j] = s;
-            }
-        }
+        scores_by_fma(Qp, Kp, a.stride_t, L, s_e);
     } else {
         ok = nm_mbar_wait(&bar_s, 0, abortp, a.status);
     }
@@ -430,19 +489,12 @@ __global__ void __launch_bounds__(TC_THREADS, 1) attention_f32_tc_kernel(const F
 #pragma unroll
             for (int j = 0; j < 16; ++j) s_e[row * E_PITCH + key0 + c + j] = e[j];
         }
-        __syncthreads();
-        if (row < L) {
-            for (int c = 0; c < 16; ++c) {
-                float x = 0.f;
-                for (int j = 0; j < L; ++j) x = __fmaf_rn(s_e[row * E_PITCH + j], __ldcg(Vp + (int64_t)j * a.stride_t + part * 16 + c), x);
-                out[c] = x * rinv;
-            }
-        }
+        output_by_fma(Vp, a.stride_t, L, s_e, rinv, out);
     } else {
         ok = nm_mbar_wait(&bar_o, 0, abortp, a.status) && ok;
         __syncwarp();
         nm_tc_fence_after();
-uint32_t h0[16], h1[16], mid[16], low[16];
+        uint32_t h0[16], h1[16], mid[16], low[16];
         const uint32_t o = t_row + (uint32_t)(part * 16);
         nm_tmem_ld16_sync(o, h0);
         if (steps > 4) nm_tmem_ld16_sync(o + 64, h1);

@@ -153,3 +153,15 @@ def test_attention_replay_takes_the_table_of_its_time(ctx, L):
     torch.cuda.synchronize()
     ctx.check_device_status()
     assert torch.equal(out, ref)
+
+
+@pytest.mark.parametrize("B,L", [(8, 128), (8, 37)])
+def test_not_finite_attention_takes_no_longer_than_a_plain_one(ctx, B, L):
+    """Products on the CUDA cores: 2 to 4 times the finite call; with each operand from memory it was 40 times."""
+    h = 12
+    load_tables_both(ctx, 64, {"exp": (-8.0, 0.0), "recip": (L / 16.0, float(L))})
+    x = torch.from_numpy(nm_inputs.matrix((B * L, 3 * h * 64), L, "f32", 0.8)).cuda()
+    out = torch.empty(B * L, h * 64, device="cuda")
+    finite = time_of(lambda: ctx.attention_pwl(x, out, B, L, h, 64))
+    x[:, 5::64] = float("nan")
+    assert time_of(lambda: ctx.attention_pwl(x, out, B, L, h, 64)) < 8 * finite
