@@ -184,8 +184,8 @@ nm_status nm_linear_pwl(nm_ctx* ctx, const nm_linear_desc* desc, void* stream);
  * (NM_ERR_INVALID_ARG otherwise).
  * algo: 0 = pick; 1 = the plain CUDA-core kernel; 2 = tensor-core kernel that streams K and V (d = 64, L a multiple
  * of 128); 3 = tensor-core kernel that keeps the whole score block in tensor memory (d = 64, L in {128, 256, 384, 512}).
- * Picked for d = 64: fp32 the tensor cores up to L = 128 (three bf16 terms per operand), a tiled CUDA-core kernel as
- * long as 32 rows of scores fit shared memory (L up to 1408);
+ * Picked for d = 64: fp32 the tensor cores (three bf16 terms per operand) for L from 65 to 128 and, where B * heads does not
+ * exceed the GPU's SMs, for shorter sequences, otherwise a tiled CUDA-core kernel as long as 32 rows of scores fit shared memory (L up to 1408);
  * 16-bit types the streaming kernel at any L.  At multiples of 128 it rounds the probabilities e_j to the storage type
  * before the second product; at other lengths they keep 24 bits (fp16: 22), and all sums are fp32 everywhere. */
 typedef struct {

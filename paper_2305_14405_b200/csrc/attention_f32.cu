@@ -523,6 +523,15 @@ __global__ void __launch_bounds__(TC_THREADS, 1) attention_f32_tc_kernel(const F
 int score_pitch(int L) { return (L + KB - 1) / KB * KB + 4; }
 size_t smem_bytes(int L) { return sizeof(float) * (2 * (size_t)NM_MAX_SEGMENTS + (QB + 2 * KB) * TP + (size_t)QB * score_pitch(L)); }
 
+// Is the tensor-core kernel the faster one?  It holds one CTA, 128 rows, per SM whatever L is; the other one four, and up to
+// 64 keys it needs one or two of 32 rows.  So with 65 to 128 keys always (4 to 1536 (batch, head) pairs: 0.37 to 1.05 of the other's time),
+// with less if one round takes all pairs (L 16, 37, 64: 96 pairs 0.71, 0.70, 0.73; 12 pairs 0.80, 1.06, 1.14), not with more rounds
+// (192 pairs 1.01, 1.22, 1.29; 1536 pairs 57 us against 31, 86 against 61, 97 against 63).
+bool use_tc(const nm_attn_desc* d, int sms)
+{
+    return d->L <= 128 && (d->L > 64 || (int64_t)d->B * d->heads <= sms);
+}
+
 }  // namespace
 
 bool nm_attention_f32_supported(const nm_attn_desc* d)
@@ -542,7 +551,7 @@ nm_status nm_launch_attention_f32(nm_ctx* ctx, const nm_attn_desc* d, cudaStream
     a.stride_b = d->stride_b; a.stride_t = d->stride_t; a.scale = d->scale;
     a.t_exp = ctx->d_tables + d->exp_slot; a.t_rcp = ctx->d_tables + d->recip_slot;
     a.status = ctx->d_status;
-    const bool tc = d->L <= 128;
+    const bool tc = use_tc(d, ctx->sm_count);
     const int64_t blocks = (int64_t)(tc ? 1 : a.q_blocks) * d->heads * d->B;
     if (blocks > 0x7fffffffLL) return NM_ERR_UNSUPPORTED;
     auto kern = tc ? attention_f32_tc_kernel : attention_f32_kernel;
