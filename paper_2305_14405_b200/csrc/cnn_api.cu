@@ -28,6 +28,7 @@ struct ConvGeom {
     int Hp, Wp;       // CONV_ROWTAP, CONV_PAIRTAP: extent of the padded input copy
     int pair_rows;    // CONV_PAIRTAP: rows of it that are pairs
     size_t a_bytes, w_bytes;
+    size_t ws_bytes;  // of the workspace that is asked for: enough for the forced tensor-core kernels too
 };
 
 bool conv_geom(const nm_conv_desc* d, ConvGeom* g)
@@ -43,18 +44,11 @@ bool conv_geom(const nm_conv_desc* d, ConvGeom* g)
     g->M = (int64_t)d->N * g->Ho * g->Wo;
     g->pad_w = false;
     g->Hp = g->Wp = 0;
-    g->a_bytes = g->w_bytes = 0;
+    g->a_bytes = g->w_bytes = g->ws_bytes = 0;
     if (d->kh == 1 && d->kw == 1 && d->stride == 1 && d->pad == 0 && d->Cin % 8 == 0) {
         g->path = CONV_DIRECT;
     } else if (d->Cin % 64 == 0 && d->algo != 1) {
         g->path = CONV_IMPLICIT;
-    } else if (d->Cin <= 4 && d->kw <= 8 && d->kh <= 8 && d->stride == 2 && d->algo == 0 && d->Cout <= 128 && d->pad <= 64) {
-        // (wider outputs keep the row pairs: all weights have to stay in shared memory; so do forced kernels)
-        g->path = CONV_STEM;
-        g->Hp = d->H;
-        g->Wp = (d->W + d->pad + 1) & ~1;
-        g->a_bytes = align256((size_t)d->N * g->Hp * g->Wp * 4 * 2);
-        g->w_bytes = align256((size_t)d->Cout * ((d->kh + 1) / 2) * 64 * 2);
     } else if (d->Cin <= 4 && d->kw <= 8 && d->stride == 2 && d->algo != 1) {
         g->path = CONV_PAIRTAP;
         // Output row oy reads pair rows oy .. oy + kh / 2 - 1, output pixel ox pixels 2 ox .. 2 ox + 7.  The last row of an odd
@@ -66,6 +60,14 @@ bool conv_geom(const nm_conv_desc* d, ConvGeom* g)
         g->Wp = (g->Wo - 1) * 2 + 8;
         g->a_bytes = align256((size_t)d->N * g->Hp * g->Wp * 8 * 2);
         g->w_bytes = align256((size_t)d->Cout * pairs * 64 * 2);
+        if (d->algo == 0 && d->kh <= 8 && d->Cout <= 128 && d->pad <= 64) {
+            // (wider outputs keep the row pairs: all weights have to stay in shared memory; so do forced kernels)
+            g->ws_bytes = g->a_bytes + g->w_bytes;
+            g->path = CONV_STEM;
+            g->Hp = d->H;
+            g->Wp = (d->W + d->pad + 1) & ~1;
+            g->a_bytes = align256((size_t)d->N * g->Hp * g->Wp * 4 * 2);
+        }
     } else if (d->Cin <= 8 && d->kw <= 8 && d->algo != 1) {
         g->path = CONV_ROWTAP;
         // rows 0 .. (Ho-1)*s + kh - 1 and pixels 0 .. (Wo-1)*s + 7 of the padded copy are read
@@ -80,6 +82,7 @@ bool conv_geom(const nm_conv_desc* d, ConvGeom* g)
         g->a_bytes = align256((size_t)g->M * g->Kpad * 2);
         g->w_bytes = g->pad_w ? align256((size_t)d->Cout * g->Kpad * 2) : 0;
     }
+    if (g->ws_bytes < g->a_bytes + g->w_bytes) g->ws_bytes = g->a_bytes + g->w_bytes;
     return true;
 }
 
@@ -109,7 +112,7 @@ size_t nm_conv2d_workspace_bytes(const nm_conv_desc* d)
 {
     ConvGeom g;
     if (!d || !conv_geom(d, &g)) return 0;
-    return g.a_bytes + g.w_bytes;
+    return g.ws_bytes;
 }
 
 nm_status nm_conv2d_pwl(nm_ctx* ctx, const nm_conv_desc* d, void* workspace, size_t ws_bytes, void* stream)

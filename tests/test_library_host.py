@@ -177,3 +177,16 @@ def test_tensor_memory_is_allocated_before_the_next_kernel_may_start():
             assert trigger > 0 and "__syncthreads();" in rest[:trigger], (name, text[:m.start()].count("\n") + 1)
             seen += 1
     assert seen >= 8
+
+
+def test_a_workspace_for_the_chosen_convolution_is_enough_for_the_forced_ones(lib):
+    """What the chosen kernel asks for holds what forced tensor-core kernels take, whatever form a first layer has."""
+    for N, H, W, Cin, Cout, k, stride, pad in [(2, 64, 48, 3, 64, 7, 2, 3), (128, 224, 224, 3, 64, 7, 2, 3), (3, 17, 40, 1, 8, 3, 2, 1), (1, 20, 20, 4, 128, 1, 2, 0),
+                                               (1, 30, 31, 4, 72, 2, 2, 40), (2, 40, 24, 3, 136, 7, 2, 3), (2, 31, 30, 3, 64, 9, 2, 4), (5, 33, 33, 5, 64, 3, 2, 1),
+                                               (4, 8, 8, 64, 64, 3, 1, 1), (4, 8, 8, 64, 64, 1, 1, 0)]:
+        need = []
+        for algo in (0, 2, 3, nm.algo_split(2, 64)):
+            d = nm.ConvDesc()
+            d.N, d.H, d.W, d.Cin, d.Cout, d.kh, d.kw, d.stride, d.pad, d.dtype, d.algo = N, H, W, Cin, Cout, k, k, stride, pad, nm.F16, algo
+            need.append(int(lib.nm_conv2d_workspace_bytes(C.byref(d))))
+        assert need[0] >= max(need), (need, N, H, W, Cin, Cout, k)
