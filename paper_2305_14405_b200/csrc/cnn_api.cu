@@ -60,7 +60,7 @@ bool conv_geom(const nm_conv_desc* d, ConvGeom* g)
         g->Wp = (g->Wo - 1) * 2 + 8;
         g->a_bytes = align256((size_t)d->N * g->Hp * g->Wp * 8 * 2);
         g->w_bytes = align256((size_t)d->Cout * pairs * 64 * 2);
-        if (d->algo == 0 && d->kh <= 8 && d->Cout <= 128 && d->pad <= 64) {
+        if (d->algo == 0 && d->kh <= 8 && d->Cout <= 128 && d->pad <= 64 && nm_conv_stem_pays(g->Wo, g->Ho, d->N, d->Cout)) {
             // (wider outputs keep the row pairs: all weights have to stay in shared memory; so do forced kernels)
             g->ws_bytes = g->a_bytes + g->w_bytes;
             g->path = CONV_STEM;

@@ -439,8 +439,10 @@ nm_status nm_launch_pad_pairs(nm_ctx* ctx, const void* x, void* xp, const void* 
 nm_status nm_launch_pad_stem(nm_ctx* ctx, const void* x, void* xp, const void* w, void* wp, nm_dtype dt, int Nb, int H, int W, int Cin,
                              int pad, int Wp, int Cout, int kh, int kw, cudaStream_t st)
 {
-    const int64_t rows = (int64_t)Nb * H, most = 16LL * ctx->sm_count;
-    const unsigned grid = (unsigned)(rows < most ? rows : most);
+    // a block per image row, and for few rows enough for the weights (one image of 16 x 16, 128 outputs: 12.7 -> 9.3 us)
+    const int64_t rows = (int64_t)Nb * H, w_blocks = ((int64_t)Cout * ((kh + 1) / 2) * 64 + 127) / 128, most = 16LL * ctx->sm_count;
+    const int64_t blocks = rows > w_blocks ? rows : w_blocks;
+    const unsigned grid = (unsigned)(blocks < most ? blocks : most);
     NmLaunchScope scope(ctx, NM_KERNEL_IM2COL, ((double)rows * W * Cin + (double)rows * Wp * 4) * nm_dtype_size(dt), st);
     if (dt == NM_F16) pad_stem_kernel<__half><<<grid, 128, 0, st>>>((const __half*)x, (__half*)xp, (const __half*)w, (__half*)wp, rows, W, Cin, pad, Wp, Cout, kh, kw);
     else pad_stem_kernel<__nv_bfloat16><<<grid, 128, 0, st>>>((const __nv_bfloat16*)x, (__nv_bfloat16*)xp, (const __nv_bfloat16*)w, (__nv_bfloat16*)wp, rows, W, Cin, pad, Wp, Cout, kh, kw);

@@ -40,6 +40,13 @@ void choose_patch(int Wo, int Ho, int N, int* TW, int* TH, int* NB)
     }
 }
 
+int64_t count_patches(int Wo, int Ho, int N)
+{
+    int tw, th, nb;
+    choose_patch(Wo, Ho, N, &tw, &th, &nb);
+    return (int64_t)ceil_div(Wo, tw) * ceil_div(Ho, th) * ceil_div(N, nb);
+}
+
 // Patch geometry and epilogue operands common to both kernels; returns the number of patches.
 int64_t fill_args(nm_ctx* ctx, const NmConvTc* c, NmChain chain, TcArgs* a)
 {
@@ -196,9 +203,7 @@ nm_status launch_sel(nm_ctx* ctx, const NmConvTc* c, NmChain chain, cudaStream_t
     if (c->stem_kh) return c->Cout <= 64 ? launch_halo<T, 64, STEM>(ctx, c, chain, st) : launch_halo<T, 128, STEM>(ctx, c, chain, st);
     TileChoice t;
     if (c->algo == 0) {
-        int tw, th, nb;
-        choose_patch(c->Wo, c->Ho, c->N, &tw, &th, &nb);
-        const int64_t patches = (int64_t)ceil_div(c->Wo, tw) * ceil_div(c->Ho, th) * ceil_div(c->N, nb);
+        const int64_t patches = count_patches(c->Wo, c->Ho, c->N);
         if (use_halo(c, patches, ctx->sm_count)) {
             const nm_status e = c->Cout <= 64 ? launch_halo<T, 64, HALO3X3>(ctx, c, chain, st) : launch_halo<T, 128, HALO3X3>(ctx, c, chain, st);
             if (e != NM_ERR_UNSUPPORTED) return e;
@@ -221,6 +226,17 @@ nm_status launch_sel(nm_ctx* ctx, const NmConvTc* c, NmChain chain, cudaStream_t
 }
 
 }  // namespace
+
+// Is the patch-wise form of a first layer (STEM) faster than the row pairs'?  Its patch is 8 x 16 pixels of one image, theirs leaves as few
+// rows empty as it can and may hold several images.  Few patches, up to four a SM with 64 columns and one with 128: it is (0.73 to 1.00
+// of the time and 0.91 to 1.03).  Beyond, by patches over patches of the row pairs, its time over theirs with the copies, 64 to 2048 images:
+// 64 columns 1.0: 0.65 to 0.86, 1.43: 0.90 to 0.93, 1.7: 0.97 to 1.01, 2.0 (8 x 8 outputs): 0.75 to 0.89, 2.66 (17 x 17): 1.14 to 1.25, 3.16 (9 x 9): 0.98
+// to 1.10; 128 columns 1.0: 0.78 to 0.92, 1.33: 1.00 to 1.04, 1.43: 1.11, 1.78: 1.01 to 1.26, 2.66: 1.37 to 1.61, 3.16: 1.10 to 1.50.
+bool nm_conv_stem_pays(int Wo, int Ho, int N, int Cout)
+{
+    const int64_t patches = (int64_t)ceil_div(Wo, 8) * ceil_div(Ho, 16) * N;
+    return patches <= (Cout <= 64 ? 4 : 1) * 148 || (double)patches <= (Cout <= 64 ? 2.0 : 1.3) * (double)count_patches(Wo, Ho, N);
+}
 
 nm_status nm_launch_conv_tc(nm_ctx* ctx, const NmConvTc* c, cudaStream_t st, NmChain chain)
 {

@@ -766,7 +766,7 @@ struct NmConvTc {
     int sw, sh, pw, ph;
     int taps_y, taps_x, cblocks;
     int last_row_jump;
-    int stem_kh;    // first layer (NM_STEM): filter rows; a_* describe the copy {4 W, H, N, 1}, ph and pw are the padding
+    int stem_kh;    // first layer, patch-wise form: filter rows; a_* describe the copy {4 W, H, N, 1}, ph and pw are the padding
     const void* w;
     int64_t ldw, Ktot;
     int N, Ho, Wo, Cout;
@@ -779,6 +779,7 @@ struct NmConvTc {
     double flops;   // 2 * pixels * Cout * (taps * Cin) of the convolution itself, for the launch records
 };
 nm_status nm_launch_conv_tc(nm_ctx* ctx, const NmConvTc* c, cudaStream_t st, NmChain chain = NmChain());
+bool nm_conv_stem_pays(int Wo, int Ho, int N, int Cout);   // which form of a first layer is the faster one
 // zero-padded copies that let a few-channel first layer run as an implicit GEMM: x [N,H,W,Cin] -> xp [N,Hp,Wp,8]
 // (border of `pad` pixels, channels Cin..7 zero) and w [Cout,kh,kw,Cin] -> wp [Cout,kh,8,8]
 nm_status nm_launch_pad_input(nm_ctx* ctx, const void* x, void* xp, nm_dtype dt, int Nb, int H, int W, int Cin, int pad,

@@ -38,3 +38,21 @@ def test_the_forms_of_the_first_layer_agree_in_every_bit(nm, ctx, dtype, N, H, W
         ctx.check_device_status()
         outs.append(out.nan_to_num(12345.0))
     assert torch.equal(*outs)
+
+
+@pytest.mark.parametrize("N,H,Cout,patchwise", [(1, 16, 128, True), (64, 18, 128, True), (512, 16, 64, True), (512, 18, 64, False), (512, 24, 64, True),
+                                                (512, 24, 128, False), (64, 34, 64, True), (128, 34, 64, False), (128, 18, 128, False), (512, 32, 128, True), (512, 48, 128, False), (64, 66, 64, True),
+                                                (64, 66, 128, False), (64, 100, 128, False), (8, 224, 64, True)])
+def test_the_form_follows_the_patches(nm, ctx, N, H, Cout, patchwise):  # noqa: F811
+    """Outputs that leave much of a fixed patch empty go to the row pairs (three launches instead of two), with the same result."""
+    x, w, b, _ = operands(N, H, H, 3, Cout, 7, 7, torch.float16, H)
+    outs = []
+    for algo, launches in ((nm.ALGO_AUTO, 2 if patchwise else 3), (nm.ALGO_TC, 3)):
+        out = torch.full((N, (H - 1) // 2 + 1, (H - 1) // 2 + 1, Cout), float("nan"), device="cuda").half()
+        d = ctx.conv_desc(x, w, out, 2, 3, bias=b, slot=nm.SLOT_RELU, algo=algo)
+        ctx.launch_count(reset=True)
+        ctx.conv2d_pwl(d, torch.empty(ctx.conv2d_workspace_bytes(d), dtype=torch.uint8, device="cuda"))
+        assert ctx.launch_count() == launches
+        ctx.check_device_status()
+        outs.append(out)
+    assert torch.equal(*outs) and outs[0].isfinite().all()
