@@ -38,16 +38,16 @@
 // ONE form (L <= 128, a single 128-key chunk): the scores and the accumulator do not share columns (128 | 64, and P behind
 // them: 256 columns, two CTAs per SM), so the one Q K^T of sweep 1 serves sweep 2 as well, and nothing is fetched or
 // multiplied twice in what is then a latency-bound kernel (B 1, L 128, 16 heads: 6.4 -> 4.9 us).  All of V is fetched at once and P V
-// runs once, over all keys.  Two softmax warps share 32 rows, half of the blocks of 16 keys each; the second one's sums go on from the
-// first one's, in the order that one warp would take (int8 24 layers, 128 tokens: 889 -> 849 us; with several chunks per tile, where
+// runs once, over all keys.  DUO (launch_one says when): two softmax warps share 32 rows, half of the blocks of 16 keys each; the second one's
+// sums go on from the first one's, in the order that one warp would take, so that the forms agree in every bit (int8 24 layers, 128 tokens: 889 -> 849 us; with several chunks per tile, where
 // the shared-memory pipe is the bound, two warps per quarter lose: B 32, L 512, 12 heads 70.8 -> 80.1).  RAGGED and ONE: the first two
 // terms of a block of 16 keys take the place of its scores, the third goes behind the accumulator, and P V takes the smallest
-// terms first, instead of one product per 64 keys (B 32, L 100, 12 heads: 15.0 -> 12.8 us; B 1, L 37: 5.3).
+// terms first, instead of one product per 64 keys (B 32, L 100, 12 heads: 15.0 -> 12.6 us; B 1, L 37: 4.6).
 //
 //   warp 0            control: TMA loads (K chunks through two stages, V chunks through one) and the tcgen05.mma
 //                     for S = Q K_c^T and O += P_c V_c (V as an MN-major operand).  It sleeps in a named barrier
 //                     (bar.sync) that the softmax warps signal with bar.arrive, so hand-offs cost no polling.
-//   warps 1..4 (ONE: 1..8)  softmax, one (two) per tensor-memory lane quarter: tcgen05.ld, row maximum (sweep 1); PWL exp, row
+//   warps 1..4 (DUO: 1..8)  softmax, one (two) per tensor-memory lane quarter: tcgen05.ld, row maximum (sweep 1); PWL exp, row
 //                     sum, P tile (sweep 2); PWL reciprocal, scaling, store (optionally as int8 codes for the int8
 //                     encoder).
 #include <string.h>
@@ -176,14 +176,19 @@ __device__ __forceinline__ void load_first_v(const LoadCtx& c, const Tile& t)
     for (int i = 0; i < c.v_chunks; ++i) nm_tma_load_3d(c.v_st + i * STAGE, c.tmV, t.g * HD, i * CK, t.b, c.bar_v_full);
 }
 
-// Threads of a CTA: the control warp and one or (ONE) two softmax warps per lane quarter.
-template <bool ONE> constexpr int CTA_THREADS = ONE ? 288 : 160;
+// Forms: several 128-key chunks; ONE: a single one; DUO: a single one, with two softmax warps per lane quarter instead of one.
+enum Form { MANY, ONE_CHUNK, DUO_CHUNK };
+// Threads of a CTA: the control warp and the softmax warps.
+template <Form FORM> constexpr int CTA_THREADS = FORM == DUO_CHUNK ? 288 : 160;
 
-template <typename T, bool CLAMP_HI, bool RAGGED, bool ONE>
-__global__ void __launch_bounds__(CTA_THREADS<ONE>, RAGGED || ONE ? 2 : 3)
+// PER_SM: CTAs that an SM holds, by registers and tensor memory three, with 256 columns two.  RAGGED and DUO: two with 96 registers, of which
+// 24 bytes spill, or one with 162.
+template <typename T, bool CLAMP_HI, bool RAGGED, Form FORM, int PER_SM>
+__global__ void __launch_bounds__(CTA_THREADS<FORM>, PER_SM)
 attention_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                         const __grid_constant__ CUtensorMap tmV, const SArgs a)
 {
+    constexpr bool ONE = FORM != MANY, DUO = FORM == DUO_CHUNK;
     constexpr uint32_t IDESC_QK = nm_idesc(1, AT<T>::fmt, 0, 0, BQ, CK);   // S chunk: 128 x 64
     constexpr uint32_t IDESC_PV = nm_idesc(1, AT<T>::fmt, 0, 1, BQ, HD);   // O: 128 x 64, V MN-major
     constexpr uint32_t IDESC_QK1 = nm_idesc(1, AT<T>::fmt, 0, 0, BQ, 2 * CK);   // sweep 1: 128 x 128
@@ -196,17 +201,17 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
     constexpr uint32_t P_COLS = RAGGED ? 128 : 32;
     constexpr int TERMS = RAGGED ? ProbTerms<T>::N : 1;
     constexpr bool SCALED = RAGGED && std::is_same<T, __half>::value;
-    constexpr int NT = CTA_THREADS<ONE>;
-    constexpr int LD = ONE ? 16 : 32;   // scores read at a time
+    constexpr int NT = CTA_THREADS<FORM>;
+    constexpr int LD = DUO ? 16 : 32;   // scores that sweep 1 reads at a time
 
     extern __shared__ uint8_t smem_raw[];
     __shared__ uint64_t bar_q, bar_drain;
     __shared__ uint64_t bar_k_full[2], bar_k1_full[2], bar_v_full, bar_s_full, bar_p_empty;
     __shared__ uint32_t tmem_slot, tmem_slot_p;
     __shared__ int abort_flag;
-    // ONE: the two warps' row maxima (SCALED: and minima), and what they pass on to add a row up as one of them would
-    __shared__ float s_pair[ONE ? 2 : 1][2][BQ];
-    __shared__ float4 s_sum[ONE ? 9 : 1][ONE ? BQ : 1];
+    // DUO: the two warps' row maxima (SCALED: and minima), and what they pass on to add a row up as one of them would
+    __shared__ float s_pair[DUO ? 2 : 1][2][BQ];
+    __shared__ float4 s_sum[DUO ? 9 : 1][DUO ? BQ : 1];
 
     const int L = a.L;
     const int n = RAGGED ? (L + CK - 1) / CK : L / CK;                    // 64-key chunks of sweep 2
@@ -450,8 +455,8 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
         // One row per thread.  A warp never blocks on the others: it signals the control warp with bar.arrive.
         const int q = warp & 3;
         const int row = q * 32 + lane;
-        const int part = ONE ? (warp - 1) >> 2 : 0;   // which of the two warps that share 32 rows, half of the blocks of 16 keys each
-        const int blocks = RAGGED ? (L + 15) / 16 : 8, first = part * ((blocks + 1) / 2), last = part ? blocks : (blocks + 1) / 2;   // ONE: its blocks
+        const int part = DUO ? (warp - 1) >> 2 : 0;   // which of the two warps that share 32 rows, half of the blocks of 16 keys each
+        const int blocks = RAGGED ? (L + 15) / 16 : 8, first = part * ((blocks + 1) / 2), last = part || !DUO ? blocks : (blocks + 1) / 2;   // ONE: its blocks
         const uint32_t bar_sc = 2, bar_pr = 3, bar_oc = 6;
         // this row's value of the other warp, which takes the same steps
         [[maybe_unused]] auto swap = [&](float (*buf)[BQ], float v) {
@@ -506,9 +511,9 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
 #pragma unroll
                     for (int hh = 0; hh < 4; ++hh) {   // 128 keys: the scores span [S | O]
                         uint32_t r[LD];
-                        const int key = ONE ? (first + hh) * 16 : hh * 32;
-                        if (ONE && first + hh >= last) continue;   // no keys there
-                        if constexpr (ONE) nm_tmem_ld16_sync(t_row + (uint32_t)key, r);
+                        const int key = DUO ? (first + hh) * 16 : hh * 32;
+                        if (DUO ? first + hh >= last : RAGGED && ONE && key >= L) continue;   // no keys there
+                        if constexpr (DUO) nm_tmem_ld16_sync(t_row + (uint32_t)key, r);
                         else nm_tmem_ld32_sync(t_row + (uint32_t)key, r);
                         if (!ONE && hh == 3) {   // all of it is in registers: the control warp may overwrite S
                             nm_tc_fence_before();
@@ -537,8 +542,8 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                     asm volatile("bar.arrive %0, %1;" ::"r"(bar_sc), "n"(NT) : "memory");
                 }
             }
-            if constexpr (ONE) m = fmaxf(m, swap(s_pair[0], m));
-            if constexpr (ONE && SCALED) lowest = fminf(lowest, swap(s_pair[1], lowest));
+            if constexpr (DUO) m = fmaxf(m, swap(s_pair[0], m));
+            if constexpr (DUO && SCALED) lowest = fminf(lowest, swap(s_pair[1], lowest));
             // RAGGED: the scores are scaled and rounded before the maximum is subtracted, and the segment number is clamped on
             // both sides, as on the CUDA cores.  Otherwise one FMA does both, and its result must not lie above 0, which is what
             // bounds the segment number there: the product is rounded up.  Rounded to nearest, fma(m, scale, -m scale) lies up
@@ -546,7 +551,7 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
             const float neg_ms = RAGGED ? -__fmul_rn(m, a.scale) : -__fmul_ru(m, a.scale);
             const uint64_t neg_ms2 = nm_pack2(neg_ms, neg_ms);
             float sum0 = 0.f, sum1 = 0.f, sum2 = 0.f, sum3 = 0.f;
-            [[maybe_unused]] int groups = 0;   // ONE: groups of 8 keys that the second warp has put into s_sum
+            [[maybe_unused]] int groups = 0;   // DUO: groups of 8 keys that the second warp has put into s_sum
             // SCALED: the power of two that brings the largest |e| this row can have to 2^14 .. 2^15 (below the table the first
             // segment goes on), and its inverse; an fp16 term then loses nothing to the narrow exponent
             [[maybe_unused]] float up = 1.f, down = 1.f;
@@ -561,7 +566,7 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
             // ---- sweep 2: e = PWL_exp(s - m), row sum, P tiles.
             // W scores of this thread's row -> exponentials, in groups of 8.  MASKED: keys from `lim` on lie beyond L; they take
             // the maximum as their score (which keeps the table index in range) and the exponential 0.
-            constexpr int W = RAGGED ? 16 : LD;   // (with several terms of P, 32 keys at a time spill)
+            constexpr int W = RAGGED || ONE ? 16 : 32;   // (with several terms of P, 32 keys at a time spill)
             auto exponentials = [&](uint32_t* r, int lim, auto masked, auto&& use) {
                 constexpr bool MASKED = decltype(masked)::value;
                 if constexpr (MASKED) {
@@ -607,7 +612,7 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                             if (jj * 8 + k + 1 >= lim) e[k + 1] = 0.f;
                         }
                     }
-                    if (ONE && part == 1) {   // (to be added up behind the first warp's)
+                    if (DUO && part == 1) {   // (to be added up behind the first warp's)
                         s_sum[groups++][row] = make_float4(e[0] + e[4], e[1] + e[5], e[2] + e[6], e[3] + e[7]);
                     } else {
                         sum0 += e[0] + e[4];
@@ -731,7 +736,7 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                 }
             }
             float sum = (sum0 + sum1) + (sum2 + sum3);
-            if constexpr (ONE) {
+            if constexpr (DUO) {
                 // Added up in the order that one warp would take, so that the last bit does not depend on the split (an int8
                 // network's codes do on that bit): the second warp goes on from the first one's four sums.
                 float* const total = &s_pair[0][0][row];   // (the maxima have been read: both warps are at the barrier below)
@@ -761,8 +766,8 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                       (size_t)g * HD;
             const uint32_t o_addr = t_row + O_OFF;
 #pragma unroll
-            for (int j2 = 0; j2 < (ONE ? HD / 32 : HD / 16); ++j2) {   // 16 channels at a time
-                const int jj = ONE ? 2 * part + j2 : j2;
+            for (int j2 = 0; j2 < (DUO ? HD / 32 : HD / 16); ++j2) {   // 16 channels at a time
+                const int jj = DUO ? 2 * part + j2 : j2;
                 uint32_t r0[16];
                 if (ok && live) {
                     nm_tmem_ld16_sync(o_addr + (uint32_t)(jj * 16), r0);
@@ -773,7 +778,7 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                         for (int k = 0; k < 16; ++k) r0[k] = __float_as_uint(__uint_as_float(r0[k]) + __uint_as_float(r1[k]));
                     }
                 }
-                if (j2 == (ONE ? HD / 32 : HD / 16) - 1 && more) {
+                if (j2 == (DUO ? HD / 32 : HD / 16) - 1 && more) {
                     // all of O is in registers: the control warp may start the next tile's sweep 1 over [S | O]
                     nm_tc_fence_before();
                     asm volatile("bar.arrive %0, %1;" ::"r"(bar_oc), "n"(NT) : "memory");
@@ -830,7 +835,7 @@ nm_status make_map(nm_ctx* ctx, CUtensorMap* m, const void* ptr, nm_dtype dt, co
     return r == CUDA_SUCCESS ? NM_OK : NM_ERR_CUDA;
 }
 
-template <typename T, bool CLAMP_HI, bool RAGGED, bool ONE>
+template <typename T, bool CLAMP_HI, bool RAGGED, Form FORM, int PER_SM>
 nm_status launch(nm_ctx* ctx, const nm_attn_desc* d, cudaStream_t st, int8_t* out_q, float q_inv_scale)
 {
     SArgs a;
@@ -863,23 +868,23 @@ nm_status launch(nm_ctx* ctx, const nm_attn_desc* d, cudaStream_t st, int8_t* ou
     if ((s = make_map(ctx, &tmQ, d->Q, d->dtype, d, BQ)) != NM_OK) return s;
     if ((s = make_map(ctx, &tmK, d->K, d->dtype, d, CK)) != NM_OK) return s;
     if ((s = make_map(ctx, &tmV, d->V, d->dtype, d, CK)) != NM_OK) return s;
-    auto kern = attention_stream_kernel<T, CLAMP_HI, RAGGED, ONE>;
+    auto kern = attention_stream_kernel<T, CLAMP_HI, RAGGED, FORM, PER_SM>;
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
         return NM_ERR_CUDA;
     const int64_t tiles = (int64_t)d->B * d->heads * ((d->L + BQ - 1) / BQ);
     if (tiles > 0x7fffffffLL) return NM_ERR_SHAPE;
-    // persistent: one resident wave of CTAs, each walking over tiles.  Three CTAs per SM (RAGGED, ONE: two) by the launch
-    // bounds (registers) and by tensor memory (3 x 160 or 2 x 256 of 512 columns); fewer if the exp table makes the
-    // shared memory larger (233472 bytes per SM, 1 KB reserved per CTA).
-    int64_t per_sm = 233472 / (int64_t)(smem + 1024 + (ONE ? 22 * 1024 : 1536));
-    if (per_sm > (RAGGED || ONE ? 2 : 3)) per_sm = RAGGED || ONE ? 2 : 3;
+    // persistent: one resident wave of CTAs, each walking over tiles; by the launch bounds (registers), by tensor memory
+    // (3 x 160 or 2 x 256 of 512 columns) and, if the exp table makes the shared memory larger, by that (233472 bytes per SM,
+    // 1 KB reserved per CTA).
+    int64_t per_sm = 233472 / (int64_t)(smem + 1024 + (FORM == DUO_CHUNK ? 22 * 1024 : 1536));
+    if (per_sm > PER_SM) per_sm = PER_SM;
     if (per_sm < 1) per_sm = 1;
     int64_t grid = (int64_t)ctx->sm_count * per_sm;
     if (grid > tiles) grid = tiles;
     cudaLaunchConfig_t cfg;
     memset(&cfg, 0, sizeof(cfg));
     cfg.gridDim = dim3((unsigned)grid);
-    cfg.blockDim = dim3(CTA_THREADS<ONE>);
+    cfg.blockDim = dim3(CTA_THREADS<FORM>);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
@@ -890,6 +895,21 @@ nm_status launch(nm_ctx* ctx, const nm_attn_desc* d, cudaStream_t st, int8_t* ou
     NmLaunchScope scope(ctx, NM_KERNEL_ATTENTION_TC, 4.0 * (double)d->B * d->heads * (double)d->L * d->L * HD, st);
     if (cudaLaunchKernelEx(&cfg, kern, tmQ, tmK, tmV, a) != cudaSuccess) return NM_ERR_CUDA;
     return cudaGetLastError() == cudaSuccess ? NM_OK : NM_ERR_CUDA;
+}
+
+// The form for a (batch, head) of one chunk.  Two softmax warps halve the chain of one head, one warp gets more heads through an SM.  us, one
+// warp, two with two CTAs per SM, two with one (bf16, 12 heads a sequence):
+//   L 37    B 1 5.2, 5.3, 4.6   B 12 5.9, 6.1, 5.3   B 24 7.4, 7.2, 10.1   B 32 8.6, 9.8, 13.0   B 128 21.1, 24.5, 34.2
+//   L 100   B 1 6.9, 7.7, 6.4   B 12 7.6, 8.2, 6.8   B 24 9.8, 11.0, 13.1  B 32 12.6, 14.7, 17.1 B 128 35.6, 43.4, 48.4
+//   L 24    B 24 7.1, 6.2       L 64   B 16 7.4, 7.7   (two with two, up to 48 keys, as long as one round takes all heads)
+//   L 128   B 1 5.3, 5.3        B 12 5.7, 5.5        B 24 8.1, 8.0         B 32 9.5, 9.7         B 128 27.0, 28.0   (unmasked: no spills with two)
+template <typename T, bool CLAMP_HI, bool RAGGED>
+nm_status launch_one(nm_ctx* ctx, const nm_attn_desc* d, cudaStream_t st, int8_t* out_q, float q_inv_scale)
+{
+    const int64_t heads = (int64_t)d->B * d->heads;
+    if (RAGGED && heads <= ctx->sm_count) return launch<T, CLAMP_HI, RAGGED, DUO_CHUNK, RAGGED ? 1 : 2>(ctx, d, st, out_q, q_inv_scale);
+    if (heads <= 2 * ctx->sm_count && (!RAGGED || d->L <= 48)) return launch<T, CLAMP_HI, RAGGED, DUO_CHUNK, 2>(ctx, d, st, out_q, q_inv_scale);
+    return launch<T, CLAMP_HI, RAGGED, ONE_CHUNK, 2>(ctx, d, st, out_q, q_inv_scale);
 }
 
 }  // namespace
@@ -915,7 +935,7 @@ nm_status nm_launch_attention_stream(nm_ctx* ctx, const nm_attn_desc* d, cudaStr
     const bool clamp_hi = ctx->h_tables[d->exp_slot].x_max < 0.0f;
     const bool ragged = d->L % 128 != 0, one = d->L <= 128;
 #define NM_ATTN_FORM(T, CH, RG)                                                                                       \
-    (one ? launch<T, CH, RG, true>(ctx, d, st, out_q, q_inv_scale) : launch<T, CH, RG, false>(ctx, d, st, out_q, q_inv_scale))
+    (one ? launch_one<T, CH, RG>(ctx, d, st, out_q, q_inv_scale) : launch<T, CH, RG, MANY, RG ? 2 : 3>(ctx, d, st, out_q, q_inv_scale))
 #define NM_ATTN_CASE(T) (ragged ? NM_ATTN_FORM(T, true, true) : clamp_hi ? NM_ATTN_FORM(T, true, false) : NM_ATTN_FORM(T, false, false))
     if (d->dtype == NM_BF16) return NM_ATTN_CASE(__nv_bfloat16);
     return NM_ATTN_CASE(__half);

@@ -133,3 +133,22 @@ def test_probabilities_keep_their_bits(nm, ctx):
     ctx.attention_pwl(qkv, out, B, L, h, 64)
     ctx.check_device_status()
     assert (out != want).double().mean() < 4e-4
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float16])
+@pytest.mark.parametrize("L", [1, 16, 17, 33, 48, 49, 64, 100, 127, 128])
+@pytest.mark.parametrize("exp_range", [(-8.0, 0.0), (-6.0, -0.5)])
+def test_sequences_do_not_depend_on_the_batch(ctx, dtype, L, exp_range):
+    """One or two softmax warps, one or two CTAs per SM: the form follows the number of (batch, head) pairs, every bit stays."""
+    h, most = 12, 30   # 12, 144, 156, 288, 300 and 360 pairs on 148 SMs
+    load_tables_both(ctx, 64, {"exp": exp_range, "recip": (max(L / 16.0, 0.5), float(max(L, 2)))})
+    g = torch.Generator(device="cuda").manual_seed(L)
+    x = (torch.randn((most * L, 3 * 64 * h), generator=g, device="cuda") * 0.8).to(dtype)
+    outs = []
+    for B in (most, 25, 24, 13, 12, 1):
+        out = torch.full((most * L, 64 * h), float("nan"), device="cuda").to(dtype)
+        ctx.attention_pwl(x, out, B, L, h, 64)
+        ctx.check_device_status()
+        assert out[:B * L].isfinite().all() and out[B * L:].isnan().all()
+        outs.append(out[:B * L])
+    assert all(torch.equal(outs[0][:o.shape[0]], o) for o in outs)
