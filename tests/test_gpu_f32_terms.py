@@ -34,7 +34,34 @@ def test_linear_precision(ctx, M, N, K):
     assert err < 4 * 1.55e-8 + 7.4e-9 * (K / 64) ** 0.5 + 2.5e-8
 
 
-@pytest.mark.parametrize("a_exp,w_exp", [(0, 0), (-110, 0), (0, -110), (-110, 100), (40, 40), (100, -100)])
+@pytest.mark.parametrize("M,N", [(64, 256), (1024, 768)])
+@pytest.mark.parametrize("K", [16, 64, 768, 3072])
+@pytest.mark.parametrize("kind", ["normal", "positive", "uniform"])
+def test_linear_is_no_less_accurate_than_a_chain_of_fmas(nm, ctx, M, N, K, kind):
+    """Operands of one sign, too, where the truncations do not average out: test_linear_precision's bound, and the plain kernel's error
+    (measured: at most 1.2e-7 against 6e-8 at K = 16 to 1e-6 at K = 3072)."""
+    A, W = [torch.from_numpy(nm_inputs.matrix(s, K, "f32", d)).cuda() for s, d in (((M, K), 1.0), ((N, K), 0.02))]
+    if kind != "normal":
+        A, W = A.abs(), W.abs()
+    if kind == "uniform":   # the fractional part of a wide normal distribution
+        A, W = (50 * A).frac(), (2500 * W).frac()
+    ref = A.double() @ W.double().t()
+    errs = [((linear(ctx, A, W, algo).double() - ref).norm() / ref.norm()).item() for algo in (nm.ALGO_AUTO, nm.ALGO_SIMT)]
+    assert errs[0] < 4 * 1.55e-8 + 7.4e-9 * (K / 64) ** 0.5 + 2.5e-8 and errs[0] < errs[1], errs
+
+
+@pytest.mark.parametrize("e", [-126, -128, -130, -133, -136])
+def test_linear_of_subnormal_operands(ctx, e):
+    """The first term of an operand of 2^-126 2^-n has 8 - n bits, so the products that are left out are up to 2^(n - 26) of
+    the whole one, at most 2^-18; the operand itself is a multiple of 2^(n - 23) of its size."""
+    A, W = [torch.from_numpy(nm_inputs.matrix(s, 7, "f32", 1.0)).cuda() for s in ((72, 200), (68, 200))]
+    A = (A.sign().double() * (1 + A.abs().double() % 1) * 2.0 ** e).float()
+    ref = A.double() @ W.double().t()
+    for got, want in ((linear(ctx, A, W * 2.0 ** 100), ref * 2.0 ** 100), (linear(ctx, W * 2.0 ** 100, A), ref.t() * 2.0 ** 100)):
+        assert ((got.double() - want).norm() / want.norm()).item() < 1e-7 + 2.0 ** (min(-126 - e, 8) - 26)
+
+
+@pytest.mark.parametrize("a_exp,w_exp", [(0, 0), (-118, 100), (-122, 100), (100, -122), (-110, 0), (0, -110), (-110, 100), (40, 40), (100, -100)])
 def test_linear_exponents(ctx, a_exp, w_exp):
     """The terms' scaling keeps the range of fp32: the same result times a power of two."""
     A, W = [torch.from_numpy(nm_inputs.matrix(s, 7, "f32", 1.0)).cuda() for s in ((70, 200), (68, 200))]
@@ -131,6 +158,37 @@ def test_attention(nm, ctx, L, n, odd):
     with np.errstate(invalid="ignore"):
         row = np.max(np.where(f, np.abs(ref), 0.0), axis=1, keepdims=True)
     assert (np.abs(got - ref)[f] <= (2e-5 * np.maximum(scale, row))[f]).all()
+
+
+@pytest.mark.parametrize("L", [1, 16, 17, 33, 64, 65, 100, 128, 200])
+@pytest.mark.parametrize("positive", [False, True])
+@pytest.mark.parametrize("B", [4, 16])
+def test_attention_precision(nm, ctx, B, L, positive):
+    """Against float64 with the same tables.  B 4: the tensor cores up to L = 128, 0.6e-7 to 1.2e-7 measured (without the products m m', h l', l h' of P V
+    it would be 2e-6); the tiled kernel beyond and, with 192 heads, up to 64 keys: 1.0e-7 to 1.9e-7, 2.8e-7 with 200.  The plain kernel has more."""
+    h = 12
+    tabs = load_tables_both(ctx, 64, {"exp": (-8.0, 0.0), "recip": (max(L / 16.0, 0.5), float(max(L, 2)))})
+    x = torch.from_numpy(nm_inputs.matrix((B * L, 3 * h * 64), L, "f32", 0.8)).cuda()
+    if positive:
+        x[:, 2 * h * 64:].abs_()
+    q, k, v = [t.double().view(B, L, h, 64).transpose(1, 2) for t in x.split(h * 64, 1)]
+
+    def pwl(z, name, lo, hi):
+        kk, bb = [torch.from_numpy(t).cuda().double() for t in (tabs[name].k, tabs[name].b)]
+        i = ((z - lo) * (64 / (hi - lo))).floor().clamp(0, 63).long()
+        return kk[i] * z + bb[i]
+
+    s = (q @ k.transpose(-1, -2)) * 0.125
+    e = pwl(s - s.amax(-1, keepdim=True), "exp", -8.0, 0.0)
+    ref = ((e @ v) * pwl(e.sum(-1, keepdim=True), "recip", max(L / 16.0, 0.5), float(max(L, 2)))).transpose(1, 2).reshape(B * L, h * 64)
+    errs = []
+    for algo in (nm.ALGO_AUTO, nm.ALGO_SIMT):
+        out = torch.full((B * L, h * 64), float("nan"), device="cuda")
+        ctx.attention_pwl(x, out, B, L, h, 64, algo=algo)
+        ctx.check_device_status()
+        errs.append(((out.double() - ref).norm() / ref.norm()).item())
+    terms = L <= 128 and (L > 64 or B * h <= 148)
+    assert errs[0] < (1.5e-7 if terms else 2.5e-7 if L <= 128 else 3.5e-7) and errs[0] < 1.03 * errs[1], errs
 
 
 @pytest.mark.parametrize("L", [37, 128, 200])
