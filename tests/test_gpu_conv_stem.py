@@ -2,6 +2,7 @@
 import pytest
 import torch
 
+import test_gpu_cnn_paths
 from test_gpu_cnn_paths import conv_both, ctx, operands  # noqa: F401
 
 pytestmark = pytest.mark.gpu
@@ -56,3 +57,21 @@ def test_the_form_follows_the_patches(nm, ctx, N, H, Cout, patchwise):  # noqa: 
         ctx.check_device_status()
         outs.append(out)
     assert torch.equal(*outs) and outs[0].isfinite().all()
+
+
+# 136 columns; nine filter rows; outputs that leave too much of a patch empty
+@pytest.mark.parametrize("N,H,W,Cin,Cout,kh,kw,pad", [(2, 40, 24, 3, 136, 7, 7, 3), (2, 31, 30, 3, 64, 9, 7, 4), (1, 33, 20, 4, 136, 3, 3, 1),
+                                                      (128, 34, 34, 3, 64, 7, 7, 3), (200, 18, 18, 3, 128, 5, 5, 2)])
+def test_row_pairs_read_no_row_outside_the_window(nm, ctx, N, H, W, Cin, Cout, kh, kw, pad):  # noqa: F811
+    test_gpu_cnn_paths.test_first_layer_reads_no_row_outside_the_window(nm, ctx, N, H, W, Cin, Cout, kh, kw, pad)
+
+
+# 600 patches each: two channel blocks, whose weights stay in shared memory; three, whose weights pass through a ring; one to compare
+@pytest.mark.parametrize("dtype", [torch.float16, torch.bfloat16])
+@pytest.mark.parametrize("Cin", [64, 128, 192])
+@pytest.mark.parametrize("Cout,res", [(64, False), (40, True)])
+def test_halo_of_64_columns(nm, ctx, dtype, Cin, Cout, res):  # noqa: F811
+    """Few outputs, so that all products of a patch come from one issuing lane."""
+    x, w, b, g = operands(40, 48, 40, Cin, Cout, 3, 3, dtype, Cin)
+    r = torch.randn((40, 48, 40, Cout), generator=g, device="cuda").to(dtype) if res else None
+    conv_both(nm, ctx, x, w, b, 1, 1, r)
