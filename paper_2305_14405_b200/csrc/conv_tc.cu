@@ -104,7 +104,7 @@ nm_status make_tmaps_out(nm_ctx* ctx, CUtensorMap* tmO, CUtensorMap* tmR, const 
 
 // Is the halo form (linear_tc_kernel.cuh) the faster one?  3 x 3, stride 1, padding 1, at least two rounds of CTA pairs, and less
 // time by the bytes a tile takes from L2 (50 a clock) and the tensor core's cycles, although its fixed 8 x 16 patch wastes rows
-// that the free patch does not: 128 images, 56 x 56, 64 -> 64: 52 us against 77; 28 x 28, 128 -> 128: 39.2 against
+// that the free patch does not: 128 images, 56 x 56, 64 -> 64: 35 us against 77; 28 x 28, 128 -> 128: 39.2 against
 // 44.8.  Wider outputs are bound by the tensor core in either form.
 bool use_halo(const NmConvTc* c, int64_t free_patches, int sms)
 {
@@ -115,7 +115,7 @@ bool use_halo(const NmConvTc* c, int64_t free_patches, int sms)
     if (halo_patches < 2LL * 2 * sms) return false;
     const int bn = c->Cout <= 64 ? 64 : 128;
     const double b_bytes = bn / 2 * ROW_BYTES, taps = 9.0 * c->cblocks, mma = bn == 64 ? 160.0 : 256.0;
-    const double w_stream = bn == 64 && c->cblocks == 1 ? 0.0 : taps * b_bytes;
+    const double w_stream = bn == 64 && c->cblocks <= 2 ? 0.0 : taps * b_bytes;   // (up to 18 weight tiles stay in shared memory)
     const double feed_free = taps * (A_BYTES + b_bytes) / 50, feed_halo = (c->cblocks * (double)HALO_BYTES + w_stream) / 50;
     const double t_free = (double)free_patches * (feed_free > taps * mma ? feed_free : taps * mma);
     const double t_halo = (double)halo_patches * (feed_halo > taps * mma ? feed_halo : taps * mma);

@@ -11,9 +11,11 @@
 // Bound by the shared-memory port with 128 columns: per K-block of 64 k the terms' stores take 768 cycles, the products' operand reads
 // 1536, the fp32 fetch 1390 beside them; 2700 were measured.  The fetch loop must not spill (beside 200 KB of shared memory the L1 is
 // too small to hold a spilled register: 5000 cycles), hence the two chunks at a time, the one walking pointer and the tail apart.
+// (8 bytes do spill, a value written once before the loop; with 128 columns it is the partial last K-block's, without which none does.)
 // Relative errors against float64 here and with packed FMAs on the CUDA cores, which this kernel replaced: 1024 x 768 x 768
-// 9.0e-8 and 2.5e-7, x 3072 1.2e-7 and 2.5e-7, 128 x 768 x 256 8.1e-8 and 9.7e-8.  Times: 1024 x 2304 x 768 24.5 us and 84.3,
-// 1024 x 768 x 3072 42.3 and 132.0, 40 x 768 x 3072 14.2 and 24.0, 128 x 768 x 256 7.3 and 7.6.
+// 9.0e-8 and 2.5e-7, x 3072 1.2e-7 and 2.5e-7, 128 x 768 x 256 8.1e-8 and 9.7e-8; operands of one sign 8.0e-8 and 1.1e-7, 9.1e-8
+// and 6.7e-8, 8.0e-8 and 5.0e-8.  Times: 1024 x 2304 x 768 24.4 us and 84.5, 1024 x 768 x 3072 42.8 and 132.1, 40 x 768 x 3072 13.0
+// and 24.0, 128 x 768 x 256 7.4 and 7.6.
 #include "f32_terms.cuh"
 #include "linear_split_kernel.cuh"
 

@@ -1,5 +1,5 @@
-"""GPU parity, the fp32 path on the CUDA cores: linear operator (packed FMA tiles, K split over clusters) and attention
-(score block in shared memory)."""
+"""GPU parity, the fp32 path: the linear operator on the tensor cores (bf16 terms, K split over clusters) and the plain kernel, attention
+with terms and with the score block in shared memory."""
 import numpy as np
 import pytest
 import torch
