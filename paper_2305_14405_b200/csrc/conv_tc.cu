@@ -147,6 +147,9 @@ nm_status launch_halo(nm_ctx* ctx, const NmConvTc* c, NmChain chain, cudaStream_
     if (s != NM_OK) return s;
     s = make_tmaps_out(ctx, &tmO, &tmR, c, cv);
     if (s != NM_OK) return s;
+    if constexpr (FORM == HALO3X3 && BN == 64) {
+        if (a.w_resident) return launch_kernel<T, T, true, BN, true, HALO_RESIDENT>(ctx, tmA, tmW, tmO, tmR, a, smem, c->flops, st);
+    }
     return launch_kernel<T, T, true, BN, true, FORM>(ctx, tmA, tmW, tmO, tmR, a, smem, c->flops, st);
 }
 

@@ -64,7 +64,7 @@ constexpr int HALO_W = 10, HALO_H = 18;                    // input pixels of a 
 constexpr int HALO_LOAD = HALO_W * HALO_H * ROW_BYTES;     // bytes of one halo box
 constexpr int HALO_BYTES = (HALO_LOAD + 1023) / 1024 * 1024;
 constexpr int MAX_W_STAGES = 18;
-enum { NO_HALO = 0, HALO3X3 = 1, STEM = 2 };               // forms of the A operand's load
+enum { NO_HALO, HALO3X3, STEM, HALO_RESIDENT };            // forms of the A operand's load (HALO_RESIDENT: all weights in shared memory, 64 columns)
 constexpr int STEM_PITCH = (2 * 7 + 8) * 4 * 2;            // bytes of an image row of a patch
 constexpr int STEM_BYTES = ((2 * 15 + 8) * STEM_PITCH + 1023) / 1024 * 1024;
 
@@ -231,10 +231,11 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     // one's MMAs, 281 and less (128 images, 28 x 28, 128 -> 128, 3 x 3: 45.6 -> 39.2 us).  With 256 columns the tensor core
     // covers it, and all lanes, whose stage numbers and descriptors stay in uniform registers, are 1 % faster.
     constexpr bool ONE_LANE = BN < 256;
-    // The halo forms' issuer has many products between two waits; with 64 columns, where all weights stay in shared memory, all lanes
+    // The halo forms' issuer has many products between two waits; with 64 columns and all weights in shared memory all lanes
     // wait and one elected lane issues a patch's products unrolled, 45 cycles each instead of 70 (128 images: 56 x 56, 64 -> 64,
-    // 3 x 3: 50 -> 35 us, the first layer 131 -> 97; 28 x 28, 128 -> 128, with a wait per tap: 38 -> 43, so one lane there).
-    constexpr bool ONE_ISSUER = ONE_LANE && HALO != STEM && !(HALO && BN == 64);
+    // 3 x 3: 50 -> 35 us, the first layer 131 -> 97; with a wait per tap one lane is the better: 28 x 28, 128 -> 128 38 us against 43,
+    // 56 x 56, 192 -> 64 163 against 195).
+    constexpr bool ONE_ISSUER = ONE_LANE && HALO != STEM && HALO != HALO_RESIDENT;
     // Several accumulators per tile (TcArgs::acc_steps): matrices of few columns.
     constexpr bool MULTI = BN == 64 && !CONV && !TcIn<InT>::is_int;
     const uint32_t buf_cols = MULTI ? BN * (uint32_t)a.accs : BN;
@@ -478,7 +479,7 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                             }
                             __syncwarp();
                         }
-                        else if (!ONE_ISSUER && a.w_resident) {   // channel block cb's nine weight tiles lie behind one another
+                        else if constexpr (HALO == HALO_RESIDENT) {   // channel block cb's nine weight tiles lie behind one another
                             for (int i = 0; wait_w && ok && i < 9; ++i)
                                 ok = issue_vote(nm_mbar_wait(&bar_wfull[9 * cb + i], 0, abortp, a.status));
                             if (!ok) break;
