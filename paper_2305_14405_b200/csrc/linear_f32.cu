@@ -11,11 +11,11 @@
 // Bound by the shared-memory port with 128 columns: per K-block of 64 k the terms' stores take 768 cycles, the products' operand reads
 // 1536, the fp32 fetch 1390 beside them; 2700 were measured.  The fetch loop must not spill (beside 200 KB of shared memory the L1 is
 // too small to hold a spilled register: 5000 cycles), hence the two chunks at a time, the one walking pointer and the tail apart.
-// (8 bytes do spill, a value written once before the loop; with 128 columns it is the partial last K-block's, without which none does.)
+// (By -Xptxas -v 8 bytes spill with 128 columns, none with 64; with a partial last K-block, a kernel of its own, 16 and 12.)
 // Relative errors against float64 here and with packed FMAs on the CUDA cores, which this kernel replaced: 1024 x 768 x 768
 // 9.0e-8 and 2.5e-7, x 3072 1.2e-7 and 2.5e-7, 128 x 768 x 256 8.1e-8 and 9.7e-8; operands of one sign 8.0e-8 and 1.1e-7, 9.1e-8
-// and 6.7e-8, 8.0e-8 and 5.0e-8.  Times: 1024 x 2304 x 768 24.4 us and 84.5, 1024 x 768 x 3072 42.8 and 132.1, 40 x 768 x 3072 13.0
-// and 24.0, 128 x 768 x 256 7.4 and 7.6.
+// and 6.7e-8, 8.0e-8 and 5.0e-8.  Times: 1024 x 2304 x 768 23.9 us and 84.5, 1024 x 768 x 3072 42.3 and 132.1, 40 x 768 x 3072 12.4
+// and 24.0, 128 x 768 x 256 6.9 and 7.6, 200 x 768 x 16 6.4 and 5.9 (the set-up of tensor memory and barriers).
 #include "f32_terms.cuh"
 #include "linear_split_kernel.cuh"
 
@@ -45,7 +45,7 @@ template <int BN> struct F32Tile {
 // at a time, those without such a sum passed over; 4 x 4 chains per lane, the operands 16 k at a time through the warp's own CHAIN_WORDS of
 // shared memory, one buffer filling while the other is multiplied.  1024 x 768 x 3072, 48 us alone: one row of NaN or infinities 258 to 274 us,
 // nothing but NaN 521 (each such sum by its row's thread, from memory: 2240 and 28400); 37 x 768 x 3072, 16 us: 45 and 72.  The finite
-// product pays for the code with 0.5 us of 42.3 (8 x 4 chains, which need 40 more registers: with 1.3 us, and 360 and 369 us).
+// product pays for the code with up to 1 % (8 x 4 chains, which need 40 more registers: with 3 %, and 360 and 369 us).
 constexpr int CHAIN_K = 16, CHAIN_PITCH = CHAIN_K + 4, CHAIN_BUF = 64 * CHAIN_PITCH, CHAIN_WORDS = 2 * CHAIN_BUF;
 
 template <int COLS>
@@ -118,7 +118,11 @@ __device__ __forceinline__ void fma_chains(const float* A, const float* W, int64
     }
 }
 
-template <int BN>
+// TAIL: K is no multiple of a K-block.  A kernel of its own, so that the fetch loop over whole K-blocks keeps its registers: with the last
+// K-block's loads in flight together in the same kernel 1024 x 768 x 3072 took 45.9 us instead of 42.3.  us with the last K-block's loads
+// one after another behind branches, so, and with packed FMAs: 128 x 256 x 200 9.8, 7.6, 8.6; 200 x 768 x 16 8.6, 6.4, 5.9;
+// 16384 x 768 x 16 68.7, 52.3, 58.6.  Without a partial K-block 128 x 768 x 256 7.4 -> 6.9, 40 x 768 x 3072 12.8 -> 12.4.
+template <int BN, bool TAIL>
 __global__ void __launch_bounds__(F_THREADS, 1)
 linear_f32_kernel(const float* __restrict__ A, const float* __restrict__ W, int64_t lda, int64_t ldw, const SplitArgs s)
 {
@@ -189,7 +193,7 @@ linear_f32_kernel(const float* __restrict__ A, const float* __restrict__ W, int6
         const int64_t stepA = 16 * lda, stepW = 16 * ldw;
         const float* pA = A + (m0 + r0) * lda + c4 + (int64_t)kb0 * FBK;   // row 0 in the K-block that is fetched next
         const float* pW = W + (n0 + r0) * ldw + c4 + (int64_t)kb0 * FBK;
-        const int full = min(kb1, (int)(a.K / FBK));   // K-blocks that are all there end here
+        const int full = TAIL ? min(kb1, (int)(a.K / FBK)) : kb1;   // K-blocks that are all there end here
         // (one pointer walks along the rows: an address per row would be kept in registers)
         const float* pf = pW;
         uint32_t mask = kb0 < full ? exists : 0u;
@@ -225,7 +229,7 @@ linear_f32_kernel(const float* __restrict__ A, const float* __restrict__ W, int6
         for (int kb = kb0; kb < kb1; ++kb) {
             if (!nm_mbar_wait(&bar_empty[stage], phase ^ 1u, abortp, a.status)) { ok = false; break; }
             const uint32_t dst = dst0 + (uint32_t)(stage * T::STAGE_BYTES);
-            if (kb < full) {
+            if (!TAIL || kb < full) {
 #pragma unroll
                 for (int i = 0; i < T::CHUNKS; i += T::GROUP) {
                     uint2 h[T::GROUP], m[T::GROUP], l[T::GROUP];
@@ -244,24 +248,32 @@ linear_f32_kernel(const float* __restrict__ A, const float* __restrict__ W, int6
 #pragma unroll
                     for (int j = 0; j < T::GROUP; ++j) put(dst + place(i + j), i < BN / 16 ? T::B_BYTES : A_BYTES, h[j], m[j], l[j]);
                 }
-            } else {
-                // K ends in this one: zeros beyond it, and the last one to three k of a row, whose end may be the memory's, singly
+            } else if constexpr (TAIL) {
+                // K ends in this one: zeros beyond it, and the last one to three k of a row, whose end may be the memory's, singly.
+                // Predicated loads, as many in flight as the registers hold: behind branches each waits for the one before.
                 const int left = (int)a.K - (kb * FBK + c4);
-#pragma unroll 4
-                for (int i = 0; i < T::CHUNKS; ++i) {
-                    const float* p = (i < BN / 16 ? W + (n0 + r0 + 16 * i) * ldw : A + (m0 + r0 + 16 * i - BN) * lda) + (int64_t)kb * FBK + c4;
-                    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-                    if (exists & (1u << i)) {
-                        if (left >= 4) v = __ldcg(reinterpret_cast<const float4*>(p));
-                        else {
-                            if (left > 0) v.x = __ldcg(p);
-                            if (left > 1) v.y = __ldcg(p + 1);
-                            if (left > 2) v.z = __ldcg(p + 2);
-                        }
+                const uint32_t whole = left >= 4 ? exists : 0u, ends = left > 0 && left < 4 ? exists : 0u;
+#pragma unroll
+                for (int i = 0; i < T::CHUNKS; i += T::AHEAD) {
+#pragma unroll
+                    for (int j = 0; j < T::AHEAD; ++j) {
+                        if (i + j == 0) pf = pW;   // (both have come to this K-block)
+                        if (i + j == BN / 16) pf = pA;
+                        float4& v = reg[j];
+                        v = make_float4(0.f, 0.f, 0.f, 0.f);
+                        asm volatile("{\n\t.reg .pred p, x, y, z;\n\tsetp.ne.u32 p, %5, 0;\n\tsetp.ne.u32 x, %6, 0;\n\tsetp.gt.and.s32 y, %7, 1, x;\n\tsetp.gt.and.s32 z, %7, 2, x;\n\t"
+                                     "@p ld.global.cg.v4.f32 {%0, %1, %2, %3}, [%4];\n\t@x ld.global.cg.f32 %0, [%4];\n\t"
+                                     "@y ld.global.cg.f32 %1, [%4 + 4];\n\t@z ld.global.cg.f32 %2, [%4 + 8];\n\t}"
+                                     : "+f"(v.x), "+f"(v.y), "+f"(v.z), "+f"(v.w)
+                                     : "l"(pf), "r"(whole & (1u << (i + j))), "r"(ends & (1u << (i + j))), "r"(left));
+                        pf += i + j < BN / 16 ? stepW : stepA;
                     }
-                    uint2 h, m, l;
-                    nm_f32_terms4(v, h, m, l);
-                    put(dst + place(i), i < BN / 16 ? T::B_BYTES : A_BYTES, h, m, l);
+#pragma unroll
+                    for (int j = 0; j < T::AHEAD; ++j) {
+                        uint2 h, m, l;
+                        nm_f32_terms4(reg[j], h, m, l);
+                        put(dst + place(i + j), i + j < BN / 16 ? T::B_BYTES : A_BYTES, h, m, l);
+                    }
                 }
             }
             nm_fence_proxy_async();
@@ -416,16 +428,17 @@ F32Choice choose_f32(int64_t M, int64_t N, int k_blocks, const int* resident)
 template <int BN>
 nm_status launch_f32(nm_ctx* ctx, const nm_linear_desc* d, SplitArgs& s, cudaLaunchConfig_t& cfg, cudaLaunchAttribute* attr, cudaStream_t st)
 {
+    auto kern = d->K % FBK == 0 ? linear_f32_kernel<BN, false> : linear_f32_kernel<BN, true>;
     const int64_t n_tiles = (d->N + BN - 1) / BN, tiles = (d->M + BM - 1) / BM * n_tiles;
     s.t.num_n_tiles = (int)n_tiles;
     s.t.num_tiles = (int)tiles;
-    if (cudaFuncSetAttribute(linear_f32_kernel<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, F32Tile<BN>::SMEM) != cudaSuccess)
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, F32Tile<BN>::SMEM) != cudaSuccess)
         return NM_ERR_CUDA;
     cfg.dynamicSmemBytes = F32Tile<BN>::SMEM;
     cfg.numAttrs = split_launch_attrs(ctx, attr, s.S);
     cfg.gridDim = dim3((unsigned)(tiles * s.S));
     NmLaunchScope scope(ctx, NM_KERNEL_LINEAR_TC, 2.0 * (double)d->M * (double)d->N * (double)d->K, st);
-    if (cudaLaunchKernelEx(&cfg, linear_f32_kernel<BN>, (const float*)d->A, (const float*)d->W, d->lda, d->ldw, s) != cudaSuccess)
+    if (cudaLaunchKernelEx(&cfg, kern, (const float*)d->A, (const float*)d->W, d->lda, d->ldw, s) != cudaSuccess)
         return NM_ERR_CUDA;
     return cudaGetLastError() == cudaSuccess ? NM_OK : NM_ERR_CUDA;
 }
@@ -466,13 +479,13 @@ nm_status nm_launch_linear_f32(nm_ctx* ctx, const nm_linear_desc* d, cudaStream_
     int* resident = ctx->f32_resident;
     if (__atomic_load_n(&resident[0], __ATOMIC_ACQUIRE) == 0) {
         cfg.dynamicSmemBytes = F32Tile<64>::SMEM;
-        if (cudaFuncSetAttribute(linear_f32_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, F32Tile<64>::SMEM) != cudaSuccess)
+        if (cudaFuncSetAttribute(linear_f32_kernel<64, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, F32Tile<64>::SMEM) != cudaSuccess)
             return NM_ERR_CUDA;
         for (int S = 1; S <= 8; ++S) {
             int n = 0;
             cfg.numAttrs = split_launch_attrs(ctx, attr, S);
             cfg.gridDim = dim3((unsigned)(S * ctx->sm_count));
-            if (cudaOccupancyMaxActiveClusters(&n, linear_f32_kernel<64>, &cfg) != cudaSuccess) {
+            if (cudaOccupancyMaxActiveClusters(&n, linear_f32_kernel<64, false>, &cfg) != cudaSuccess) {
                 (void)cudaGetLastError();
                 n = S == 1 ? ctx->sm_count : 0;
             }

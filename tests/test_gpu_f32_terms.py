@@ -61,6 +61,23 @@ def test_linear_of_subnormal_operands(ctx, e):
         assert ((got.double() - want).norm() / want.norm()).item() < 1e-7 + 2.0 ** (min(-126 - e, 8) - 26)
 
 
+# K that ends in a K-block of 64: within a group of four, at its end, one block and several, one CTA and splits; rows and columns cut off
+@pytest.mark.parametrize("K", [1, 2, 3, 4, 5, 15, 63, 65, 66, 127, 130, 199, 1031])
+@pytest.mark.parametrize("M,N", [(1, 4), (130, 68), (2000, 1540)])
+def test_linear_partial_k_block(nm, ctx, M, N, K):
+    """What lies behind a row's end is neither added nor, behind the last row, read (the tensors end there).  Each sum's error is bounded
+    by the magnitudes of its products, since single sums, of which there may be few, can be small: four truncations of 2^-23, a chain of K / 64
+    roundings, that of the result and what is left out, 2^-24 each."""
+    kp = K + -K % 4
+    A, W = [torch.full(((r - 1) * kp + K + 1,), float("nan"), device="cuda")[:-1] for r in (M, N)]
+    a, w = [torch.as_strided(t, (r, K), (kp, 1)) for t, r in ((A, M), (W, N))]
+    a.copy_(torch.from_numpy(nm_inputs.matrix((M, K), K, "f32", 1.0)))
+    w.copy_(torch.from_numpy(nm_inputs.matrix((N, K), K + 1, "f32", 0.02)))
+    ref = a.double() @ w.double().t()
+    size = a.double().abs() @ w.double().abs().t()
+    assert ((linear(ctx, a, w).double() - ref).abs() <= (4 * 2.0 ** -23 + (K / 64 + 3) * 2.0 ** -24) * size).all()
+
+
 @pytest.mark.parametrize("a_exp,w_exp", [(0, 0), (-118, 100), (-122, 100), (100, -122), (-110, 0), (0, -110), (-110, 100), (40, 40), (100, -100)])
 def test_linear_exponents(ctx, a_exp, w_exp):
     """The terms' scaling keeps the range of fp32: the same result times a power of two."""
